@@ -10,7 +10,7 @@
 //   layer 2:  D2[128, 128-column chunk j of Cout2]   = T[slot] x W2[chunk j]^T          for every chunk j
 //             E2: + bias2, * scale2, + residual * s_res, ReLU, round, clamp -> tile buffer -> TMA store
 //
-// Warps (whole warps walk the schedules, lane 0 issues):
+// Warps (whole warps walk the schedules, an elected lane issues):
 //   0      TMA producer of layer 1 (input patches, weight ring), and of all resident weights before the kernel
 //          orders itself behind its predecessor in the stream;
 //   1      MMA issue of layer 1 (owns the TMEM allocation);
@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
   __shared__ __align__(8) unsigned long long tb_full[kFMaxTb], tb_empty[kFMaxTb];
   __shared__ __align__(8) unsigned long long buf_full[kFMaxSlots], store_ready[kFMaxSlots];
   __shared__ __align__(8) unsigned long long w1_full, w2_full, mma_turn;
-  __shared__ uint32_t tap_shift16[kMaxTaps];
   __shared__ uint32_t tmem_holder;
   __shared__ int abort_flag;
 
@@ -141,7 +140,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     else if (lane == 19) prefetch_tensormap(&tmB2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
-    if (lane0) {
+    if (elect_one()) {
       // layer-2 weights: one K-major tile of bn2 x Cout1 bytes per chunk
       const uint32_t bar2 = smem_u32(&w2_full);
       mbar_arrive_expect_tx(bar2, (uint32_t)chunks * p.l2.b_tile_bytes);
@@ -177,7 +176,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
       else if (lane == 17) prefetch_tensormap(&tmY);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (threadIdx.x >= 32 && (int)threadIdx.x - 32 < p.l1.taps) tap_shift16[threadIdx.x - 32] = p.l1.tap_shift16[threadIdx.x - 32];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     tcgen05_fence_before();
     asm volatile("bar.arrive 3, %0;" ::"r"(kFThreads) : "memory");
@@ -204,7 +202,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       const int q0 = ti.qt * q.tw - q.pad_w, p0 = ti.pt * q.th - q.pad_h;
       for (int c = 0; c < q.C_pad && ok; c += q.bk) {
         if (!mbar_wait(aempty0 + stage * 8u, phase ^ 1u, abortp)) { ok = false; break; }
-        if (lane0) {
+        if (elect_one()) {
           const uint32_t bar = afull0 + stage * 8u;
           mbar_arrive_expect_tx(bar, q.a_sub_bytes);
           tma_load_4d(a_dst, &tmA, bar, c, q0, p0, ti.img);
@@ -214,7 +212,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
         if (q.b_mode == kBRing) {
           for (int tap = 0; tap < q.taps; tap += q.b_T) {
             if (!mbar_wait(bempty0 + bs * 8u, bphase ^ 1u, abortp)) { ok = false; break; }
-            if (lane0) {
+            if (elect_one()) {
               const uint32_t bbar = bfull0 + bs * 8u;
               mbar_arrive_expect_tx(bbar, b_tx);
               tma_load_3d(b_dst, &tmB1, bbar, c, 0, tap);
@@ -234,17 +232,14 @@ __global__ void __launch_bounds__(kFThreads, 1)
     ra.a_full = smem_u32(&a_full[0]); ra.a_empty = smem_u32(&a_empty[0]);
     ra.b_full = smem_u32(&b_full[0]); ra.b_empty = smem_u32(&b_empty[0]);
     ra.acc_full = smem_u32(&acc1_full[0]); ra.acc_empty = smem_u32(&acc1_empty[0]);
-    ra.bres_full = smem_u32(&w1_full); ra.tap_shift16 = tap_shift16; ra.turn = smem_u32(&mma_turn);
-    bool ok;
-    if (p.l1.ksteps == 4) ok = mma_role<4>(p.l1, ra, 0);
-    else if (p.l1.ksteps == 2) ok = mma_role<2>(p.l1, ra, 0);
-    else ok = mma_role<1>(p.l1, ra, 0);
+    ra.bres_full = smem_u32(&w1_full); ra.turn = smem_u32(&mma_turn);
+    const bool ok = mma_role(p.l1, ra, 0);
     if (!ok && lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutMma); }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ layer-2 MMA issue: T[slot] x W2[chunk]^T
     const UmmaParams& q = p.l2;
-    const uint64_t hi = ((uint64_t)q.desc_hi << 32) | (1ull << 16);
-    const uint64_t t_d0 = hi | (((base + p.off_tb) >> 4) & 0x3fffu), w_d0 = hi | (((base + p.off_w2) >> 4) & 0x3fffu);
+    const uint32_t hi = q.desc_hi;
+    const uint32_t t_d0 = kDescLbo | (((base + p.off_tb) >> 4) & 0x3fffu), w_d0 = kDescLbo | (((base + p.off_w2) >> 4) & 0x3fffu);
     const uint32_t tb16 = p.tb_bytes >> 4, wt16 = q.b_tile_bytes >> 4;
     const uint32_t tbf0 = smem_u32(&tb_full[0]), tbe0 = smem_u32(&tb_empty[0]);
     const uint32_t a2f0 = smem_u32(&acc2_full[0]), a2e0 = smem_u32(&acc2_empty[0]);
@@ -253,22 +248,20 @@ __global__ void __launch_bounds__(kFThreads, 1)
     bool ok = mbar_wait(smem_u32(&w2_full), 0u, abortp);
     for (int k = 0; k < my_tiles && ok; ++k) {
       if (!mbar_wait(tbf0 + slot * 8u, tpar, abortp)) { ok = false; break; }
-      const uint64_t t_d = t_d0 + slot * tb16;
+      const uint32_t t_d = t_d0 + slot * tb16;
       const int jb = k == 0 ? j0 : 0, je = k == my_tiles - 1 ? j1 : chunks;  // this CTA's chunks of the tile
-      uint64_t w_d = w_d0 + (uint32_t)jb * wt16;
+      uint32_t w_d = w_d0 + (uint32_t)jb * wt16;
       for (int j = jb; j < je; ++j, w_d += wt16) {
         if (!mbar_wait(a2e0 + g * 8u, gpar, abortp)) { ok = false; break; }
         tcgen05_fence_after();
-        if (lane0) {
+        if (elect_one()) {
           const uint32_t d_tmem = tmem_base + g * (uint32_t)kFAcc2Cols;
-          if (q.ksteps == 4) umma_i8_block<4>(d_tmem, t_d, w_d, q.idesc, 0u);
-          else if (q.ksteps == 2) umma_i8_block<2>(d_tmem, t_d, w_d, q.idesc, 0u);
-          else umma_i8_block<1>(d_tmem, t_d, w_d, q.idesc, 0u);
+          umma_i8_block(d_tmem, t_d, w_d, hi, q.idesc, 0u, q.ksteps);
           umma_commit(a2f0 + g * 8u);
         }
         if (++g == (uint32_t)kFE2Groups) { g = 0; gpar ^= 1u; }
       }
-      if (lane0) umma_commit(tbe0 + slot * 8u);  // T[slot] may be overwritten once these MMAs have read it
+      if (elect_one()) umma_commit(tbe0 + slot * 8u);  // T[slot] may be overwritten once these MMAs have read it
       if (++slot == ntb) { slot = 0; tpar ^= 1u; }
     }
     if (!ok && lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutMma); }
@@ -297,7 +290,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     ItemIter ld, st;
     ld.init(h, t0, j0, my_items);
     st.init(h, t0, j0, my_items);
-    if (lane0)
+    if (elect_one())
       for (uint32_t s = 0; s < nslots && !ld.done(); ++s, ld.next(h, chunks)) load_residual(ld, s);
     else
       for (uint32_t s = 0; s < nslots && !ld.done(); ++s) ld.next(h, chunks);
@@ -306,7 +299,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     bool ok = true;
     for (; !st.done(); st.next(h, chunks)) {
       if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
-      if (lane0) {
+      if (elect_one()) {
         uint32_t src = base + q.off_bufs + slot * q.tile8_bytes;
         for (int pn = 0, c = q.c_off + st.j * q.bn; pn < q.panels; ++pn, c += pw, src += panel_bytes)
           tma_store_4d(&tmY, src, c, st.ti.qt * h.tw, st.ti.pt * h.th, st.ti.img);
@@ -318,7 +311,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       prev_slot = (int)slot;
       if (++slot == nslots) { slot = 0; spar ^= 1u; }
     }
-    if (lane0) bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
+    if (elect_one()) bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
     if (!ok && lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutStore); }
   } else if (warp < kFCtrlWarps + 4) {
     // ------------------------------------------------------------------ E1: layer-1 accumulator -> T[slot]
@@ -478,11 +471,7 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   a.R = d1.R; a.S = d1.S; a.taps = d1.R * d1.S;
   a.halo_sw = 1; a.halo_e = 0; a.c_true = d1.C;
   a.a_mode = kAHalo;
-  a.row16 = (unsigned)(d1.dil_h * ht.twb) * (unsigned)(BK1 >> 4);
-  a.col16 = (unsigned)d1.dil_w * (unsigned)(BK1 >> 4);
-  a.fast_taps = (d1.R == 3 && d1.S == 3) ? 9 : ((d1.R == 5 && d1.S == 5) ? 25 : 0);
-  for (int r = 0; r < d1.R; ++r)
-    for (int t = 0; t < d1.S; ++t) a.tap_shift16[r * d1.S + t] = (unsigned)((r * d1.dil_h * ht.twb + t * d1.dil_w) * BK1) >> 4;
+  a.in16 = (unsigned)d1.dil_w * (unsigned)(BK1 >> 4); a.out16 = (unsigned)(d1.dil_h * ht.twb) * (unsigned)(BK1 >> 4); a.tap_inner = d1.S;
   a.c_blocks = (d1.C + BK1 - 1) / BK1;
   a.C_pad = a.c_blocks * BK1;
   a.k_iters = a.taps * a.c_blocks; a.splits = 1; a.kps = a.k_iters; a.kb = 1;

@@ -51,33 +51,29 @@ namespace {
 
 // The MMA lanes of the leader CTA of a pair (halo tiles, weight ring): the same schedule as mma_role, with
 // tcgen05.mma.cta_group::2 over both CTAs' tiles and commits that arrive in both CTAs.
-template <int kSteps>
 __device__ __forceinline__ bool mma_role_pair(const UmmaParams& p, const MmaRoleArgs& r, const int who, const int vblock,
                                               const int vgrid) {
   TileIterT<true> ti;
   const int L = p.mma_lanes;
-  const bool lane0 = (threadIdx.x & 31u) == 0;
   ti.init(p, vblock + who * vgrid, L * vgrid, 0);
   const uint32_t nstages = (uint32_t)p.stages, nbst = (uint32_t)p.b_stages;
-  const uint64_t hi = ((uint64_t)p.desc_hi << 32) | (1ull << 16);
-  const uint64_t a_d0 = hi | (((r.base + p.off_a) >> 4) & 0x3fffu), bring_d0 = hi | (((r.base + p.off_bring) >> 4) & 0x3fffu);
+  const uint32_t hi = p.desc_hi;
+  const uint32_t a_d0 = kDescLbo | (((r.base + p.off_a) >> 4) & 0x3fffu), bring_d0 = kDescLbo | (((r.base + p.off_bring) >> 4) & 0x3fffu);
   const uint32_t stage16 = p.a_stage_bytes >> 4, bsub16 = p.b_sub_bytes >> 4, btile16 = p.b_tile_bytes >> 4;
   const uint32_t idesc = p.idesc;
-  const int taps = p.taps, c_blocks = p.c_blocks, bT = p.b_T;
+  const int taps = p.taps, c_blocks = p.c_blocks, bT = p.b_T, inner = p.tap_inner;
+  const bool four = p.ksteps == 4;  // K blocks of 128 bytes, else 64 (the plan pairs no narrower ones)
+  const uint32_t in16 = p.in16, out16 = p.out16;
   const uint32_t spt = (uint32_t)c_blocks, bpt = (uint32_t)(p.b_chunks * c_blocks);
   const uint32_t skip_a = (uint32_t)(L - 1) * spt, skip_b = (uint32_t)(L - 1) * bpt;
   uint32_t stage = ((uint32_t)who * spt) % nstages, phase = (((uint32_t)who * spt) / nstages) & 1u;
   uint32_t bs = ((uint32_t)who * bpt) % nbst, bphase = (((uint32_t)who * bpt) / nbst) & 1u;
-  uint64_t a_d = a_d0 + stage * stage16, bring_d = bring_d0 + bs * bsub16;
+  uint32_t a_d = a_d0 + stage * stage16, bring_d = bring_d0 + bs * bsub16;
   const uint32_t nacc = (uint32_t)p.nacc;
   uint32_t ab = (uint32_t)who % nacc, acc_par = 1u ^ (((uint32_t)who / nacc) & 1u);
   uint32_t my_k = 0;
   const uint32_t turn_next = r.turn + (uint32_t)((who + 1) % L) * 8u;
   const uint32_t turn_mine = r.turn + (uint32_t)who * 8u;
-  const bool fast9 = p.fast_taps == 9 && bT == 3;
-  uint32_t shift9[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) shift9[t] = fast9 ? r.tap_shift16[t] : 0u;
   for (; ti.tile < r.total_tiles; ti.next(p)) {
     if (!mbar_wait(r.acc_empty + ab * 8u, acc_par, r.abortp)) return false;
     if (who == 0) { if (my_k > 0 && !mbar_wait(turn_mine, (my_k - 1) & 1u, r.abortp)) return false; }
@@ -88,55 +84,37 @@ __device__ __forceinline__ bool mma_role_pair(const UmmaParams& p, const MmaRole
     for (int cb = 0; cb < c_blocks; ++cb) {
       if (!mbar_wait(r.a_full + stage * 8u, phase, r.abortp)) return false;
       const bool last_cb = cb == c_blocks - 1;
-      tcgen05_fence_after();
-      if (fast9) {
-        // 3x3 in ring stages of one filter row each: straight-line issue with the shifts in registers
-#pragma unroll
-        for (int row = 0; row < 3; ++row) {
-          if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
-          tcgen05_fence_after();
-          if (lane0) {
-            if (last_cb && row == 2) mbar_arrive(turn_next);
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-              const uint64_t ad = a_d + shift9[3 * row + t], bd = bring_d + (uint32_t)t * btile16;
-              umma_i8_pair(d_tmem, ad, bd, idesc, (row == 0 && t == 0) ? accum : 1u);
-#pragma unroll
-              for (int k = 1; k < kSteps; ++k) umma_i8_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
-            }
-            umma_commit_pair(r.b_empty + bs * 8u);
-          }
-          accum = 1;
-          bring_d += bsub16;
-          if (++bs == nbst) { bs = 0; bphase ^= 1u; bring_d = bring_d0; }
-        }
-      }
-      for (int tap0 = 0; !fast9 && tap0 < taps; tap0 += bT) {
+      uint32_t a_row = a_d, a_tap = a_d;
+      int left = inner;
+      for (int tap0 = 0; tap0 < taps; tap0 += bT) {
         if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
         tcgen05_fence_after();
         const int nt = min(bT, taps - tap0);
-        if (lane0) {
-          if (last_cb && tap0 + bT >= taps) mbar_arrive(turn_next);
-          uint64_t bd = bring_d;
-          for (int t = 0; t < nt; ++t, bd += btile16) {
-            const uint64_t ad = a_d + r.tap_shift16[tap0 + t];
-            umma_i8_pair(d_tmem, ad, bd, idesc, accum);
-#pragma unroll
-            for (int k = 1; k < kSteps; ++k) umma_i8_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
-            accum = 1;
+        if (last_cb && tap0 + bT >= taps && elect_one()) mbar_arrive(turn_next);
+        uint32_t bd = bring_d;
+        for (int t = 0; t < nt; ++t, bd += btile16) {
+          if (elect_one()) {
+            umma_i8_pair(d_tmem, a_tap, bd, hi, idesc, accum);
+            umma_i8_pair(d_tmem, a_tap + 2, bd + 2, hi, idesc, 1u);
+            if (four) {
+              umma_i8_pair(d_tmem, a_tap + 4, bd + 4, hi, idesc, 1u);
+              umma_i8_pair(d_tmem, a_tap + 6, bd + 6, hi, idesc, 1u);
+            }
           }
-          umma_commit_pair(r.b_empty + bs * 8u);
+          accum = 1;
+          a_tap += in16;
+          if (--left == 0) { left = inner; a_row += out16; a_tap = a_row; }
         }
-        accum = 1;
+        if (elect_one()) umma_commit_pair(r.b_empty + bs * 8u);
         bring_d += bsub16;
         if (++bs == nbst) { bs = 0; bphase ^= 1u; bring_d = bring_d0; }
       }
-      if (lane0) umma_commit_pair(r.a_empty + stage * 8u);
+      if (elect_one()) umma_commit_pair(r.a_empty + stage * 8u);
       a_d += stage16;
       if (++stage == nstages) { stage = 0; phase ^= 1u; a_d = a_d0; }
     }
     ++my_k;
-    if (lane0) umma_commit_pair(r.acc_full + ab * 8u);
+    if (elect_one()) umma_commit_pair(r.acc_full + ab * 8u);
     ab += (uint32_t)L;
     while (ab >= nacc) { ab -= nacc; acc_par ^= 1u; }
     stage += skip_a;
@@ -167,7 +145,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
                                                                         // lane between two uses, so no phase can be skipped
   __shared__ __align__(8) unsigned long long bres_full;
   __shared__ __align__(8) unsigned long long mma_turn[kMmaWarps];
-  __shared__ uint32_t tap_shift16[kMaxTaps];  // halo: descriptor start offset of a tap, in 16-byte units
   __shared__ uint32_t tmem_holder;
   __shared__ int abort_flag;
 
@@ -255,7 +232,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         tmem_relinquish();
       }
     }
-    if (p.a_mode == kAHalo && threadIdx.x >= 32 && threadIdx.x - 32 < p.taps) tap_shift16[threadIdx.x - 32] = p.tap_shift16[threadIdx.x - 32];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if constexpr (kCta2) {
       // bias and scale of every channel, once per CTA (zero beyond Cout; one scale replicated if per tensor)
@@ -278,7 +254,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   volatile int* abortp = &abort_flag;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ A / B producer (whole warp; lane 0 issues)
+    // ------------------------------------------------------------------ A / B producer (whole warp; an elected lane issues)
     TileIterT<kCta2> ti;
     ti.init(p, vblock, vgrid, cta_rank);
     const uint32_t nstages = (uint32_t)p.stages, nbst = (uint32_t)p.b_stages;
@@ -293,8 +269,8 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       // laid out [tap][bn rows][bk bytes], i.e. one K-major operand tile per tap
       const uint32_t bar = smem_u32(&bres_full);
       uint32_t dst = base;
-      if (!lane0) {
-        // only lane 0 issues
+      if (!elect_one()) {
+        // only an elected lane issues
       } else if (p.a_mode == kAHalo && p.halo_sw == 2) {
         mbar_arrive_expect_tx(bar, (uint32_t)(p.n_tiles * p.c_blocks * p.taps) * p.b_tile_bytes);
         // pixel-pair taps: tap t' of a filter row covers s = 2t' - e and 2t' - e + 1, whose weights are 2C
@@ -316,7 +292,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         for (int c = 0; c < p.C_pad && ok; c += p.bk) {
           if (!mbar_wait(aempty0 + stage * 8u, phase ^ 1u, abortp)) { ok = false; break; }
           const uint32_t bar = afull0 + stage * 8u;
-          if (!lane0) {
+          if (!elect_one()) {
           } else if constexpr (kCta2) {
             // the leader's barrier counts the bytes of both CTAs' patches
             if (cta_rank == 0) mbar_arrive_expect_tx(bar, 2u * p.a_sub_bytes);
@@ -333,7 +309,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
             for (int tap = 0; tap < p.taps; tap += p.b_T) {
               if (!mbar_wait(bempty0 + bs * 8u, bphase ^ 1u, abortp)) { ok = false; break; }
               const uint32_t bbar = bfull0 + bs * 8u;
-              if (!lane0) {
+              if (!elect_one()) {
               } else if constexpr (kCta2) {
                 if (cta_rank == 0) mbar_arrive_expect_tx(bbar, 2u * b_tx);
                 tma_load_3d_pair(b_dst, &tmB, map_to_cta(bbar, 0), c, n0, tap);
@@ -373,13 +349,13 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
           const int nsub = min(p.kb, p.kps - it);
           if (!mbar_wait(aempty0 + stage * 8u, phase ^ 1u, abortp)) { ok = false; break; }
           const uint32_t bar = afull0 + stage * 8u;
-          if (lane0) mbar_arrive_expect_tx(bar, (uint32_t)nsub * sub_tx);
+          if (elect_one()) mbar_arrive_expect_tx(bar, (uint32_t)nsub * sub_tx);
           uint32_t dst = a_dst, bdst = a_dst + b_in_stage;
           for (int j = 0; j < nsub; ++j) {
-            if (!lane0) {
+            if (!elect_one()) {
             } else if (p.a_mode == kAIm2col) tma_load_im2col_4d(dst, &tmA, bar, c, w0, h0, img, (unsigned short)off_w, (unsigned short)off_h);
             else tma_load_2d(dst, &tmA, bar, c, m0);
-            if (lane0 && p.b_mode == kBStage) tma_load_3d(bdst, &tmB, bar, c, tap, n0);
+            if (p.b_mode == kBStage && elect_one()) tma_load_3d(bdst, &tmB, bar, c, tap, n0);
             dst += p.a_sub_bytes;
             bdst += p.b_sub_bytes;
             c += p.bk;
@@ -399,7 +375,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       atomicOr(p.status, kTimeoutProducer);
     }
   } else if (warp == 1 || warp == 4 || (warp == 5 && p.mma_lanes == 3)) {
-    // ------------------------------------------------------------------ MMA issuers (warps 1, 4 and 5; lane 0 issues)
+    // ------------------------------------------------------------------ MMA issuers (warps 1, 4 and 5; an elected lane issues)
     const int who = warp == 1 ? 0 : warp - 3;
     MmaRoleArgs ra;
     ra.base = base; ra.tmem_base = tmem_base; ra.total_tiles = total_tiles; ra.abortp = abortp;
@@ -407,14 +383,12 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     ra.a_full = smem_u32(&a_full[0]); ra.a_empty = smem_u32(&a_empty[0]);
     ra.b_full = smem_u32(&b_full[0]); ra.b_empty = smem_u32(&b_empty[0]);
     ra.acc_full = smem_u32(&acc_full[0]); ra.acc_empty = smem_u32(&acc_empty[0]);
-    ra.bres_full = smem_u32(&bres_full); ra.tap_shift16 = tap_shift16; ra.turn = smem_u32(&mma_turn[0]);
+    ra.bres_full = smem_u32(&bres_full); ra.turn = smem_u32(&mma_turn[0]);
     bool ok = true;
     if constexpr (kCta2) {
-      if (cta_rank == 0) ok = p.ksteps == 4 ? mma_role_pair<4>(p, ra, who, vblock, vgrid) : mma_role_pair<2>(p, ra, who, vblock, vgrid);
+      if (cta_rank == 0) ok = mma_role_pair(p, ra, who, vblock, vgrid);
     } else {
-      if (p.ksteps == 4) ok = mma_role<4>(p, ra, who);
-      else if (p.ksteps == 2) ok = mma_role<2>(p, ra, who);
-      else ok = mma_role<1>(p, ra, who);
+      ok = mma_role(p, ra, who);
     }
     if (!ok && lane0) {
       abort_flag = 1;
@@ -434,7 +408,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       for (; ti.tile < total_tiles; ti.next(p)) {
         if (!mbar_wait(bempty0 + slot * 8u, par, abortp)) { ok = false; break; }
         const uint32_t bar = bfull0 + slot * 8u;
-        if (!lane0) {
+        if (!elect_one()) {
         } else if (p.res_mode == kResTma && ti.valid) {
           uint32_t dst = base + p.off_bufs + slot * p.tile8_bytes;
           mbar_arrive_expect_tx(bar, p.res_tx_bytes);
@@ -467,7 +441,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
       for (; ti.tile < total_tiles; ti.next(p)) {
         if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
-        if (!lane0) {
+        if (!elect_one()) {
         } else if (p.out8) {
           uint32_t src = base + p.off_bufs + slot * p.tile8_bytes;
           if (!ti.valid) {
@@ -487,7 +461,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         }
         if (++slot == nslots) { slot = 0; spar ^= 1u; }
       }
-      if (p.out8 && lane0) {
+      if (p.out8 && elect_one()) {
         bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
         if (prev_slot >= 0) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
       }
@@ -769,15 +743,11 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     p.S = ht.s_eff; p.taps = d.R * ht.s_eff; p.pad_w = ht.pad_w_eff;
     p.halo_sw = ht.sw; p.halo_e = ht.e;
     const int dil_w = paired ? 1 : d.dil_w;
-    p.row16 = (unsigned)(d.dil_h * ht.twb) * (unsigned)(BK >> 4);
-    p.col16 = (unsigned)dil_w * (unsigned)(BK >> 4);
-    p.fast_taps = (!paired && d.R == 3 && ht.s_eff == 3) ? 9 : ((!paired && d.R == 5 && ht.s_eff == 5) ? 25 : ((paired && d.R == 7 && ht.s_eff == 4) ? 28 : 0));
-    for (int r = 0; r < d.R; ++r)
-      for (int t = 0; t < ht.s_eff; ++t) {
-        // tap order = order of the weight tiles in shared memory: (r, s) normally, (t', r) for pixel pairs
-        const int tap = paired ? t * d.R + r : r * ht.s_eff + t;
-        p.tap_shift16[tap] = (unsigned)((r * d.dil_h * ht.twb + t * dil_w) * BK) >> 4;
-      }
+    // tap order = order of the weight tiles in shared memory: (r, s) normally, (t', r) for pixel pairs
+    const unsigned row16 = (unsigned)(d.dil_h * ht.twb) * (unsigned)(BK >> 4), col16 = (unsigned)dil_w * (unsigned)(BK >> 4);
+    p.in16 = paired ? row16 : col16;
+    p.out16 = paired ? col16 : row16;
+    p.tap_inner = paired ? d.R : ht.s_eff;
   }
   p.c_blocks = (c_eff + BK - 1) / BK;
   p.C_pad = p.c_blocks * BK;

@@ -35,19 +35,19 @@ __global__ void __launch_bounds__(128, 1) mma_rate_kernel(int bn, int chains, in
   tcgen05_fence_after();
   const uint32_t tmem_base = tmem_holder;
   if (warp == 0) {
-    const uint64_t hi = ((uint64_t)((unsigned)((8 * 128) >> 4) | (1u << 14) | (2u << 29)) << 32) | (1ull << 16);
-    const uint64_t a_d = hi | ((base >> 4) & 0x3fffu), b_d = hi | (((base + kBM * 128) >> 4) & 0x3fffu);
+    const uint32_t hi = (uint32_t)((8 * 128) >> 4) | (1u << 14) | (2u << 29);
+    const uint32_t a_d = kDescLbo | ((base >> 4) & 0x3fffu), b_d = kDescLbo | (((base + kBM * 128) >> 4) & 0x3fffu);
     const uint32_t idesc = (2u << 4) | (1u << 10) | ((unsigned)(bn >> 3) << 17) | ((unsigned)(kBM >> 4) << 24);
     const uint32_t stride = bn < 32 ? 32u : (uint32_t)bn;
     const long long t0 = clock64();
-    if (lane == 0) {
+    {
       int chain = 0;
       for (int i = 0; i < instructions; ++i) {
         const uint32_t k = (uint32_t)(i & 3) * 2u;
-        umma_i8(tmem_base + (uint32_t)chain * stride, a_d + k, b_d + k, idesc, i >= chains ? 1u : 0u);
+        if (elect_one()) umma_i8(tmem_base + (uint32_t)chain * stride, a_d + k, b_d + k, hi, idesc, i >= chains ? 1u : 0u);
         if (++chain == chains) chain = 0;
       }
-      umma_commit(smem_u32(&done_bar));
+      if (elect_one()) umma_commit(smem_u32(&done_bar));
     }
     __syncwarp();
     const bool ok = mbar_wait(smem_u32(&done_bar), 0u, &abort_flag);

@@ -24,7 +24,7 @@ constexpr int kMaxStages = 8;           // A stages
 constexpr int kMaxBStages = 8;          // weight ring
 constexpr int kMaxAcc = 4;
 constexpr int kMaxSlots = 8;            // 8-bit tile buffers over all groups
-constexpr int kMaxTaps = 64;            // halo mode keeps a descriptor offset per tap in shared memory
+constexpr int kMaxTaps = 64;            // halo mode: filter taps (one TMA box holds all taps of resident weights)
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 constexpr int kSmemLimit = 232448;                           // 227 KiB opt-in maximum per CTA
 constexpr int kStaticSmemReserve = 2048;                     // barriers, tap table and flags
@@ -62,7 +62,6 @@ struct UmmaParams {
   int k_iters, kb;           // plain/im2col: taps * c_blocks (tap, block) iterations, kb of them per A stage
   int tw, th, twb, hb;       // halo: tile and patch extents in pixels (pixel pairs along W when halo_sw == 2)
   int halo_sw, halo_e, c_true;  // halo: stride along W (1 or 2), parity of pad_w, channels per input pixel
-  unsigned int tap_shift16[kMaxTaps];  // halo: descriptor start offset of every tap, in 16-byte units
   int p_tiles, q_tiles;      // halo: tiles per image column / row
   int stages, b_stages;      // A stages, weight-ring stages
   int nacc, acc_stride, tmem_cols;  // TMEM accumulators, columns between them, allocation (power of two)
@@ -80,8 +79,10 @@ struct UmmaParams {
   int cta2;                  // 1: CTA pairs (clusters of two) issue tcgen05.mma.cta_group::2 over two m tiles that
                              // share the n tile; each CTA holds its own A patch and half of the weight tile rows
   int m_tiles_real;          // cta2: number of real m tiles (m_tiles counts pairs)
-  int fast_taps;             // halo: tap count of a filter whose issue loop is unrolled (3x3, 5x5, 7 x 4 pairs), else 0
-  unsigned int row16, col16; // halo: descriptor shift, in 16-byte units, of one filter row / one filter column
+  // halo: the taps of a filter are walked in the order of their weight tiles, `tap_inner` of them at a time; the
+  // patch descriptor moves by in16 (16-byte units) from one tap to the next and by out16 from one group to the next
+  unsigned int in16, out16;
+  int tap_inner;
   int mma_lanes;             // 3 with four accumulators (narrow tiles are bound by the issue rate of a lone lane), else 2
   int epi_split;             // 1: every epilogue group takes a share of the columns of every tile (short launches)
   int b_T, b_chunks;         // weight ring: filter taps per ring stage (one TMA operation), stages per channel block
@@ -203,10 +204,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Low word of a shared-memory matrix descriptor: (start address >> 4) | kDescLbo, the leading-byte-offset field
+// (bits 16-29), unused for swizzled K-major tiles, set to 1.
+constexpr uint32_t kDescLbo = 1u << 16;
+
+// One lane of a converged warp.  The control roles issue under this predicate and never under "lane == 0": the
+// compiler knows that an elected branch holds a single thread and keeps the operands of tcgen05.mma, of the TMA
+// copies and of their barriers in uniform registers, where a lane-number branch costs some twenty moves per
+// instruction.  With 32-bit descriptor words and rolled tap loops a kernel shrinks from 240 to 75 KB of code and the
+// issuing warps stop being the limit: 3x3 64->64 at 300x300 63.3 -> 53.5 us (batch 16), 3x3 512->512 at 7x7 18.9 ->
+// 15.1 us, 3x3 64->64 + 1x1 64->256 + residual at 56x56 38.2 -> 32.3 us (batch 64), one 14x14 layer 5.3 -> 4.4 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+  return pred != 0;
+}
+
 // Waits are warp collective: every role runs as a whole converged warp (its loop counters, addresses and
-// descriptors then are warp-uniform values, which the instructions that take uniform operands, tcgen05.mma and
-// the TMA copies, need: computed by a single diverged lane they cost a dozen extra moves per instruction),
-// all 32 lanes poll, and the votes make the outcome uniform by construction.
+// descriptors then are warp-uniform values), all 32 lanes poll, and the votes make the outcome uniform by
+// construction.
 // Slow path of a wait, out of line to keep the role loops small.  Gives up after about
 // kWaitLimitNs or when another role of this CTA has already given up; the caller then records the
 // site and leaves its loop.  The wall clock is only read once the wait has lasted a while.
@@ -335,12 +351,13 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t addr, uint32_t cols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
 }
-__device__ __forceinline__ void umma_i8_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_i8_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %4, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // arrives on the barrier at this offset in both CTAs of the pair once the MMAs issued so far have completed
@@ -350,53 +367,38 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
                : "memory");
 }
 
-// D[tmem] (+)= A[smem desc] * B[smem desc]^T, 8-bit integer inputs, int32 accumulate.  The issuing
-// lane retires about one instruction every six cycles, so the issue path is kept to the bare
-// instruction: descriptors live in 64-bit registers and the always-accumulate form has a constant
-// predicate.
-__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// D[tmem] (+)= A[smem desc] * B[smem desc]^T, 8-bit integer inputs, int32 accumulate.  Both operands' descriptors
+// share the constant high word; only low words (start address >> 4 | kDescLbo) are computed, with 32-bit additions.
+__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void umma_i8_acc(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
+__device__ __forceinline__ void umma_i8_acc(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
       "setp.eq.u32 p, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc)
       : "memory");
 }
 
-// kSteps instructions over one K block of kSteps * 32 bytes: +2 in 16-byte address units per step.
-template <int kSteps>
-__device__ __forceinline__ void umma_i8_block(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate_first) {
-  umma_i8(d_tmem, a_desc, b_desc, idesc, accumulate_first);
-#pragma unroll
-  for (int k = 1; k < kSteps; ++k) umma_i8_acc(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc);
-}
-
-// All taps of an R x S filter (kTrans: tap order (s, r) of the pixel-pair view, else (r, s)) on one channel block
-// against resident weight tiles, fully unrolled: the descriptor shift of tap (r, s) is r * row16 + s * col16.
-template <int kR, int kS, bool kTrans, int kSteps>
-__device__ __forceinline__ void issue_taps(uint32_t d_tmem, uint64_t a_d, uint32_t row16, uint32_t col16, uint64_t bres,
-                                           uint32_t btile16, uint32_t idesc, uint32_t accumulate_first) {
-  uint32_t coff[kS];
-#pragma unroll
-  for (int t = 0; t < kS; ++t) coff[t] = (uint32_t)t * col16;
-  uint64_t rowb = a_d;  // descriptor of filter row r, advanced by additions
-#pragma unroll
-  for (int r = 0; r < kR; ++r) {
-#pragma unroll
-    for (int t = 0; t < kS; ++t) {
-      const int tap = kTrans ? t * kR + r : r * kS + t;  // position of the tap's weight tile
-      umma_i8_block<kSteps>(d_tmem, rowb + coff[t], bres + (uint32_t)tap * btile16, idesc,
-                            (r == 0 && t == 0) ? accumulate_first : 1u);
+// The instructions of one K block of ksteps * 32 bytes (ksteps = 1, 2 or 4, uniform): +2 in 16-byte address units
+// per step.
+__device__ __forceinline__ void umma_i8_block(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                              uint32_t accumulate_first, int ksteps) {
+  umma_i8(d_tmem, a_lo, b_lo, hi, idesc, accumulate_first);
+  if (ksteps > 1) {
+    umma_i8_acc(d_tmem, a_lo + 2, b_lo + 2, hi, idesc);
+    if (ksteps > 2) {
+      umma_i8_acc(d_tmem, a_lo + 4, b_lo + 4, hi, idesc);
+      umma_i8_acc(d_tmem, a_lo + 6, b_lo + 6, hi, idesc);
     }
-    rowb += row16;
   }
 }
 
@@ -656,14 +658,11 @@ __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile&
 struct MmaRoleArgs {
   uint32_t base, tmem_base;
   uint32_t a_full, a_empty, b_full, b_empty, acc_full, acc_empty, bres_full, turn;
-  const uint32_t* tap_shift16;
   int first_tile, tile_step, total_tiles;  // this CTA's work items: first_tile, first_tile + tile_step, ... below total_tiles
   volatile int* abortp;
 };
 
-// The single MMA-issuing lane.  kSteps (K block bytes / 32) is a compile-time constant so that the
-// instructions of one K block are straight-line code.  Returns false if a wait gave up.
-template <int kSteps>
+// One MMA-issuing warp (an elected lane issues).  Returns false if a wait gave up.
 __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs& r, const int who) {
   // This lane's tiles are lt = who, who + kMmaWarps, ... of the CTA's sequence; the stage, weight-ring
   // and accumulator positions of a tile follow from lt alone.  A parity wait is only meaningful for
@@ -672,15 +671,11 @@ __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs&
   // and the accumulator wait run ahead of that.
   TileIterT<false> ti;
   const int L = p.mma_lanes;
-  const bool lane0 = (threadIdx.x & 31u) == 0;  // the whole warp walks the schedule, this lane issues
   ti.init(p, r.first_tile + who * r.tile_step, L * r.tile_step);
   const uint32_t nstages = (uint32_t)p.stages, nbst = (uint32_t)p.b_stages;
-  // descriptors: high word constant; low word = start address >> 4 (shared memory ends below 256 KiB,
-  // the 14-bit field never wraps) plus the leading-byte-offset field (bits 16-29), unused for swizzled
-  // K-major tiles and set to 1
-  const uint64_t hi = ((uint64_t)p.desc_hi << 32) | (1ull << 16);
-  const uint64_t a_d0 = hi | (((r.base + p.off_a) >> 4) & 0x3fffu), bring_d0 = hi | (((r.base + p.off_bring) >> 4) & 0x3fffu);
-  const uint64_t bres_d0 = hi | ((r.base >> 4) & 0x3fffu);
+  const uint32_t hi = p.desc_hi;
+  const uint32_t a_d0 = kDescLbo | (((r.base + p.off_a) >> 4) & 0x3fffu), bring_d0 = kDescLbo | (((r.base + p.off_bring) >> 4) & 0x3fffu);
+  const uint32_t bres_d0 = kDescLbo | ((r.base >> 4) & 0x3fffu);
   const uint32_t stage16 = p.a_stage_bytes >> 4, asub16 = p.a_sub_bytes >> 4, bsub16 = p.b_sub_bytes >> 4, btile16 = p.b_tile_bytes >> 4;
   const uint32_t idesc = p.idesc;
   const int taps = p.taps, c_blocks = p.c_blocks, k_iters = p.kps, kb = p.kb;  // k iterations of one work item
@@ -693,18 +688,16 @@ __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs&
   uint32_t stage = ((uint32_t)who * spt) % nstages, phase = (((uint32_t)who * spt) / nstages) & 1u;
   uint32_t bs = 0, bphase = 0;
   if (ring) { bs = ((uint32_t)who * bpt) % nbst; bphase = (((uint32_t)who * bpt) / nbst) & 1u; }
-  uint64_t a_d = a_d0 + stage * stage16;
-  uint64_t bring_d = bring_d0 + bs * bsub16;
+  uint32_t a_d = a_d0 + stage * stage16;
+  uint32_t bring_d = bring_d0 + bs * bsub16;
   const uint32_t nacc = (uint32_t)p.nacc;
   uint32_t ab = (uint32_t)who % nacc, acc_par = 1u ^ (((uint32_t)who / nacc) & 1u);  // accumulator and the parity of its empty barrier
   uint32_t my_k = 0;  // number of tiles this lane has issued
   const uint32_t turn_next = r.turn + (uint32_t)((who + 1) % L) * 8u;  // the next lane's turn barrier
   const uint32_t turn_mine = r.turn + (uint32_t)who * 8u;
   if (p.b_mode == kBResident && !mbar_wait(r.bres_full, 0u, r.abortp)) return false;
-  const int fast_taps = halo ? p.fast_taps : 0;  // 9: 3x3, 25: 5x5, 28: 7x7 as pixel pairs, else 0
-  uint32_t shift9[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) shift9[t] = fast_taps == 9 ? r.tap_shift16[t] : 0u;
+  const uint32_t in16 = p.in16, out16 = p.out16;
+  const int inner = p.tap_inner, ksteps = p.ksteps;
   for (; ti.tile < r.total_tiles; ti.next(p)) {
     if (!mbar_wait(r.acc_empty + ab * 8u, acc_par, r.abortp)) return false;
     // turn[w] counts the tiles the other lane has finished waiting for: tile number k of lane 0 needs
@@ -715,101 +708,60 @@ __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs&
     const uint32_t d_tmem = r.tmem_base + ab * (uint32_t)p.acc_stride;
     uint32_t accum = 0;
     // resident weights: tile (nt, cb, tap) sits at ((nt * c_blocks + cb) * taps + tap) * b_tile_bytes
-    const uint64_t bres_nt = bres_d0 + (uint32_t)(ti.nt * c_blocks * taps) * btile16;
+    const uint32_t bres_nt = bres_d0 + (uint32_t)(ti.nt * c_blocks * taps) * btile16;
     if (halo) {
-      uint64_t bres = bres_nt;  // (cb, tap) is exactly the order of the loops below
+      uint32_t bres = bres_nt;  // (cb, tap) is exactly the order of the loops below
       for (int cb = 0; cb < c_blocks; ++cb) {
         if (!mbar_wait(r.a_full + stage * 8u, phase, r.abortp)) return false;
         const bool last_cb = cb == c_blocks - 1;
-        if (last_cb && !ring && lane0) mbar_arrive(turn_next);  // this tile's last wait is behind us
+        if (last_cb && !ring && elect_one()) mbar_arrive(turn_next);  // this tile's last wait is behind us
         tcgen05_fence_after();
-        if (ring && bT == 1) {
-          // (kept apart from the multi-tap loop below: every extra instruction of this lone lane costs ~6 cycles)
-          for (int tap = 0; tap < taps; ++tap) {
-            if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
-            tcgen05_fence_after();
-            if (lane0) {
-              if (last_cb && tap == taps - 1) mbar_arrive(turn_next);
-              umma_i8_block<kSteps>(d_tmem, a_d + r.tap_shift16[tap], bring_d, idesc, accum);
-              umma_commit(r.b_empty + bs * 8u);
-            }
-            accum = 1;
-            bring_d += bsub16;
-            if (++bs == nbst) { bs = 0; bphase ^= 1u; bring_d = bring_d0; }
-          }
-        } else if (ring && fast_taps == 9 && bT == 3) {
-          // 3x3 in ring stages of one filter row each: straight-line issue with the shifts in registers
-#pragma unroll
-          for (int row = 0; row < 3; ++row) {
-            if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
-            tcgen05_fence_after();
-            if (lane0) {
-              if (last_cb && row == 2) mbar_arrive(turn_next);
-#pragma unroll
-              for (int t = 0; t < 3; ++t)
-                umma_i8_block<kSteps>(d_tmem, a_d + shift9[3 * row + t], bring_d + (uint32_t)t * btile16, idesc, (row == 0 && t == 0) ? accum : 1u);
-              umma_commit(r.b_empty + bs * 8u);
-            }
-            accum = 1;
-            bring_d += bsub16;
-            if (++bs == nbst) { bs = 0; bphase ^= 1u; bring_d = bring_d0; }
-          }
-        } else if (ring) {
+        uint32_t a_row = a_d, a_tap = a_d;  // descriptor of the filter row's first tap, of this tap
+        int left = inner;
+        if (ring) {
           for (int tap0 = 0; tap0 < taps; tap0 += bT) {
             if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
             tcgen05_fence_after();
             const int nt = min(bT, taps - tap0);
-            if (lane0) {
-              if (last_cb && tap0 + bT >= taps) mbar_arrive(turn_next);
-              uint64_t bd = bring_d;
-              for (int t = 0; t < nt; ++t, bd += btile16) {
-                umma_i8_block<kSteps>(d_tmem, a_d + r.tap_shift16[tap0 + t], bd, idesc, accum);
-                accum = 1;
-              }
-              umma_commit(r.b_empty + bs * 8u);
+            if (last_cb && tap0 + bT >= taps && elect_one()) mbar_arrive(turn_next);
+            uint32_t bd = bring_d;
+            for (int t = 0; t < nt; ++t, bd += btile16) {
+              if (elect_one()) umma_i8_block(d_tmem, a_tap, bd, hi, idesc, accum, ksteps);
+              accum = 1;
+              a_tap += in16;
+              if (--left == 0) { left = inner; a_row += out16; a_tap = a_row; }
             }
-            accum = 1;
+            if (elect_one()) umma_commit(r.b_empty + bs * 8u);
             bring_d += bsub16;
             if (++bs == nbst) { bs = 0; bphase ^= 1u; bring_d = bring_d0; }
           }
-        } else if (fast_taps == 9) {
-          // common filters: tap shifts in registers, straight-line issue (this lane pays ~6 cycles per
-          // instruction, more per branch, and a shared-memory load per tap otherwise)
-          // 3x3: the nine shifts live in registers (measured faster than forming them by additions)
-          if (lane0) {
-#pragma unroll
-            for (int tap = 0; tap < 9; ++tap)
-              umma_i8_block<kSteps>(d_tmem, a_d + shift9[tap], bres + (uint32_t)tap * btile16, idesc, tap == 0 ? accum : 1u);
-          }
-          accum = 1;
-          bres += 9u * btile16;
-        } else if (fast_taps == 25) {
-          if (lane0) issue_taps<5, 5, false, kSteps>(d_tmem, a_d, p.row16, p.col16, bres, btile16, idesc, accum);
-          accum = 1;
-          bres += 25u * btile16;
-        } else if (fast_taps == 28) {
-          if (lane0) issue_taps<7, 4, true, kSteps>(d_tmem, a_d, p.row16, p.col16, bres, btile16, idesc, accum);
-          accum = 1;
-          bres += 28u * btile16;
         } else {
-          if (lane0) {
-            uint64_t bt = bres;
-#pragma unroll 3
-            for (int tap = 0; tap < taps; ++tap) {
-              umma_i8_block<kSteps>(d_tmem, a_d + r.tap_shift16[tap], bt, idesc, accum);
-              accum = 1;
-              bt += btile16;
+          if (elect_one()) {
+            uint32_t bt = bres;
+            for (int t0 = 0; t0 < taps; t0 += inner, a_row += out16) {
+              uint32_t at = a_row;
+              if (ksteps == 1) {  // (the run-time step count costs the one-instruction block a tenth of its rate)
+                for (int t = 0; t < inner; ++t, at += in16, bt += btile16) {
+                  umma_i8(d_tmem, at, bt, hi, idesc, accum);
+                  accum = 1;
+                }
+              } else {
+                for (int t = 0; t < inner; ++t, at += in16, bt += btile16) {
+                  umma_i8_block(d_tmem, at, bt, hi, idesc, accum, ksteps);
+                  accum = 1;
+                }
+              }
             }
           }
           accum = 1;
           bres += (uint32_t)taps * btile16;
         }
-        if (lane0) umma_commit(r.a_empty + stage * 8u);
+        if (elect_one()) umma_commit(r.a_empty + stage * 8u);
         a_d += stage16;
         if (++stage == nstages) { stage = 0; phase ^= 1u; a_d = a_d0; }
       }
     } else {
-      uint64_t bres_tap = bres_nt, bres = bres_nt;  // iterations run over taps with the channel blocks innermost
+      uint32_t bres_tap = bres_nt, bres = bres_nt;  // iterations run over taps with the channel blocks innermost
       int cb = 0;
       if (p.splits > 1) {
         const int it0 = ti.sp * k_iters, tap0 = p.fd_cblocks.div(it0);
@@ -821,25 +773,32 @@ __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs&
       for (int it = 0; it < k_iters;) {
         const int nsub = min(kb, k_iters - it);
         if (!mbar_wait(r.a_full + stage * 8u, phase, r.abortp)) return false;
-        if (it + nsub >= k_iters && lane0) mbar_arrive(turn_next);  // this tile's last wait is behind us
+        if (it + nsub >= k_iters && elect_one()) mbar_arrive(turn_next);  // this tile's last wait is behind us
         tcgen05_fence_after();
-        uint64_t sa = a_d, sb = a_d + b_off16;
-        for (int j = 0; j < nsub; ++j) {
-          if (lane0) umma_i8_block<kSteps>(d_tmem, sa, b_in_stage ? sb : bres, idesc, accum);
-          accum = 1;
-          sa += asub16;
-          sb += bsub16;
-          bres += (uint32_t)taps * btile16;
-          if (++cb == c_blocks) { cb = 0; bres_tap += btile16; bres = bres_tap; }
+        uint32_t sa = a_d, sb = a_d + b_off16;
+        if (b_in_stage) {
+          if (elect_one())
+            for (int j = 0; j < nsub; ++j, sa += asub16, sb += bsub16) {
+              umma_i8_block(d_tmem, sa, sb, hi, idesc, accum, ksteps);
+              accum = 1;
+            }
+        } else {
+          for (int j = 0; j < nsub; ++j, sa += asub16) {
+            if (elect_one()) umma_i8_block(d_tmem, sa, bres, hi, idesc, accum, ksteps);
+            accum = 1;
+            bres += (uint32_t)taps * btile16;
+            if (++cb == c_blocks) { cb = 0; bres_tap += btile16; bres = bres_tap; }
+          }
         }
-        if (lane0) umma_commit(r.a_empty + stage * 8u);
+        accum = 1;
+        if (elect_one()) umma_commit(r.a_empty + stage * 8u);
         it += nsub;
         a_d += stage16;
         if (++stage == nstages) { stage = 0; phase ^= 1u; a_d = a_d0; }
       }
     }
     ++my_k;
-    if (lane0) umma_commit(r.acc_full + ab * 8u);
+    if (elect_one()) umma_commit(r.acc_full + ab * 8u);
     ab += (uint32_t)L;
     while (ab >= nacc) { ab -= nacc; acc_par ^= 1u; }
     // step over the stages and ring tiles of the other lanes' tiles
