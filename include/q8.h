@@ -41,7 +41,7 @@ typedef enum q8_dtype { Q8_U8 = 0, Q8_S8 = 1, Q8_S32 = 2, Q8_F32 = 3 } q8_dtype;
 
 /* Which convolution kernel to use. */
 typedef enum q8_conv_algo {
-  Q8_ALGO_AUTO = 0,   /* tensor-core kernel when the shape allows it, else direct */
+  Q8_ALGO_AUTO = 0,   /* TMA-fed tensor-core kernel when the shape allows it, else the gathering one or direct */
   Q8_ALGO_UMMA = 1,   /* tcgen05 implicit GEMM; Q8_ERR_UNSUPPORTED if not eligible */
   Q8_ALGO_DIRECT = 2  /* CUDA-core direct convolution, any shape */
 } q8_conv_algo;
@@ -173,8 +173,8 @@ typedef struct q8_conv_desc {
  * Host only. */
 int q8_conv2d_workspace_bytes(const q8_conv_desc* d, size_t* bytes);
 
-/* Which kernel q8_conv2d would pick for `d`: writes Q8_ALGO_UMMA or
- * Q8_ALGO_DIRECT.  Host only. */
+/* Whether q8_conv2d would take the TMA-fed kernel for `d`: writes Q8_ALGO_UMMA if so, else Q8_ALGO_DIRECT.
+ * Host only. */
 int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo);
 
 /* x: device NHWC (x_type).  w: device KRSC s8.  bias: device s32[K] or NULL.
@@ -184,7 +184,8 @@ int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo);
  * slower for the shapes that would split).  Contents undefined afterwards.
  * Alignment: the tensor-core kernel needs x, w, y, residual 16-byte aligned, C
  * a multiple of 16, and for u8/s8 output y_ldc and y_c_offset multiples of 16;
- * Q8_ALGO_AUTO falls back to the direct kernel otherwise.
+ * Q8_ALGO_AUTO otherwise runs a tensor-core kernel that gathers its operands
+ * byte by byte (K up to 4096), or the direct kernel for the smallest calls.
  * Errors: Q8_ERR_INVALID_ARG (null/extent/enum, R*S*C > 65793 which could
  * overflow int32), Q8_ERR_UNSUPPORTED (Q8_ALGO_UMMA on an ineligible shape),
  * Q8_ERR_WORKSPACE, Q8_ERR_CUDA.  Nothing is launched on error. */

@@ -175,6 +175,11 @@ int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32
   }
   if (!ok) {
     if (d->algo == Q8_ALGO_UMMA) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
+    // Few outputs with a short reduction finish before the gathering kernel has set up its pipeline (1x1 of 5 -> 8
+    // channels at 8x8: 2.6 against 3.5 us; 20 -> 16 at 32x32: 3.3 against 3.9; 5 -> 32 on 8 x 28x28: 4.1 both).  From 27
+    // products or 100 000 outputs on they take longer (3x3 of 3 -> 8 on 2 x 17x19: 4.9 against 3.8 us).
+    const bool tiny = (long long)d->R * d->S * d->C <= 24 && a.M * d->K <= 100000;
+    if (d->K <= 4096 && !tiny) return launch_conv_gather(a);
     return launch_conv_direct(a);
   }
   return launch_conv_umma(a);
