@@ -78,6 +78,7 @@ class QuantNetwork:
         self.info = {"input": (q8.Q8_S8, self._factor("input"))}
         self.bufs["input"] = torch.empty(self.shape["input"], dtype=torch.int8, device=device)
         ws_bytes = 0
+        w_maxima = self._weight_maxima(folded, per_channel, device)
         for L in layers:
             t_in, q_in = self.info[L.src[0]]
             n, h, w_, c = self.shape[L.src[0]]
@@ -100,7 +101,7 @@ class QuantNetwork:
                 elif self.shape[L.name][3] != sp.K:
                     ldc = self.shape[L.name][3]  # padded with zero channels
                 qc = pipeline.prepare_conv(wf.contiguous(), bf, (n, h, w_, c), q_in, q_y, t_in, y_type, sp.relu, sp.stride,
-                                           sp.pad, sp.dil, q_res, res_type, ldc, off, per_channel=per_channel)
+                                           sp.pad, sp.dil, q_res, res_type, ldc, off, per_channel=per_channel, w_maxabs=w_maxima[L.name])
                 self.convs[L.name] = qc
                 self.info[L.name] = (y_type, qc.q_y)
                 ws_bytes = max(ws_bytes, q8.q8_conv2d_workspace_bytes(qc.desc))
@@ -140,6 +141,24 @@ class QuantNetwork:
                 self.outputs[L.name] = self.bufs[L.name][..., :L.conv.K]
         for first in self.fused_with:   # the tensor between two layers of one launch is never written
             self.outputs.pop(first, None)
+        self._capture(device)
+
+    def _weight_maxima(self, folded, per_channel, device):
+        """max|w| of every convolution (a list per output channel with per_channel), read back in one copy."""
+        convs = [L for L in self.layers if L.op == "conv"]
+        sizes = [L.conv.K if per_channel else 1 for L in convs]
+        slots = torch.zeros(sum(sizes), dtype=torch.float32, device=device)
+        for L, part in zip(convs, slots.split(sizes)):
+            w = folded[L.name][0].contiguous()
+            if per_channel:
+                q8.q8_calibrate_maxabs_rows(w, part)
+            else:
+                q8.q8_calibrate_maxabs(w, part)
+        host, out, at = slots.cpu().tolist(), {}, 0
+        for L, n in zip(convs, sizes):
+            out[L.name] = host[at:at + n] if per_channel else host[at]
+            at += n
+        return out
 
     # ---- host bookkeeping ---------------------------------------------------------------------------
     def _shapes(self, in_shape):
@@ -325,8 +344,33 @@ class QuantNetwork:
         self.run_quantized()
         return self.outputs
 
+    def _capture(self, device):
+        """Records the layers once as a CUDA graph over the network's own buffers.  Called layer by layer from Python a
+        forward costs the host 10 to 25 us per layer, more than the GPU spends on it: Inception-v3 at batch 64 took
+        2.98 ms against 1.4 ms of kernels, ResNet-50 at batch 1 1.25 ms against 0.35 ms.  The graph holds no caller
+        pointer (the input quantization, which reads the caller's images, stays outside) and no allocation."""
+        with torch.cuda.device(device):
+            side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                # relaxed: kernels may be loaded on first use while they are recorded, other threads are unaffected
+                graph.capture_begin(capture_error_mode="relaxed")
+                try:
+                    self._run_layers()
+                finally:
+                    graph.capture_end()
+            torch.cuda.current_stream().wait_stream(side)
+        self.graph = graph
+
     def run_quantized(self):
-        """Everything after the input quantization (the part a CUDA graph replays)."""
+        """Everything after the input quantization, on the current stream.  Inside a caller's own capture the layers are
+        enqueued one by one and become part of the caller's graph."""
+        if torch.cuda.is_current_stream_capturing():
+            self._run_layers()
+        else:
+            self.graph.replay()
+
+    def _run_layers(self):
         if self.n_streams == 1:
             for L in self.layers:
                 self._launch(L, self.workspaces[0])

@@ -54,12 +54,14 @@ class QuantConv:
 
 def prepare_conv(w, b, in_shape, q_x, q_y, x_type=q8.Q8_U8, y_type=q8.Q8_U8, relu=True, stride=(1, 1), pad=(0, 0),
                  dil=(1, 1), q_res=None, res_type=q8.Q8_U8, y_ldc=0, y_c_offset=0, algo=q8.Q8_ALGO_AUTO,
-                 per_channel=False) -> QuantConv:
+                 per_channel=False, w_maxabs=None) -> QuantConv:
     """w: folded FP32 weights KRSC on the device, b: folded FP32 bias [K] or None.
 
     q_y is the output factor; for y_type F32 the layer dequantizes (q_y is taken as 1).
     per_channel: one weight factor per output channel (max|w[k]| / 127) instead of the paper's one per tensor;
     the bias and the requantisation multiplier then carry the factor of their channel.
+    w_maxabs: max|w| on the host (a list of K values with per_channel) where the caller has it, as a network does that
+    reads the maxima of all its layers back in one copy; else it is computed and read back here.
     """
     N, H, W, Cin = in_shape
     K, R, S, C2 = w.shape
@@ -68,16 +70,16 @@ def prepare_conv(w, b, in_shape, q_x, q_y, x_type=q8.Q8_U8, y_type=q8.Q8_U8, rel
         q_y = 1.0
     b_q = None
     if per_channel:
-        slots = torch.zeros(K, dtype=torch.float32, device=w.device)
-        q8.q8_calibrate_maxabs_rows(w, slots)
-        q_w = [q8.q8_factor(m, 7) for m in slots.cpu().tolist()]
+        if w_maxabs is None:
+            w_maxabs = q8.q8_calibrate_maxabs_rows(w, torch.zeros(K, dtype=torch.float32, device=w.device)).cpu().tolist()
+        q_w = [q8.q8_factor(m, 7) for m in w_maxabs]
         w_q = q8.q8_quantize_rows(w, torch.tensor(q_w, dtype=torch.float32, device=w.device), q8.Q8_S8)
         if b is not None:
             q_b = torch.tensor([q8.q8_bias_factor(q_x, qk) for qk in q_w], dtype=torch.float32, device=w.device)
             b_q = q8.q8_quantize_rows(b.reshape(K, 1).contiguous(), q_b, q8.Q8_S32).reshape(K)
         scale = torch.tensor([q8.q8_requant_scale(q_x, qk, q_y) for qk in q_w], dtype=torch.float32, device=w.device)
     else:
-        q_w = q8.q8_factor(tensor_maxabs(w), 7)
+        q_w = q8.q8_factor(tensor_maxabs(w) if w_maxabs is None else w_maxabs, 7)
         w_q = q8.q8_quantize(w, q_w, q8.Q8_S8)
         if b is not None:
             b_q = q8.q8_quantize(b, q8.q8_bias_factor(q_x, q_w), q8.Q8_S32)
