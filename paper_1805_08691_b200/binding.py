@@ -95,8 +95,15 @@ def _check(rc):
         raise Q8Error(rc, lib.q8_last_error().decode())
 
 
+_raw_stream, _get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle of torch.cuda.current_stream() without the Stream object around it (5 us against 0.2 us a call,
+    # more than the rest of a call's marshalling)
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_get_device())
 
 
 def _dev(t, what):
@@ -104,7 +111,7 @@ def _dev(t, what):
         return None
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
         raise TypeError(f"{what}: expected a contiguous CUDA tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def q8_version():
