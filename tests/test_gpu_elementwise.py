@@ -202,3 +202,24 @@ def test_global_average_pool(q8, H, W, C, dt):
     x = g.integers(lo, hi, (3, H, W, C)).astype(dt)
     got = q8.q8_avgpool2d(_cuda(x), (H, W), (1, 1), (0, 0), False).cpu().numpy()
     assert np.array_equal(got, o.pool(x, "avg", (H, W), (1, 1), (0, 0), False))
+
+
+@pytest.mark.parametrize("q", [1.0, 0.0196078, 3.0e-9, 2.0 ** -59, 2.0 ** -61, 1e-40, 2.0 ** 99, 3e36])
+def test_quantize_neighbours_of_ties(q8, q):
+    """Quotients one to three units in the last place around every rounding boundary of the 8-bit range, zeros, denormals,
+    non-finite values: the reciprocal-based quotient (factors 2^-60 to 2^100) and the division (others) must both give
+    the IEEE quotient's code.  Sizes leave a remainder below four and a last block that is not full."""
+    q = float(np.float32(q))
+    with np.errstate(all="ignore"):
+        h = ((np.arange(-300, 301) + 0.5) * np.float64(q)).astype(np.float32)
+        near = [h]
+        for up in (np.float32(np.inf), np.float32(-np.inf)):
+            v = h
+            for _ in range(3):
+                v = np.nextafter(v, up)
+                near.append(v)
+        extra = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-45, -1e-40, 3.4e38, -3.4e38], dtype=np.float32)
+        x = np.concatenate(near + [extra])
+    for t, ot in ((0, o.U8), (1, o.S8)):
+        got = q8.q8_quantize(torch.from_numpy(x).cuda(), q, t).cpu().numpy()
+        assert np.array_equal(got, o.quantize(x, q, ot)), (q, t)
