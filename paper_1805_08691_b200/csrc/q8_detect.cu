@@ -161,6 +161,26 @@ __device__ __forceinline__ float exp_fixed(float x) {
   return __fmul_rn(p, __int_as_float(((int)k + 127) << 23));
 }
 
+// The same for x <= 0 (or NaN), in fewer instructions: the upper clamp cannot apply; adding 1.5 * 2^23 rounds x log2 e to
+// the nearest integer, ties to even, and leaves that integer in the low mantissa bits, from where it shifts into the
+// exponent of the scale.  Identical results.
+__device__ __forceinline__ float exp_fixed_neg(float x) {
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(x) : "f"(x), "f"(-87.0f));
+  const float t = __fadd_rn(__fmul_rn(x, 1.44269504088896341f), 12582912.0f);
+  const float k = __fsub_rn(t, 12582912.0f);
+  float r = __fmaf_rn(-k, 0.693145751953125f, x);
+  r = __fmaf_rn(-k, 1.42860682030941723e-6f, r);
+  float p = 1.0f / 5040.0f;
+  p = __fmaf_rn(p, r, 1.0f / 720.0f);
+  p = __fmaf_rn(p, r, 1.0f / 120.0f);
+  p = __fmaf_rn(p, r, 1.0f / 24.0f);
+  p = __fmaf_rn(p, r, 1.0f / 6.0f);
+  p = __fmaf_rn(p, r, 0.5f);
+  p = __fmaf_rn(p, r, 1.0f);
+  p = __fmaf_rn(p, r, 1.0f);
+  return __fmul_rn(p, __int_as_float((__float_as_int(t) << 23) + 0x3f800000));
+}
+
 constexpr int kMaxSources = 8;
 constexpr int kRegClasses = 24;   // class counts up to this keep a box's logits in registers
 struct DetSources {
@@ -205,11 +225,29 @@ __global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __gri
   const bool in_regs = classes <= kRegClasses;
   if (in_regs) {
     float* st = stage[threadIdx.x >> 5];
+    const float* x0 = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), 0));
+    if (__all_sync(0xffffffffu, x == x0 + lane * classes)) {  // the warp's boxes lie one after the other
+      float t[kRegClasses];
+#pragma unroll
+      for (int c = 0; c < kRegClasses; ++c)
+        if (c < classes) t[c] = __ldg(x0 + c * 32 + lane);
+#pragma unroll
+      for (int c = 0; c < kRegClasses; ++c)
+        if (c < classes) st[c * 32 + lane] = t[c];
+    } else {
     const unsigned int inv = 65536u / (unsigned)classes + 1u;  // k / classes for k < 32 * 24
-    for (int k0 = 0; k0 < 32 * classes; k0 += 32) {
-      const int k = k0 + lane, box = (int)(((unsigned)k * inv) >> 16);
-      const float* xb = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), box));
-      st[k] = __ldg(xb + (k - box * classes));
+    for (int c0 = 0; c0 < classes; c0 += 8) {  // eight loads in flight
+      float t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = (c0 + u) * 32 + lane, box = min((int)(((unsigned)k * inv) >> 16), 31);
+        const float* xb = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), box));
+        if (c0 + u < classes) t[u] = __ldg(xb + (k - box * classes));
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (c0 + u < classes) st[(c0 + u) * 32 + lane] = t[u];
+    }
     }
   }
   const float4 pr = __ldg(priors + q);
@@ -221,17 +259,16 @@ __global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __gri
   if (live) boxes[(size_t)n * P + p] = make_float4(__fsub_rn(cx, hw), __fsub_rn(cy, hh), __fadd_rn(cx, hw), __fadd_rn(cy, hh));
   float* pr_out = prob + (size_t)n * classes * P + p;
   unsigned int* mk = masks + (size_t)n * classes * PW + (p >> 5);
-  auto emit = [&](int c, float e, float sum, float floor_e) {
-    if (c == background) return;
-    bool cand = live && !(e < floor_e);
-    float v = 0.0f;
+  // the candidate bits of class c
+  auto emit = [&](int c, float e, float sum, float floor_e) -> unsigned int {
+    bool cand = live && !(e < floor_e) && c != background;
+    if (!__any_sync(0xffffffffu, cand)) return 0u;
     if (cand) {
-      v = __fdiv_rn(e, sum);
+      const float v = __fdiv_rn(e, sum);
       cand = v > conf_thresh;
+      if (cand) pr_out[(size_t)c * P] = v;
     }
-    const unsigned int bits = __ballot_sync(0xffffffffu, cand);
-    if (cand) pr_out[(size_t)c * P] = v;
-    if (lane == 0) mk[(size_t)c * PW] = bits;
+    return __ballot_sync(0xffffffffu, cand);
   };
   if (in_regs) {
     __syncwarp();
@@ -246,20 +283,28 @@ __global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __gri
 #pragma unroll
     for (int c = 0; c < kRegClasses; ++c)
       if (c < classes) {
-        e[c] = exp_fixed(__fsub_rn(e[c], m));
+        e[c] = exp_fixed_neg(__fsub_rn(e[c], m));
         sum = __fadd_rn(sum, e[c]);
       }
     const float floor_e = 0.99f * conf_thresh * sum;
+    unsigned int word = 0;  // lane c keeps the bits of class c
 #pragma unroll
     for (int c = 0; c < kRegClasses; ++c)
-      if (c < classes) emit(c, e[c], sum, floor_e);
+      if (c < classes) {
+        const unsigned int bits = emit(c, e[c], sum, floor_e);
+        if (lane == c) word = bits;
+      }
+    if (lane < classes) mk[(size_t)lane * PW] = word;
   } else {
     float m = x[0];
     for (int c = 1; c < classes; ++c) m = x[c] > m ? x[c] : m;
     float sum = 0.0f;
-    for (int c = 0; c < classes; ++c) sum = __fadd_rn(sum, exp_fixed(__fsub_rn(x[c], m)));
+    for (int c = 0; c < classes; ++c) sum = __fadd_rn(sum, exp_fixed_neg(__fsub_rn(x[c], m)));
     const float floor_e = 0.99f * conf_thresh * sum;
-    for (int c = 0; c < classes; ++c) emit(c, exp_fixed(__fsub_rn(x[c], m)), sum, floor_e);
+    for (int c = 0; c < classes; ++c) {
+      const unsigned int bits = emit(c, exp_fixed_neg(__fsub_rn(x[c], m)), sum, floor_e);
+      if (lane == 0) mk[(size_t)c * PW] = bits;
+    }
   }
 }
 
@@ -307,8 +352,10 @@ constexpr int kSelCap = 2048;        // keys handed to the per-class sort
 __device__ int select_bin(const int* hist, int need, int* below) {
   const int lane = threadIdx.x & 31;
   constexpr int kPer = kSelBins / 32;
-  int local = 0;
-  for (int j = 0; j < kPer; ++j) local += hist[lane * kPer + j];
+  static_assert(kPer == 64, "two bins per lane below");
+  int local = 0;  // lane l owns bins 64 l .. 64 l + 63; each starts at another one, so that the banks differ
+#pragma unroll 16
+  for (int j = 0; j < kPer; ++j) local += hist[lane * kPer + ((j + lane) & (kPer - 1))];
   int incl = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -317,19 +364,21 @@ __device__ int select_bin(const int* hist, int need, int* below) {
   }
   const unsigned int reached = __ballot_sync(0xffffffffu, incl >= need);
   const int src = reached ? __ffs(reached) - 1 : 31;
-  int bin = 0, bel = 0;
-  if (lane == src) {
-    int cum = incl - local, j = 0;
-    for (; j < kPer - 1; ++j) {
-      const int h = hist[lane * kPer + j];
-      if (cum + h >= need) break;
-      cum += h;
-    }
-    bin = lane * kPer + j;
-    bel = cum;
+  const int before = __shfl_sync(0xffffffffu, incl - local, src);
+  // the 64 bins of that lane, two per lane
+  const int h0 = hist[src * kPer + 2 * lane], h1 = hist[src * kPer + 2 * lane + 1];
+  int sum2 = h0 + h1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, sum2, o);
+    if (lane >= o) sum2 += v;
   }
-  *below = __shfl_sync(0xffffffffu, bel, src);
-  return __shfl_sync(0xffffffffu, bin, src);
+  const unsigned int r2 = __ballot_sync(0xffffffffu, before + sum2 >= need);
+  const int s2 = r2 ? __ffs(r2) - 1 : 31;
+  const int base = before + sum2 - h0 - h1;
+  const bool first = base + h0 >= need;
+  *below = __shfl_sync(0xffffffffu, first ? base : base + h0, s2);
+  return src * kPer + 2 * s2 + (__shfl_sync(0xffffffffu, first ? 1 : 0, s2) ? 0 : 1);
 }
 
 __device__ __forceinline__ unsigned long long nms_key(float s, int p) {
@@ -795,7 +844,7 @@ int q8_detection_output(int n_sources, const float* const* loc, const int* loc_s
   {
     // room for every kept key and, where that is smaller, for the selection that is sorted (a power of two)
     const int most = fg * nms_top_k;
-    int cap = 1, sort_cap = 512;
+    int cap = 1, sort_cap = 1024;
     while (cap < most) cap <<= 1;
     while (sort_cap < 2 * (keep_top_k < most ? keep_top_k : most)) sort_cap <<= 1;
     if (sort_cap >= cap) sort_cap = cap;
