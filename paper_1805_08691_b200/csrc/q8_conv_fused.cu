@@ -61,7 +61,7 @@ struct ItemIter {
   }
 };
 
-template <int kOut1, int kOut2>
+template <int kOut1, int kOut2, bool kUniform>
 __global__ void __launch_bounds__(kFThreads, 1)
     conv_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
                       const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmRes,
@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     EpiTile t;
     t.s_bias = s_bias1;
     t.s_scale = s_scale1;
+    t.scale = s_scale1[0];
     const int pp = row / q.twb, qq = row - pp * q.twb;  // accumulator row -> pixel of the patch grid
     t.smem_ok = pp < q.th && qq < q.tw;
     t.srow = t.smem_ok ? pp * q.tw + qq : 0;
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       tcgen05_fence_after();
       t.buf = base_ptr + p.off_tb + (size_t)slot * p.tb_bytes;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)p.acc1_col + ab * (uint32_t)q.acc_stride;
-      epilogue_row<kOut1, kResTma, false>(q, t, taddr, acce0 + ab * 8u, lane, 0, nchunk);
+      epilogue_row<kOut1, kResTma, false, kUniform>(q, t, taddr, acce0 + ab * 8u, lane, 0, nchunk);
       fence_proxy_async_smem();  // the tile is read by the tensor core (async proxy)
       mbar_arrive(tbf0 + slot * 8u);
       if (++ab == nacc) { ab = 0; apar ^= 1u; }
@@ -354,6 +355,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     EpiTile t;
     t.s_bias = s_bias2;
     t.s_scale = s_scale2;
+    t.scale = s_scale2[0];
     t.srow = row;                               // T rows are the tile's pixels in dense order
     t.smem_ok = row < p.l1.th * p.l1.tw;
     epi_row_setup(q, t);
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       tcgen05_fence_after();
       t.n0 = j * q.bn;
       t.buf = base_ptr + q.off_bufs + (size_t)slot * q.tile8_bytes;
-      epilogue_row<kOut2, kResTma, false>(q, t, taddr, acce, lane, 0, nchunk);
+      epilogue_row<kOut2, kResTma, false, kUniform>(q, t, taddr, acce, lane, 0, nchunk);
       fence_proxy_async_smem();
       mbar_arrive(ready0 + slot * 8u);
       apar ^= 1u;
@@ -396,10 +398,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
   }
 }
 
-template <int kOut1, int kOut2>
+template <int kOut1, int kOut2, bool kUniform>
 int launch_fused_variant(const CUtensorMap& tmA, const CUtensorMap& tmB1, const CUtensorMap& tmB2, const CUtensorMap& tmRes,
                          const CUtensorMap& tmY, const FusedParams& p, size_t dyn, int grid, cudaStream_t stream) {
-  auto kernel = conv_fused_kernel<kOut1, kOut2>;
+  auto kernel = conv_fused_kernel<kOut1, kOut2, kUniform>;
   static std::atomic<bool> configured[kMaxDevices];
   const int dev = current_device();
   if (dev < 0 || !configured[dev].load(std::memory_order_acquire)) {
@@ -659,12 +661,20 @@ int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void
 
   const long long items = (long long)p.l1.m_tiles * p.l2.n_tiles;
   const int grid = (int)(items < sm_count() ? items : sm_count());
+  // one multiplier per tensor in both layers, or per-channel arrays (a lone one is staged once per channel)
+  const bool uniform = d1.scale_count == 1 && d2.scale_count == 1;
+#define Q8_FUSED(OUT1, OUT2)                                                                                           \
+  do {                                                                                                                 \
+    if (uniform) return launch_fused_variant<OUT1, OUT2, true>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);  \
+    return launch_fused_variant<OUT1, OUT2, false>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);              \
+  } while (0)
   if (d1.y_type == Q8_U8) {
-    if (d2.y_type == Q8_U8) return launch_fused_variant<Q8_U8, Q8_U8>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);
-    return launch_fused_variant<Q8_U8, Q8_S8>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);
+    if (d2.y_type == Q8_U8) Q8_FUSED(Q8_U8, Q8_U8);
+    Q8_FUSED(Q8_U8, Q8_S8);
   }
-  if (d2.y_type == Q8_U8) return launch_fused_variant<Q8_S8, Q8_U8>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);
-  return launch_fused_variant<Q8_S8, Q8_S8>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);
+  if (d2.y_type == Q8_U8) Q8_FUSED(Q8_S8, Q8_U8);
+  Q8_FUSED(Q8_S8, Q8_S8);
+#undef Q8_FUSED
 }
 
 }  // namespace q8

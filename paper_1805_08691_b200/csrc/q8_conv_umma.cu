@@ -131,7 +131,7 @@ __device__ __forceinline__ bool mma_role_pair(const UmmaParams& p, const MmaRole
 // G epilogue groups; one instantiation per output type and residual source keeps a single epilogue
 // body in each kernel (several of them in one kernel made the register allocator spill).
 // kCta2: the CTA-pair variant (its cta_group::2 instructions make the kernel launchable as clusters of two only).
-template <int G, int kOut, int kRes, bool kCta2>
+template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
 __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     conv_umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmRes, const __grid_constant__ CUtensorMap tmY,
@@ -478,6 +478,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     EpiTile t;
     t.s_bias = s_bias;
     t.s_scale = s_scale;
+    t.scale = s_scale[0];
     // halo tiles: accumulator row -> pixel (pp, qq) of the patch grid; rows right of the tile are dropped
     int pp = 0, qq = 0;
     t.srow = row;
@@ -529,7 +530,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       }
       t.buf = p.nbuf > 0 ? base_ptr + p.off_bufs + (size_t)slot * p.tile8_bytes : nullptr;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * (uint32_t)p.acc_stride;
-      epilogue_row<kOut, kRes, kCta2>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1);
+      epilogue_row<kOut, kRes, kCta2, kUniform>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1);
       if (p.nbuf > 0) {
         // this thread's reads and writes of the buffer are done; the store thread takes over
         if (p.out8) fence_proxy_async_smem();
@@ -554,10 +555,10 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------ host
-template <int G, int kOut, int kRes, bool kCta2>
+template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
 int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmRes, const CUtensorMap& tmY,
                    const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
-  auto kernel = conv_umma_kernel<G, kOut, kRes, kCta2>;
+  auto kernel = conv_umma_kernel<G, kOut, kRes, kCta2, kUniform>;
   static std::atomic<bool> configured[kMaxDevices];  // per instantiation and device (the attribute is per device)
   const int dev = current_device();
   if (dev < 0 || !configured[dev].load(std::memory_order_acquire)) {
@@ -603,7 +604,11 @@ int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtenso
 template <int G>
 int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmRes, const CUtensorMap& tmY,
                   const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
-#define Q8_LAUNCH(OUT, RES) return launch_variant<G, OUT, RES, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream)
+#define Q8_LAUNCH(OUT, RES)                                                                                       \
+  do {                                                                                                            \
+    if (p.scale_count == 1) return launch_variant<G, OUT, RES, false, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream); \
+    return launch_variant<G, OUT, RES, false, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream);                 \
+  } while (0)
   // kResTma stands for "a residual through the tile buffers, or none"
   const bool global_res = p.res_mode == kResGlobal;
   if (p.y_type == Q8_U8) {
@@ -618,7 +623,7 @@ int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensor
     if (global_res) Q8_LAUNCH(Q8_F32, kResGlobal);
     Q8_LAUNCH(Q8_F32, kResTma);
   }
-  Q8_LAUNCH(Q8_S32, kResTma);
+  return launch_variant<G, Q8_S32, kResTma, false, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream);
 #undef Q8_LAUNCH
 }
 
@@ -1034,18 +1039,22 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   if (p.cta2) {
     // planned only for 8-bit outputs, residual by TMA or none.  These are the large 3x3 layers, which seldom
     // take a residual: their kernels keep that choice at compile time.
+#define Q8_PAIR_LAUNCH(GG, OUT, RES)                                                                                      \
+  do {                                                                                                                   \
+    if (p.scale_count == 1) return launch_variant<GG, OUT, RES, true, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream); \
+    return launch_variant<GG, OUT, RES, true, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);                      \
+  } while (0)
 #define Q8_PAIR(GG)                                                                                                      \
   do {                                                                                                                   \
-    if (d.y_type == Q8_U8) {                                                                                             \
-      if (res_mode == kResTma) return launch_variant<GG, Q8_U8, kResTma, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream); \
-      return launch_variant<GG, Q8_U8, kResNone, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);                    \
-    }                                                                                                                    \
-    if (res_mode == kResTma) return launch_variant<GG, Q8_S8, kResTma, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream); \
-    return launch_variant<GG, Q8_S8, kResNone, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);                      \
+    if (d.y_type == Q8_U8 && res_mode == kResTma) Q8_PAIR_LAUNCH(GG, Q8_U8, kResTma);                                    \
+    if (d.y_type == Q8_U8) Q8_PAIR_LAUNCH(GG, Q8_U8, kResNone);                                                          \
+    if (res_mode == kResTma) Q8_PAIR_LAUNCH(GG, Q8_S8, kResTma);                                                         \
+    Q8_PAIR_LAUNCH(GG, Q8_S8, kResNone);                                                                                 \
   } while (0)
     if (G == 2) Q8_PAIR(2);
     Q8_PAIR(4);
 #undef Q8_PAIR
+#undef Q8_PAIR_LAUNCH
   }
   if (G == 2) return launch_groups<2>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);
   return launch_groups<4>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);
