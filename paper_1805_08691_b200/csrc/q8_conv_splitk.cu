@@ -26,7 +26,10 @@ struct ReduceParams {
 
 // One thread per four consecutive channels of one pixel (K % 4 == 0): 16-byte loads of the partial sums.
 template <int kVec>
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(const ReduceParams p) {
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constant__ ReduceParams p) {
+  // set-up overlaps the kernel that writes the partial sums; the next one may do the same with this
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int kg = p.K / kVec;
   const long long total = p.M * kg;
   const long long nthreads = (long long)gridDim.x * blockDim.x;
@@ -85,8 +88,18 @@ int launch_splitk_reduce(const ConvArgs& a, int splits) {
   const long long items = a.M * (vec ? a.d.K / 4 : a.d.K);
   long long blocks = (items + 255) / 256;
   if (blocks > 148ll * 8) blocks = 148ll * 8;
-  if (vec) splitk_reduce_kernel<4><<<(int)blocks, 256, 0, a.stream>>>(p);
-  else splitk_reduce_kernel<1><<<(int)blocks, 256, 0, a.stream>>>(p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = a.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const int rc = check_cuda(vec ? cudaLaunchKernelEx(&cfg, splitk_reduce_kernel<4>, p) : cudaLaunchKernelEx(&cfg, splitk_reduce_kernel<1>, p),
+                            "splitk_reduce_kernel");
+  if (rc != Q8_OK) return rc;
   return check_launch("splitk_reduce_kernel");
 }
 

@@ -672,6 +672,22 @@ int umma_plan_splits(const q8_conv_desc& d, int P, int Q, long long M) {
 }
 
 namespace {
+// Tile width of a launch whose tiles of the default width would leave SMs without work: the narrowest of 16, 32, 64 and
+// 128 columns that still gives every tile an SM of its own, else the default.  Such a launch lasts as long as one CTA
+// takes to stream its operands, and a narrower tile streams fewer weights (1x1 1024->256 on one 14x14 image: two 256-wide
+// tiles 11.9 us even with the reduction split, 32 tiles of 16 columns 4.6 us; 3x3 512->512 on one 7x7 image 10.1 -> 7.6).
+// Short reductions gain less than the extra CTAs cost: up to 256 products stay as they are (1x1 256->1024 at 14x14 4.27
+// against 4.64 us), up to 512 take half of the SMs at most (512->2048 at 7x7 4.7 against 5.2 us with all).
+int narrow_bn(int bn, int K, int kgemm, long long m_tiles) {
+  if (kgemm <= 256) return bn;
+  const long long most = kgemm <= 512 ? sm_count() / 2 : sm_count();
+  for (int w = 16; w < bn && w <= 128; w *= 2)
+    if (m_tiles * ((K + w - 1) / w) <= most) return w;
+  return bn;
+}
+}  // namespace
+
+namespace {
 constexpr int kPlanNoFit = -1000;  // internal: this tile shape needs more shared memory than an SM has
 int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_halo);
 
@@ -689,7 +705,16 @@ int launch_conv_umma_impl(const ConvArgs& a, int splits) {
 
 int launch_conv_umma(const ConvArgs& a) {
   const q8_conv_desc& d = a.d;
-  const int splits = umma_plan_splits(d, a.P, a.Q, a.M);
+  int splits = umma_plan_splits(d, a.P, a.Q, a.M);
+  if (splits > 1) {
+    // Narrow tiles against a split of the default ones, by the operand bytes a CTA streams (~60 per cycle); a split
+    // pays ~6000 cycles for its second kernel.
+    const int bn = pick_bn(d.K, d.R * d.S * d.C), kg = d.R * d.S * d.C;
+    const long long m_tiles = (a.M + kBM - 1) / kBM;
+    const double t_split = (double)kg / splits * (kBM + bn) / 60.0 + 6000.0;
+    const double t_narrow = (double)kg * (kBM + narrow_bn(bn, d.K, kg, m_tiles)) / 60.0;
+    if (t_narrow <= t_split) splits = 1;
+  }
   const size_t need = splits > 1 ? (size_t)splits * (size_t)a.M * d.K * sizeof(int) : 0;
   if (splits > 1 && d.y_type != Q8_S32 && a.workspace && a.workspace_bytes >= need && aligned16(a.workspace)) {
     // pass 1: raw partial accumulators of every split into the workspace; pass 2: sum, bias, epilogue
@@ -728,11 +753,12 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   const int BK = pick_bk(c_eff) < bk_cap ? pick_bk(c_eff) : bk_cap;
   int BN = pick_bn(d.K, d.R * d.S * d.C);
   {
-    // Few output tiles (small images with many channels): 128-wide tiles run the tensor pipe at the same rate
-    // per column as 256-wide ones, and twice as many CTAs get work.
+    // Few output tiles (small images, small batches): narrower ones, so that more CTAs get work.
     const long long m_tiles = p.a_mode == kAHalo ? (long long)d.N * ((a.P + ht.th - 1) / ht.th) * ((a.Q + ht.tw - 1) / ht.tw)
                                                  : (a.M + kBM - 1) / kBM;
-    if (splits == 1 && BN == 256 && d.K % 256 == 0 && m_tiles * (d.K / 256) * 2 <= sm_count()) BN = 128;
+    // (only where the tiles of the default width do not outnumber half of the SMs, and not for pixel pairs, whose plan
+    // keeps the weights of the default tiles resident)
+    if (splits == 1 && !paired && m_tiles * ((d.K + BN - 1) / BN) * 2 <= sm_count()) BN = narrow_bn(BN, d.K, d.R * d.S * d.C, m_tiles);
   }
   {
     const int want = tune_env("Q8_BN", BN, 16, 256);
@@ -816,7 +842,9 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   // Weights stay resident when the whole layer's B operand is small: no per-tile weight traffic at all.
   // A tile of bn*bk bytes keeps every tap tile aligned to the swizzle pattern.
   const unsigned b_all = (unsigned)(p.n_tiles * p.c_blocks * p.taps) * p.b_tile_bytes;
-  const int can_reside = (b_all <= 80u * 1024u && p.taps <= 256 && p.b_tile_bytes % (8u * BK) == 0) ? 1 : 0;
+  // A launch of one item per CTA needs one tile of columns only, not the weights of all of them.
+  const long long n_items = (long long)p.m_tiles * p.n_tiles * splits;
+  const int can_reside = (b_all <= 80u * 1024u && (paired || p.n_tiles == 1 || n_items > sm_count()) && p.taps <= 256 && p.b_tile_bytes % (8u * BK) == 0) ? 1 : 0;
   const bool resident = tune_env("Q8_BRES", can_reside, 0, can_reside) != 0;
   p.b_mode = resident ? kBResident : (p.a_mode == kAHalo ? kBRing : kBStage);
   const unsigned bres_bytes = resident ? round_up(b_all, 1024u) : 0u;
