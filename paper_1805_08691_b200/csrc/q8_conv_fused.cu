@@ -128,7 +128,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
       s_bias2[i] = (p.l2.bias && i < p.l2.K) ? p.l2.bias[i] : 0;
       s_scale2[i] = p.l2.scale_count == 1 ? p.l2.scale[0] : (i < p.l2.K ? p.l2.scale[i] : 0.f);
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("bar.sync 3, %0;" ::"r"(kFThreads) : "memory");
     tcgen05_fence_after();
   } else if (warp == 0) {
@@ -155,7 +154,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
       }
     }
     __syncwarp();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("bar.arrive 1, %0;" ::"r"(kFCtrlWarps * 32) : "memory");
     asm volatile("bar.arrive 3, %0;" ::"r"(kFThreads) : "memory");
   } else {
@@ -176,7 +174,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
       else if (lane == 17) prefetch_tensormap(&tmY);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     tcgen05_fence_before();
     asm volatile("bar.arrive 3, %0;" ::"r"(kFThreads) : "memory");
     asm volatile("bar.sync 1, %0;" ::"r"(kFCtrlWarps * 32) : "memory");
@@ -198,6 +195,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
     uint32_t bs = 0, bphase = 0, b_dst = bring0;
     const uint32_t b_tx = (uint32_t)q.b_T * q.b_tile_bytes;
     bool ok = true;
+    // activations from here on: this warp and the residual's wait for the previous kernel, the others follow their loads
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int k = 0; k < my_tiles && ok; ++k, ti.next(q)) {
       const int q0 = ti.qt * q.tw - q.pad_w, p0 = ti.pt * q.th - q.pad_h;
       for (int c = 0; c < q.C_pad && ok; c += q.bk) {
@@ -290,6 +289,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     ItemIter ld, st;
     ld.init(h, t0, j0, my_items);
     st.init(h, t0, j0, my_items);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (elect_one())
       for (uint32_t s = 0; s < nslots && !ld.done(); ++s, ld.next(h, chunks)) load_residual(ld, s);
     else

@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     else if (lane == 18) prefetch_tensormap(&tmB);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // everything the previous kernel wrote is visible from here
     if constexpr (kCta2) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
       cluster_sync_all();  // the peer's barriers exist before anything signals them
       asm volatile("bar.arrive 1, %0;" ::"r"(nthreads) : "memory");
     } else {
@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         tmem_relinquish();
       }
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     if constexpr (kCta2) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
       // bias and scale of every channel, once per CTA (zero beyond Cout; one scale replicated if per tensor)
       for (int i = threadIdx.x - 32; i < p.k_pad; i += nthreads - 32) {
         s_bias[i] = (p.bias && i < p.K) ? p.bias[i] : 0;
@@ -264,6 +264,10 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     uint32_t stage = 0, phase = 0, a_dst = a0;
     uint32_t bs = 0, bphase = 0, b_dst = bring0;
     bool ok = true;
+    // Everything the previous kernel wrote is visible from here.  The roles wait for it themselves, as late as they
+    // touch global memory, so that their set-up runs while that kernel drains; the MMA warps and the store warp only
+    // ever follow loads of this warp and need no wait of their own.
+    if constexpr (!kCta2) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.b_mode == kBResident) {
       // every weight tile of the layer, once: one load per (n tile, channel block) brings all taps,
       // laid out [tap][bn rows][bk bytes], i.e. one K-major operand tile per tap
@@ -405,6 +409,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       bool ok = true;
       const int pw = 1 << p.pw_shift;
       const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
+      if constexpr (!kCta2) asm volatile("griddepcontrol.wait;" ::: "memory");
       for (; ti.tile < total_tiles; ti.next(p)) {
         if (!mbar_wait(bempty0 + slot * 8u, par, abortp)) { ok = false; break; }
         const uint32_t bar = bfull0 + slot * 8u;
