@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   const int vblock = kCta2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int vgrid = kCta2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const int total_tiles = p.m_tiles * p.n_tiles * p.splits;  // work items
-  const int slots = p.epi_split ? p.nbuf : G * p.nbuf;  // split mode: nbuf counts the buffers of the CTA
+  // pair kernels (G = 4): 1 << pair_shift groups share the columns of a tile, G >> pair_shift teams take alternate ones
+  const int slots = kCta2 ? (G >> p.pair_shift) * p.nbuf : (p.epi_split ? p.nbuf : G * p.nbuf);  // split mode: nbuf counts the buffers of the CTA
 
   // Programmatic dependent launch: the next kernel of the stream may be scheduled onto SMs as they fall idle
   // (it waits below, like this one, before it touches global memory), and this kernel's own set-up (barriers,
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   } else {
     if (warp == 1) {
       // one arrival per epilogue warp that reads the accumulator: a group's four, or all of them in split mode
-      if (lane < p.nacc) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), (p.epi_split ? 4 * G : 4) * (kCta2 ? 2 : 1)); }
+      if (lane < p.nacc) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), kCta2 ? 8 << p.pair_shift : (p.epi_split ? 4 * G : 4)); }
       else if (lane >= 8 && lane - 8 < kMmaWarps) mbar_init(smem_u32(&mma_turn[lane - 8]), 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (warp == 2) {
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       else if (lane == 16 && p.res_mode == kResTma) prefetch_tensormap(&tmRes);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (warp == 3) {
-      if (lane < slots) mbar_init(smem_u32(&store_ready[lane]), p.epi_split ? G * kGroupThreads : kGroupThreads);
+      if (lane < slots) mbar_init(smem_u32(&store_ready[lane]), kCta2 ? kGroupThreads << p.pair_shift : (p.epi_split ? G * kGroupThreads : kGroupThreads));
       else if (lane == 16 && p.out8) prefetch_tensormap(&tmY);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       const uint32_t nslots = (uint32_t)slots;
       uint32_t slot = 0, spar = 0;  // tile lt uses buffer lt % (G*nbuf); its use number (lt / (G*nbuf)) gives the parity
       int prev_slot = -1;
-      const bool one_each = !p.epi_split && p.nbuf == 1;
+      const bool one_each = (kCta2 || !p.epi_split) && p.nbuf == 1;
       bool ok = true;
       const int pw = 1 << p.pw_shift;
       const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
@@ -513,13 +514,19 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     // split mode: every group works on every tile and takes the chunks [ch0, ch1) of its columns, so that a
     // launch with one or two tiles per CTA does not leave three of four groups idle
     const bool split = p.epi_split != 0;
-    const int tile_step = split ? 1 : G;
+    const int team = kCta2 ? g >> p.pair_shift : (split ? 0 : g);
+    const int tile_step = kCta2 ? G >> p.pair_shift : (split ? 1 : G);
     const int nchunk_all = p.bn >> 4;
-    const int ch0 = split ? (g * nchunk_all) / G : 0, ch1 = split ? ((g + 1) * nchunk_all) / G : nchunk_all;
-    uint32_t ab = split ? 0u : (uint32_t)g % nacc, acc_par = split ? 0u : ((uint32_t)g / nacc) & 1u;
-    uint32_t slot = split ? 0u : (uint32_t)g, slot_par = 0;
+    int ch0 = split ? (g * nchunk_all) / G : 0, ch1 = split ? ((g + 1) * nchunk_all) / G : nchunk_all;
+    if constexpr (kCta2) {
+      const int member = g - (team << p.pair_shift);
+      ch0 = (member * nchunk_all) >> p.pair_shift;
+      ch1 = ((member + 1) * nchunk_all) >> p.pair_shift;
+    }
+    uint32_t ab = (uint32_t)team % nacc, acc_par = ((uint32_t)team / nacc) & 1u;
+    uint32_t slot = (uint32_t)team, slot_par = 0;
     TileIterT<kCta2> ti;
-    ti.init(p, vblock + (split ? 0 : g) * vgrid, tile_step * vgrid, cta_rank);
+    ti.init(p, vblock + team * vgrid, tile_step * vgrid, cta_rank);
     for (; ti.tile < total_tiles; ti.next(p)) {
       bool ok = mbar_wait(accf0 + ab * 8u, acc_par, abortp);
       if (p.nbuf > 0 && ok) ok = mbar_wait(bfull0 + slot * 8u, slot_par, abortp);
@@ -885,10 +892,13 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
       {
         const long long items = (long long)p.m_tiles * p.n_tiles, clusters = sm_count() / 2;
         const long long per = (items + (items < clusters ? items : clusters) - 1) / (items < clusters ? items : clusters);
-        p.epi_split = tune_env("Q8_SPLIT", per <= 2 ? 1 : 0, 0, 1);
-        G = tune_env("Q8_G", (BN > 128 && !p.epi_split) ? 2 : 4, 2, 4);
-        if (G == 3) G = 4;
-        if (G > p.nacc && !p.epi_split) G = 2;
+        // Teams: a launch of at most two items per pair has one team of all groups.  Tiles above 128 columns leave two
+        // accumulators, hence two teams, and with two groups each an accumulator is back in half the time (3x3 128->192
+        // at 73x73, batch 64: 62.3 -> 55.4 us).  Four teams for narrower tiles (128->128 at 150x150 as teams of two:
+        // 74 -> 108 us, what a tile costs a group beside its columns is paid twice).
+        p.pair_shift = per <= 2 ? 2 : (BN > 128 ? 1 : 0);
+        p.epi_split = p.pair_shift == 2;
+        G = 4;
       }
       p.b_tile_bytes = (unsigned)((BN / 2) * BK);   // this CTA's half of the weight rows
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
@@ -908,7 +918,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
       // Weight ring stages of several filter taps, one TMA operation each (the copy engine spends ~600 cycles
       // per operation whatever its size): as many taps as fit in about 48 KiB while two such stages fit beside
       // two activation stages and one tile buffer per epilogue group, spread evenly over a channel block.
-      const unsigned fixed = bres_bytes + (use_bufs ? (unsigned)(p.epi_split ? 2 : G) * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
+      const unsigned fixed = bres_bytes + (use_bufs ? (unsigned)(p.epi_split ? 2 : (p.cta2 ? G >> p.pair_shift : G)) * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
       const unsigned avail = budget > fixed ? budget - fixed : 0u;
       int T = (int)(48u * 1024u / p.b_tile_bytes);
       if (T > (int)(avail / (2u * p.b_tile_bytes))) T = (int)(avail / (2u * p.b_tile_bytes));
@@ -933,12 +943,13 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   }
   p.nbuf = 0;
   if (use_bufs) {
-    // two buffers per group when that still leaves a comfortable pipeline
-    p.nbuf = (budget >= bres_bytes + 2u * G * p.tile8_bytes + 2u * min_pipe && 2 * G <= kMaxSlots) ? 2 : 1;
+    // two buffers per group (team) when that still leaves a comfortable pipeline
+    const unsigned teams = p.cta2 ? (unsigned)(G >> p.pair_shift) : (unsigned)G;
+    p.nbuf = (budget >= bres_bytes + 2u * teams * p.tile8_bytes + 2u * min_pipe && 2 * teams <= (unsigned)kMaxSlots) ? 2 : 1;
     p.nbuf = tune_env("Q8_NBUF", p.nbuf, 1, p.nbuf);
     if (p.epi_split) p.nbuf = 2;  // one buffer per tile in flight; a CTA has at most two tiles
   }
-  const unsigned buf_bytes = (unsigned)(p.epi_split ? p.nbuf : G * p.nbuf) * p.tile8_bytes;
+  const unsigned buf_bytes = (unsigned)(p.epi_split ? p.nbuf : (p.cta2 ? G >> p.pair_shift : G) * p.nbuf) * p.tile8_bytes;
   if (budget < bres_bytes + buf_bytes + min_pipe) return kPlanNoFit;
   unsigned rest = budget - bres_bytes - buf_bytes;
   p.b_stages = 0;
@@ -1092,7 +1103,6 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     if (res_mode == kResTma) Q8_PAIR_LAUNCH(GG, Q8_S8, kResTma);                                                         \
     Q8_PAIR_LAUNCH(GG, Q8_S8, kResNone);                                                                                 \
   } while (0)
-    if (G == 2) Q8_PAIR(2);
     Q8_PAIR(4);
 #undef Q8_PAIR
 #undef Q8_PAIR_LAUNCH

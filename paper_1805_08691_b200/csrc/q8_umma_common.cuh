@@ -84,6 +84,7 @@ struct UmmaParams {
   unsigned int in16, out16;
   int tap_inner;
   int mma_lanes;             // 3 with four accumulators (narrow tiles are bound by the issue rate of a lone lane), else 2
+  int pair_shift;            // cta2: log2 of the epilogue groups that share the columns of a tile
   int epi_split;             // 1: every epilogue group takes a share of the columns of every tile (short launches)
   int b_T, b_chunks;         // weight ring: filter taps per ring stage (one TMA operation), stages per channel block
   unsigned int a_stage_bytes;
