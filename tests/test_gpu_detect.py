@@ -155,3 +155,20 @@ def test_detection_output_refuses_what_it_cannot_hold(q8):
     with pytest.raises(q8.Q8Error) as e:
         q8.q8_detection_output([(loc[:, :100], conf[:, :100], 1)], pri[:100], nets.SSD300_VARIANCES, 3, nms_top_k=600)
     assert e.value.code == 2
+
+
+@pytest.mark.parametrize("shape", [(2, 9000, 21, 0.3, 0, 0.01, 0.45, 400, 200), (1, 16000, 3, 0.01, 0, 0.01, 0.3, 512, 2000),
+                                   (2, 1200, 24, 1.0, -1, 0.02, 0.45, 100, 50), (2, 1200, 25, 1.0, 3, 0.02, 0.45, 100, 50),
+                                   (1, 15000, 41, 0.2, 0, 0.001, 0.45, 400, 7000), (1, 16384, 9, 0.5, 0, 0.01, 0.9, 512, 16384)])
+def test_detection_output_selection_limits(q8, shape):
+    """Sizes at the edges of the candidate masks, of the classes a decoding warp keeps in registers, and of the
+    selections: (images, boxes, classes, logit spread, background, confidence, overlap, nms_top_k, keep_top_k)."""
+    N, P, classes, spread, background, conf_thresh, nms_thresh, top, keep = shape
+    g = np.random.default_rng(P + classes)
+    centre, size = g.uniform(0.1, 0.9, (P, 2)), g.uniform(0.02, 0.2, (P, 2))
+    priors = np.concatenate([centre, size], 1).astype(np.float32)
+    loc = g.normal(0, 0.5, (N, P, 4)).astype(np.float32)
+    conf = (g.normal(0, 1, (N, P, classes)) * spread).astype(np.float32)
+    conf[:, ::7] = conf[:, :1]                                         # equal probabilities
+    _compare(q8, loc, conf, priors, [P], [1], background=background, conf_thresh=conf_thresh, nms_thresh=nms_thresh,
+             nms_top_k=top, keep_top_k=keep)

@@ -1,0 +1,42 @@
+"""GPU parity of the launch plans that a layer's size selects, against the CPU oracle, bit-exact: narrow column tiles of
+every width, and CTA pairs whose epilogue groups share a tile's columns, both with one multiplier per channel."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as o
+
+pytestmark = pytest.mark.gpu
+U8, S8 = 0, 1
+
+CASES = [
+    # name, N,H,W,C,K,R,S,pad, y type, residual
+    ("narrow_16", 1, 14, 14, 1024, 256, 1, 1, (0, 0), U8, True),
+    ("narrow_16_halo", 1, 7, 7, 512, 512, 3, 3, (1, 1), S8, False),
+    ("narrow_32_ragged", 4, 14, 14, 640, 528, 1, 1, (0, 0), U8, True),
+    ("narrow_32_short_reduction", 1, 7, 7, 512, 2048, 1, 1, (0, 0), U8, True),
+    ("narrow_64_ragged", 4, 14, 14, 576, 1008, 1, 1, (0, 0), S8, False),
+    ("narrow_128", 16, 14, 14, 768, 512, 1, 1, (0, 0), U8, False),
+    ("pair_256_shared", 14, 53, 53, 128, 512, 3, 3, (1, 1), U8, True),
+    ("pair_144_shared_odd_chunks", 44, 37, 37, 128, 144, 3, 3, (1, 1), S8, False),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
+def test_plan_matches_oracle(q8, case):
+    name, N, H, W, C, K, R, S, pad, ytype, res = case
+    g = np.random.default_rng(sum(map(ord, name)))
+    x = g.integers(0, 256, (N, H, W, C), dtype=np.uint8)
+    w = g.integers(-128, 128, (K, R, S, C)).astype(np.int8)
+    bias = g.integers(-5000, 5000, K).astype(np.int32)
+    acc = o.conv_acc(x, w, bias, (1, 1), pad, (1, 1), threads=8)
+    resid = g.integers(0, 256, acc.shape, dtype=np.uint8) if res else None
+    scale = (g.uniform(0.5, 1.5, K) * 100.0 / max(1, np.abs(acc).max())).astype(np.float32)
+    want = o.epilogue(acc, scale, resid, 0.37 if res else 0.0, ytype == U8, o.U8 if ytype == U8 else o.S8)
+    d = q8.make_conv_desc(N, H, W, C, K, R, S, (1, 1), pad, (1, 1), U8, U8, ytype, ytype == U8, K)
+    args = [torch.from_numpy(a).cuda() for a in (x, w, bias, scale)]
+    rd = torch.from_numpy(resid).cuda() if res else None
+    for _ in range(2):   # twice: the second launch follows the first in the stream
+        y = q8.q8_conv2d(d, *args, rd, 0.37 if res else 0.0)
+    q8.q8_read_status()
+    assert np.array_equal(y.cpu().numpy(), want)
