@@ -940,7 +940,7 @@ struct HaloTile {
 // Stride 2 along W needs no data movement: with W even, NHWC memory is also a tensor of pixel pairs with 2C
 // channels, and output column q reads pairs q + t' - pad', t' = 0 .. S'-1, i.e. a stride-1 filter of
 // S' = ceil((S + e) / 2) taps (e = pad_w & 1).  Stride along H is served by tiles of one output row.
-bool choose_halo_tile(const q8_conv_desc& d, int P, int Q, HaloTile* out) {
+bool search_halo_tile(const q8_conv_desc& d, int P, int Q, HaloTile* out) {
   const int sw = d.stride_w;
   if (sw != 1 && sw != 2) return false;
   int s_eff = d.S, pad_eff = d.pad_w, e = 0, dil_w = d.dil_w;
@@ -980,6 +980,25 @@ bool choose_halo_tile(const q8_conv_desc& d, int P, int Q, HaloTile* out) {
   if (best.tw == 0) return false;
   *out = best;
   return true;
+}
+
+// A call asks for the tile of its descriptor three or four times, and the search costs up to 2 us on a wide image, which a
+// small layer's launch does not hide: the last tiles found are kept per thread, by the descriptor's values, on which alone
+// they depend (3x3 64->64 on a 4x120 image, batch 1: 6.7 -> 4.4 us of host time per call).
+bool choose_halo_tile(const q8_conv_desc& d, int P, int Q, HaloTile* out) {
+  struct Entry { q8_conv_desc d; HaloTile t; int state; };  // state 0: empty, 1: no tile, 2: tile
+  static thread_local Entry cache[64];
+  unsigned int h = 2166136261u;
+  const int32_t key[] = {d.N, d.H, d.W, d.C, d.K, d.R, d.S, d.stride_h, d.stride_w, d.pad_h, d.pad_w, d.dil_h, d.dil_w};
+  for (int32_t v : key) h = (h ^ (unsigned int)v) * 16777619u;
+  Entry& e = cache[(h ^ (h >> 16)) & 63u];
+  if (e.state == 0 || memcmp(&e.d, &d, sizeof(d)) != 0) {
+    e.t = HaloTile{};
+    e.state = search_halo_tile(d, P, Q, &e.t) ? 2 : 1;
+    e.d = d;
+  }
+  if (e.state == 2) *out = e.t;
+  return e.state == 2;
 }
 
 }  // namespace
