@@ -89,6 +89,18 @@ int validate_desc(const q8_conv_desc* d, int* P, int* Q) {
   return Q8_OK;
 }
 
+// Few outputs with a short reduction: the direct kernel finishes before a tensor-core kernel has set up its pipeline (1x1 of
+// 5 -> 8 channels at 8x8: 2.6 against 3.5 us gathered; 20 -> 16 at 32x32: 3.3 against 3.9; 5 -> 32 on 8 x 28x28: 4.1 both).
+// From 27 products or 100 000 outputs on it takes longer (3x3 of 3 -> 8 on 2 x 17x19: 4.9 against 3.8 us).
+bool tiny_call(const ConvArgs& a) { return (long long)a.d.R * a.d.S * a.d.C <= 24 && a.M * a.d.K <= 100000; }
+
+// 8-bit rows off the 16-byte grid that are short and have short reductions: gathering the operands is cheaper than moving
+// the rows through shared memory (1x1 64 -> 9 at 56x56, batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32 7.2
+// against 7.1; 64 -> 15 at 112x112, batch 8 8.4 against 7.3; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).
+bool short_rows(const ConvArgs& a) {
+  const long long products = (long long)a.d.R * a.d.S * a.d.C;
+  return products <= 64 && (a.d.K <= 16 ? products * a.M <= 4000000 : a.d.K <= 32 && a.M <= 128);
+}
 }  // namespace
 }  // namespace q8
 
@@ -170,16 +182,16 @@ int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32
   if (ok) {
     const bool out8 = d->y_type == Q8_U8 || d->y_type == Q8_S8;
     if (!aligned16(x) || !aligned16(w)) { ok = false; why = "x or w not 16-byte aligned"; }
-    else if (out8 && (!aligned16(y) || a.ldc % 16 || a.c_off % 16)) { ok = false; why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; }
-    else if (a.residual && !aligned16(a.residual)) { ok = false; why = "residual not 16-byte aligned"; }
+    else if (d->algo == Q8_ALGO_UMMA || !out8) {
+      if (out8 && (!aligned16(y) || a.ldc % 16 || a.c_off % 16)) { ok = false; why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; }
+      else if (a.residual && !aligned16(a.residual)) { ok = false; why = "residual not 16-byte aligned"; }
+    }
+    // (8-bit rows off the 16-byte grid: the epilogue warps move them, see rows_out)
+    else if (rows_unaligned(a) && (tiny_call(a) || short_rows(a))) ok = false;
   }
   if (!ok) {
     if (d->algo == Q8_ALGO_UMMA) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
-    // Few outputs with a short reduction finish before the gathering kernel has set up its pipeline (1x1 of 5 -> 8
-    // channels at 8x8: 2.6 against 3.5 us; 20 -> 16 at 32x32: 3.3 against 3.9; 5 -> 32 on 8 x 28x28: 4.1 both).  From 27
-    // products or 100 000 outputs on they take longer (3x3 of 3 -> 8 on 2 x 17x19: 4.9 against 3.8 us).
-    const bool tiny = (long long)d->R * d->S * d->C <= 24 && a.M * d->K <= 100000;
-    if (d->K <= 4096 && !tiny) return launch_conv_gather(a);
+    if (d->K <= 4096 && !tiny_call(a)) return launch_conv_gather(a);
     return launch_conv_direct(a);
   }
   return launch_conv_umma(a);

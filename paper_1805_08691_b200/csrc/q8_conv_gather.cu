@@ -1,5 +1,6 @@
 // Quantized convolution on the tensor cores for layers that TMA cannot address: channel counts that are no multiple
-// of 16 (a three-channel image, pruned layers), pointers or output slices off the 16-byte grid, strides above 8.
+// of 16 (a three-channel image, pruned layers), inputs or weights off the 16-byte grid, strides above 8; and, being cheaper
+// to start, short reductions into few channels whose 8-bit rows are off that grid.
 //
 //   D[128 pixels, BN channels] (int32, TMEM) = A[128, Kp] (gathered) x B[BN, Kp]^T (gathered)
 //

@@ -528,6 +528,26 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     TileIterT<kCta2> ti;
     ti.init(p, vblock + team * vgrid, tile_step * vgrid, cta_rank);
     for (; ti.tile < total_tiles; ti.next(p)) {
+      auto place = [&] {  // the tile's pixel and columns of this thread
+        t.n0 = ti.nt * p.bn;
+        t.y_off = (long long)ti.sp * p.split_stride;
+        if (p.a_mode == kAHalo) {
+          const int pr = ti.pt * p.th + pp, qc = ti.qt * p.tw + qq;
+          t.row_ok = t.smem_ok && pr < p.P && qc < p.Q && ti.valid;
+          t.m = ((long long)ti.img * p.P + pr) * p.Q + qc;
+        } else {
+          t.m = (long long)ti.mt * kBM + row;
+          t.row_ok = t.m < p.M;
+        }
+      };
+      RowMove mv;
+      if constexpr (kRes == kResRows) {  // one buffer per group, shared where groups share tiles: their columns are disjoint
+        place();
+        t.buf = base_ptr + p.off_bufs + (split ? (size_t)0 : (size_t)g * p.tile8_bytes);
+        mv.init(p, t.n0, ch0, ch1);
+        if (p.res_mode != kResNone) rows_in(p, t, mv, lane);  // while the accumulator is being formed
+        __syncwarp();
+      }
       bool ok = mbar_wait(accf0 + ab * 8u, acc_par, abortp);
       if (p.nbuf > 0 && ok) ok = mbar_wait(bfull0 + slot * 8u, slot_par, abortp);
       if (!ok) {
@@ -538,19 +558,17 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         break;
       }
       tcgen05_fence_after();
-      t.n0 = ti.nt * p.bn;
-      t.y_off = (long long)ti.sp * p.split_stride;
-      if (p.a_mode == kAHalo) {
-        const int pr = ti.pt * p.th + pp, qc = ti.qt * p.tw + qq;
-        t.row_ok = t.smem_ok && pr < p.P && qc < p.Q && ti.valid;
-        t.m = ((long long)ti.img * p.P + pr) * p.Q + qc;
-      } else {
-        t.m = (long long)ti.mt * kBM + row;
-        t.row_ok = t.m < p.M;
+      if constexpr (kRes != kResRows) {
+        place();
+        t.buf = p.nbuf > 0 ? base_ptr + p.off_bufs + (size_t)slot * p.tile8_bytes : nullptr;
       }
-      t.buf = p.nbuf > 0 ? base_ptr + p.off_bufs + (size_t)slot * p.tile8_bytes : nullptr;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * (uint32_t)p.acc_stride;
       epilogue_row<kOut, kRes, kCta2, kUniform>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1);
+      if constexpr (kRes == kResRows) {
+        __syncwarp();
+        rows_out(p, t, mv, lane);
+        __syncwarp();  // the buffer is read before the next tile's rows go into it
+      }
       if (p.nbuf > 0) {
         // this thread's reads and writes of the buffer are done; the store thread takes over
         if (p.out8) fence_proxy_async_smem();
@@ -632,11 +650,11 @@ int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensor
   // kResTma stands for "a residual through the tile buffers, or none"
   const bool global_res = p.res_mode == kResGlobal;
   if (p.y_type == Q8_U8) {
-    if (global_res) Q8_LAUNCH(Q8_U8, kResGlobal);
+    if (!p.out8) Q8_LAUNCH(Q8_U8, kResRows);
     Q8_LAUNCH(Q8_U8, kResTma);
   }
   if (p.y_type == Q8_S8) {
-    if (global_res) Q8_LAUNCH(Q8_S8, kResGlobal);
+    if (!p.out8) Q8_LAUNCH(Q8_S8, kResRows);
     Q8_LAUNCH(Q8_S8, kResTma);
   }
   if (p.y_type == Q8_F32) {
@@ -723,9 +741,13 @@ int launch_conv_umma_impl(const ConvArgs& a, int splits) {
 }
 }  // namespace
 
+bool rows_unaligned(const ConvArgs& a) {
+  return (a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8) && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16 || (a.residual && !aligned16(a.residual)));
+}
+
 int launch_conv_umma(const ConvArgs& a) {
   const q8_conv_desc& d = a.d;
-  int splits = umma_plan_splits(d, a.P, a.Q, a.M);
+  int splits = rows_unaligned(a) ? 1 : umma_plan_splits(d, a.P, a.Q, a.M);
   if (splits > 1) {
     // Narrow tiles against a split of the default ones, by the operand bytes a CTA streams (~60 per cycle); a split
     // pays ~6000 cycles for its second kernel.
@@ -763,7 +785,10 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
 
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   int res_mode = kResNone;
-  if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResTma : kResGlobal;
+  if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResTma : (out8 ? kResRows : kResGlobal);
+  // 8-bit rows off the 16-byte grid are moved by the epilogue warps, in both directions if in one
+  const bool rows = out8 && (rows_unaligned(a) || res_mode == kResRows);
+  if (rows && a.residual) res_mode = kResRows;
   UmmaParams p;
   memset(&p, 0, sizeof(p));
   HaloTile ht = {0, 0, 0, 0, 0.0, 1, d.S, d.pad_w, 0};
@@ -845,7 +870,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
 
   // ---- shared memory plan: [resident weights] [A stages] [weight ring] [8-bit tile buffers] [bias, scale]
-  const bool use_bufs = out8 || res_mode == kResTma;
+  const bool use_bufs = (out8 && !rows) || res_mode == kResTma;
   // Launches with at most two work items per CTA cannot keep several groups busy on different tiles: there all
   // four groups share every tile, each taking a quarter of its columns (any tile width, both accumulators).
   {
@@ -883,7 +908,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     // as pairs, 135 us with three lanes).
     const long long pair_items = (long long)((p.m_tiles + 1) / 2) * p.n_tiles;
     const bool can = p.a_mode == kAHalo && !paired && p.b_mode == kBRing && BN >= 96 && BN % 32 == 0 && out8 &&
-                     res_mode != kResGlobal && splits == 1 && (BK == 128 || BK == 64) &&
+                     !rows && splits == 1 && (BK == 128 || BK == 64) &&
                      (!p.epi_split || tune_env("Q8_CTA2SPLIT", 0, 0, 1)) &&
                      pair_items >= tune_env("Q8_CTA2MIN", 2 * (sm_count() / 2), 1, 1 << 30);
     if (can && tune_env("Q8_CTA2", 1, 0, 1)) {
@@ -904,6 +929,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
     }
   }
+  const unsigned row_bytes = rows ? (unsigned)(p.epi_split ? 1 : G) * p.tile8_bytes : 0u;
   p.b_T = 1;
   p.b_chunks = p.taps;
   unsigned min_pipe;
@@ -918,7 +944,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
       // Weight ring stages of several filter taps, one TMA operation each (the copy engine spends ~600 cycles
       // per operation whatever its size): as many taps as fit in about 48 KiB while two such stages fit beside
       // two activation stages and one tile buffer per epilogue group, spread evenly over a channel block.
-      const unsigned fixed = bres_bytes + (use_bufs ? (unsigned)(p.epi_split ? 2 : (p.cta2 ? G >> p.pair_shift : G)) * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
+      const unsigned fixed = bres_bytes + row_bytes + (use_bufs ? (unsigned)(p.epi_split ? 2 : (p.cta2 ? G >> p.pair_shift : G)) * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
       const unsigned avail = budget > fixed ? budget - fixed : 0u;
       int T = (int)(48u * 1024u / p.b_tile_bytes);
       if (T > (int)(avail / (2u * p.b_tile_bytes))) T = (int)(avail / (2u * p.b_tile_bytes));
@@ -949,7 +975,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     p.nbuf = tune_env("Q8_NBUF", p.nbuf, 1, p.nbuf);
     if (p.epi_split) p.nbuf = 2;  // one buffer per tile in flight; a CTA has at most two tiles
   }
-  const unsigned buf_bytes = (unsigned)(p.epi_split ? p.nbuf : (p.cta2 ? G >> p.pair_shift : G) * p.nbuf) * p.tile8_bytes;
+  const unsigned buf_bytes = row_bytes + (unsigned)(p.epi_split ? p.nbuf : (p.cta2 ? G >> p.pair_shift : G) * p.nbuf) * p.tile8_bytes;
   if (budget < bres_bytes + buf_bytes + min_pipe) return kPlanNoFit;
   unsigned rest = budget - bres_bytes - buf_bytes;
   p.b_stages = 0;
@@ -1052,7 +1078,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     cr = encode_rows(&tmRes, const_cast<void*>(a.residual), d.K, d.K, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
     if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: residual tensor map rejected (CUresult %d)", (int)cr);
   }
-  if (out8) {
+  if (out8 && !rows) {
     cr = encode_rows(&tmY, a.y, a.c_off + d.K, a.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
     if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: output tensor map rejected (CUresult %d)", (int)cr);
   }
@@ -1077,7 +1103,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   p.res_signed = d.res_type == Q8_S8;
   p.res_scale = a.residual_scale;
   p.y = a.y; p.y_type = d.y_type; p.ldc = a.ldc; p.c_off = a.c_off; p.relu = d.relu;
-  p.out8 = out8 ? 1 : 0;
+  p.out8 = out8 && !rows ? 1 : 0;
   p.y_vec = out8 ? 1 : (aligned16(a.y) && a.ldc % 4 == 0 && a.c_off % 4 == 0);
   p.status = status;
 

@@ -56,6 +56,7 @@ struct ConvArgs {
 
 // Eligibility of the tensor-core kernel for a descriptor (pointer alignment checked at launch).
 bool umma_shape_eligible(const q8_conv_desc& d, const char** why);
+bool rows_unaligned(const ConvArgs& a);  // 8-bit output or residual rows that TMA cannot address
 int launch_conv_umma(const ConvArgs& a);
 // Number of split-K parts the tensor-core kernel uses for this layer when it is given a workspace of
 // splits * M * K int32 (1: none).  Host only.

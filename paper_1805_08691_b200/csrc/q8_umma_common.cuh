@@ -37,7 +37,7 @@ enum StatusBits : unsigned int {
   kTimeoutStore = 16u,
 };
 
-enum ResMode : int { kResNone = 0, kResTma = 1, kResGlobal = 2 };
+enum ResMode : int { kResNone = 0, kResTma = 1, kResGlobal = 2, kResRows = 3 };
 enum AMode : int { kAPlain = 0, kAIm2col = 1, kAHalo = 2 };
 enum BMode : int { kBStage = 0, kBResident = 1, kBRing = 2 };
 
@@ -488,7 +488,8 @@ __device__ __forceinline__ void epi_row_setup(const UmmaParams& p, EpiTile& t) {
 }
 
 // One 16-column chunk of one accumulator row.  kOut: Q8_U8, Q8_S8, Q8_S32 or Q8_F32.  kRes: kResNone, kResTma
-// (a residual from the tile buffer if p.res_mode says so, else none: decided at run time) or kResGlobal.  Fewer
+// (a residual from the tile buffer if p.res_mode says so, else none: decided at run time), kResGlobal (fp32 outputs) or
+// kResRows (8-bit rows that TMA cannot address: as kResTma, but the warps fill and empty the buffer themselves).  Fewer
 // distinct kernels matter more than one uniform branch per chunk: a launch of another kernel function than
 // the one before it starts with cold instruction caches, which costs a layer of a network 2 to 6 us, so the
 // layers with and without a residual sum share their kernels.  (One straight-line arm per case, chosen per
@@ -547,14 +548,14 @@ __device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTil
 #pragma unroll
   for (int j = 0; j < 8; ++j) unpack_f2(v2[j], v[2 * j], v[2 * j + 1]);
   unsigned int rw[4] = {0u, 0u, 0u, 0u};
-  if (kRes == kResTma && (kOut == Q8_U8 || kOut == Q8_S8)) {
+  if (kRes == kResRows ? p.res_mode != kResNone : (kRes == kResTma && (kOut == Q8_U8 || kOut == Q8_S8))) {
     // the tile buffer always exists for 8-bit outputs: its bytes are read ahead of the (uniform) branch on
     // whether they are a residual, so that the load is in flight with those of bias and scale
     const uint4 rv = *reinterpret_cast<const uint4*>(t.buf + off);
     rw[0] = rv.x; rw[1] = rv.y; rw[2] = rv.z; rw[3] = rv.w;
   }
-  if (kRes == kResGlobal || (kRes == kResTma && p.res_mode != kResNone)) {
-    if (kRes == kResTma) {
+  if (kRes == kResGlobal || ((kRes == kResTma || kRes == kResRows) && p.res_mode != kResNone)) {
+    if (kRes == kResTma || kRes == kResRows) {
       if (kOut != Q8_U8 && kOut != Q8_S8) {
         const uint4 rv = *reinterpret_cast<const uint4*>(t.buf + off);
         rw[0] = rv.x; rw[1] = rv.y; rw[2] = rv.z; rw[3] = rv.w;
@@ -660,6 +661,92 @@ __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile&
       }
       epilogue_chunk<kOut, kRes, kUniform>(p, t, ch + 1, rb, us);
     }
+  }
+}
+
+// 8-bit tensors whose rows TMA cannot address (channel counts, pitches, offsets or pointers off the 16-byte grid): a warp
+// moves the rows of its 32 accumulator rows between global memory and the group's tile buffer itself.  Neighbouring lanes
+// take neighbouring words of a row, `lpr` lanes a row (a power of two that covers it, so that narrow rows share a pass);
+// the global words are aligned ones, the buffer's follow from two of them by a funnel shift.  Only words that hold a byte
+// of the row are touched, and on the way out bytes outside it are never written.  Columns c0 .. c0 + nb - 1 of the tile.
+// (Against gathered operands: 3x3 128 -> 100 at 28x28, batch 32 46.0 -> 9.4 us; 1x1 64 -> 250 at 56x56, batch 16 118 ->
+// 17.9 us, as long as 256 channels take, with a residual sum 138 -> 28.6 us; partial words inside the loop over rows,
+// a residual fetched after the accumulator: 32.6 and 51.9 us.)
+struct RowMove {
+  int c0, nb, lpr_shift;
+  __device__ __forceinline__ void init(const UmmaParams& p, int n0, int ch0, int ch1) {
+    c0 = ch0 * 16;
+    nb = min(ch1 * 16, p.K - n0) - c0;
+    const int words = (nb + 3) >> 2;
+    lpr_shift = words > 16 ? 5 : (words > 8 ? 4 : (words > 4 ? 3 : (words > 2 ? 2 : (words > 1 ? 1 : 0))));
+  }
+};
+
+__device__ __forceinline__ uint32_t row_buf_offset(const UmmaParams& p, int srow, int col) {
+  const uint32_t rb = (uint32_t)srow << p.pw_shift;
+  return rb + (((uint32_t)(col & ((1 << p.pw_shift) - 1))) ^ (((rb >> 7) & (uint32_t)p.pmask) << 4)) +
+         (uint32_t)(col >> p.pw_shift) * ((uint32_t)kBM << p.pw_shift);
+}
+
+// Residual rows into the buffer, four passes of loads in flight.  All lanes of the warp call it.
+__device__ __forceinline__ void rows_in(const UmmaParams& p, const EpiTile& t, const RowMove& mv, int lane) {
+  constexpr int U = 4;
+  const int lpr = 1 << mv.lpr_shift, sub = lane & (lpr - 1), per_pass = 32 >> mv.lpr_shift;
+  const unsigned char* mine = p.res + t.m * p.K + t.n0 + mv.c0;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += U * per_pass) {
+    uintptr_t at[U];
+    int srow[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = r0 + u * per_pass + (lane >> mv.lpr_shift);
+      at[u] = (uintptr_t)__shfl_sync(0xffffffffu, (unsigned long long)mine, r & 31);
+      srow[u] = __shfl_sync(0xffffffffu, t.row_ok ? t.srow : -1, r & 31);
+      if (r >= 32) srow[u] = -1;
+    }
+#pragma unroll 1
+    for (int k = sub; 4 * k < mv.nb; k += lpr) {
+      unsigned int lo[U], hi[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int head = (int)(at[u] & 3u);
+        const unsigned int* g = reinterpret_cast<const unsigned int*>(at[u] - head) + k;
+        lo[u] = hi[u] = 0u;
+        if (srow[u] >= 0) lo[u] = g[0];
+        if (srow[u] >= 0 && 4 * (k + 1) - head < mv.nb) hi[u] = g[1];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (srow[u] >= 0)
+          *reinterpret_cast<unsigned int*>(t.buf + row_buf_offset(p, srow[u], mv.c0 + 4 * k)) = __funnelshift_r(lo[u], hi[u], 8 * (int)(at[u] & 3u));
+    }
+  }
+}
+
+// Output rows out of the buffer: the whole words of each row by its group of lanes, the up to three bytes before and after
+// them by the lane whose row it is (partial words in the loop over rows doubled its length).  All lanes call it.
+__device__ __forceinline__ void rows_out(const UmmaParams& p, const EpiTile& t, const RowMove& mv, int lane) {
+  const int lpr = 1 << mv.lpr_shift, sub = lane & (lpr - 1);
+  unsigned char* mine = static_cast<unsigned char*>(p.y) + t.m * p.ldc + p.c_off + t.n0 + mv.c0;
+  for (int r0 = 0; r0 < 32; r0 += 32 >> mv.lpr_shift) {
+    const int r = r0 + (lane >> mv.lpr_shift);
+    unsigned char* g = reinterpret_cast<unsigned char*>(__shfl_sync(0xffffffffu, (unsigned long long)mine, r));
+    const int srow = __shfl_sync(0xffffffffu, t.row_ok ? t.srow : -1, r);
+    const int head = (int)(0u - (unsigned)(uintptr_t)g) & 3;   // bytes before the first whole word
+    const int end = srow < 0 ? 0 : mv.nb - 3;
+    for (int b = head + 4 * sub; b < end; b += 4 * lpr) {
+      // bytes b .. b + 3 of the row, from the buffer words that hold byte b and byte b + 3
+      const unsigned int lo = *reinterpret_cast<const unsigned int*>(t.buf + row_buf_offset(p, srow, mv.c0 + (b & ~3)));
+      const unsigned int hi = *reinterpret_cast<const unsigned int*>(t.buf + row_buf_offset(p, srow, mv.c0 + ((b + 3) & ~3)));
+      *reinterpret_cast<unsigned int*>(g + b) = __funnelshift_r(lo, hi, 8 * head);
+    }
+  }
+  if (!t.row_ok || mv.nb <= 0) return;
+  const int head = min((int)(0u - (unsigned)(uintptr_t)mine) & 3, mv.nb), tail = head + ((mv.nb - head) & ~3);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (j < head) mine[j] = t.buf[row_buf_offset(p, t.srow, mv.c0 + j)];
+    if (tail + j < mv.nb) mine[tail + j] = t.buf[row_buf_offset(p, t.srow, mv.c0 + tail + j)];
   }
 }
 
