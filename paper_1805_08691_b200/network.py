@@ -30,6 +30,7 @@ for the fused residual sum; all tensor arithmetic runs in the library's kernels.
                                       tensors) are re-expressed and copied in by q8_concat_branch; a concat nested
                                       in another is a slice of the outer buffer and shares its factor
 """
+from operator import attrgetter
 from typing import Dict, List
 
 import numpy as np
@@ -40,7 +41,13 @@ from . import binding as q8
 from . import pipeline
 
 
+_LAUNCH_ARGS = attrgetter("w_q", "b_q", "scale", "res_scale", "desc")
+
+
 class QuantNetwork:
+    """The layer list is fixed at construction.  What the layers run with may be replaced afterwards, in whole
+    (`convs[name] = ...`, `convs[name].w_q = ...`, `bufs`, `l2`, `workspaces`) or in place: the next forward uses it."""
+
     def __init__(self, layers, folded: Dict[str, tuple], maxima: Dict[str, float], in_shape, device="cuda",
                  per_channel=False, streams=1, fuse=True, sum_policy="max"):
         """folded[name] = (w KRSC, b K) FP32 device tensors; maxima: calibrated max-abs of "input", every layer
@@ -141,7 +148,8 @@ class QuantNetwork:
                 self.outputs[L.name] = self.bufs[L.name][..., :L.conv.K]
         for first in self.fused_with:   # the tensor between two layers of one launch is never written
             self.outputs.pop(first, None)
-        self._capture(device)
+        self.device, self.recorded = device, None
+        self._record()
 
     def _weight_maxima(self, folded, per_channel, device):
         """max|w| of every convolution (a list per output channel with per_channel), read back in one copy."""
@@ -344,12 +352,28 @@ class QuantNetwork:
         self.run_quantized()
         return self.outputs
 
-    def _capture(self, device):
+    def _launch_state(self):
+        """What the recorded launches hold by value: addresses, descriptors and factors.  Contents that change in place
+        (weights of the same tensor) need no mention, the launches read them."""
+        w, bias, scale, res_scale, desc = zip(*map(_LAUNCH_ARGS, self.convs.values()))
+        l2 = self.l2.values()
+        given = [t is not None for t in bias + tuple(self.workspaces)]
+        tensors = [t for t in bias + tuple(self.workspaces) if t is not None]
+        tensors += w
+        tensors += scale
+        tensors += self.bufs.values()
+        tensors += [mult for _, _, mult in l2]
+        return (list(map(torch.Tensor.data_ptr, tensors)), given, res_scale, b"".join(desc), [t[:2] for t in l2],
+                list(self.info.values()))
+
+    def _record(self):
         """Records the layers once as a CUDA graph over the network's own buffers.  Called layer by layer from Python a
         forward costs the host 10 to 25 us per layer, more than the GPU spends on it: Inception-v3 at batch 64 took
         2.98 ms against 1.4 ms of kernels, ResNet-50 at batch 1 1.25 ms against 0.35 ms.  The graph holds no caller
         pointer (the input quantization, which reads the caller's images, stays outside) and no allocation."""
-        with torch.cuda.device(device):
+        state = self._launch_state()
+        self.recorded = None
+        with torch.cuda.device(self.device):
             side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
             side.wait_stream(torch.cuda.current_stream())
             with torch.cuda.stream(side):
@@ -360,15 +384,18 @@ class QuantNetwork:
                 finally:
                     graph.capture_end()
             torch.cuda.current_stream().wait_stream(side)
-        self.graph = graph
+        self.graph, self.recorded = graph, state
 
     def run_quantized(self):
         """Everything after the input quantization, on the current stream.  Inside a caller's own capture the layers are
         enqueued one by one and become part of the caller's graph."""
         if torch.cuda.is_current_stream_capturing():
             self._run_layers()
-        else:
-            self.graph.replay()
+            return
+        # (in time for the launch only where the GPU is idle: 20 us for 54 convolutions)
+        if self._launch_state() != self.recorded:
+            self._record()
+        self.graph.replay()
 
     def _run_layers(self):
         if self.n_streams == 1:
