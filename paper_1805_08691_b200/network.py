@@ -149,7 +149,10 @@ class QuantNetwork:
         for first in self.fused_with:   # the tensor between two layers of one launch is never written
             self.outputs.pop(first, None)
         self.device, self.recorded = device, None
-        self._record()
+        try:
+            self._record()
+        except q8.Q8Error:
+            pass    # a layer the library refuses is reported by the forward that would launch it
 
     def _weight_maxima(self, folded, per_channel, device):
         """max|w| of every convolution (a list per output channel with per_channel), read back in one copy."""
@@ -409,21 +412,24 @@ class QuantNetwork:
         for st in self.side_streams:
             st.wait_event(fork)
         done: Dict[str, torch.cuda.Event] = {}
-        for L in self.layers:
-            sid = self.stream_of[L.name]
-            st = streams[sid]
-            for t in self.deps[L.name]:
-                if t in done and self.stream_of[t] != sid:
-                    st.wait_event(done[t])
-            with torch.cuda.stream(st):
-                self._launch(L, self.workspaces[sid])
-            ev = torch.cuda.Event()
-            ev.record(st)
-            done[L.name] = ev
-        for st in self.side_streams:
-            join = torch.cuda.Event()
-            join.record(st)
-            main.wait_event(join)
+        try:
+            for L in self.layers:
+                sid = self.stream_of[L.name]
+                st = streams[sid]
+                for t in self.deps[L.name]:
+                    if t in done and self.stream_of[t] != sid:
+                        st.wait_event(done[t])
+                with torch.cuda.stream(st):
+                    self._launch(L, self.workspaces[sid])
+                ev = torch.cuda.Event()
+                ev.record(st)
+                done[L.name] = ev
+        finally:
+            # also when a layer has raised: a capture with streams that were not joined cannot be ended
+            for st in self.side_streams:
+                join = torch.cuda.Event()
+                join.record(st)
+                main.wait_event(join)
 
     def _launch(self, L, workspace):
         b = self.bufs

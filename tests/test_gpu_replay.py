@@ -155,3 +155,35 @@ def test_what_is_replaced_after_construction_takes_effect(q8, change):
     if change is not _buffer:
         assert any(not torch.equal(before[k], want[k]) for k in want)
     q8.q8_read_status()
+
+
+@pytest.mark.parametrize("layer", ["stem", "m0_3x1", "m1_3x3_s2"])
+def test_a_layer_that_is_refused_raises_its_own_error(q8, layer):
+    """... from the forward that would launch it, whichever stream it is on; the network works again once it is mended."""
+    net = _network("inception", streams=4)
+    x = _images("inception", 1)
+    want = _one_by_one(net, x)
+    stride = net.convs[layer].desc.stride_h
+    net.convs[layer].desc.stride_h = 0
+    for _ in range(2):
+        with pytest.raises(q8.Q8Error) as e:
+            net.forward(x)
+        assert e.value.code == 1
+    net.convs[layer].desc.stride_h = stride
+    _poison(net)
+    _assert_same(_snapshot(net.forward(x)), want)
+    q8.q8_read_status()
+
+
+def test_a_refused_layer_does_not_prevent_construction(q8, monkeypatch):
+    def refuse(*a, **k):
+        raise q8.Q8Error(2, "refused")
+    with monkeypatch.context() as m:
+        m.setattr(network.q8, "q8_maxpool2d", refuse)
+        net = _network("inception", streams=4)
+        x = _images("inception", 1)
+        with pytest.raises(q8.Q8Error, match="refused"):
+            net.forward(x)
+    want = _one_by_one(net, x)
+    _poison(net)
+    _assert_same(_snapshot(net.forward(x)), want)
