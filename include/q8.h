@@ -58,6 +58,26 @@ const char* q8_last_error(void);
 int q8_read_status(void* stream);
 
 /* ------------------------------------------------------------------------
+ * Recording (the paper has no counterpart): library calls enqueued once and replayed as one CUDA graph, for hosts
+ * that run the same calls over and over and would pay more for enqueueing a short kernel than the GPU for running it.
+ *  - q8_record_begin creates n_streams streams, writes them to streams[] (host array) and starts recording what is
+ *    enqueued on streams[0], and on the others once they wait for an event recorded on it.  The streams belong to this
+ *    recording alone.  Calls of other threads and work on other streams are neither recorded nor restricted.
+ *  - q8_record_end ends the recording, destroys its streams (streams[] is cleared) and writes the replayable graph
+ *    to *graph; streams[0] must wait for the last event of each other stream used.  graph NULL: the recording is
+ *    abandoned, whatever state it is in.
+ *  - q8_record_replay enqueues the recorded calls on `stream`.  The graph holds the addresses and host values of the
+ *    calls; what the addresses point to is read when it runs.  One graph is replayed by one thread at a time.
+ *  - q8_record_free releases a graph (NULL: nothing), also while it still runs.
+ * The CUDA driver keeps a graph's launch data in memory of its own.  q8_read_status, q8_static_workspace_bytes and the
+ * first q8_conv2d_static_workspace on a device may not be recorded.
+ * Errors: Q8_ERR_INVALID_ARG (null pointer, n_streams < 1), Q8_ERR_CUDA (among others: a stream was not joined). */
+int q8_record_begin(int n_streams, void** streams);
+int q8_record_end(int n_streams, void** streams, void** graph);
+int q8_record_replay(void* graph, void* stream);
+int q8_record_free(void* graph);
+
+/* ------------------------------------------------------------------------
  * Calibration (Sec. "8-bit Low Precision Inference", calibration paragraph:
  * each tensor's factor is max|r| / (2^p - 1)).
  * ---------------------------------------------------------------------- */

@@ -23,7 +23,7 @@ EXPORTS = ["q8_version", "q8_last_error", "q8_read_status", "q8_calibrate_maxabs
            "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d", "q8_static_workspace_bytes",
            "q8_conv2d_static_workspace", "q8_conv2d_then_1x1_supported", "q8_conv2d_then_1x1", "q8_int8_mma_rate", "q8_selftest_bounded_wait", "q8_concat", "q8_concat_branch", "q8_calibrate_maxabs_rows", "q8_quantize_rows", "q8_quantize_pad_image", "q8_pool_out_extent",
            "q8_maxpool2d", "q8_avgpool2d", "q8_l2norm", "q8_add_relu_quantize", "q8_detection_output_workspace_bytes",
-           "q8_detection_output"]
+           "q8_detection_output", "q8_record_begin", "q8_record_end", "q8_record_replay", "q8_record_free"]
 
 
 class Q8Error(RuntimeError):
@@ -85,6 +85,10 @@ lib.q8_add_relu_quantize.argtypes = [_vp, _vp, _sz, _f, _vp, _vp]
 lib.q8_detection_output_workspace_bytes.argtypes = [_i] * 6 + [C.POINTER(_sz)]
 lib.q8_detection_output.argtypes = [_i, C.POINTER(_vp), _ip, C.POINTER(_vp), _ip, _ip, _ip, _vp, _fp, _i, _i, _i, _f, _f, _i, _i,
                                     _vp, _sz, _vp, _vp, _vp]
+lib.q8_record_begin.argtypes = [_i, C.POINTER(_vp)]
+lib.q8_record_end.argtypes = [_i, C.POINTER(_vp), C.POINTER(_vp)]
+lib.q8_record_replay.argtypes = [_vp, _vp]
+lib.q8_record_free.argtypes = [_vp]
 for _n in EXPORTS[2:]:
     getattr(lib, _n).restype = C.c_int
 lib.q8_static_workspace_bytes.restype = C.c_size_t
@@ -124,6 +128,28 @@ def q8_last_error():
 
 def q8_read_status():
     _check(lib.q8_read_status(_stream()))
+
+
+def q8_record_begin(n_streams):
+    """Raw handles of the recording's streams (a ctypes array, to be handed to q8_record_end)."""
+    streams = (C.c_void_p * max(n_streams, 1))()
+    _check(lib.q8_record_begin(n_streams, streams))
+    return streams
+
+
+def q8_record_end(streams, keep=True):
+    """The graph of the recording, or None with keep=False (the recording is abandoned)."""
+    graph = C.c_void_p()
+    _check(lib.q8_record_end(len(streams), streams, C.byref(graph) if keep else None))
+    return graph.value
+
+
+def q8_record_replay(graph):
+    _check(lib.q8_record_replay(graph, _stream()))
+
+
+def q8_record_free(graph):
+    _check(lib.q8_record_free(graph))
 
 
 def q8_calibrate_maxabs(x, running_max):

@@ -30,6 +30,7 @@ for the fused residual sum; all tensor arithmetic runs in the library's kernels.
                                       tensors) are re-expressed and copied in by q8_concat_branch; a concat nested
                                       in another is a slice of the outer buffer and shares its factor
 """
+import threading
 from operator import attrgetter
 from typing import Dict, List
 
@@ -42,6 +43,30 @@ from . import pipeline
 
 
 _LAUNCH_ARGS = attrgetter("w_q", "b_q", "scale", "res_scale", "desc")
+
+
+class _Recording:
+    """What `enqueue(streams)` enqueues, recorded on streams of its own (not the framework's pooled ones, on which another
+    thread may be working) and replayed on the current stream."""
+
+    def __init__(self, n_streams, device, enqueue):
+        self.graph = None
+        handles = q8.q8_record_begin(n_streams)
+        try:
+            streams = [torch.cuda.ExternalStream(h, device=device) for h in handles]
+            with torch.cuda.stream(streams[0]):
+                enqueue(streams)
+        except BaseException:
+            q8.q8_record_end(handles, keep=False)
+            raise
+        self.graph = q8.q8_record_end(handles)
+
+    def replay(self):
+        q8.q8_record_replay(self.graph)
+
+    def __del__(self):
+        if self.graph is not None:
+            q8.lib.q8_record_free(self.graph)
 
 
 class QuantNetwork:
@@ -148,7 +173,7 @@ class QuantNetwork:
                 self.outputs[L.name] = self.bufs[L.name][..., :L.conv.K]
         for first in self.fused_with:   # the tensor between two layers of one launch is never written
             self.outputs.pop(first, None)
-        self.device, self.recorded = device, None
+        self.recording, self.recorded, self.lock = None, None, threading.Lock()
         try:
             self._record()
         except q8.Q8Error:
@@ -374,20 +399,11 @@ class QuantNetwork:
         forward costs the host 10 to 25 us per layer, more than the GPU spends on it: Inception-v3 at batch 64 took
         2.98 ms against 1.4 ms of kernels, ResNet-50 at batch 1 1.25 ms against 0.35 ms.  The graph holds no caller
         pointer (the input quantization, which reads the caller's images, stays outside) and no allocation."""
-        state = self._launch_state()
-        self.recorded = None
-        with torch.cuda.device(self.device):
-            side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
-            side.wait_stream(torch.cuda.current_stream())
-            with torch.cuda.stream(side):
-                # relaxed: kernels may be loaded on first use while they are recorded, other threads are unaffected
-                graph.capture_begin(capture_error_mode="relaxed")
-                try:
-                    self._run_layers()
-                finally:
-                    graph.capture_end()
-            torch.cuda.current_stream().wait_stream(side)
-        self.graph, self.recorded = graph, state
+        state, device = self._launch_state(), self.bufs["input"].device
+        self.recording = self.recorded = None
+        with torch.cuda.device(device):
+            self.recording = _Recording(self.n_streams, device, self._run_layers)
+        self.recorded = state
 
     def run_quantized(self):
         """Everything after the input quantization, on the current stream.  Inside a caller's own capture the layers are
@@ -396,20 +412,21 @@ class QuantNetwork:
             self._run_layers()
             return
         # (in time for the launch only where the GPU is idle: 20 us for 54 convolutions)
-        if self._launch_state() != self.recorded:
-            self._record()
-        self.graph.replay()
+        with self.lock:
+            if self._launch_state() != self.recorded:
+                self._record()
+            self.recording.replay()
 
-    def _run_layers(self):
+    def _run_layers(self, streams=None):
         if self.n_streams == 1:
             for L in self.layers:
                 self._launch(L, self.workspaces[0])
             return
         main = torch.cuda.current_stream()
-        streams = [main] + self.side_streams
+        streams = streams or [main] + self.side_streams
         fork = torch.cuda.Event()
         fork.record(main)
-        for st in self.side_streams:
+        for st in streams[1:]:
             st.wait_event(fork)
         done: Dict[str, torch.cuda.Event] = {}
         try:
@@ -426,7 +443,7 @@ class QuantNetwork:
                 done[L.name] = ev
         finally:
             # also when a layer has raised: a capture with streams that were not joined cannot be ended
-            for st in self.side_streams:
+            for st in streams[1:]:
                 join = torch.cuda.Event()
                 join.record(st)
                 main.wait_event(join)

@@ -95,3 +95,10 @@ def test_kernel_selection_rules():
     assert q8.q8_conv2d_query_algo(q8.make_conv_desc(32, 56, 56, 64, 64, 3, 3, pad=(1, 1))) == U
     assert q8.q8_conv2d_query_algo(q8.make_conv_desc(1, 8, 8, 3, 8, 3, 3, pad=(1, 1))) == q8.Q8_ALGO_DIRECT
     assert q8.q8_conv2d_query_algo(q8.make_conv_desc(32, 56, 56, 64, 64, 3, 3, pad=(1, 1), algo=q8.Q8_ALGO_DIRECT)) == q8.Q8_ALGO_DIRECT
+
+
+def test_recording_requests_are_checked_on_the_host():
+    assert _code(q8.q8_record_begin, 0) == 1
+    assert _code(q8.q8_record_replay, None) == 1
+    assert q8.lib.q8_record_end(1, (C.c_void_p * 1)(), None) == 1
+    q8.q8_record_free(None)

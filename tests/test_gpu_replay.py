@@ -1,6 +1,8 @@
 """QuantNetwork.forward replays recorded launches: it must give what its layers launched one by one give, bit for bit, for
 new images, on any stream, inside a caller's capture, and after any of the tensors, descriptors or factors that the
 layers run with has been replaced."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -187,3 +189,41 @@ def test_a_refused_layer_does_not_prevent_construction(q8, monkeypatch):
     want = _one_by_one(net, x)
     _poison(net)
     _assert_same(_snapshot(net.forward(x)), want)
+
+
+def test_recording_leaves_other_threads_alone(q8, monkeypatch):
+    """While the launches of a network are recorded, another thread's work on any stream of the framework's pool runs (it is
+    not recorded), and it may draw random numbers."""
+    pool = [torch.cuda.Stream() for _ in range(32)]
+    counts = [torch.zeros(1, device="cuda") for _ in pool]
+    torch.cuda.synchronize()
+    failed, rounds, launch = [], [], network.q8.q8_maxpool2d
+
+    def work():
+        try:
+            for st, c in zip(pool, counts):
+                with torch.cuda.stream(st):
+                    c.add_(1)
+            torch.rand(4, device="cuda")
+        except Exception as e:
+            failed.append(e)
+
+    def maxpool(*a, **k):
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        rounds.append(1)
+        return launch(*a, **k)
+
+    with monkeypatch.context() as m:
+        m.setattr(network.q8, "q8_maxpool2d", maxpool)
+        net = _network("inception", streams=4)
+    assert rounds and not failed
+    for st, c in zip(pool, counts):
+        st.synchronize()
+        assert c.item() == len(rounds)
+    x = _images("inception", 1)
+    want = _one_by_one(net, x)
+    _poison(net)
+    _assert_same(_snapshot(net.forward(x)), want)
+    assert [c.item() for c in counts] == [len(rounds)] * len(pool)
