@@ -405,6 +405,13 @@ class QuantNetwork:
             self.recording = _Recording(self.n_streams, device, self._run_layers)
         self.recorded = state
 
+    def __getstate__(self):
+        """A copy (single-stream networks can be copied and pickled) records its own launches in its first forward."""
+        return {**self.__dict__, "recording": None, "recorded": None, "lock": None}
+
+    def __setstate__(self, state):
+        self.__dict__.update(state, lock=threading.Lock())
+
     def run_quantized(self):
         """Everything after the input quantization, on the current stream.  Inside a caller's own capture the layers are
         enqueued one by one and become part of the caller's graph."""

@@ -1,6 +1,8 @@
 """QuantNetwork.forward replays recorded launches: it must give what its layers launched one by one give, bit for bit, for
 new images, on any stream, inside a caller's capture, and after any of the tensors, descriptors or factors that the
 layers run with has been replaced."""
+import copy
+import pickle
 import threading
 
 import numpy as np
@@ -227,3 +229,14 @@ def test_recording_leaves_other_threads_alone(q8, monkeypatch):
     _poison(net)
     _assert_same(_snapshot(net.forward(x)), want)
     assert [c.item() for c in counts] == [len(rounds)] * len(pool)
+
+
+@pytest.mark.parametrize("duplicate", [copy.deepcopy, lambda net: pickle.loads(pickle.dumps(net))], ids=["deepcopy", "pickle"])
+def test_a_copied_network_runs_on_its_own_tensors(q8, duplicate):
+    net = _network("bottlenecks", streams=1)
+    x, y = _images("bottlenecks", 1), _images("bottlenecks", 2)
+    want_x, want_y = _one_by_one(net, x), _one_by_one(net, y)
+    twin = duplicate(net)
+    a, b = net.forward(x), twin.forward(y)
+    _assert_same(_snapshot(a), want_x)
+    _assert_same(_snapshot(b), want_y)
