@@ -189,12 +189,14 @@ int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32
     // (8-bit rows off the 16-byte grid: the epilogue warps move them, see rows_out)
     else if (rows_unaligned(a) && (tiny_call(a) || short_rows(a))) ok = false;
   }
-  if (!ok) {
-    if (d->algo == Q8_ALGO_UMMA) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
-    if (d->K <= 4096 && !tiny_call(a)) return launch_conv_gather(a);
-    return launch_conv_direct(a);
+  if (ok) {
+    rc = launch_conv_umma(a);
+    if (rc != kPlanNoFit) return rc;
+    why = "no tile shape of this layer fits in shared memory";
   }
-  return launch_conv_umma(a);
+  if (d->algo == Q8_ALGO_UMMA) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
+  if (d->K <= 4096 && !tiny_call(a)) return launch_conv_gather(a);
+  return launch_conv_direct(a);
 }
 
 int q8_conv2d_then_1x1_supported(const q8_conv_desc* d1, const q8_conv_desc* d2, int* supported) {

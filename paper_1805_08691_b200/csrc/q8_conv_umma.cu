@@ -669,6 +669,16 @@ bool is_plain(const q8_conv_desc& d) {
   return d.R == 1 && d.S == 1 && d.stride_h == 1 && d.stride_w == 1 && d.pad_h == 0 && d.pad_w == 0;
 }
 
+// im2col tensor maps: corners are 8-bit signed, tap offsets 8-bit unsigned, strides at most 8.
+bool im2col_open(const q8_conv_desc& d, const char** why) {
+  const int up_w = d.pad_w - (d.S - 1) * d.dil_w, up_h = d.pad_h - (d.R - 1) * d.dil_h;
+  if (d.pad_w > 128 || d.pad_h > 128 || up_w < -128 || up_h < -128 || up_w > 127 || up_h > 127) { *why = "padding/dilation outside the im2col corner range"; return false; }
+  if ((d.S - 1) * d.dil_w > 255 || (d.R - 1) * d.dil_h > 255) { *why = "filter extent outside the im2col offset range"; return false; }
+  if (d.stride_h > 8 || d.stride_w > 8) { *why = "stride > 8"; return false; }
+  if ((long long)d.N * d.H * d.W * d.C < 131072) { *why = "activation tensor smaller than 128 KiB"; return false; }
+  return true;
+}
+
 }  // namespace
 
 bool umma_shape_eligible(const q8_conv_desc& d, const char** why) {
@@ -679,14 +689,7 @@ bool umma_shape_eligible(const q8_conv_desc& d, const char** why) {
   if (is_plain(d)) return true;
   HaloTile ht;
   const int P = conv_out_extent(d.H, d.pad_h, d.dil_h, d.R, d.stride_h), Q = conv_out_extent(d.W, d.pad_w, d.dil_w, d.S, d.stride_w);
-  if (choose_halo_tile(d, P, Q, &ht)) return true;
-  // im2col tensor maps: corners are 8-bit signed, tap offsets 8-bit unsigned, strides at most 8
-  const int up_w = d.pad_w - (d.S - 1) * d.dil_w, up_h = d.pad_h - (d.R - 1) * d.dil_h;
-  if (d.pad_w > 128 || d.pad_h > 128 || up_w < -128 || up_h < -128 || up_w > 127 || up_h > 127) { *why = "padding/dilation outside the im2col corner range"; return false; }
-  if ((d.S - 1) * d.dil_w > 255 || (d.R - 1) * d.dil_h > 255) { *why = "filter extent outside the im2col offset range"; return false; }
-  if (d.stride_h > 8 || d.stride_w > 8) { *why = "stride > 8"; return false; }
-  if ((long long)d.N * d.H * d.W * d.C < 131072) { *why = "activation tensor smaller than 128 KiB"; return false; }
-  return true;
+  return choose_halo_tile(d, P, Q, &ht) || im2col_open(d, why);
 }
 
 // Split-K plan: layers whose output tiles cannot occupy a quarter of the SMs split the reduction over
@@ -725,24 +728,39 @@ int narrow_bn(int bn, int K, int kgemm, long long m_tiles) {
 }
 }  // namespace
 
-namespace {
-constexpr int kPlanNoFit = -1000;  // internal: this tile shape needs more shared memory than an SM has
-int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_halo);
-
-// Tries tile shapes from the preferred one down: halo patches of dilated filters on wide channel blocks can
-// exceed shared memory, narrower channel blocks shrink them; im2col loads need the least.
-int launch_conv_umma_impl(const ConvArgs& a, int splits) {
-  static const struct { int bk_cap; bool halo; } kTries[] = {{128, true}, {64, true}, {32, true}, {128, false}, {64, false}};
-  for (const auto& t : kTries) {
-    const int rc = launch_conv_umma_plan(a, splits, t.bk_cap, t.halo);
-    if (rc != kPlanNoFit) return rc;
-  }
-  return fail(Q8_ERR_UNSUPPORTED, "conv_umma: no tile shape of this layer fits in shared memory");
-}
-}  // namespace
-
 bool rows_unaligned(const ConvArgs& a) {
   return (a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8) && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16 || (a.residual && !aligned16(a.residual)));
+}
+
+namespace {
+// How a layer runs: tiles, shared memory and pipeline depths.  Decided from the descriptor and the alignment of the
+// pointers alone, so that it can be asked for without a device.
+struct UmmaPlan {
+  UmmaParams p;
+  HaloTile ht;
+  int G, res_mode, pw, c_eff;
+  bool rows, paired, resident;
+  size_t dyn;
+};
+
+bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, UmmaPlan* plan);
+
+// Tries tile shapes from the preferred one down: halo patches of dilated filters on wide channel blocks can
+// exceed shared memory, narrower channel blocks shrink them; im2col loads need the least, where they are open.
+bool plan_conv(const ConvArgs& a, int splits, UmmaPlan* plan) {
+  static const struct { int bk_cap; bool halo; } kTries[] = {{128, true}, {64, true}, {32, true}, {128, false}, {64, false}};
+  const char* why;
+  for (const auto& t : kTries)
+    if ((t.halo || is_plain(a.d) || im2col_open(a.d, &why)) && plan_tiles(a, splits, t.bk_cap, t.halo, plan)) return true;
+  return false;
+}
+
+int launch_planned(const ConvArgs& a, int splits);
+}  // namespace
+
+bool umma_fits(const ConvArgs& a) {
+  UmmaPlan plan;
+  return plan_conv(a, 1, &plan);
 }
 
 int launch_conv_umma(const ConvArgs& a) {
@@ -768,30 +786,26 @@ int launch_conv_umma(const ConvArgs& a) {
     part.c_off = 0;
     part.bias = nullptr;
     part.residual = nullptr;
-    int rc = launch_conv_umma_impl(part, splits);
-    if (rc != Q8_OK) return rc;
-    return launch_splitk_reduce(a, splits);
+    const int rc = launch_planned(part, splits);
+    if (rc == Q8_OK) return launch_splitk_reduce(a, splits);
+    if (rc != kPlanNoFit) return rc;
   }
-  return launch_conv_umma_impl(a, 1);
+  return launch_planned(a, 1);
 }
 
 namespace {
-int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_halo) {
+bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, UmmaPlan* plan) {
   const q8_conv_desc& d = a.d;
-  const DriverFns& fn = driver_fns();
-  if (!fn.tiled || !fn.im2col) return fail(Q8_ERR_CUDA, "conv_umma: cuTensorMapEncode* entry points not available");
-  unsigned int* status = status_word_device_ptr();
-  if (!status) return fail(Q8_ERR_CUDA, "conv_umma: status word not available");
-
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   int res_mode = kResNone;
   if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResTma : (out8 ? kResRows : kResGlobal);
   // 8-bit rows off the 16-byte grid are moved by the epilogue warps, in both directions if in one
   const bool rows = out8 && (rows_unaligned(a) || res_mode == kResRows);
   if (rows && a.residual) res_mode = kResRows;
-  UmmaParams p;
+  UmmaParams& p = plan->p;
   memset(&p, 0, sizeof(p));
-  HaloTile ht = {0, 0, 0, 0, 0.0, 1, d.S, d.pad_w, 0};
+  HaloTile& ht = plan->ht;
+  ht = {0, 0, 0, 0, 0.0, 1, d.S, d.pad_w, 0};
   p.a_mode = is_plain(d) ? kAPlain : ((allow_halo && tune_env("Q8_HALO", 1, 0, 1) && choose_halo_tile(d, a.P, a.Q, &ht)) ? kAHalo : kAIm2col);
   const bool paired = p.a_mode == kAHalo && ht.sw == 2;  // input read as pixel pairs with 2C channels
   const int c_eff = paired ? 2 * d.C : d.C;
@@ -809,7 +823,6 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     const int want = tune_env("Q8_BN", BN, 16, 256);
     if (want % 16 == 0) BN = want;
   }
-  const CUtensorMapSwizzle swz = swizzle_for_bytes(BK);
   p.bn = BN; p.bk = BK; p.ksteps = BK / 32;
   p.P = a.P; p.Q = a.Q; p.PQ = a.P * a.Q; p.M = (int)a.M; p.K = d.K;
   p.stride_h = d.stride_h; p.stride_w = d.stride_w; p.pad_h = d.pad_h; p.pad_w = d.pad_w; p.dil_h = d.dil_h; p.dil_w = d.dil_w;
@@ -976,7 +989,7 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
     if (p.epi_split) p.nbuf = 2;  // one buffer per tile in flight; a CTA has at most two tiles
   }
   const unsigned buf_bytes = row_bytes + (unsigned)(p.epi_split ? p.nbuf : (p.cta2 ? G >> p.pair_shift : G) * p.nbuf) * p.tile8_bytes;
-  if (budget < bres_bytes + buf_bytes + min_pipe) return kPlanNoFit;
+  if (budget < bres_bytes + buf_bytes + min_pipe) return false;
   unsigned rest = budget - bres_bytes - buf_bytes;
   p.b_stages = 0;
   if (p.b_mode == kBRing) {
@@ -993,9 +1006,29 @@ int launch_conv_umma_plan(const ConvArgs& a, int splits, int bk_cap, bool allow_
   p.off_bufs = p.off_bring + (unsigned)p.b_stages * p.b_sub_bytes;
   p.off_chan = p.off_bufs + buf_bytes;
   size_t dyn = 1024u + p.off_chan + chan_bytes;
-  if (dyn > (size_t)(kSmemLimit - kStaticSmemReserve)) return kPlanNoFit;
+  if (dyn > (size_t)(kSmemLimit - kStaticSmemReserve)) return false;
   // at least 120 KiB so that one CTA owns an SM and with it the whole TMEM
-  if (dyn < 120 * 1024) dyn = 120 * 1024;
+  plan->dyn = dyn < 120 * 1024 ? 120 * 1024 : dyn;
+  plan->G = G; plan->res_mode = res_mode; plan->pw = pw; plan->c_eff = c_eff;
+  plan->rows = rows; plan->paired = paired; plan->resident = resident;
+  return true;
+}
+
+int launch_planned(const ConvArgs& a, int splits) {
+  const q8_conv_desc& d = a.d;
+  UmmaPlan plan;
+  if (!plan_conv(a, splits, &plan)) return kPlanNoFit;
+  const DriverFns& fn = driver_fns();
+  if (!fn.tiled || !fn.im2col) return fail(Q8_ERR_CUDA, "conv_umma: cuTensorMapEncode* entry points not available");
+  unsigned int* status = status_word_device_ptr();
+  if (!status) return fail(Q8_ERR_CUDA, "conv_umma: status word not available");
+  UmmaParams& p = plan.p;
+  const HaloTile& ht = plan.ht;
+  const int BK = p.bk, BN = p.bn, G = plan.G, res_mode = plan.res_mode, pw = plan.pw, c_eff = plan.c_eff;
+  const bool rows = plan.rows, paired = plan.paired, resident = plan.resident;
+  const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
+  const size_t dyn = plan.dyn;
+  const CUtensorMapSwizzle swz = swizzle_for_bytes(BK);
 
   // ---- tensor maps
   CUtensorMap tmA, tmB, tmRes, tmY;

@@ -57,6 +57,10 @@ struct ConvArgs {
 // Eligibility of the tensor-core kernel for a descriptor (pointer alignment checked at launch).
 bool umma_shape_eligible(const q8_conv_desc& d, const char** why);
 bool rows_unaligned(const ConvArgs& a);  // 8-bit output or residual rows that TMA cannot address
+// Whether one of its tile shapes fits the layer (decided without a device).
+bool umma_fits(const ConvArgs& a);
+// kPlanNoFit (nothing recorded as an error) where none does, else a q8_status.
+constexpr int kPlanNoFit = -1000;
 int launch_conv_umma(const ConvArgs& a);
 // Number of split-K parts the tensor-core kernel uses for this layer when it is given a workspace of
 // splits * M * K int32 (1: none).  Host only.

@@ -40,3 +40,23 @@ def test_plan_matches_oracle(q8, case):
         y = q8.q8_conv2d(d, *args, rd, 0.37 if res else 0.0)
     q8.q8_read_status()
     assert np.array_equal(y.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("K", [32, 33])
+@pytest.mark.parametrize("ytype", [U8, S8])
+def test_layer_that_no_tile_of_the_tma_fed_kernel_fits(q8, K, ytype):
+    """Filter rows 70 apart with stride 2: a halo patch exceeds shared memory, and im2col maps end at 128 rows."""
+    g = np.random.default_rng(K)
+    x = g.integers(0, 256, (1, 200, 128, 16), dtype=np.uint8)
+    w = g.integers(-128, 128, (K, 3, 1, 16)).astype(np.int8)
+    scale = np.float32(1e-3)
+    want = o.conv2d(x, w, None, scale, stride=(2, 1), dil=(70, 1), relu=True, y_type=o.U8 if ytype == U8 else o.S8, threads=8)
+    d = q8.make_conv_desc(1, 200, 128, 16, K, 3, 1, (2, 1), (0, 0), (70, 1), U8, U8, ytype, True)
+    args = [torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), None, torch.tensor([scale], device="cuda")]
+    y = q8.q8_conv2d(d, *args)
+    q8.q8_read_status()
+    assert np.array_equal(y.cpu().numpy(), want)
+    d.algo = q8.Q8_ALGO_UMMA
+    with pytest.raises(q8.Q8Error) as e:
+        q8.q8_conv2d(d, *args)
+    assert e.value.code == 2
