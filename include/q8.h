@@ -193,9 +193,26 @@ typedef struct q8_conv_desc {
  * Host only. */
 int q8_conv2d_workspace_bytes(const q8_conv_desc* d, size_t* bytes);
 
-/* Whether q8_conv2d would take the TMA-fed kernel for `d`: writes Q8_ALGO_UMMA if so, else Q8_ALGO_DIRECT.
- * Host only. */
+/* Whether q8_conv2d would take the TMA-fed kernel for `d`, given 16-byte aligned pointers and no residual: writes
+ * Q8_ALGO_UMMA if so, else Q8_ALGO_DIRECT (the call then takes another kernel, or with d->algo = Q8_ALGO_UMMA is
+ * refused).  Host only. */
 int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo);
+
+/* How q8_conv2d would run `d`, given 16-byte aligned pointers, q8_conv2d_workspace_bytes() bytes of scratch and a
+ * residual or none: an aid for tests and tuning, whose answers may change with the library.  Host only (without a
+ * device the plan is that of a B200).  Errors: Q8_ERR_INVALID_ARG; Q8_ERR_UNSUPPORTED where the call is refused. */
+typedef enum q8_conv_kernel { Q8_KERNEL_DIRECT = 0, Q8_KERNEL_GATHER = 1, Q8_KERNEL_TMA = 2 } q8_conv_kernel;
+typedef struct q8_conv_plan {
+  int32_t kernel;           /* q8_conv_kernel; the fields below are zero unless it is Q8_KERNEL_TMA */
+  int32_t tile_n;           /* output channels of a tile */
+  int32_t operand;          /* activations as 0: a matrix, 1: im2col loads, 2: halo patches */
+  int32_t splits;           /* parts of the reduction, 1: not split */
+  int32_t weights;          /* 0: staged with the activations, 1: resident in shared memory, 2: in a ring of their own */
+  int32_t cta_pair;         /* 1: CTA pairs share the weights of a tile */
+  int32_t shared_groups;    /* epilogue groups that share the columns of a tile */
+  int32_t moved_rows;       /* 1: 8-bit rows off the 16-byte grid, moved by the epilogue warps */
+} q8_conv_plan;
+int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan);
 
 /* x: device NHWC (x_type).  w: device KRSC s8.  bias: device s32[K] or NULL.
  * scale: device fp32[scale_count].  residual: device [N,P,Q,K] dense (res_type)

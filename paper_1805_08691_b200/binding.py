@@ -14,13 +14,14 @@ from . import build as _build
 
 Q8_U8, Q8_S8, Q8_S32, Q8_F32 = 0, 1, 2, 3
 Q8_ALGO_AUTO, Q8_ALGO_UMMA, Q8_ALGO_DIRECT = 0, 1, 2
+Q8_KERNEL_DIRECT, Q8_KERNEL_GATHER, Q8_KERNEL_TMA = 0, 1, 2
 Q8_OK = 0
 STATUS_NAMES = {0: "Q8_OK", 1: "Q8_ERR_INVALID_ARG", 2: "Q8_ERR_UNSUPPORTED", 3: "Q8_ERR_ALIGNMENT",
                 4: "Q8_ERR_WORKSPACE", 5: "Q8_ERR_CUDA", 6: "Q8_ERR_TIMEOUT", 7: "Q8_ERR_NONFINITE"}
 TORCH_DTYPES = {Q8_U8: torch.uint8, Q8_S8: torch.int8, Q8_S32: torch.int32, Q8_F32: torch.float32}
 EXPORTS = ["q8_version", "q8_last_error", "q8_read_status", "q8_calibrate_maxabs", "q8_factor", "q8_requant_scale",
            "q8_bias_factor", "q8_quantize", "q8_quantize_pad_channels", "q8_dequantize", "q8_fold_bn",
-           "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d", "q8_static_workspace_bytes",
+           "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d_query_plan", "q8_conv2d", "q8_static_workspace_bytes",
            "q8_conv2d_static_workspace", "q8_conv2d_then_1x1_supported", "q8_conv2d_then_1x1", "q8_int8_mma_rate", "q8_selftest_bounded_wait", "q8_concat", "q8_concat_branch", "q8_calibrate_maxabs_rows", "q8_quantize_rows", "q8_quantize_pad_image", "q8_pool_out_extent",
            "q8_maxpool2d", "q8_avgpool2d", "q8_l2norm", "q8_add_relu_quantize", "q8_detection_output_workspace_bytes",
            "q8_detection_output", "q8_record_begin", "q8_record_end", "q8_record_replay", "q8_record_free"]
@@ -36,6 +37,11 @@ class q8_conv_desc(C.Structure):
     _fields_ = [(n, C.c_int32) for n in (
         "N", "H", "W", "C", "K", "R", "S", "stride_h", "stride_w", "pad_h", "pad_w", "dil_h", "dil_w",
         "x_type", "res_type", "y_type", "relu", "scale_count", "y_ldc", "y_c_offset", "algo")]
+
+
+class q8_conv_plan(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in (
+        "kernel", "tile_n", "operand", "splits", "weights", "cta_pair", "shared_groups", "moved_rows")]
 
 
 def _load():
@@ -65,6 +71,7 @@ lib.q8_dequantize.argtypes = [_vp, _i, _sz, _f, _vp, _vp]
 lib.q8_fold_bn.argtypes = [_vp] * 6 + [C.c_double, _i, _sz, _vp, _vp, _vp]
 lib.q8_conv2d_workspace_bytes.argtypes = [C.POINTER(q8_conv_desc), C.POINTER(_sz)]
 lib.q8_conv2d_query_algo.argtypes = [C.POINTER(q8_conv_desc), _ip]
+lib.q8_conv2d_query_plan.argtypes = [C.POINTER(q8_conv_desc), _i, C.POINTER(q8_conv_plan)]
 lib.q8_conv2d.argtypes = [C.POINTER(q8_conv_desc), _vp, _vp, _vp, _vp, _vp, _f, _vp, _vp, _sz, _vp]
 lib.q8_static_workspace_bytes.argtypes = []
 lib.q8_selftest_bounded_wait.argtypes = [C.c_uint, _vp]
@@ -244,6 +251,12 @@ def q8_conv2d_query_algo(d):
     a = C.c_int()
     _check(lib.q8_conv2d_query_algo(C.byref(d), C.byref(a)))
     return a.value
+
+
+def q8_conv2d_query_plan(d, residual=False):
+    p = q8_conv_plan()
+    _check(lib.q8_conv2d_query_plan(C.byref(d), int(residual), C.byref(p)))
+    return p
 
 
 def q8_conv2d(d, x, w, bias, scale, residual=None, residual_scale=0.0, y=None, workspace=None):

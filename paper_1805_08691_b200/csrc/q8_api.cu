@@ -101,6 +101,45 @@ bool short_rows(const ConvArgs& a) {
   const long long products = (long long)a.d.R * a.d.S * a.d.C;
   return products <= 64 && (a.d.K <= 16 ? products * a.M <= 4000000 : a.d.K <= 32 && a.M <= 128);
 }
+
+// The kernel a call takes, from its descriptor and the alignment of its pointers; `why` is set where the TMA-fed one is
+// not taken.  That kernel may still find no tile that fits (umma_fits, or kPlanNoFit from its launch); route_off_tma then
+// says what takes its place.
+enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRouteTma };
+
+Route route_off_tma(const ConvArgs& a) {
+  if (a.d.algo == Q8_ALGO_UMMA) return kRouteRefused;
+  return a.d.K <= 4096 && !tiny_call(a) ? kRouteGather : kRouteDirect;
+}
+
+Route conv_route(const ConvArgs& a, const char** why) {
+  const q8_conv_desc& d = a.d;
+  if (d.algo == Q8_ALGO_DIRECT) return kRouteDirect;
+  if (!umma_shape_eligible(d, why)) return route_off_tma(a);
+  if (!aligned16(a.x) || !aligned16(a.w)) { *why = "x or w not 16-byte aligned"; return route_off_tma(a); }
+  const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
+  if (d.algo == Q8_ALGO_UMMA || !out8) {
+    if (out8 && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16)) { *why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; return route_off_tma(a); }
+    if (a.residual && !aligned16(a.residual)) { *why = "residual not 16-byte aligned"; return route_off_tma(a); }
+  } else if (rows_unaligned(a) && (tiny_call(a) || short_rows(a))) {
+    return route_off_tma(a);  // (other 8-bit rows off the 16-byte grid: the epilogue warps move them, see rows_out)
+  }
+  return kRouteTma;
+}
+
+// The call a descriptor describes, with pointers that stand for 16-byte aligned ones.
+int described_call(const q8_conv_desc* d, bool residual, ConvArgs* a) {
+  *a = ConvArgs{};
+  const int rc = validate_desc(d, &a->P, &a->Q);
+  if (rc != Q8_OK) return rc;
+  a->d = *d;
+  a->M = (long long)d->N * a->P * a->Q;
+  a->x = reinterpret_cast<const void*>(256); a->w = reinterpret_cast<const int8_t*>(256); a->y = reinterpret_cast<void*>(256);
+  a->residual = residual && d->y_type != Q8_S32 ? reinterpret_cast<const void*>(256) : nullptr;
+  a->ldc = d->y_ldc == 0 ? d->K : d->y_ldc;
+  a->c_off = d->y_c_offset;
+  return Q8_OK;
+}
 }  // namespace
 }  // namespace q8
 
@@ -146,13 +185,27 @@ int q8_conv2d_workspace_bytes(const q8_conv_desc* d, size_t* bytes) {
 
 int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo) {
   clear_error();
-  int P, Q;
-  int rc = validate_desc(d, &P, &Q);
+  ConvArgs a;
+  const int rc = described_call(d, false, &a);
   if (rc != Q8_OK) return rc;
   if (!algo) return fail(Q8_ERR_INVALID_ARG, "q8_conv2d_query_algo: null pointer");
   const char* why = nullptr;
-  if (d->algo == Q8_ALGO_DIRECT) *algo = Q8_ALGO_DIRECT;
-  else *algo = umma_shape_eligible(*d, &why) ? Q8_ALGO_UMMA : Q8_ALGO_DIRECT;
+  *algo = conv_route(a, &why) == kRouteTma && umma_fits(a) ? Q8_ALGO_UMMA : Q8_ALGO_DIRECT;
+  return Q8_OK;
+}
+
+int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan) {
+  clear_error();
+  ConvArgs a;
+  const int rc = described_call(d, residual != 0, &a);
+  if (rc != Q8_OK) return rc;
+  if (!plan) return fail(Q8_ERR_INVALID_ARG, "q8_conv2d_query_plan: null pointer");
+  memset(plan, 0, sizeof(*plan));
+  const char* why = "";
+  Route route = conv_route(a, &why);
+  if (route == kRouteTma && !umma_describe(a, plan)) { route = route_off_tma(a); why = "no tile shape of this layer fits in shared memory"; }
+  if (route == kRouteRefused) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
+  plan->kernel = route == kRouteTma ? Q8_KERNEL_TMA : (route == kRouteGather ? Q8_KERNEL_GATHER : Q8_KERNEL_DIRECT);
   return Q8_OK;
 }
 
@@ -176,27 +229,16 @@ int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32
   a.workspace = workspace; a.workspace_bytes = workspace_bytes;
   a.stream = as_stream(stream);
 
-  if (d->algo == Q8_ALGO_DIRECT) return launch_conv_direct(a);
   const char* why = "";
-  bool ok = umma_shape_eligible(*d, &why);
-  if (ok) {
-    const bool out8 = d->y_type == Q8_U8 || d->y_type == Q8_S8;
-    if (!aligned16(x) || !aligned16(w)) { ok = false; why = "x or w not 16-byte aligned"; }
-    else if (d->algo == Q8_ALGO_UMMA || !out8) {
-      if (out8 && (!aligned16(y) || a.ldc % 16 || a.c_off % 16)) { ok = false; why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; }
-      else if (a.residual && !aligned16(a.residual)) { ok = false; why = "residual not 16-byte aligned"; }
-    }
-    // (8-bit rows off the 16-byte grid: the epilogue warps move them, see rows_out)
-    else if (rows_unaligned(a) && (tiny_call(a) || short_rows(a))) ok = false;
-  }
-  if (ok) {
+  Route route = conv_route(a, &why);
+  if (route == kRouteTma) {
     rc = launch_conv_umma(a);
     if (rc != kPlanNoFit) return rc;
+    route = route_off_tma(a);
     why = "no tile shape of this layer fits in shared memory";
   }
-  if (d->algo == Q8_ALGO_UMMA) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
-  if (d->K <= 4096 && !tiny_call(a)) return launch_conv_gather(a);
-  return launch_conv_direct(a);
+  if (route == kRouteRefused) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
+  return route == kRouteGather ? launch_conv_gather(a) : launch_conv_direct(a);
 }
 
 int q8_conv2d_then_1x1_supported(const q8_conv_desc* d1, const q8_conv_desc* d2, int* supported) {

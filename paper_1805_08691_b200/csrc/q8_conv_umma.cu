@@ -763,9 +763,11 @@ bool umma_fits(const ConvArgs& a) {
   return plan_conv(a, 1, &plan);
 }
 
-int launch_conv_umma(const ConvArgs& a) {
+namespace {
+// Parts of the reduction a call runs in, given scratch for them.
+int call_splits(const ConvArgs& a) {
   const q8_conv_desc& d = a.d;
-  int splits = rows_unaligned(a) ? 1 : umma_plan_splits(d, a.P, a.Q, a.M);
+  int splits = rows_unaligned(a) || d.y_type == Q8_S32 ? 1 : umma_plan_splits(d, a.P, a.Q, a.M);
   if (splits > 1) {
     // Narrow tiles against a split of the default ones, by the operand bytes a CTA streams (~60 per cycle); a split
     // pays ~6000 cycles for its second kernel.
@@ -775,19 +777,44 @@ int launch_conv_umma(const ConvArgs& a) {
     const double t_narrow = (double)kg * (kBM + narrow_bn(bn, d.K, kg, m_tiles)) / 60.0;
     if (t_narrow <= t_split) splits = 1;
   }
-  const size_t need = splits > 1 ? (size_t)splits * (size_t)a.M * d.K * sizeof(int) : 0;
-  if (splits > 1 && d.y_type != Q8_S32 && a.workspace && a.workspace_bytes >= need && aligned16(a.workspace)) {
-    // pass 1: raw partial accumulators of every split into the workspace; pass 2: sum, bias, epilogue
-    ConvArgs part = a;
-    part.d.y_type = Q8_S32;
-    part.d.relu = 0;
-    part.y = a.workspace;
-    part.ldc = d.K;
-    part.c_off = 0;
-    part.bias = nullptr;
-    part.residual = nullptr;
-    const int rc = launch_planned(part, splits);
-    if (rc == Q8_OK) return launch_splitk_reduce(a, splits);
+  return splits;
+}
+
+// The first pass of a split: raw partial accumulators of every part into the workspace.
+ConvArgs partial_call(const ConvArgs& a) {
+  ConvArgs part = a;
+  part.d.y_type = Q8_S32;
+  part.d.relu = 0;
+  part.y = a.workspace;
+  part.ldc = a.d.K;
+  part.c_off = 0;
+  part.bias = nullptr;
+  part.residual = nullptr;
+  return part;
+}
+}  // namespace
+
+bool umma_describe(const ConvArgs& a, q8_conv_plan* out) {
+  UmmaPlan plan;
+  int splits = call_splits(a);
+  if (splits > 1 && !plan_conv(partial_call(a), splits, &plan)) splits = 1;
+  if (splits == 1 && !plan_conv(a, 1, &plan)) return false;
+  out->tile_n = plan.p.bn;
+  out->operand = plan.p.a_mode;
+  out->splits = splits;
+  out->weights = plan.p.b_mode;
+  out->cta_pair = plan.p.cta2;
+  out->shared_groups = plan.p.cta2 ? 1 << plan.p.pair_shift : (plan.p.epi_split ? plan.G : 1);
+  out->moved_rows = plan.rows;
+  return true;
+}
+
+int launch_conv_umma(const ConvArgs& a) {
+  const int splits = call_splits(a);
+  const size_t need = splits > 1 ? (size_t)splits * (size_t)a.M * a.d.K * sizeof(int) : 0;
+  if (splits > 1 && a.workspace && a.workspace_bytes >= need && aligned16(a.workspace)) {
+    const int rc = launch_planned(partial_call(a), splits);
+    if (rc == Q8_OK) return launch_splitk_reduce(a, splits);  // pass 2: sum, bias, epilogue
     if (rc != kPlanNoFit) return rc;
   }
   return launch_planned(a, 1);

@@ -57,8 +57,9 @@ struct ConvArgs {
 // Eligibility of the tensor-core kernel for a descriptor (pointer alignment checked at launch).
 bool umma_shape_eligible(const q8_conv_desc& d, const char** why);
 bool rows_unaligned(const ConvArgs& a);  // 8-bit output or residual rows that TMA cannot address
-// Whether one of its tile shapes fits the layer (decided without a device).
+// Whether one of its tile shapes fits the layer, and which (decided without a device).
 bool umma_fits(const ConvArgs& a);
+bool umma_describe(const ConvArgs& a, q8_conv_plan* out);
 // kPlanNoFit (nothing recorded as an error) where none does, else a q8_status.
 constexpr int kPlanNoFit = -1000;
 int launch_conv_umma(const ConvArgs& a);

@@ -97,6 +97,43 @@ def test_kernel_selection_rules():
     assert q8.q8_conv2d_query_algo(q8.make_conv_desc(32, 56, 56, 64, 64, 3, 3, pad=(1, 1), algo=q8.Q8_ALGO_DIRECT)) == q8.Q8_ALGO_DIRECT
 
 
+D, G, T = q8.Q8_KERNEL_DIRECT, q8.Q8_KERNEL_GATHER, q8.Q8_KERNEL_TMA
+U8, S8, S32, F32 = q8.Q8_U8, q8.Q8_S8, q8.Q8_S32, q8.Q8_F32
+
+ROUTES = [
+    # kernel, N,H,W,C,K,R,S, further descriptor fields
+    (T, 32, 56, 56, 64, 64, 3, 3, dict(pad=(1, 1))),
+    (T, 32, 56, 56, 64, 250, 1, 1, {}),                                # 8-bit rows off the 16-byte grid: moved by the warps
+    (T, 32, 56, 56, 64, 256, 1, 1, dict(y_ldc=300, y_c_offset=13)),
+    (G, 1, 56, 56, 64, 9, 1, 1, {}),                                   # ... unless short, with a short reduction
+    (T, 1, 56, 56, 64, 9, 1, 1, dict(y_type=F32)),
+    (D, 1, 8, 8, 16, 9, 1, 1, {}),                                     # ... or tiny
+    (T, 1, 8, 8, 16, 16, 1, 1, {}),
+    (G, 2, 28, 28, 100, 120, 3, 3, dict(pad=(1, 1))),
+    (D, 1, 8, 8, 3, 8, 1, 1, {}),
+    (D, 2, 9, 9, 16, 5000, 1, 1, {}),
+    (G, 1, 200, 128, 16, 32, 3, 1, dict(stride=(2, 1), dil=(70, 1))),  # no tile fits
+]
+
+
+@pytest.mark.parametrize("route", ROUTES, ids=lambda r: "x".join(map(str, r[1:8])) + "".join(f"_{v}" for v in r[8].values()))
+def test_queries_follow_the_dispatch(route):
+    kernel, fields, more = route[0], route[1:8], route[8]
+    d = q8.make_conv_desc(*fields, **more)
+    assert q8.q8_conv2d_query_plan(d).kernel == kernel
+    assert (q8.q8_conv2d_query_algo(d) == q8.Q8_ALGO_UMMA) == (kernel == T)
+    d.algo = q8.Q8_ALGO_DIRECT
+    assert q8.q8_conv2d_query_plan(d).kernel == D and q8.q8_conv2d_query_algo(d) == q8.Q8_ALGO_DIRECT
+    # asked for by name, the TMA-fed kernel also refuses rows off the grid
+    d.algo = q8.Q8_ALGO_UMMA
+    ldc = d.y_ldc or d.K
+    if kernel == T and (d.y_type == F32 or (ldc % 16 == 0 and d.y_c_offset % 16 == 0)):
+        assert q8.q8_conv2d_query_plan(d).kernel == T and q8.q8_conv2d_query_algo(d) == q8.Q8_ALGO_UMMA
+    elif kernel == T or d.C % 16 or d.K > 4096 or d.y_type in (U8, S8):
+        assert q8.q8_conv2d_query_algo(d) == q8.Q8_ALGO_DIRECT
+        assert _code(q8.q8_conv2d_query_plan, d) == 2
+
+
 def test_recording_requests_are_checked_on_the_host():
     assert _code(q8.q8_record_begin, 0) == 1
     assert q8.lib.q8_record_replay(None, None) == 1
