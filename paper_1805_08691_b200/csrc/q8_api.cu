@@ -109,7 +109,7 @@ enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRouteTma };
 
 Route route_off_tma(const ConvArgs& a) {
   if (a.d.algo == Q8_ALGO_UMMA) return kRouteRefused;
-  return a.d.K <= 4096 && !tiny_call(a) ? kRouteGather : kRouteDirect;
+  return gather_addressable(a.d) && !tiny_call(a) ? kRouteGather : kRouteDirect;
 }
 
 Route conv_route(const ConvArgs& a, const char** why) {

@@ -392,6 +392,14 @@ int launch_gather_variant(const GatherParams& p, size_t dyn, cudaStream_t stream
 
 }  // namespace
 
+// The channel arrays of 4096 outputs fit beside the stages.  Positions in a row of input pixels, padding included, are
+// 32-bit byte offsets, and rows past the last pixel are told by a row number below -2^28; wider images and filters stay
+// with the direct kernel, whose addresses are 64-bit.
+bool gather_addressable(const q8_conv_desc& d) {
+  const long long row = ((long long)d.W + 2ll * d.pad_w + (long long)d.S * d.dil_w) * d.C;
+  return d.K <= 4096 && row < (1ll << 30) && d.H + 2ll * d.pad_h < (1ll << 28) && (long long)d.R * d.dil_h < (1ll << 28);
+}
+
 int launch_conv_gather(const ConvArgs& a) {
   const q8_conv_desc& d = a.d;
   GatherParams p;

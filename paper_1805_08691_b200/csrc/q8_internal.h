@@ -69,8 +69,9 @@ int umma_plan_splits(const q8_conv_desc& d, int P, int Q, long long M);
 // Sums the split-K partial accumulators in a.workspace, adds the bias and applies the epilogue of `a`.
 int launch_splitk_reduce(const ConvArgs& a, int splits);
 int launch_conv_direct(const ConvArgs& a);
-// Tensor-core kernel that gathers its operands byte by byte (q8_conv_gather.cu): any alignment, any shape up to 4096
-// output channels.
+// Tensor-core kernel that gathers its operands byte by byte (q8_conv_gather.cu): any alignment, any shape whose rows it can
+// address.
+bool gather_addressable(const q8_conv_desc& d);
 int launch_conv_gather(const ConvArgs& a);
 // A stride-1 convolution followed by a 1x1 convolution over its output, in one launch (q8_conv_fused.cu).
 // Descriptors validated by the caller; `why` names the first reason a pair cannot run fused.

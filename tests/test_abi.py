@@ -113,6 +113,10 @@ ROUTES = [
     (D, 1, 8, 8, 3, 8, 1, 1, {}),
     (D, 2, 9, 9, 16, 5000, 1, 1, {}),
     (G, 1, 200, 128, 16, 32, 3, 1, dict(stride=(2, 1), dil=(70, 1))),  # no tile fits
+    (G, 1, 1, 1 << 19, 1025, 8, 1, 1, dict(stride=(1, 1 << 14))),
+    (D, 1, 1, 1 << 21, 1025, 8, 1, 1, dict(stride=(1, 1 << 17))),      # rows of more than 2^30 bytes, with and
+    (D, 1, 1, 1000, 1025, 8, 1, 1, dict(stride=(1, 1 << 17), pad=(0, 1 << 20))),   # without their padding
+    (D, 1, 300, 8, 5, 64, 2, 2, dict(dil=(1 << 28, 1), pad=(1 << 27, 0))),        # filter rows 2^28 apart
 ]
 
 
