@@ -170,16 +170,13 @@ int q8_read_status(void* stream) {
 
 int q8_conv2d_workspace_bytes(const q8_conv_desc* d, size_t* bytes) {
   clear_error();
-  int P, Q;
-  int rc = validate_desc(d, &P, &Q);
+  ConvArgs a;
+  const int rc = described_call(d, false, &a);
   if (rc != Q8_OK) return rc;
   if (!bytes) return fail(Q8_ERR_INVALID_ARG, "q8_conv2d_workspace_bytes: null pointer");
-  *bytes = 0;
-  if (d->algo != Q8_ALGO_DIRECT && d->y_type != Q8_S32) {
-    const long long M = (long long)d->N * P * Q;
-    const int splits = umma_plan_splits(*d, P, Q, M);
-    if (splits > 1) *bytes = (size_t)splits * (size_t)M * (size_t)d->K * sizeof(int32_t);
-  }
+  const char* why = nullptr;
+  const int splits = conv_route(a, &why) == kRouteTma ? umma_splits(a) : 1;
+  *bytes = splits > 1 ? (size_t)splits * (size_t)a.M * (size_t)d->K * sizeof(int32_t) : 0;
   return Q8_OK;
 }
 

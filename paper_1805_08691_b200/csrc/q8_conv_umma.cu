@@ -692,26 +692,6 @@ bool umma_shape_eligible(const q8_conv_desc& d, const char** why) {
   return choose_halo_tile(d, P, Q, &ht) || im2col_open(d, why);
 }
 
-// Split-K plan: layers whose output tiles cannot occupy a quarter of the SMs split the reduction over
-// (tap, channel block) iterations into `splits` equal parts; every part writes raw int32 partial sums
-// (integer addition is associative, so the result stays bit exact).  Only the plain and im2col operand
-// paths split.  Returns 1 when the layer runs unsplit.
-int umma_plan_splits(const q8_conv_desc& d, int P, int Q, long long M) {
-  if (!umma_shape_eligible(d, nullptr)) return 1;
-  HaloTile ht;
-  if (!is_plain(d) && choose_halo_tile(d, P, Q, &ht)) return 1;
-  const int BK = pick_bk(d.C), BN = pick_bn(d.K, d.R * d.S * d.C);
-  const long long tiles = ((M + kBM - 1) / kBM) * ((d.K + BN - 1) / BN);
-  const int k_iters = d.R * d.S * ((d.C + BK - 1) / BK);
-  const int sms = sm_count();
-  // a split costs a second (small) kernel and the partial-sum traffic: it pays once most SMs would idle
-  if (tiles * 4 > sms) return 1;
-  int best = 1;
-  for (int sp = 2; sp <= 16 && tiles * sp <= sms; ++sp)
-    if (k_iters % sp == 0 && k_iters / sp >= 4) best = sp;
-  return best;
-}
-
 namespace {
 // Tile width of a launch whose tiles of the default width would leave SMs without work: the narrowest of 16, 32, 64 and
 // 128 columns that still gives every tile an SM of its own, else the default.  Such a launch lasts as long as one CTA
@@ -764,22 +744,6 @@ bool umma_fits(const ConvArgs& a) {
 }
 
 namespace {
-// Parts of the reduction a call runs in, given scratch for them.
-int call_splits(const ConvArgs& a) {
-  const q8_conv_desc& d = a.d;
-  int splits = rows_unaligned(a) || d.y_type == Q8_S32 ? 1 : umma_plan_splits(d, a.P, a.Q, a.M);
-  if (splits > 1) {
-    // Narrow tiles against a split of the default ones, by the operand bytes a CTA streams (~60 per cycle); a split
-    // pays ~6000 cycles for its second kernel.
-    const int bn = pick_bn(d.K, d.R * d.S * d.C), kg = d.R * d.S * d.C;
-    const long long m_tiles = (a.M + kBM - 1) / kBM;
-    const double t_split = (double)kg / splits * (kBM + bn) / 60.0 + 6000.0;
-    const double t_narrow = (double)kg * (kBM + narrow_bn(bn, d.K, kg, m_tiles)) / 60.0;
-    if (t_narrow <= t_split) splits = 1;
-  }
-  return splits;
-}
-
 // The first pass of a split: raw partial accumulators of every part into the workspace.
 ConvArgs partial_call(const ConvArgs& a) {
   ConvArgs part = a;
@@ -792,13 +756,44 @@ ConvArgs partial_call(const ConvArgs& a) {
   part.residual = nullptr;
   return part;
 }
+
+// Split-K plan: layers whose output tiles cannot occupy a quarter of the SMs split the reduction over
+// (tap, channel block) iterations into equal parts; every part writes raw int32 partial sums (integer addition is
+// associative, so the result stays bit exact).  Only the plain and im2col operand paths split.  Returns the parts a call
+// runs in, given scratch for them: 1 where it runs unsplit.
+int split_parts(const ConvArgs& a) {
+  const q8_conv_desc& d = a.d;
+  if (d.y_type == Q8_S32 || rows_unaligned(a) || !umma_shape_eligible(d, nullptr)) return 1;
+  HaloTile ht;
+  if (!is_plain(d) && choose_halo_tile(d, a.P, a.Q, &ht)) return 1;
+  const int kg = d.R * d.S * d.C, BK = pick_bk(d.C), BN = pick_bn(d.K, kg);
+  const long long m_tiles = (a.M + kBM - 1) / kBM, tiles = m_tiles * ((d.K + BN - 1) / BN);
+  const int k_iters = d.R * d.S * ((d.C + BK - 1) / BK);
+  const int sms = sm_count();
+  // a split costs a second (small) kernel and the partial-sum traffic: it pays once most SMs would idle
+  if (tiles * 4 > sms) return 1;
+  int splits = 1;
+  for (int sp = 2; sp <= 16 && tiles * sp <= sms; ++sp)
+    if (k_iters % sp == 0 && k_iters / sp >= 4) splits = sp;
+  if (splits == 1) return 1;
+  // Narrow tiles against the split of the default ones, by the operand bytes a CTA streams (~60 per cycle); a split
+  // pays ~6000 cycles for its second kernel.
+  const double t_split = (double)kg / splits * (kBM + BN) / 60.0 + 6000.0;
+  const double t_narrow = (double)kg * (kBM + narrow_bn(BN, d.K, kg, m_tiles)) / 60.0;
+  return t_narrow <= t_split ? 1 : splits;
+}
 }  // namespace
+
+int umma_splits(const ConvArgs& a) {
+  const int splits = split_parts(a);
+  UmmaPlan plan;
+  return splits > 1 && plan_conv(partial_call(a), splits, &plan) ? splits : 1;
+}
 
 bool umma_describe(const ConvArgs& a, q8_conv_plan* out) {
   UmmaPlan plan;
-  int splits = call_splits(a);
-  if (splits > 1 && !plan_conv(partial_call(a), splits, &plan)) splits = 1;
-  if (splits == 1 && !plan_conv(a, 1, &plan)) return false;
+  const int splits = umma_splits(a);
+  if (!plan_conv(splits > 1 ? partial_call(a) : a, splits, &plan)) return false;
   out->tile_n = plan.p.bn;
   out->operand = plan.p.a_mode;
   out->splits = splits;
@@ -810,9 +805,8 @@ bool umma_describe(const ConvArgs& a, q8_conv_plan* out) {
 }
 
 int launch_conv_umma(const ConvArgs& a) {
-  const int splits = call_splits(a);
-  const size_t need = splits > 1 ? (size_t)splits * (size_t)a.M * a.d.K * sizeof(int) : 0;
-  if (splits > 1 && a.workspace && a.workspace_bytes >= need && aligned16(a.workspace)) {
+  const int splits = a.workspace && aligned16(a.workspace) ? split_parts(a) : 1;
+  if (splits > 1 && a.workspace_bytes >= (size_t)splits * (size_t)a.M * a.d.K * sizeof(int)) {
     const int rc = launch_planned(partial_call(a), splits);
     if (rc == Q8_OK) return launch_splitk_reduce(a, splits);  // pass 2: sum, bias, epilogue
     if (rc != kPlanNoFit) return rc;

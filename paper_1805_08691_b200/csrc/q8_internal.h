@@ -63,9 +63,9 @@ bool umma_describe(const ConvArgs& a, q8_conv_plan* out);
 // kPlanNoFit (nothing recorded as an error) where none does, else a q8_status.
 constexpr int kPlanNoFit = -1000;
 int launch_conv_umma(const ConvArgs& a);
-// Number of split-K parts the tensor-core kernel uses for this layer when it is given a workspace of
+// Number of split-K parts the TMA-fed kernel uses for this call when it is given a workspace of
 // splits * M * K int32 (1: none).  Host only.
-int umma_plan_splits(const q8_conv_desc& d, int P, int Q, long long M);
+int umma_splits(const ConvArgs& a);
 // Sums the split-K partial accumulators in a.workspace, adds the bias and applies the epilogue of `a`.
 int launch_splitk_reduce(const ConvArgs& a, int splits);
 int launch_conv_direct(const ConvArgs& a);

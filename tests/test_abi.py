@@ -138,6 +138,16 @@ def test_queries_follow_the_dispatch(route):
         assert _code(q8.q8_conv2d_query_plan, d) == 2
 
 
+@pytest.mark.parametrize("shape,parts", [((64, 1, 1, 8192, 1008, 1, 1), 16), ((64, 1, 1, 2048, 1008, 1, 1), 1), ((1, 14, 14, 1024, 256, 1, 1), 1),
+                                         ((1, 64, 74, 2048, 256, 1, 1), 1), ((8, 7, 7, 6144, 512, 1, 1), 12), ((2, 10, 10, 8192, 9, 1, 1), 1)])
+def test_scratch_is_asked_for_by_the_layers_that_split(shape, parts):
+    d = q8.make_conv_desc(*shape)
+    assert q8.q8_conv2d_query_plan(d).splits == parts
+    assert q8.q8_conv2d_workspace_bytes(d) == (parts * shape[0] * shape[1] * shape[2] * shape[4] * 4 if parts > 1 else 0)
+    d.y_type, d.relu = S32, 0
+    assert q8.q8_conv2d_workspace_bytes(d) == 0
+
+
 def test_recording_requests_are_checked_on_the_host():
     assert _code(q8.q8_record_begin, 0) == 1
     assert q8.lib.q8_record_replay(None, None) == 1

@@ -230,19 +230,25 @@ def test_forced_umma_rejects_ineligible_shapes(q8):
 
 
 SPLITK_CASES = [
-    # name, N,H,W,C,K,R,S,stride,pad, y type, residual, relu
-    ("fc_c2048_k1000_f32", 64, 1, 1, 2048, 1000, 1, 1, 1, 0, F32, None, False),
-    ("3x3_7x7_c512_k512_res", 8, 7, 7, 512, 512, 3, 3, 1, 1, U8, "u8", True),
-    ("1x1_c2048_k512", 8, 7, 7, 2048, 512, 1, 1, 1, 0, U8, None, True),
-    ("3x3s2_c256_k256_s8", 4, 15, 15, 256, 256, 3, 3, 2, 1, S8, None, False),
-    ("1x1_c1024_k24_slice", 2, 10, 10, 1024, 24, 1, 1, 1, 0, F32, None, True),
+    # name, N,H,W,C,K,R,S,stride,pad, y type, residual, relu, channels of the tensor the output is a slice of (0: none), parts
+    ("fc_c8192_k1000_f32", 64, 1, 1, 8192, 1000, 1, 1, 1, 0, F32, None, False, 0, 16),
+    ("3x3_7x7_c512_k512_res", 8, 7, 7, 512, 512, 3, 3, 1, 1, U8, "u8", True, 0, 9),
+    ("1x1_c6144_k512", 8, 7, 7, 6144, 512, 1, 1, 1, 0, U8, None, True, 0, 12),
+    ("3x3s2_c512_k256_s8", 4, 15, 15, 512, 256, 3, 3, 2, 1, S8, None, False, 0, 9),
+    ("1x1_c8192_k27_f32", 2, 10, 10, 8192, 27, 1, 1, 1, 0, F32, None, True, 0, 16),
+    ("1x1_c8192_k24_slice", 2, 10, 10, 8192, 24, 1, 1, 1, 0, U8, "u8", True, 64, 16),
+    # layers that narrow tiles serve better than a split: the scratch they are given stays untouched
+    ("fc_c2048_k1000_f32", 64, 1, 1, 2048, 1000, 1, 1, 1, 0, F32, None, False, 0, 1),
+    ("1x1_c2048_k512", 8, 7, 7, 2048, 512, 1, 1, 1, 0, U8, None, True, 0, 1),
+    ("3x3s2_c256_k256_s8", 4, 15, 15, 256, 256, 3, 3, 2, 1, S8, None, False, 0, 1),
+    ("1x1_c1024_k24_slice", 2, 10, 10, 1024, 24, 1, 1, 1, 0, F32, None, True, 0, 1),
 ]
 
 
 @pytest.mark.parametrize("case", SPLITK_CASES, ids=[c[0] for c in SPLITK_CASES])
 def test_split_k_matches_oracle_and_unsplit(q8, case):
     """Layers with few output tiles split the reduction when given a workspace; the result must not change."""
-    name, N, H, W, C, K, R, S, st, pad, ytype, res, relu = case
+    name, N, H, W, C, K, R, S, st, pad, ytype, res, relu, wide, parts = case
     g = np.random.default_rng(sum(map(ord, name)))
     x = g.integers(0, 256, (N, H, W, C), dtype=np.uint8)
     w = g.integers(-128, 128, (K, R, S, C)).astype(np.int8)
@@ -253,13 +259,21 @@ def test_split_k_matches_oracle_and_unsplit(q8, case):
     scale = np.float32(100.0 / max(1, np.abs(acc).max()))
     rs = 0.37 if resid is not None else 0.0
     want = o.epilogue(acc, scale, resid, rs, relu, OT[ytype])
-    d = q8.make_conv_desc(N, H, W, C, K, R, S, (st, st), (pad, pad), (1, 1), U8, U8, ytype, relu)
+    d = q8.make_conv_desc(N, H, W, C, K, R, S, (st, st), (pad, pad), (1, 1), U8, U8, ytype, relu, 1, wide, 16 if wide else 0)
     nbytes = q8.q8_conv2d_workspace_bytes(d)
-    assert nbytes > 0, "this shape is expected to split"
-    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    assert nbytes == (parts * N * P * Q * K * 4 if parts > 1 else 0) and q8.q8_conv2d_query_plan(d, bool(res)).splits == parts
+    room = 16 * N * P * Q * K * 4
+    ws = torch.full((room,), 0xA5, dtype=torch.uint8, device="cuda")
     args = (_cuda(x), _cuda(w), _cuda(bias), torch.tensor([scale], device="cuda"), _cuda(resid) if res else None, rs)
     y_split = q8.q8_conv2d(d, *args, workspace=ws)
     y_plain = q8.q8_conv2d(d, *args)
     q8.q8_read_status()
-    assert np.array_equal(_bits(y_split.cpu().numpy()), _bits(want))
-    assert np.array_equal(_bits(y_plain.cpu().numpy()), _bits(want))
+    lo = 16 if wide else 0
+    assert np.array_equal(_bits(np.ascontiguousarray(y_split.cpu().numpy()[..., lo:lo + K])), _bits(want))
+    assert np.array_equal(_bits(np.ascontiguousarray(y_plain.cpu().numpy()[..., lo:lo + K])), _bits(want))
+    # every partial sum was written by the first pass, nothing beyond them
+    partials = ws[:nbytes].view(torch.int32).view(parts, -1) if parts > 1 else None
+    if parts > 1:
+        acc0 = torch.from_numpy(acc.reshape(-1, K) - bias).cuda().view(-1)
+        assert torch.equal(partials.sum(0, dtype=torch.int32), acc0)
+    assert bool((ws[nbytes:] == 0xA5).all())

@@ -30,8 +30,8 @@ def _case(q8, N, H, W, C, K, R, pad, ytype, with_res, seed):
     return d, x, w, b, scale, res
 
 
-@pytest.mark.parametrize("shape", [(64, 1, 1, 2048, 1000, 1, 0, F32, False), (8, 7, 7, 512, 512, 3, 1, U8, True)],
-                         ids=["fc_2048_1000_f32", "3x3_7x7_512_res_u8"])
+@pytest.mark.parametrize("shape", [(64, 1, 1, 8192, 1000, 1, 0, F32, False), (8, 7, 7, 512, 512, 3, 1, U8, True)],
+                         ids=["fc_8192_1000_f32", "3x3_7x7_512_res_u8"])
 def test_static_workspace_matches_caller_workspace_twice(q8, shape):
     N, H, W, C, K, R, pad, ytype, with_res = shape
     for call in range(2):  # second call: the built-in array still holds the first call's partial sums
@@ -65,10 +65,12 @@ def test_static_workspace_refuses_oversized_layers_and_runs_unsplit_ones(q8):
     with pytest.raises(q8.Q8Error) as e:
         q8.q8_conv2d_static_workspace(d, x, w, b, scale)
     assert e.value.code == 4 and "built-in" in str(e.value)
-    # a layer that needs no scratch simply runs
-    d, x, w, b, scale, res = _case(q8, 2, 16, 16, 64, 64, 3, 1, U8, False, seed=8)
-    assert q8.q8_conv2d_workspace_bytes(d) == 0
-    got = q8.q8_conv2d_static_workspace(d, x, w, b, scale)
-    want = q8.q8_conv2d(d, x, w, b, scale)
-    q8.q8_read_status()
-    assert torch.equal(got, want)
+    # layers that need no scratch simply run: with many tiles, and with few where narrow ones are better than a split
+    # (1x1 2048 -> 256 on 4736 pixels: a split would need 18.5 MiB)
+    for shape in [(2, 16, 16, 64, 64, 3, 1), (1, 64, 74, 2048, 256, 1, 0)]:
+        d, x, w, b, scale, res = _case(q8, *shape, U8, False, seed=8)
+        assert q8.q8_conv2d_workspace_bytes(d) == 0
+        got = q8.q8_conv2d_static_workspace(d, x, w, b, scale)
+        want = q8.q8_conv2d(d, x, w, b, scale)
+        q8.q8_read_status()
+        assert torch.equal(got, want)
