@@ -47,9 +47,12 @@ int q8_record_end(int n_streams, void** streams, void** graph) {
   cudaGraphExec_t exec = nullptr;
   int rc = check_cuda(cudaStreamEndCapture(as_stream(streams[0]), &recorded), "q8_record_end: end capture");
   if (rc == Q8_OK && graph) rc = check_cuda(cudaGraphInstantiate(&exec, recorded, 0), "q8_record_end: instantiate");
+  // the launch data goes to the device now, not with the first replay
+  if (exec) rc = check_cuda(cudaGraphUpload(exec, as_stream(streams[0])), "q8_record_end: upload");
   if (recorded) cudaGraphDestroy(recorded);
   destroy_streams(n_streams, streams);
   if (rc == Q8_OK && graph) *graph = exec;
+  else if (exec) cudaGraphExecDestroy(exec);
   if (rc != Q8_OK) cudaGetLastError();  // a recording that cannot be ended leaves its error to the next launch otherwise
   return graph ? rc : Q8_OK;
 }
