@@ -106,13 +106,13 @@ def _check(rc):
         raise Q8Error(rc, lib.q8_last_error().decode())
 
 
-_raw_stream, _get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# torch.cuda.current_stream() without the Stream object around the handle (5 us against 0.2 us a call, more than the rest
+# of a call's marshalling); a torch without these private entry points takes the public one
+_raw_stream, _get_device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
 
 
 def _stream():
-    # the raw handle of torch.cuda.current_stream() without the Stream object around it (5 us against 0.2 us a call,
-    # more than the rest of a call's marshalling)
-    if not torch.cuda.is_initialized():
+    if _raw_stream is None or _get_device is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_get_device())
 

@@ -3,6 +3,8 @@ validation turns bad requests into documented error codes without launching anyt
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -146,6 +148,14 @@ def test_scratch_is_asked_for_by_the_layers_that_split(shape, parts):
     assert q8.q8_conv2d_workspace_bytes(d) == (parts * shape[0] * shape[1] * shape[2] * shape[4] * 4 if parts > 1 else 0)
     d.y_type, d.relu = S32, 0
     assert q8.q8_conv2d_workspace_bytes(d) == 0
+
+
+@pytest.mark.parametrize("name", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_private_torch_entry_points_are_optional(name):
+    code = (f"import torch; delattr(torch._C, {name!r}); import types; import paper_1805_08691_b200.binding as b; "
+            "torch.cuda.is_initialized = lambda: True; torch.cuda.current_stream = lambda: types.SimpleNamespace(cuda_stream=77); "
+            "assert b._stream() == 77")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
 
 
 def test_recording_requests_are_checked_on_the_host():
