@@ -943,22 +943,15 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
     const long long pair_items = (long long)((p.m_tiles + 1) / 2) * p.n_tiles;
     const bool can = p.a_mode == kAHalo && !paired && p.b_mode == kBRing && BN >= 96 && BN % 32 == 0 && out8 &&
                      !rows && splits == 1 && (BK == 128 || BK == 64) &&
-                     (!p.epi_split || tune_env("Q8_CTA2SPLIT", 0, 0, 1)) &&
-                     pair_items >= tune_env("Q8_CTA2MIN", 2 * (sm_count() / 2), 1, 1 << 30);
+                     !p.epi_split && pair_items >= tune_env("Q8_CTA2MIN", 2 * (sm_count() / 2), 1, 1 << 30);
     if (can && tune_env("Q8_CTA2", 1, 0, 1)) {
       p.cta2 = 1;
-      p.m_tiles = (p.m_tiles + 1) / 2;              // work items are pairs of m tiles
-      {
-        const long long items = (long long)p.m_tiles * p.n_tiles, clusters = sm_count() / 2;
-        const long long per = (items + (items < clusters ? items : clusters) - 1) / (items < clusters ? items : clusters);
-        // Teams: a launch of at most two items per pair has one team of all groups.  Tiles above 128 columns leave two
-        // accumulators, hence two teams, and with two groups each an accumulator is back in half the time (3x3 128->192
-        // at 73x73, batch 64: 62.3 -> 55.4 us).  Four teams for narrower tiles (128->128 at 150x150 as teams of two:
-        // 74 -> 108 us, what a tile costs a group beside its columns is paid twice).
-        p.pair_shift = per <= 2 ? 2 : (BN > 128 ? 1 : 0);
-        p.epi_split = p.pair_shift == 2;
-        G = 4;
-      }
+      p.m_tiles = (p.m_tiles + 1) / 2;              // work items are pairs of m tiles, more than two per pair of SMs
+      // Teams: tiles above 128 columns leave two accumulators, hence two teams, and with two groups each an accumulator is
+      // back in half the time (3x3 128->192 at 73x73, batch 64: 62.3 -> 55.4 us).  Four teams for narrower tiles (128->128
+      // at 150x150 as teams of two: 74 -> 108 us, what a tile costs a group beside its columns is paid twice).
+      p.pair_shift = BN > 128 ? 1 : 0;
+      G = 4;
       p.b_tile_bytes = (unsigned)((BN / 2) * BK);   // this CTA's half of the weight rows
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
     }

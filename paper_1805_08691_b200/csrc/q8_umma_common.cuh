@@ -994,7 +994,7 @@ FastDiv make_fastdiv(int d) {
 // shared-memory or TMEM plan does not hold.
 //   Q8_PDL 0/1 dependent launch, Q8_HALO 0/1 halo tiles, Q8_BN tile width (multiple of 16), Q8_LANES 2/3 MMA warps,
 //   Q8_SPLIT 0/1 column-split epilogue (only where the plan allows it), Q8_G 2/4 epilogue groups, Q8_BRES 0 weights
-//   not resident, Q8_CTA2 0 no CTA pairs, Q8_CTA2SPLIT, Q8_CTA2MIN pair-mode thresholds, Q8_BT taps per weight-ring
+//   not resident, Q8_CTA2 0 no CTA pairs, Q8_CTA2MIN pair-mode threshold, Q8_BT taps per weight-ring
 //   stage, Q8_KB channel blocks per A stage, Q8_NBUF tile buffers per group, Q8_BSTAGES / Q8_STAGES ring depths (at
 //   most what fits), Q8_GRID number of CTAs (at most the default).
 int tune_env(const char* name, int dflt, int lo, int hi) {
