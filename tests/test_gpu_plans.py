@@ -10,21 +10,24 @@ pytestmark = pytest.mark.gpu
 U8, S8 = 0, 1
 
 CASES = [
-    # name, N,H,W,C,K,R,S,pad, y type, residual
-    ("narrow_16", 1, 14, 14, 1024, 256, 1, 1, (0, 0), U8, True),
-    ("narrow_16_halo", 1, 7, 7, 512, 512, 3, 3, (1, 1), S8, False),
-    ("narrow_32_ragged", 4, 14, 14, 640, 528, 1, 1, (0, 0), U8, True),
-    ("narrow_32_short_reduction", 1, 7, 7, 512, 2048, 1, 1, (0, 0), U8, True),
-    ("narrow_64_ragged", 4, 14, 14, 576, 1008, 1, 1, (0, 0), S8, False),
-    ("narrow_128", 16, 14, 14, 768, 512, 1, 1, (0, 0), U8, False),
-    ("pair_256_shared", 14, 53, 53, 128, 512, 3, 3, (1, 1), U8, True),
-    ("pair_144_shared_odd_chunks", 44, 37, 37, 128, 144, 3, 3, (1, 1), S8, False),
+    # name, N,H,W,C,K,R,S,pad, y type, residual, tile width, CTA pair, groups that share a tile's columns
+    ("narrow_16", 1, 14, 14, 1024, 256, 1, 1, (0, 0), U8, True, 16, 0, 1),
+    ("narrow_16_halo", 1, 7, 7, 512, 512, 3, 3, (1, 1), S8, False, 16, 0, 1),
+    ("narrow_32_ragged", 4, 14, 14, 640, 528, 1, 1, (0, 0), U8, True, 32, 0, 1),
+    ("narrow_32_short_reduction", 1, 7, 7, 512, 2048, 1, 1, (0, 0), U8, True, 32, 0, 1),
+    ("narrow_64_ragged", 4, 14, 14, 576, 1008, 1, 1, (0, 0), S8, False, 64, 0, 4),
+    ("narrow_128", 16, 14, 14, 768, 512, 1, 1, (0, 0), U8, False, 128, 0, 4),
+    ("pair_256_shared", 14, 53, 53, 128, 512, 3, 3, (1, 1), U8, True, 256, 1, 2),
+    ("pair_160_five_chunks_a_group", 44, 37, 37, 128, 160, 3, 3, (1, 1), S8, False, 160, 1, 2),
+    ("pair_224_seven_chunks_a_group", 30, 37, 37, 96, 224, 3, 3, (1, 1), S8, True, 224, 1, 2),
+    ("pair_96_alone", 44, 37, 37, 128, 96, 3, 3, (1, 1), U8, False, 96, 1, 1),
+    ("wide_144_single_cta", 44, 37, 37, 128, 144, 3, 3, (1, 1), S8, False, 144, 0, 1),
 ]
 
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
 def test_plan_matches_oracle(q8, case):
-    name, N, H, W, C, K, R, S, pad, ytype, res = case
+    name, N, H, W, C, K, R, S, pad, ytype, res, tile_n, pair, shared = case
     g = np.random.default_rng(sum(map(ord, name)))
     x = g.integers(0, 256, (N, H, W, C), dtype=np.uint8)
     w = g.integers(-128, 128, (K, R, S, C)).astype(np.int8)
@@ -34,6 +37,8 @@ def test_plan_matches_oracle(q8, case):
     scale = (g.uniform(0.5, 1.5, K) * 100.0 / max(1, np.abs(acc).max())).astype(np.float32)
     want = o.epilogue(acc, scale, resid, 0.37 if res else 0.0, ytype == U8, o.U8 if ytype == U8 else o.S8)
     d = q8.make_conv_desc(N, H, W, C, K, R, S, (1, 1), pad, (1, 1), U8, U8, ytype, ytype == U8, K)
+    plan = q8.q8_conv2d_query_plan(d, res)
+    assert (plan.kernel, plan.tile_n, plan.cta_pair, plan.shared_groups) == (q8.Q8_KERNEL_TMA, tile_n, pair, shared)
     args = [torch.from_numpy(a).cuda() for a in (x, w, bias, scale)]
     rd = torch.from_numpy(resid).cuda() if res else None
     for _ in range(2):   # twice: the second launch follows the first in the stream

@@ -19,11 +19,11 @@ CASES = [
     ("k60_strided", 2, 57, 57, 64, 60, 1, 1, 2, (0, 0), U8, False, False, 0, 0, 0),
     ("k100_halo_long", 32, 56, 56, 32, 100, 3, 3, 1, (1, 1), U8, True, False, 0, 0, 0),
     ("k250_long", 16, 57, 57, 64, 250, 1, 1, 1, (0, 0), S8, True, False, 0, 0, 0),
-    ("k250_shared_tile", 2, 28, 28, 640, 250, 1, 1, 1, (0, 0), U8, True, True, 0, 0, 0),
+    ("k250_shared_tile", 4, 28, 28, 640, 250, 1, 1, 1, (0, 0), U8, True, True, 0, 0, 0),
     ("k500_two_tiles", 6, 28, 28, 320, 500, 3, 3, 1, (1, 1), U8, False, False, 0, 0, 0),
     ("k301_narrow", 1, 14, 14, 1024, 301, 1, 1, 1, (0, 0), U8, True, False, 0, 0, 0),
     ("k256_odd_slice", 4, 33, 33, 128, 256, 1, 1, 1, (0, 0), U8, True, False, 13, 6, 1),
-    ("k64_pairs_of_pixels", 2, 64, 64, 16, 61, 7, 7, 2, (3, 3), U8, False, True, 3, 2, 3),
+    ("k61_pairs_of_pixels", 2, 30, 240, 16, 61, 7, 7, 2, (3, 3), U8, False, True, 3, 2, 3),
     ("k24_slice_aligned_pitch", 2, 33, 33, 64, 24, 1, 1, 1, (0, 0), U8, True, False, 24, 16, 0),
 ]
 
@@ -42,6 +42,10 @@ def test_rows_off_the_grid_match_oracle(q8, case):
     want = o.epilogue(acc, scale if per_channel else scale[0], resid, 0.37 if res else 0.0, ytype == U8, o.U8 if ytype == U8 else o.S8)
     ldc = K + extra
     d = q8.make_conv_desc(N, H, W, C, K, R, S, (st, st), pad, (1, 1), U8, U8, ytype, ytype == U8, K if per_channel else 1, ldc, c_off)
+    plan = q8.q8_conv2d_query_plan(d, res)
+    assert plan.kernel == q8.Q8_KERNEL_TMA and plan.moved_rows
+    assert plan.shared_groups == (4 if name in ("k250_shared_tile", "k60_strided", "k500_two_tiles", "k256_odd_slice", "k61_pairs_of_pixels") else 1)
+    assert plan.operand == (1 if "strided" in name else (2 if R > 1 else 0))
     rows = N * P * Q
     buf = torch.full((64 + rows * ldc + 64,), 7, dtype=q8.TORCH_DTYPES[ytype], device="cuda")
     y = buf[64 + shift:64 + shift + rows * ldc].view(N, P, Q, ldc)
