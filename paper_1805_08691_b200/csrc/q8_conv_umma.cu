@@ -860,6 +860,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
     p.tap_inner = paired ? d.R : ht.s_eff;
   }
   p.c_blocks = (c_eff + BK - 1) / BK;
+  if (paired && p.c_blocks != 1) return false;  // the weights of a pixel pair are one block of 2C channels
   p.C_pad = p.c_blocks * BK;
   p.k_iters = p.taps * p.c_blocks;
   p.splits = splits;

@@ -115,6 +115,7 @@ ROUTES = [
     (D, 1, 8, 8, 3, 8, 1, 1, {}),
     (D, 2, 9, 9, 16, 5000, 1, 1, {}),
     (G, 1, 200, 128, 16, 32, 3, 1, dict(stride=(2, 1), dil=(70, 1))),  # no tile fits
+    (G, 1, 60, 60, 32, 32, 7, 1, dict(stride=(2, 2), pad=(2, 0), dil=(9, 1))),   # nor in whole pixel pairs
     (G, 1, 1, 1 << 19, 1025, 8, 1, 1, dict(stride=(1, 1 << 14))),
     (D, 1, 1, 1 << 21, 1025, 8, 1, 1, dict(stride=(1, 1 << 17))),      # rows of more than 2^30 bytes, with and
     (D, 1, 1, 1000, 1025, 8, 1, 1, dict(stride=(1, 1 << 17), pad=(0, 1 << 20))),   # without their padding
@@ -138,6 +139,14 @@ def test_queries_follow_the_dispatch(route):
     elif kernel == T or d.C % 16 or d.K > 4096 or d.y_type in (U8, S8):
         assert q8.q8_conv2d_query_algo(d) == q8.Q8_ALGO_DIRECT
         assert _code(q8.q8_conv2d_query_plan, d) == 2
+
+
+@pytest.mark.parametrize("K", [8, 16])
+def test_pixel_pairs_are_never_cut_into_channel_blocks(K):
+    """A patch of whole 64-byte pixel pairs does not fit here: the layer takes im2col loads, not narrower blocks of pairs."""
+    d = q8.make_conv_desc(2, 95, 198, 32, K, 7, 1, (2, 2), (2, 0), (3, 1))
+    plan = q8.q8_conv2d_query_plan(d)
+    assert (plan.kernel, plan.operand) == (T, 1)
 
 
 @pytest.mark.parametrize("shape,parts", [((64, 1, 1, 8192, 1008, 1, 1), 16), ((64, 1, 1, 2048, 1008, 1, 1), 1), ((1, 14, 14, 1024, 256, 1, 1), 1),

@@ -65,3 +65,19 @@ def test_layer_that_no_tile_of_the_tma_fed_kernel_fits(q8, K, ytype):
     with pytest.raises(q8.Q8Error) as e:
         q8.q8_conv2d(d, *args)
     assert e.value.code == 2
+
+
+@pytest.mark.parametrize("shape", [(2, 95, 198, 32, 8, 3), (2, 95, 198, 32, 16, 3), (1, 60, 60, 32, 32, 9), (1, 95, 60, 64, 48, 6)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_pixel_pairs_whose_patch_does_not_fit(q8, shape):
+    """Stride-2 filters of tall dilated columns: the patch of pixel pairs exceeds shared memory."""
+    N, H, W, C, K, dil = shape
+    g = np.random.default_rng(K)
+    x = g.integers(0, 256, (N, H, W, C), dtype=np.uint8)
+    w = g.integers(-128, 128, (K, 7, 1, C)).astype(np.int8)
+    scale = np.float32(4e-4)
+    want = o.conv2d(x, w, None, scale, stride=(2, 2), pad=(2, 0), dil=(dil, 1), relu=True, y_type=o.U8, threads=8)
+    d = q8.make_conv_desc(N, H, W, C, K, 7, 1, (2, 2), (2, 0), (dil, 1), U8, U8, U8, True)
+    y = q8.q8_conv2d(d, torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), None, torch.tensor([scale], device="cuda"))
+    q8.q8_read_status()
+    assert np.array_equal(y.cpu().numpy(), want)
