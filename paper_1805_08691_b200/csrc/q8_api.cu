@@ -121,8 +121,8 @@ Route conv_route(const ConvArgs& a, const char** why) {
   if (d.algo == Q8_ALGO_UMMA || !out8) {
     if (out8 && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16)) { *why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; return route_off_tma(a); }
     if (a.residual && !aligned16(a.residual)) { *why = "residual not 16-byte aligned"; return route_off_tma(a); }
-  } else if (rows_unaligned(a) && (tiny_call(a) || short_rows(a))) {
-    return route_off_tma(a);  // (other 8-bit rows off the 16-byte grid: the epilogue warps move them, see rows_out)
+  } else if (rows_off_tma(a) && (tiny_call(a) || short_rows(a))) {
+    return route_off_tma(a);  // (other 8-bit rows that TMA cannot store: the epilogue warps move them, see rows_out)
   }
   return kRouteTma;
 }

@@ -712,6 +712,10 @@ bool rows_unaligned(const ConvArgs& a) {
   return (a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8) && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16 || (a.residual && !aligned16(a.residual)));
 }
 
+bool rows_off_tma(const ConvArgs& a) {
+  return rows_unaligned(a) || ((a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8) && a.d.K % 16);
+}
+
 namespace {
 // How a layer runs: tiles, shared memory and pipeline depths.  Decided from the descriptor and the alignment of the
 // pointers alone, so that it can be asked for without a device.
@@ -820,8 +824,8 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   int res_mode = kResNone;
   if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResTma : (out8 ? kResRows : kResGlobal);
-  // 8-bit rows off the 16-byte grid are moved by the epilogue warps, in both directions if in one
-  const bool rows = out8 && (rows_unaligned(a) || res_mode == kResRows);
+  // 8-bit rows that TMA cannot address are moved by the epilogue warps, in both directions if in one
+  const bool rows = out8 && (rows_off_tma(a) || res_mode == kResRows);
   if (rows && a.residual) res_mode = kResRows;
   UmmaParams& p = plan->p;
   memset(&p, 0, sizeof(p));
@@ -1106,8 +1110,9 @@ int launch_planned(const ConvArgs& a, int splits) {
   if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: weight tensor map rejected (CUresult %d)", (int)cr);
 
   // Residual and output tiles: [M][channels] matrices, or for halo tiles (channels, Q, P, N) tensors whose
-  // TH x TW box lands as TH*TW dense rows.  The output map ends at the last channel this layer owns,
-  // so the store clips ragged Cout tiles and never touches a neighbouring slice of a concatenated tensor.
+  // TH x TW box lands as TH*TW dense rows.  The output map ends at the last channel this layer owns, a multiple of 16
+  // (stores are clipped in units of 16 bytes), so the store clips ragged Cout tiles and never touches a neighbouring
+  // slice of a concatenated tensor.
   auto encode_rows = [&](CUtensorMap* tm, void* ptr, int channels, int ld, CUtensorMapL2promotion promo) -> CUresult {
     if (p.a_mode == kAHalo) {
       cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)a.Q, (cuuint64_t)a.P, (cuuint64_t)d.N};

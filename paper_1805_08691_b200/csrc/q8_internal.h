@@ -56,7 +56,10 @@ struct ConvArgs {
 
 // Eligibility of the tensor-core kernel for a descriptor (pointer alignment checked at launch).
 bool umma_shape_eligible(const q8_conv_desc& d, const char** why);
-bool rows_unaligned(const ConvArgs& a);  // 8-bit output or residual rows that TMA cannot address
+bool rows_unaligned(const ConvArgs& a);  // 8-bit output or residual rows off the 16-byte grid
+// ... or on it, but ending between two of its lines: a TMA store is clipped in units of 16 bytes and would zero the
+// channels up to the next line, which may belong to another layer's slice.
+bool rows_off_tma(const ConvArgs& a);
 // Whether one of its tile shapes fits the layer, and which (decided without a device).
 bool umma_fits(const ConvArgs& a);
 bool umma_describe(const ConvArgs& a, q8_conv_plan* out);

@@ -24,6 +24,10 @@ CASES = [
     ("k301_narrow", 1, 14, 14, 1024, 301, 1, 1, 1, (0, 0), U8, True, False, 0, 0, 0),
     ("k256_odd_slice", 4, 33, 33, 128, 256, 1, 1, 1, (0, 0), U8, True, False, 13, 6, 1),
     ("k61_pairs_of_pixels", 2, 30, 240, 16, 61, 7, 7, 2, (3, 3), U8, False, True, 3, 2, 3),
+    # rows on the grid that end off it: the channels up to the next 16-byte line belong to somebody else
+    ("k24_of_48", 2, 33, 33, 64, 24, 1, 1, 1, (0, 0), U8, False, False, 24, 0, 0),
+    ("k88_of_128_halo", 2, 40, 40, 32, 88, 3, 3, 1, (1, 1), S8, False, True, 40, 16, 0),
+    ("k3_of_16_long", 4, 80, 80, 64, 3, 3, 3, 1, (1, 1), U8, False, False, 13, 0, 0),
     ("k24_slice_aligned_pitch", 2, 33, 33, 64, 24, 1, 1, 1, (0, 0), U8, True, False, 24, 16, 0),
 ]
 
@@ -44,7 +48,7 @@ def test_rows_off_the_grid_match_oracle(q8, case):
     d = q8.make_conv_desc(N, H, W, C, K, R, S, (st, st), pad, (1, 1), U8, U8, ytype, ytype == U8, K if per_channel else 1, ldc, c_off)
     plan = q8.q8_conv2d_query_plan(d, res)
     assert plan.kernel == q8.Q8_KERNEL_TMA and plan.moved_rows
-    assert plan.shared_groups == (4 if name in ("k250_shared_tile", "k60_strided", "k500_two_tiles", "k256_odd_slice", "k61_pairs_of_pixels") else 1)
+    assert plan.shared_groups == (4 if name in ("k250_shared_tile", "k60_strided", "k500_two_tiles", "k256_odd_slice", "k61_pairs_of_pixels", "k88_of_128_halo") else 1)
     assert plan.operand == (1 if "strided" in name else (2 if R > 1 else 0))
     rows = N * P * Q
     buf = torch.full((64 + rows * ldc + 64,), 7, dtype=q8.TORCH_DTYPES[ytype], device="cuda")
@@ -55,9 +59,12 @@ def test_rows_off_the_grid_match_oracle(q8, case):
         rd = rbuf[shift:shift + rows * K].view(N, P, Q, K)
         rd.copy_(torch.from_numpy(resid).cuda())
     args = [torch.from_numpy(a).cuda() for a in (x, w, bias, scale)]
-    q8.q8_conv2d(d, *args, rd, 0.37 if res else 0.0, y)
-    q8.q8_read_status()
-    got = y.cpu().numpy()
-    assert np.array_equal(got[..., c_off:c_off + K], want)
-    assert (got[..., :c_off] == 7).all() and (got[..., c_off + K:] == 7).all()
-    assert bool((buf[:64 + shift] == 7).all()) and bool((buf[64 + shift + rows * ldc:] == 7).all())
+    algos = [q8.Q8_ALGO_AUTO] + [q8.Q8_ALGO_UMMA] * (ldc % 16 == 0 and c_off % 16 == 0 and shift == 0)
+    for d.algo in algos:
+        buf.fill_(7)
+        q8.q8_conv2d(d, *args, rd, 0.37 if res else 0.0, y)
+        q8.q8_read_status()
+        got = y.cpu().numpy()
+        assert np.array_equal(got[..., c_off:c_off + K], want)
+        assert (got[..., :c_off] == 7).all() and (got[..., c_off + K:] == 7).all()
+        assert bool((buf[:64 + shift] == 7).all()) and bool((buf[64 + shift + rows * ldc:] == 7).all())
