@@ -89,13 +89,23 @@ int validate_desc(const q8_conv_desc* d, int* P, int* Q) {
   return Q8_OK;
 }
 
-// Few outputs with a short reduction: the direct kernel finishes before a tensor-core kernel has set up its pipeline (1x1 of
-// 5 -> 8 channels at 8x8: 2.6 against 3.5 us gathered; 20 -> 16 at 32x32: 3.3 against 3.9; 5 -> 32 on 8 x 28x28: 4.1 both).
-// From 27 products or 100 000 outputs on it takes longer (3x3 of 3 -> 8 on 2 x 17x19: 4.9 against 3.8 us).
-bool tiny_call(const ConvArgs& a) { return (long long)a.d.R * a.d.S * a.d.C <= 24 && a.M * a.d.K <= 100000; }
+// Time of the direct kernel in microseconds.  A thread forms one output, tap by tap; outputs cost index arithmetic and,
+// like the products of all of them, throughput; the products of one output are a chain of loads, longer where the weights
+// of the lanes lie in different sectors.  Fitted, with gather_us, to 2600 layers with 1 to 500 output channels, filters up
+// to 7x7 and up to 8000 products (median error of both 8 %).  Taking the smaller estimate is on average 1.5 % off the
+// better kernel over the layers with C off the 16-channel grid (8.6 % with the limits in products and outputs that stood
+// here, 7 times at worst: 7x7 of 163 -> 397 channels on one pixel takes 15 us directly, 102 gathered).
+double direct_us(const ConvArgs& a) {
+  const q8_conv_desc& d = a.d;
+  const double outputs = 1e-6 * (double)a.M * d.K, taps = (double)d.R * d.S;
+  const int in_h = (d.H - 1) / d.dil_h + 1, in_w = (d.W - 1) / d.dil_w + 1;  // filter rows and columns that fit the image
+  const double seen = (double)(d.R < in_h ? d.R : in_h) * (d.S < in_w ? d.S : in_w), chain = seen * d.C;
+  const double apart = taps * d.C > 32 ? (d.K < 32 ? d.K / 32.0 : 1.0) : 0.0;
+  return 2.4 + outputs * (9.0 + 0.22 * chain) + chain * (0.033 + 0.019 * apart) + (taps > 1 ? 0.1 * seen : 0.0) + 0.03 * taps;
+}
 
-// 8-bit rows off the 16-byte grid that are short and have short reductions: gathering the operands is cheaper than moving
-// the rows through shared memory (1x1 64 -> 9 at 56x56, batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32 7.2
+// 8-bit rows that TMA cannot store, short ones with short reductions: gathering the operands (or the direct kernel) is
+// cheaper than moving the rows through shared memory (1x1 64 -> 9 at 56x56, batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32 7.2
 // against 7.1; 64 -> 15 at 112x112, batch 8 8.4 against 7.3; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).
 bool short_rows(const ConvArgs& a) {
   const long long products = (long long)a.d.R * a.d.S * a.d.C;
@@ -109,7 +119,7 @@ enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRouteTma };
 
 Route route_off_tma(const ConvArgs& a) {
   if (a.d.algo == Q8_ALGO_UMMA) return kRouteRefused;
-  return gather_addressable(a.d) && !tiny_call(a) ? kRouteGather : kRouteDirect;
+  return gather_addressable(a.d) && gather_us(a) < direct_us(a) ? kRouteGather : kRouteDirect;
 }
 
 Route conv_route(const ConvArgs& a, const char** why) {
@@ -121,8 +131,11 @@ Route conv_route(const ConvArgs& a, const char** why) {
   if (d.algo == Q8_ALGO_UMMA || !out8) {
     if (out8 && (!aligned16(a.y) || a.ldc % 16 || a.c_off % 16)) { *why = "8-bit output needs y, y_ldc, y_c_offset aligned to 16"; return route_off_tma(a); }
     if (a.residual && !aligned16(a.residual)) { *why = "residual not 16-byte aligned"; return route_off_tma(a); }
-  } else if (rows_off_tma(a) && (tiny_call(a) || short_rows(a))) {
-    return route_off_tma(a);  // (other 8-bit rows that TMA cannot store: the epilogue warps move them, see rows_out)
+  } else if (rows_off_tma(a)) {
+    // Other such rows are moved by the epilogue warps (see rows_out), which takes 5 to 6 us at the least.  The direct kernel
+    // where it is surely faster: below 4.5 us by its estimate (1x1 32 -> 44 on 108 pixels: 4.0 against 5.5 us).
+    if (short_rows(a)) return route_off_tma(a);
+    if (direct_us(a) < 4.5) return kRouteDirect;
   }
   return kRouteTma;
 }

@@ -392,6 +392,50 @@ int launch_gather_variant(const GatherParams& p, size_t dyn, cudaStream_t stream
 
 }  // namespace
 
+namespace {
+struct GatherTiles {
+  int run_taps, run_chunks, chunks;  // see GatherParams
+  int lg_cpb, nblk, bn, n_tiles;
+  long long tiles;
+};
+
+GatherTiles gather_tiles(const ConvArgs& a) {
+  const q8_conv_desc& d = a.d;
+  GatherTiles t;
+  t.run_taps = (d.dil_w == 1 || d.S == 1) ? d.S : 1;
+  t.run_chunks = (t.run_taps * d.C + 15) / 16;
+  t.chunks = (d.R * d.S / t.run_taps) * t.run_chunks;
+  t.lg_cpb = t.chunks <= 2 ? 1 : (t.chunks <= 4 ? 2 : 3);
+  t.nblk = (t.chunks + (1 << t.lg_cpb) - 1) >> t.lg_cpb;
+  // Tile width: up to 128 columns; narrower ones while most SMs would stay without a tile.  The activations are
+  // gathered again for every tile of columns, but by SMs that had nothing to do (1x1 of 200 -> 500 channels at 14x14:
+  // 30.8 us with tiles of 128 columns, 10.2 us with these).
+  const long long m_tiles = (a.M + kBM - 1) / kBM;
+  t.n_tiles = (d.K + 127) / 128;
+  while (m_tiles * t.n_tiles * 2 <= sm_count() && (d.K + 2 * t.n_tiles - 1) / (2 * t.n_tiles) > 16) t.n_tiles *= 2;
+  t.bn = ((d.K + t.n_tiles - 1) / t.n_tiles + 15) / 16 * 16;
+  t.n_tiles = (d.K + t.bn - 1) / t.bn;
+  t.tiles = m_tiles * t.n_tiles;
+  return t;
+}
+
+// Whole 16-channel chunks of a row can be stored in 16-byte pieces.
+bool gather_vec(const ConvArgs& a) {
+  const int grid = a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8 ? 16 : 4;
+  return aligned16(a.y) && a.ldc % grid == 0 && a.c_off % grid == 0;
+}
+}  // namespace
+
+// Fitted together with the direct kernel's estimate (see there).  Start-up; a K block in flight; the chunks of columns that
+// a CTA stores, dearest byte by byte; the bytes that its producers gather.
+double gather_us(const ConvArgs& a) {
+  const GatherTiles t = gather_tiles(a);
+  const double waves = (double)((t.tiles + sm_count() - 1) / sm_count()), columns = (t.bn < a.d.K ? t.bn : a.d.K) / 16.0;
+  const bool out8 = a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8;
+  const double store = gather_vec(a) ? 0.18 : (out8 ? 1.6 * (a.M < kBM ? (double)a.M / kBM : 1.0) : 0.66);
+  return 2.5 + 0.75 * t.nblk + waves * (columns * store + 4.6 * t.nblk * t.bn / 128.0 * (1 << t.lg_cpb) / 8.0);
+}
+
 // The channel arrays of 4096 outputs fit beside the stages.  Positions in a row of input pixels, padding included, are
 // 32-bit byte offsets, and rows past the last pixel are told by a row number below -2^28; wider images and filters stay
 // with the direct kernel, whose addresses are 64-bit.
@@ -413,29 +457,19 @@ int launch_conv_gather(const ConvArgs& a) {
   p.res_vec = d.K % 16 == 0 && aligned16(a.residual);
   p.res_signed = d.res_type == Q8_S8; p.res_scale = a.residual_scale;
   p.y = a.y; p.ldc = a.ldc; p.c_off = a.c_off; p.relu = d.relu;
-  const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
-  p.y_vec = aligned16(a.y) && a.ldc % (out8 ? 16 : 4) == 0 && a.c_off % (out8 ? 16 : 4) == 0;
+  p.y_vec = gather_vec(a);
   p.H = d.H; p.W = d.W; p.C = d.C; p.K = d.K; p.S = d.S;
   p.P = a.P; p.Q = a.Q; p.PQ = a.P * a.Q; p.M = (int)a.M;
   p.stride_h = d.stride_h; p.stride_w = d.stride_w; p.pad_h = d.pad_h; p.pad_w = d.pad_w; p.dil_h = d.dil_h; p.dil_w = d.dil_w;
+  const GatherTiles t = gather_tiles(a);
   p.rsc = d.R * d.S * d.C;
-  p.run_taps = (d.dil_w == 1 || d.S == 1) ? d.S : 1;
-  p.run_len = p.run_taps * d.C;
-  p.run_chunks = (p.run_len + 15) / 16;
-  p.chunks = (p.rsc / p.run_len) * p.run_chunks;
-  p.bkb = p.chunks <= 2 ? 32 : (p.chunks <= 4 ? 64 : 128);
-  p.lg_cpb = p.bkb == 32 ? 1 : (p.bkb == 64 ? 2 : 3);
-  p.nblk = (p.chunks + (1 << p.lg_cpb) - 1) >> p.lg_cpb;
+  p.run_taps = t.run_taps; p.run_len = t.run_taps * d.C; p.run_chunks = t.run_chunks; p.chunks = t.chunks;
+  p.lg_cpb = t.lg_cpb;
+  p.bkb = 16 << t.lg_cpb;
+  p.nblk = t.nblk;
   p.swz_mask = p.bkb == 128 ? 7u : (p.bkb == 64 ? 3u : 1u);
-  // Tile width: up to 128 columns; narrower ones while most SMs would stay without a tile.  The activations are
-  // gathered again for every tile of columns, but by SMs that had nothing to do (1x1 of 200 -> 500 channels at 14x14:
-  // 30.8 us with tiles of 128 columns, 10.2 us with these).
-  const long long m_tiles = (a.M + kBM - 1) / kBM;
-  p.n_tiles = (d.K + 127) / 128;
-  while (m_tiles * p.n_tiles * 2 <= sm_count() && (d.K + 2 * p.n_tiles - 1) / (2 * p.n_tiles) > 16) p.n_tiles *= 2;
-  p.bn = ((d.K + p.n_tiles - 1) / p.n_tiles + 15) / 16 * 16;
-  p.n_tiles = (d.K + p.bn - 1) / p.bn;
-  const long long tiles = m_tiles * p.n_tiles;
+  p.bn = t.bn; p.n_tiles = t.n_tiles;
+  const long long tiles = t.tiles;
   if (tiles > 0x7fffffff) return fail(Q8_ERR_UNSUPPORTED, "conv_gather: too many tiles");
   p.tiles = (int)tiles;
   p.acc_stride = 32;

@@ -75,6 +75,7 @@ int launch_conv_direct(const ConvArgs& a);
 // Tensor-core kernel that gathers its operands byte by byte (q8_conv_gather.cu): any alignment, any shape whose rows it can
 // address.
 bool gather_addressable(const q8_conv_desc& d);
+double gather_us(const ConvArgs& a);  // its estimated time
 int launch_conv_gather(const ConvArgs& a);
 // A stride-1 convolution followed by a 1x1 convolution over its output, in one launch (q8_conv_fused.cu).
 // Descriptors validated by the caller; `why` names the first reason a pair cannot run fused.

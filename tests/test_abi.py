@@ -114,6 +114,12 @@ ROUTES = [
     (G, 2, 28, 28, 100, 120, 3, 3, dict(pad=(1, 1))),
     (D, 1, 8, 8, 3, 8, 1, 1, {}),
     (D, 2, 9, 9, 16, 5000, 1, 1, {}),
+    (G, 8, 299, 299, 3, 32, 3, 3, dict(stride=(2, 2))),
+    (D, 1, 1, 1, 163, 397, 7, 7, dict(pad=(3, 3))),                    # few outputs or few products: no tensor cores
+    (D, 7, 1, 1, 64, 9, 7, 7, dict(pad=(3, 3), stride=(2, 2))),
+    (D, 9, 160, 160, 5, 1, 1, 1, {}),
+    (D, 1, 31, 9, 2, 444, 1, 1, {}),
+    (D, 1, 9, 12, 32, 44, 1, 1, {}),
     (G, 1, 200, 128, 16, 32, 3, 1, dict(stride=(2, 1), dil=(70, 1))),  # no tile fits
     (G, 1, 60, 60, 32, 32, 7, 1, dict(stride=(2, 2), pad=(2, 0), dil=(9, 1))),   # nor in whole pixel pairs
     (G, 1, 1, 1 << 19, 1025, 8, 1, 1, dict(stride=(1, 1 << 14))),
