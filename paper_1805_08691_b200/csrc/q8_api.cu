@@ -104,9 +104,12 @@ double direct_us(const ConvArgs& a) {
   return 2.4 + outputs * (9.0 + 0.22 * chain) + chain * (0.033 + 0.019 * apart) + (taps > 1 ? 0.1 * seen : 0.0) + 0.03 * taps;
 }
 
-// 8-bit rows that TMA cannot store, short ones with short reductions: gathering the operands (or the direct kernel) is
-// cheaper than moving the rows through shared memory (1x1 64 -> 9 at 56x56, batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32 7.2
-// against 7.1; 64 -> 15 at 112x112, batch 8 8.4 against 7.3; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).
+// 8-bit rows that TMA cannot store, short ones with short reductions: gathering the operands (or the direct kernel) costs
+// less than the kernel that moves such rows through shared memory, whose start-up is longer.  The gathering kernel's time
+// grows faster, by the bytes that its producers fetch (reduction x pixels) and by every 16 columns that it stores byte by
+// byte, which is what the limits are in (1x1 64 -> 9 at 56x56: batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32
+// 7.2 against 7.1; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).  Over 870 random layers whose rows TMA
+// cannot store, the kernel taken is on average 0.9 % off the fastest of the three.
 bool short_rows(const ConvArgs& a) {
   const long long products = (long long)a.d.R * a.d.S * a.d.C;
   return products <= 64 && (a.d.K <= 16 ? products * a.M <= 4000000 : a.d.K <= 32 && a.M <= 128);

@@ -17,8 +17,8 @@
 // activations.  All waits are bounded as in the other tensor-core kernels.
 //
 // Bound by the producers' instructions (some sixty per 16-byte chunk, nothing else is near a limit), hence no division
-// per chunk, rows per thread fixed at compile time and branch-free loads.  Measured against the CUDA-core kernel it
-// replaces: 3x3/2 of 3 -> 32 channels on 8 x 299x299 155 -> 12.5 us, 7x7/2 of 3 -> 64 on 224x224 134 -> 7.7 us,
+// per chunk, rows per thread fixed at compile time and branch-free loads.  Measured against the CUDA-core kernel:
+// 3x3/2 of 3 -> 32 channels on 8 x 299x299 157.7 -> 12.2 us, 7x7/2 of 3 -> 64 on 224x224 134 -> 7.7 us,
 // 3x3 of 100 -> 120 on 8 x 28x28 963 -> 26 us, 1x1 of 200 -> 500 at 14x14 32.8 -> 10.2 us.
 #include "q8_umma_common.cuh"
 

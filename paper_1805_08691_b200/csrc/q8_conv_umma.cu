@@ -3,14 +3,13 @@
 //   D[M = N*P*Q pixels, Cout] (int32, in TMEM) = A[M, R*S*C] (u8/s8) x B[Cout, R*S*C]^T (s8)
 //
 // Persistent kernel: one CTA per SM walks over output tiles of 128 accumulator rows x BN channels.
-// A lone control warp executes roughly one instruction every 6-10 cycles and every TMA operation
-// occupies the SM's copy engine for at least ~370 cycles whatever its size, so the pipeline moves
-// few, large pieces:
+// Every TMA operation occupies the SM's copy engine for at least ~370 cycles whatever its size, and a control
+// warp spends some hundred cycles on a pipeline iteration, so the pipeline moves few, large pieces:
 //
 //   A operand, three sources
 //     plain  : 1x1 / stride 1 / no padding.  The activation tensor is the [M][C] matrix itself; a
 //              stage holds several consecutive 128 x BK channel blocks (2-D tiled loads).
-//     halo   : stride 1 filters.  A tile is TH x TW output pixels of one image.  One 4-D tiled load
+//     halo   : filters of stride 1 along W, or 2 where the input can be read as pixel pairs.  A tile is TH x TW output pixels of one image.  One 4-D tiled load
 //              brings the (TH + halo) x (TW + halo) input patch of a channel block, zero filled
 //              outside the image (the exact code of 0.0 under a symmetric quantizer).  Every filter
 //              tap (r, s) is then the same patch read from a start address shifted by
@@ -22,14 +21,14 @@
 //   B operand (KRSC weights), three sources
 //     resident : the whole layer's weights sit in shared memory for the CTA's lifetime;
 //     ring     : (halo) BN x BK tiles per tap and channel block through their own ring, several taps per
-//                stage (one TMA operation) for tiles up to 128 columns;
+//                stage (one TMA operation) for tiles up to 128 columns and for CTA pairs;
 //     stage    : (plain, im2col) one BN x BK tile next to each A block of a stage.
 //
-// Roles (one lane each unless noted):
+// Roles (whole converged warps, an elected lane issues):
 //   warp 0     : TMA producer of A patches / blocks and of B tiles;
 //   warps 1, 4 : tcgen05.mma.kind::i8 issue (128 x BN x 32 per instruction, int32 accumulators in a
-//                ring of up to four TMEM buffers), alternate tiles each, so that the per-tile
-//                bookkeeping of one lane overlaps the issue of the other; tcgen05.commit releases
+//   (and 5)      ring of up to four TMEM buffers), alternate tiles each, so that the per-tile
+//                bookkeeping of one warp overlaps the issue of the other; tcgen05.commit releases
 //                stages and publishes accumulators.  Warp 1 also owns the TMEM allocation;
 //   warp 2     : hands 8-bit tile buffers to the epilogue groups, filled by TMA with the residual
 //                tile of the fused eltwise sum when there is one;
@@ -461,7 +460,8 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
           bulk_commit();
           if (one_each) {
             // one buffer per group: its group waits for it, so it is handed back as soon as it has been read (3x3
-            // 128->192 at 73x73, two groups: 65.5 -> 62.3 us; with more buffers the wait would only hold up this warp)
+            // 128->192 at 73x73, batch 64, two groups: 66.0 -> 62.3 us; with more buffers the wait would only hold up
+            // this warp)
             bulk_wait_read<0>();
             mbar_arrive(bempty0 + slot * 8u);
           } else {
@@ -900,6 +900,8 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   while (p.acc_stride < BN) p.acc_stride *= 2;
   p.nacc = 512 / p.acc_stride < kMaxAcc ? 512 / p.acc_stride : kMaxAcc;
   p.tmem_cols = p.nacc * p.acc_stride;  // a power of two in [32, 512]
+  // Three issuing warps where four accumulators allow it: 64-column tiles gain (3x3 64->64 at 300x300, batch 32: 130 ->
+  // 106 us; at 56x56, batch 64: 13.4 -> 12.4 us), wider ones are within 4 % either way (64->128 at 150x150 43.6 -> 45.4 us).
   // With two accumulators a third lane could wait on an accumulator barrier two phases ahead (the release it waits
   // for may belong to a tile that another lane has not issued yet); with four, the tile that last used the
   // accumulator was issued before this lane's previous tile.
@@ -939,12 +941,12 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   p.cta2 = 0;
   p.m_tiles_real = p.m_tiles;
   {
-    // Worth it once every SM pair has two work items (28x28 3x3 128->128, batch 64: 16.0 -> 15.0 us).  Shorter
-    // launches gain a microsecond alone but lose inside a network whose branches run on several streams
-    // (clusters need two free SMs of one pair at the same time), so they stay single CTAs.  Tile widths whose
-    // halves keep whole 16-row groups.  Layers with resident weights stay single CTAs: they are bound by the
-    // issue rate of the MMA lanes, which a third lane cures better (300x300 64->64: 167 us with two lanes, 154 us
-    // as pairs, 135 us with three lanes).
+    // Long launches only, three items per pair of SMs and more: batch 32 at 150x150 128->128 97.0 -> 78.5 us, 75x75
+    // 256->256 80.0 -> 68.0 us, batch 64 at 73x73 128->192 67.8 -> 60.1 us, at 35x35 96->96 16.5 -> 14.7 us.  At the lower
+    // end they can lose (28x28 128->128, batch 64: 11.7 -> 12.7 us), and inside a network whose branches run on several
+    // streams a cluster needs two free SMs of one pair at the same time.  Tile widths whose halves keep whole 16-row
+    // groups.  Layers with resident weights stay single CTAs: 3x3 64->64 at 300x300, batch 32 takes 106 us with them, 199 us
+    // with streamed weights, 167 us with those as pairs.
     const long long pair_items = (long long)((p.m_tiles + 1) / 2) * p.n_tiles;
     const bool can = p.a_mode == kAHalo && !paired && p.b_mode == kBRing && BN >= 96 && BN % 32 == 0 && out8 &&
                      !rows && splits == 1 && (BK == 128 || BK == 64) &&
@@ -953,7 +955,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
       p.cta2 = 1;
       p.m_tiles = (p.m_tiles + 1) / 2;              // work items are pairs of m tiles, more than two per pair of SMs
       // Teams: tiles above 128 columns leave two accumulators, hence two teams, and with two groups each an accumulator is
-      // back in half the time (3x3 128->192 at 73x73, batch 64: 62.3 -> 55.4 us).  Four teams for narrower tiles (128->128
+      // back in half the time (3x3 128->192 at 73x73, batch 64: 62.1 -> 57.3 us).  Four teams for narrower tiles (128->128
       // at 150x150 as teams of two: 74 -> 108 us, what a tile costs a group beside its columns is paid twice).
       p.pair_shift = BN > 128 ? 1 : 0;
       G = 4;

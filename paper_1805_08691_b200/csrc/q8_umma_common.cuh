@@ -27,7 +27,7 @@ constexpr int kMaxSlots = 8;            // 8-bit tile buffers over all groups
 constexpr int kMaxTaps = 64;            // halo mode: filter taps (one TMA box holds all taps of resident weights)
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 constexpr int kSmemLimit = 232448;                           // 227 KiB opt-in maximum per CTA
-constexpr int kStaticSmemReserve = 2048;                     // barriers, tap table and flags
+constexpr int kStaticSmemReserve = 2048;                     // barriers and flags
 
 enum StatusBits : unsigned int {
   kTimeoutProducer = 1u,
@@ -83,7 +83,7 @@ struct UmmaParams {
   // patch descriptor moves by in16 (16-byte units) from one tap to the next and by out16 from one group to the next
   unsigned int in16, out16;
   int tap_inner;
-  int mma_lanes;             // 3 with four accumulators (narrow tiles are bound by the issue rate of a lone lane), else 2
+  int mma_lanes;             // MMA-issuing warps: 3 with four accumulators, else 2 (see plan_tiles)
   int pair_shift;            // cta2: log2 of the epilogue groups that share the columns of a tile
   int epi_split;             // 1: every epilogue group takes a share of the columns of every tile (short launches)
   int b_T, b_chunks;         // weight ring: filter taps per ring stage (one TMA operation), stages per channel block
@@ -209,12 +209,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // (bits 16-29), unused for swizzled K-major tiles, set to 1.
 constexpr uint32_t kDescLbo = 1u << 16;
 
-// One lane of a converged warp.  The control roles issue under this predicate and never under "lane == 0": the
-// compiler knows that an elected branch holds a single thread and keeps the operands of tcgen05.mma, of the TMA
-// copies and of their barriers in uniform registers, where a lane-number branch costs some twenty moves per
-// instruction.  With 32-bit descriptor words and rolled tap loops a kernel shrinks from 240 to 75 KB of code and the
-// issuing warps stop being the limit: 3x3 64->64 at 300x300 63.3 -> 53.5 us (batch 16), 3x3 512->512 at 7x7 18.9 ->
-// 15.1 us, 3x3 64->64 + 1x1 64->256 + residual at 56x56 38.2 -> 32.3 us (batch 64), one 14x14 layer 5.3 -> 4.4 us.
+// One lane of a converged warp.  The control roles issue under this predicate and never under "lane == 0": tcgen05.mma
+// and the TMA copies take warp-uniform operands, and an elected branch tells the compiler that it holds a single thread.
+// Together with 32-bit descriptor words and rolled tap loops, timed against the branch on the lane number: 3x3 64->64 at
+// 300x300 63.3 -> 53.5 us (batch 16), 3x3 512->512 at 7x7 18.9 -> 15.1 us, 3x3 64->64 + 1x1 64->256 + residual at 56x56
+// 38.2 -> 32.3 us (batch 64), one 14x14 layer 5.3 -> 4.4 us.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
@@ -627,9 +626,9 @@ __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile&
                                              int lane, const int ch0, const int nchunk) {
   // chunks ch0 .. nchunk-1 of 16 columns each
   int ra[16], rb[16];
-  // a warp-wide reduction hands the value over in a uniform register, where the packed multiply takes it as it is; from
-  // an ordinary register it costs register pairs (1x1 64->256 at 56x56, batch 64: 18.6 us with loads, 18.2 us from a
-  // register, 17.2 us from a uniform one; 3x3 + 1x1 pair 32.0 / 30.9 / 30.3 us)
+  // passed through a warp-wide reduction, which tells the compiler that the value is the same in all lanes (1x1 64->256
+  // at 56x56, batch 64: 18.6 us with the loads, 18.2 us without the reduction, 17.2 us with it; 3x3 + 1x1 pair 32.0 /
+  // 30.9 / 30.3 us)
   const float us = kUniform ? __uint_as_float(__reduce_or_sync(0xffffffffu, __float_as_uint(t.scale))) : 0.0f;
   if (ch0 >= nchunk) {  // no columns for this warp in this tile: it still hands the accumulator back
     tcgen05_fence_before();
@@ -961,7 +960,8 @@ int pick_bn(int K, int kgemm) {
     const int n_tiles = (K + w - 1) / w;
     // cycles per 128-row block of the output: every tile of columns runs the whole reduction again (one
     // 128 x w x 32 MMA takes max(59, 0.53 w) cycles, a pipeline iteration about 550), the epilogue pays for
-    // every padded column
+    // every padded column.  Against all widths on 26 layers of the three networks' shapes the choice is the fastest
+    // or within 3 %, but for 512->2048 at 7x7, batch 64 (128 columns 9.1 us, 256 7.8 us).
     const double mma = k_steps * (0.53 * w > 59.0 ? 0.53 * w : 59.0), feed = k_iters * 550.0;
     const double cost = n_tiles * ((mma > feed ? mma : feed) + 200.0) + (double)n_tiles * w * 8.0;
     if (best_cost < 0 || cost <= best_cost) { best = w; best_cost = cost; }
