@@ -222,8 +222,8 @@ int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan
  * Alignment: Q8_ALGO_UMMA needs x, w, y, residual 16-byte aligned, C a multiple
  * of 16, and for u8/s8 output y_ldc and y_c_offset multiples of 16.
  * Q8_ALGO_AUTO takes the same kernel for any y and residual of a u8/s8 output
- * (rows off that grid, and K that are no multiple of 16, cost it more), and otherwise a tensor-core kernel that gathers its operands
- * byte by byte (K up to 4096), or the direct kernel for the smallest calls.
+ * (rows off that grid, and K that are no multiple of 16, cost it more), and otherwise a tensor-core kernel
+ * that gathers its operands byte by byte (K up to 4096) or the direct kernel, by their estimated times.
  * Errors: Q8_ERR_INVALID_ARG (null/extent/enum, R*S*C > 65793 which could
  * overflow int32), Q8_ERR_UNSUPPORTED (Q8_ALGO_UMMA on an ineligible shape),
  * Q8_ERR_WORKSPACE, Q8_ERR_CUDA.  Nothing is launched on error. */
