@@ -26,18 +26,23 @@
 //
 // Roles (whole converged warps, an elected lane issues):
 //   warp 0     : TMA producer of A patches / blocks and of B tiles;
-//   warps 1, 4 : tcgen05.mma.kind::i8 issue (128 x BN x 32 per instruction, int32 accumulators in a
-//   (and 5)      ring of up to four TMEM buffers), alternate tiles each, so that the per-tile
+//   warps 1, 2 : tcgen05.mma.kind::i8 issue (128 x BN x 32 per instruction, int32 accumulators in a
+//   (and 3)      ring of up to four TMEM buffers), alternate tiles each, so that the per-tile
 //                bookkeeping of one warp overlaps the issue of the other; tcgen05.commit releases
 //                stages and publishes accumulators.  Warp 1 also owns the TMEM allocation;
-//   warp 2     : hands 8-bit tile buffers to the epilogue groups, filled by TMA with the residual
-//                tile of the fused eltwise sum when there is one;
-//   warp 3     : sends finished 8-bit tiles to global memory with TMA stores, recycles the buffers;
-//   warps 6..  : G epilogue groups of four warps; group g owns every G-th tile of the CTA, or, in launches
+//   warps 4..  : G epilogue groups of four warps; group g owns every G-th tile of the CTA, or, in launches
 //                with at most two tiles per CTA, a share of the columns of every tile.  A thread
 //                owns one accumulator row: tcgen05.ld, + bias, requantise, + residual, ReLU, round,
-//                clamp; the 16 bytes go back into the buffer the residual came from (same swizzled
-//                position), which then is the source of the TMA store.
+//                clamp, straight to global memory; residual bytes come from there the same way, a pair of
+//                16-column chunks ahead.
+// The epilogue moved its bytes by TMA before (residual tiles into shared-memory buffers, finished tiles out of them): a
+// copy of a 128-row box occupies the copy engine for some 400 cycles, beside those of the operands, and the store of the
+// last tile, through two barriers and another warp, ended 0.8 us after its arithmetic.  Now that is 0.2 us (14x14 256->256
+// 3x3, batch 64: from the last accumulator to the end of the CTA 2.0 -> 1.8 us in all, since 32 rows a pitch apart keep the
+// load/store unit for 47 cycles an instruction; tiles of 16 columns on one image 0.9 -> 0.6 us), and the shared memory of the buffers holds operands: ResNet-50 batch 1 285 -> 252 us, batch
+// 64 722 -> 702 us, Inception-v3 batch 64 1226 -> 1164 us, 14x14 bottleneck batch 64 33.1 -> 30.6 us.  Measured and not kept:
+// rows exchanged through shared memory so that two lanes share one (64 contiguous bytes an access): 14x14 bottleneck 33.3 us,
+// 56x56 41 us; four lanes a row by tcgen05.ld.16x128b and weight rows in permuted order: 32.3 and 44 us.
 // The kernel is launched with programmatic stream serialization: its set-up overlaps the tail of the kernel
 // before it, and every global access comes after griddepcontrol.wait.
 // All hand-offs are mbarriers, there is no block-wide barrier after the prologue.  Every wait is
@@ -133,21 +138,17 @@ __device__ __forceinline__ bool mma_role_pair(const UmmaParams& p, const MmaRole
 template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
 __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     conv_umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                     const __grid_constant__ CUtensorMap tmRes, const __grid_constant__ CUtensorMap tmY,
                      const __grid_constant__ UmmaParams p) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long a_full[kMaxStages], a_empty[kMaxStages];
   __shared__ __align__(8) unsigned long long b_full[kMaxBStages], b_empty[kMaxBStages];
   __shared__ __align__(8) unsigned long long acc_full[kMaxAcc], acc_empty[kMaxAcc];
-  __shared__ __align__(8) unsigned long long buf_full[kMaxSlots], buf_empty[kMaxSlots];
-  __shared__ __align__(8) unsigned long long store_ready[kMaxSlots];  // per buffer: a buffer is recycled by the store
-                                                                        // lane between two uses, so no phase can be skipped
   __shared__ __align__(8) unsigned long long bres_full;
   __shared__ __align__(8) unsigned long long mma_turn[kMmaWarps];
   __shared__ uint32_t tmem_holder;
   __shared__ int abort_flag;
 
-  // dynamic smem: [resident weights] [A stages] [weight ring] [G*nbuf 8-bit tile buffers] [bias, scale]
+  // dynamic smem: [resident weights] [A stages] [weight ring] [tile buffers of moved rows] [bias, scale]
   const uint32_t raw_base = smem_u32(smem_raw);
   const uint32_t base = (raw_base + 1023u) & ~1023u;
   unsigned char* const base_ptr = smem_raw + (base - raw_base);
@@ -162,8 +163,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   const int vblock = kCta2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int vgrid = kCta2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const int total_tiles = p.m_tiles * p.n_tiles * p.splits;  // work items
-  // pair kernels (G = 4): 1 << pair_shift groups share the columns of a tile, G >> pair_shift teams take alternate ones
-  const int slots = kCta2 ? (G >> p.pair_shift) * p.nbuf : (p.epi_split ? p.nbuf : G * p.nbuf);  // split mode: nbuf counts the buffers of the CTA
 
   // Programmatic dependent launch: the next kernel of the stream may be scheduled onto SMs as they fall idle
   // (it waits below, like this one, before it touches global memory), and this kernel's own set-up (barriers,
@@ -212,14 +211,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       // one arrival per epilogue warp that reads the accumulator: a group's four, or all of them in split mode
       if (lane < p.nacc) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), kCta2 ? 8 << p.pair_shift : (p.epi_split ? 4 * G : 4)); }
       else if (lane >= 8 && lane - 8 < kMmaWarps) mbar_init(smem_u32(&mma_turn[lane - 8]), 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    } else if (warp == 2) {
-      if (lane < slots) { mbar_init(smem_u32(&buf_full[lane]), 1); mbar_init(smem_u32(&buf_empty[lane]), 1); }
-      else if (lane == 16 && p.res_mode == kResTma) prefetch_tensormap(&tmRes);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    } else if (warp == 3) {
-      if (lane < slots) mbar_init(smem_u32(&store_ready[lane]), kCta2 ? kGroupThreads << p.pair_shift : (p.epi_split ? G * kGroupThreads : kGroupThreads));
-      else if (lane == 16 && p.out8) prefetch_tensormap(&tmY);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -378,9 +369,9 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       abort_flag = 1;
       atomicOr(p.status, kTimeoutProducer);
     }
-  } else if (warp == 1 || warp == 4 || (warp == 5 && p.mma_lanes == 3)) {
-    // ------------------------------------------------------------------ MMA issuers (warps 1, 4 and 5; an elected lane issues)
-    const int who = warp == 1 ? 0 : warp - 3;
+  } else if (warp < kCtrlWarps) {
+    // ------------------------------------------------------------------ MMA issuers (warps 1 to 3; an elected lane issues)
+    const int who = warp - 1;
     MmaRoleArgs ra;
     ra.base = base; ra.tmem_base = tmem_base; ra.total_tiles = total_tiles; ra.abortp = abortp;
     ra.first_tile = (int)blockIdx.x; ra.tile_step = (int)gridDim.x;
@@ -389,7 +380,9 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     ra.acc_full = smem_u32(&acc_full[0]); ra.acc_empty = smem_u32(&acc_empty[0]);
     ra.bres_full = smem_u32(&bres_full); ra.turn = smem_u32(&mma_turn[0]);
     bool ok = true;
-    if constexpr (kCta2) {
+    if (who >= p.mma_lanes) {
+      // two issuing warps
+    } else if constexpr (kCta2) {
       if (cta_rank == 0) ok = mma_role_pair(p, ra, who, vblock, vgrid);
     } else {
       ok = mma_role(p, ra, who);
@@ -398,93 +391,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       abort_flag = 1;
       atomicOr(p.status, kTimeoutMma);
     }
-  } else if (warp == 2) {
-    // ------------------------------------------------------------------ tile-buffer / residual producer
-    if (p.nbuf > 0) {
-      TileIterT<kCta2> ti;
-      ti.init(p, vblock, vgrid, cta_rank);
-      const uint32_t bfull0 = smem_u32(&buf_full[0]), bempty0 = smem_u32(&buf_empty[0]);
-      const uint32_t nslots = (uint32_t)slots;
-      uint32_t slot = 0, par = 1;  // slots are used round robin over all groups: tile lt -> slot lt % (G*nbuf)
-      bool ok = true;
-      const int pw = 1 << p.pw_shift;
-      const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
-      if constexpr (!kCta2) asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (; ti.tile < total_tiles; ti.next(p)) {
-        if (!mbar_wait(bempty0 + slot * 8u, par, abortp)) { ok = false; break; }
-        const uint32_t bar = bfull0 + slot * 8u;
-        if (!elect_one()) {
-        } else if (p.res_mode == kResTma && ti.valid) {
-          uint32_t dst = base + p.off_bufs + slot * p.tile8_bytes;
-          mbar_arrive_expect_tx(bar, p.res_tx_bytes);
-          if (p.a_mode == kAHalo) {
-            for (int pn = 0, c = ti.nt * p.bn; pn < p.panels; ++pn, c += pw, dst += panel_bytes) tma_load_4d(dst, &tmRes, bar, c, ti.qt * p.tw, ti.pt * p.th, ti.img);
-          } else {
-            for (int pn = 0, c = ti.nt * p.bn; pn < p.panels; ++pn, c += pw, dst += panel_bytes) tma_load_2d(dst, &tmRes, bar, c, ti.mt * kBM);
-          }
-        } else {
-          mbar_arrive(bar);
-        }
-        if (++slot == nslots) { slot = 0; par ^= 1u; }
-      }
-      if (!ok && lane0) {
-        abort_flag = 1;
-        atomicOr(p.status, kTimeoutResidual);
-      }
-    }
-  } else if (warp == 3) {
-    // ------------------------------------------------------------------ output store / buffer recycler
-    if (p.nbuf > 0) {
-      TileIterT<kCta2> ti;
-      ti.init(p, vblock, vgrid, cta_rank);
-      const uint32_t bempty0 = smem_u32(&buf_empty[0]), ready0 = smem_u32(&store_ready[0]);
-      const uint32_t nslots = (uint32_t)slots;
-      uint32_t slot = 0, spar = 0;  // tile lt uses buffer lt % (G*nbuf); its use number (lt / (G*nbuf)) gives the parity
-      int prev_slot = -1;
-      const bool one_each = (kCta2 || !p.epi_split) && p.nbuf == 1;
-      bool ok = true;
-      const int pw = 1 << p.pw_shift;
-      const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
-      for (; ti.tile < total_tiles; ti.next(p)) {
-        if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
-        if (!elect_one()) {
-        } else if (p.out8) {
-          uint32_t src = base + p.off_bufs + slot * p.tile8_bytes;
-          if (!ti.valid) {
-            // second tile of the last pair of an odd count: nothing to store
-          } else if (p.a_mode == kAHalo) {
-            for (int pn = 0, c = p.c_off + ti.nt * p.bn; pn < p.panels; ++pn, c += pw, src += panel_bytes) tma_store_4d(&tmY, src, c, ti.qt * p.tw, ti.pt * p.th, ti.img);
-          } else {
-            for (int pn = 0, c = p.c_off + ti.nt * p.bn; pn < p.panels; ++pn, c += pw, src += panel_bytes) tma_store_2d(&tmY, src, c, ti.mt * kBM);
-          }
-          bulk_commit();
-          if (one_each) {
-            // one buffer per group: its group waits for it, so it is handed back as soon as it has been read (3x3
-            // 128->192 at 73x73, batch 64, two groups: 66.0 -> 62.3 us; with more buffers the wait would only hold up
-            // this warp)
-            bulk_wait_read<0>();
-            mbar_arrive(bempty0 + slot * 8u);
-          } else {
-            // the store before this one has read its buffer: hand that buffer back
-            bulk_wait_read<1>();
-            if (prev_slot >= 0) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
-          }
-          prev_slot = (int)slot;
-        } else {
-          mbar_arrive(bempty0 + slot * 8u);
-        }
-        if (++slot == nslots) { slot = 0; spar ^= 1u; }
-      }
-      if (p.out8 && elect_one()) {
-        bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
-        if (prev_slot >= 0 && !one_each) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
-      }
-      if (!ok && lane0) {
-        abort_flag = 1;
-        atomicOr(p.status, kTimeoutStore);
-      }
-    }
-  } else if (warp >= kCtrlWarps) {
+  } else {
     // ------------------------------------------------------------------ epilogue groups
     const int g = (warp - kCtrlWarps) >> 2;
     const int quad = warp & 3;  // TMEM lane quadrant this warp may read
@@ -497,6 +404,9 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     int pp = 0, qq = 0;
     t.srow = row;
     t.smem_ok = true;
+    t.yrow = nullptr;
+    t.rrow = nullptr;
+    t.wide = t.res_wide = false;
     if (p.a_mode == kAHalo) {
       pp = row / p.twb;  // once per thread
       qq = row - pp * p.twb;
@@ -509,8 +419,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     const uint32_t accf0 = smem_u32(&acc_full[0]);
     uint32_t acce0 = smem_u32(&acc_empty[0]);
     if constexpr (kCta2) acce0 = map_to_cta(acce0, 0);
-    const uint32_t bfull0 = smem_u32(&buf_full[0]), ready0 = smem_u32(&store_ready[0]);
-    const uint32_t nslots = (uint32_t)slots, nacc = (uint32_t)p.nacc;
+    const uint32_t nacc = (uint32_t)p.nacc;
     // split mode: every group works on every tile and takes the chunks [ch0, ch1) of its columns, so that a
     // launch with one or two tiles per CTA does not leave three of four groups idle
     const bool split = p.epi_split != 0;
@@ -524,7 +433,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       ch1 = ((member + 1) * nchunk_all) >> p.pair_shift;
     }
     uint32_t ab = (uint32_t)team % nacc, acc_par = ((uint32_t)team / nacc) & 1u;
-    uint32_t slot = (uint32_t)team, slot_par = 0;
     TileIterT<kCta2> ti;
     ti.init(p, vblock + team * vgrid, tile_step * vgrid, cta_rank);
     for (; ti.tile < total_tiles; ti.next(p)) {
@@ -534,23 +442,28 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         if (p.a_mode == kAHalo) {
           const int pr = ti.pt * p.th + pp, qc = ti.qt * p.tw + qq;
           t.row_ok = t.smem_ok && pr < p.P && qc < p.Q && ti.valid;
-          t.m = ((long long)ti.img * p.P + pr) * p.Q + qc;
+          t.m = (ti.img * p.P + pr) * p.Q + qc;
         } else {
-          t.m = (long long)ti.mt * kBM + row;
+          t.m = ti.mt * kBM + row;
           t.row_ok = t.m < p.M;
         }
       };
+      place();
+      ResPair rp = {};
       RowMove mv;
       if constexpr (kRes == kResRows) {  // one buffer per group, shared where groups share tiles: their columns are disjoint
-        place();
         t.buf = base_ptr + p.off_bufs + (split ? (size_t)0 : (size_t)g * p.tile8_bytes);
         mv.init(p, t.n0, ch0, ch1);
         if (p.res_mode != kResNone) rows_in(p, t, mv, lane);  // while the accumulator is being formed
         __syncwarp();
+      } else {
+        t.wide = p.y_wide && ((t.n0 + ch0 * 16) & 31) == 0;
+        t.res_wide = p.res_wide && ((t.n0 + ch0 * 16) & 31) == 0;
+        t.yrow = static_cast<unsigned char*>(p.y) + (long long)t.m * p.ldc + p.c_off + t.n0;
+        t.rrow = p.res + (long long)t.m * p.K + t.n0;
+        if (kRes == kResVec && p.res_mode != kResNone) load_residual(p, t, ch0, ch1, rp);  // the first bytes, likewise
       }
-      bool ok = mbar_wait(accf0 + ab * 8u, acc_par, abortp);
-      if (p.nbuf > 0 && ok) ok = mbar_wait(bfull0 + slot * 8u, slot_par, abortp);
-      if (!ok) {
+      if (!mbar_wait(accf0 + ab * 8u, acc_par, abortp)) {
         if (lane == 0) {
           abort_flag = 1;
           atomicOr(p.status, kTimeoutEpilogue);
@@ -558,26 +471,15 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         break;
       }
       tcgen05_fence_after();
-      if constexpr (kRes != kResRows) {
-        place();
-        t.buf = p.nbuf > 0 ? base_ptr + p.off_bufs + (size_t)slot * p.tile8_bytes : nullptr;
-      }
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * (uint32_t)p.acc_stride;
-      epilogue_row<kOut, kRes, kCta2, kUniform>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1);
+      epilogue_row<kOut, kRes, kCta2, kUniform, kRes == kResRows>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1, rp);
       if constexpr (kRes == kResRows) {
         __syncwarp();
         rows_out(p, t, mv, lane);
         __syncwarp();  // the buffer is read before the next tile's rows go into it
       }
-      if (p.nbuf > 0) {
-        // this thread's reads and writes of the buffer are done; the store thread takes over
-        if (p.out8) fence_proxy_async_smem();
-        mbar_arrive(ready0 + slot * 8u);
-      }
       ab += (uint32_t)tile_step;
       while (ab >= nacc) { ab -= nacc; acc_par ^= 1u; }
-      slot += (uint32_t)tile_step;
-      if (slot >= nslots) { slot -= nslots; slot_par ^= 1u; }
     }
   }
 
@@ -594,8 +496,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
 
 // ------------------------------------------------------------------------------------------ host
 template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
-int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmRes, const CUtensorMap& tmY,
-                   const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
+int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
   auto kernel = conv_umma_kernel<G, kOut, kRes, kCta2, kUniform>;
   static std::atomic<bool> configured[kMaxDevices];  // per instantiation and device (the attribute is per device)
   const int dev = current_device();
@@ -630,7 +531,7 @@ int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtenso
     attr[pdl].val.clusterDim.z = 1;
     cfg.numAttrs = pdl + 1;
   }
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB, tmRes, tmY, p);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB, p);
   if (le != cudaSuccess) {
     cudaGetLastError();
     return fail(Q8_ERR_CUDA, "conv_umma: launch failed (%s; grid %d, block %d, shared memory %zu, cluster %d)", cudaGetErrorString(le),
@@ -640,28 +541,27 @@ int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtenso
 }
 
 template <int G>
-int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmRes, const CUtensorMap& tmY,
-                  const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
+int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaParams& p, bool rows, size_t dyn, int grid, cudaStream_t stream) {
 #define Q8_LAUNCH(OUT, RES)                                                                                       \
   do {                                                                                                            \
-    if (p.scale_count == 1) return launch_variant<G, OUT, RES, false, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream); \
-    return launch_variant<G, OUT, RES, false, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream);                 \
+    if (p.scale_count == 1) return launch_variant<G, OUT, RES, false, true>(tmA, tmB, p, dyn, grid, stream); \
+    return launch_variant<G, OUT, RES, false, false>(tmA, tmB, p, dyn, grid, stream);                 \
   } while (0)
-  // kResTma stands for "a residual through the tile buffers, or none"
+  // kResVec stands for "a residual through the tile buffers, or none"
   const bool global_res = p.res_mode == kResGlobal;
   if (p.y_type == Q8_U8) {
-    if (!p.out8) Q8_LAUNCH(Q8_U8, kResRows);
-    Q8_LAUNCH(Q8_U8, kResTma);
+    if (rows) Q8_LAUNCH(Q8_U8, kResRows);
+    Q8_LAUNCH(Q8_U8, kResVec);
   }
   if (p.y_type == Q8_S8) {
-    if (!p.out8) Q8_LAUNCH(Q8_S8, kResRows);
-    Q8_LAUNCH(Q8_S8, kResTma);
+    if (rows) Q8_LAUNCH(Q8_S8, kResRows);
+    Q8_LAUNCH(Q8_S8, kResVec);
   }
   if (p.y_type == Q8_F32) {
     if (global_res) Q8_LAUNCH(Q8_F32, kResGlobal);
-    Q8_LAUNCH(Q8_F32, kResTma);
+    Q8_LAUNCH(Q8_F32, kResVec);
   }
-  return launch_variant<G, Q8_S32, kResTma, false, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, stream);
+  return launch_variant<G, Q8_S32, kResVec, false, false>(tmA, tmB, p, dyn, grid, stream);
 #undef Q8_LAUNCH
 }
 
@@ -722,7 +622,7 @@ namespace {
 struct UmmaPlan {
   UmmaParams p;
   HaloTile ht;
-  int G, res_mode, pw, c_eff;
+  int G, res_mode, c_eff;
   bool rows, paired, resident;
   size_t dyn;
 };
@@ -823,7 +723,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   const q8_conv_desc& d = a.d;
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   int res_mode = kResNone;
-  if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResTma : (out8 ? kResRows : kResGlobal);
+  if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResVec : (out8 ? kResRows : kResGlobal);
   // 8-bit rows that TMA cannot address are moved by the epilogue warps, in both directions if in one
   const bool rows = out8 && (rows_off_tma(a) || res_mode == kResRows);
   if (rows && a.residual) res_mode = kResRows;
@@ -910,8 +810,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   p.b_tile_bytes = (unsigned)(BN * BK);
   p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
 
-  // ---- shared memory plan: [resident weights] [A stages] [weight ring] [8-bit tile buffers] [bias, scale]
-  const bool use_bufs = (out8 && !rows) || res_mode == kResTma;
+  // ---- shared memory plan: [resident weights] [A stages] [weight ring] [tile buffers of moved rows] [bias, scale]
   // Launches with at most two work items per CTA cannot keep several groups busy on different tiles: there all
   // four groups share every tile, each taking a quarter of its columns (any tile width, both accumulators).
   {
@@ -978,7 +877,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
       // Weight ring stages of several filter taps, one TMA operation each (the copy engine spends ~600 cycles
       // per operation whatever its size): as many taps as fit in about 48 KiB while two such stages fit beside
       // two activation stages and one tile buffer per epilogue group, spread evenly over a channel block.
-      const unsigned fixed = bres_bytes + row_bytes + (use_bufs ? (unsigned)(p.epi_split ? 2 : (p.cta2 ? G >> p.pair_shift : G)) * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
+      const unsigned fixed = bres_bytes + row_bytes + 2u * p.a_stage_bytes;
       const unsigned avail = budget > fixed ? budget - fixed : 0u;
       int T = (int)(48u * 1024u / p.b_tile_bytes);
       if (T > (int)(avail / (2u * p.b_tile_bytes))) T = (int)(avail / (2u * p.b_tile_bytes));
@@ -1001,17 +900,8 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
     p.a_stage_bytes = (unsigned)p.kb * unit;
     min_pipe = 2u * p.a_stage_bytes;
   }
-  p.nbuf = 0;
-  if (use_bufs) {
-    // two buffers per group (team) when that still leaves a comfortable pipeline
-    const unsigned teams = p.cta2 ? (unsigned)(G >> p.pair_shift) : (unsigned)G;
-    p.nbuf = (budget >= bres_bytes + 2u * teams * p.tile8_bytes + 2u * min_pipe && 2 * teams <= (unsigned)kMaxSlots) ? 2 : 1;
-    p.nbuf = tune_env("Q8_NBUF", p.nbuf, 1, p.nbuf);
-    if (p.epi_split) p.nbuf = 2;  // one buffer per tile in flight; a CTA has at most two tiles
-  }
-  const unsigned buf_bytes = row_bytes + (unsigned)(p.epi_split ? p.nbuf : (p.cta2 ? G >> p.pair_shift : G) * p.nbuf) * p.tile8_bytes;
-  if (budget < bres_bytes + buf_bytes + min_pipe) return false;
-  unsigned rest = budget - bres_bytes - buf_bytes;
+  if (budget < bres_bytes + row_bytes + min_pipe) return false;
+  unsigned rest = budget - bres_bytes - row_bytes;
   p.b_stages = 0;
   if (p.b_mode == kBRing) {
     int bst = (int)((rest - 2u * p.a_stage_bytes) / p.b_sub_bytes);
@@ -1025,12 +915,12 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   p.off_a = bres_bytes;
   p.off_bring = p.off_a + (unsigned)p.stages * p.a_stage_bytes;
   p.off_bufs = p.off_bring + (unsigned)p.b_stages * p.b_sub_bytes;
-  p.off_chan = p.off_bufs + buf_bytes;
+  p.off_chan = p.off_bufs + row_bytes;
   size_t dyn = 1024u + p.off_chan + chan_bytes;
   if (dyn > (size_t)(kSmemLimit - kStaticSmemReserve)) return false;
   // at least 120 KiB so that one CTA owns an SM and with it the whole TMEM
   plan->dyn = dyn < 120 * 1024 ? 120 * 1024 : dyn;
-  plan->G = G; plan->res_mode = res_mode; plan->pw = pw; plan->c_eff = c_eff;
+  plan->G = G; plan->res_mode = res_mode; plan->c_eff = c_eff;
   plan->rows = rows; plan->paired = paired; plan->resident = resident;
   return true;
 }
@@ -1045,16 +935,14 @@ int launch_planned(const ConvArgs& a, int splits) {
   if (!status) return fail(Q8_ERR_CUDA, "conv_umma: status word not available");
   UmmaParams& p = plan.p;
   const HaloTile& ht = plan.ht;
-  const int BK = p.bk, BN = p.bn, G = plan.G, res_mode = plan.res_mode, pw = plan.pw, c_eff = plan.c_eff;
+  const int BK = p.bk, BN = p.bn, G = plan.G, res_mode = plan.res_mode, c_eff = plan.c_eff;
   const bool rows = plan.rows, paired = plan.paired, resident = plan.resident;
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   const size_t dyn = plan.dyn;
   const CUtensorMapSwizzle swz = swizzle_for_bytes(BK);
 
   // ---- tensor maps
-  CUtensorMap tmA, tmB, tmRes, tmY;
-  memset(&tmRes, 0, sizeof(tmRes));
-  memset(&tmY, 0, sizeof(tmY));
+  CUtensorMap tmA, tmB;
   CUresult cr;
   const cuuint32_t ones[4] = {1, 1, 1, 1};
   if (p.a_mode == kAPlain) {
@@ -1111,34 +999,6 @@ int launch_planned(const ConvArgs& a, int splits) {
   }
   if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: weight tensor map rejected (CUresult %d)", (int)cr);
 
-  // Residual and output tiles: [M][channels] matrices, or for halo tiles (channels, Q, P, N) tensors whose
-  // TH x TW box lands as TH*TW dense rows.  The output map ends at the last channel this layer owns, a multiple of 16
-  // (stores are clipped in units of 16 bytes), so the store clips ragged Cout tiles and never touches a neighbouring
-  // slice of a concatenated tensor.
-  auto encode_rows = [&](CUtensorMap* tm, void* ptr, int channels, int ld, CUtensorMapL2promotion promo) -> CUresult {
-    if (p.a_mode == kAHalo) {
-      cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)a.Q, (cuuint64_t)a.P, (cuuint64_t)d.N};
-      cuuint64_t strides[3] = {(cuuint64_t)ld, (cuuint64_t)a.Q * ld, (cuuint64_t)a.P * a.Q * ld};
-      cuuint32_t box[4] = {(cuuint32_t)pw, (cuuint32_t)ht.tw, (cuuint32_t)ht.th, 1};
-      return fn.tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, ptr, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      swizzle_for_bytes(pw), promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
-    cuuint64_t dims[2] = {(cuuint64_t)channels, (cuuint64_t)a.M};
-    cuuint64_t strides[1] = {(cuuint64_t)ld};
-    cuuint32_t box[2] = {(cuuint32_t)pw, (cuuint32_t)kBM};
-    return fn.tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, ptr, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    swizzle_for_bytes(pw), promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  };
-  if (res_mode == kResTma) {
-    cr = encode_rows(&tmRes, const_cast<void*>(a.residual), d.K, d.K, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-    if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: residual tensor map rejected (CUresult %d)", (int)cr);
-  }
-  if (out8 && !rows) {
-    cr = encode_rows(&tmY, a.y, a.c_off + d.K, a.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
-    if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: output tensor map rejected (CUresult %d)", (int)cr);
-  }
-  p.res_tx_bytes = (unsigned)BN * (p.a_mode == kAHalo ? (unsigned)(ht.tw * ht.th) : (unsigned)kBM);
-
   // instruction descriptor: D = s32 (2 << 4); A format at bit 7 (0 = u8, 1 = s8); B = s8 at bit 10;
   // both operands K-major; N/8 at bit 17; M/16 at bit 24.
   p.idesc = (2u << 4) | ((d.x_type == Q8_S8 ? 1u : 0u) << 7) | (1u << 10) | ((unsigned)(BN >> 3) << 17) |
@@ -1158,7 +1018,9 @@ int launch_planned(const ConvArgs& a, int splits) {
   p.res_signed = d.res_type == Q8_S8;
   p.res_scale = a.residual_scale;
   p.y = a.y; p.y_type = d.y_type; p.ldc = a.ldc; p.c_off = a.c_off; p.relu = d.relu;
-  p.out8 = out8 && !rows ? 1 : 0;
+  // an 8-bit row is stored and its residual loaded in whole 32-byte sectors where the pitch allows it
+  p.y_wide = out8 && !rows && (reinterpret_cast<uintptr_t>(a.y) & 31u) == 0 && a.ldc % 32 == 0 && a.c_off % 32 == 0;
+  p.res_wide = res_mode == kResVec && (reinterpret_cast<uintptr_t>(a.residual) & 31u) == 0 && d.K % 32 == 0;
   p.y_vec = out8 ? 1 : (aligned16(a.y) && a.ldc % 4 == 0 && a.c_off % 4 == 0);
   p.status = status;
 
@@ -1174,22 +1036,22 @@ int launch_planned(const ConvArgs& a, int splits) {
     // take a residual: their kernels keep that choice at compile time.
 #define Q8_PAIR_LAUNCH(GG, OUT, RES)                                                                                      \
   do {                                                                                                                   \
-    if (p.scale_count == 1) return launch_variant<GG, OUT, RES, true, true>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream); \
-    return launch_variant<GG, OUT, RES, true, false>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);                      \
+    if (p.scale_count == 1) return launch_variant<GG, OUT, RES, true, true>(tmA, tmB, p, dyn, grid, a.stream); \
+    return launch_variant<GG, OUT, RES, true, false>(tmA, tmB, p, dyn, grid, a.stream);                      \
   } while (0)
 #define Q8_PAIR(GG)                                                                                                      \
   do {                                                                                                                   \
-    if (d.y_type == Q8_U8 && res_mode == kResTma) Q8_PAIR_LAUNCH(GG, Q8_U8, kResTma);                                    \
+    if (d.y_type == Q8_U8 && res_mode == kResVec) Q8_PAIR_LAUNCH(GG, Q8_U8, kResVec);                                    \
     if (d.y_type == Q8_U8) Q8_PAIR_LAUNCH(GG, Q8_U8, kResNone);                                                          \
-    if (res_mode == kResTma) Q8_PAIR_LAUNCH(GG, Q8_S8, kResTma);                                                         \
+    if (res_mode == kResVec) Q8_PAIR_LAUNCH(GG, Q8_S8, kResVec);                                                         \
     Q8_PAIR_LAUNCH(GG, Q8_S8, kResNone);                                                                                 \
   } while (0)
     Q8_PAIR(4);
 #undef Q8_PAIR
 #undef Q8_PAIR_LAUNCH
   }
-  if (G == 2) return launch_groups<2>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);
-  return launch_groups<4>(tmA, tmB, tmRes, tmY, p, dyn, grid, a.stream);
+  if (G == 2) return launch_groups<2>(tmA, tmB, p, rows, dyn, grid, a.stream);
+  return launch_groups<4>(tmA, tmB, p, rows, dyn, grid, a.stream);
 }
 }  // namespace
 

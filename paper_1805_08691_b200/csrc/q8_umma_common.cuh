@@ -16,14 +16,13 @@ namespace q8 {
 namespace {
 
 constexpr int kBM = 128;
-constexpr int kCtrlWarps = 6;            // producer, MMA 0, buffers/residual, store, MMA 1, spare
+constexpr int kCtrlWarps = 4;            // producer, MMA 0, 1, 2
 constexpr int kCtrlThreads = kCtrlWarps * 32;
 constexpr int kMmaWarps = 3;             // at most this many MMA-issuing lanes; tile lt belongs to lane lt % mma_lanes
 constexpr int kGroupThreads = 128;      // one epilogue group
 constexpr int kMaxStages = 8;           // A stages
 constexpr int kMaxBStages = 8;          // weight ring
 constexpr int kMaxAcc = 4;
-constexpr int kMaxSlots = 8;            // 8-bit tile buffers over all groups
 constexpr int kMaxTaps = 64;            // halo mode: filter taps (one TMA box holds all taps of resident weights)
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 constexpr int kSmemLimit = 232448;                           // 227 KiB opt-in maximum per CTA
@@ -33,11 +32,9 @@ enum StatusBits : unsigned int {
   kTimeoutProducer = 1u,
   kTimeoutMma = 2u,
   kTimeoutEpilogue = 4u,
-  kTimeoutResidual = 8u,
-  kTimeoutStore = 16u,
 };
 
-enum ResMode : int { kResNone = 0, kResTma = 1, kResGlobal = 2, kResRows = 3 };
+enum ResMode : int { kResNone = 0, kResVec = 1, kResGlobal = 2, kResRows = 3 };
 enum AMode : int { kAPlain = 0, kAIm2col = 1, kAHalo = 2 };
 enum BMode : int { kBStage = 0, kBResident = 1, kBRing = 2 };
 
@@ -65,7 +62,6 @@ struct UmmaParams {
   int p_tiles, q_tiles;      // halo: tiles per image column / row
   int stages, b_stages;      // A stages, weight-ring stages
   int nacc, acc_stride, tmem_cols;  // TMEM accumulators, columns between them, allocation (power of two)
-  int nbuf;                  // 8-bit tile buffers per epilogue group (0: none)
   int m_tiles, n_tiles;
   FastDiv fd_ntiles, fd_perimg, fd_qtiles, fd_pq, fd_q;  // n_tiles, p_tiles*q_tiles, q_tiles, P*Q, Q
   int splits, kps;           // split-K: work item = (tile, split), each split runs kps of the k_iters iterations
@@ -89,7 +85,6 @@ struct UmmaParams {
   int b_T, b_chunks;         // weight ring: filter taps per ring stage (one TMA operation), stages per channel block
   unsigned int a_stage_bytes;
   unsigned int tile8_bytes;
-  unsigned int res_tx_bytes; // bytes one residual tile load delivers
   unsigned int off_a, off_bring, off_bufs, off_chan;  // from the 1 KiB aligned base; resident weights at 0
   int pw_shift, pmask, panels;  // 8-bit tiles live in smem as panels of 2^pw_shift bytes per row
   int k_pad;                 // n_tiles * bn channels of bias/scale staged in smem
@@ -100,7 +95,8 @@ struct UmmaParams {
   int res_mode, res_signed;
   float res_scale;
   void* y;
-  int y_type, y_vec, out8, ldc, c_off, relu;
+  int y_type, y_vec, ldc, c_off, relu;
+  int y_wide, res_wide;      // 8-bit rows of the output, of the residual, start on 32-byte lines
   unsigned int* status;
 };
 
@@ -279,20 +275,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
-  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-               ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-               : "memory");
-}
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-               ::"l"(map), "r"(src), "r"(c0), "r"(c1)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
@@ -468,8 +450,11 @@ struct EpiTile {
   const int* s_bias;       // smem, k_pad entries
   const float* s_scale;    // smem, k_pad entries
   float scale;             // the first of them: the multiplier of every channel when there is one per tensor
-  unsigned char* buf;      // this tile's 8-bit buffer (residual in, output out) or nullptr
-  long long m;             // output pixel (row of the [M][Cout] result) of this thread
+  unsigned char* buf;      // 8-bit tile in shared memory (kTile, kResRows)
+  unsigned char* yrow;     // this thread's row of the 8-bit output, at the tile's first channel
+  const unsigned char* rrow;  // ... of the residual
+  bool wide, res_wide;     // pairs of chunks of those rows start on 32-byte lines
+  int m;                   // output pixel (row of the [M][Cout] result, fewer than 2^31) of this thread
   long long y_off;         // element offset of this work item's output (split-K partial results), else 0
   int srow;                // row of this thread's pixel inside the 8-bit tile buffer
   uint32_t row_base, swz;  // byte offset of that row inside a panel, and the row's swizzle term (set by epi_row_setup)
@@ -477,6 +462,35 @@ struct EpiTile {
   bool row_ok;             // the pixel exists (inside the image and below M)
   bool smem_ok;            // this accumulator row maps to a pixel of the tile (always, except halo tiles)
 };
+
+// 32 bytes of one row, a whole sector.
+__device__ __forceinline__ void store_32(unsigned char* g, const uint4& a, const uint4& b) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(g), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+__device__ __forceinline__ void load_32(const unsigned char* g, uint4& a, uint4& b) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+               : "l"(g)
+               : "memory");
+}
+
+// Residual bytes of the chunks ch and ch + 1 of this thread's row (zero where there are none).
+struct ResPair { uint4 a, b; };
+__device__ __forceinline__ void load_residual(const UmmaParams& p, const EpiTile& t, int ch, int nchunk, ResPair& r) {
+  r.a = r.b = make_uint4(0u, 0u, 0u, 0u);
+  const int nb = t.n0 + ch * 16;
+  if (!t.row_ok || nb >= p.K) return;
+  const unsigned char* g = t.rrow + ch * 16;
+  const bool two = ch + 1 < nchunk && nb + 16 < p.K;
+  if (t.res_wide && two) {
+    load_32(g, r.a, r.b);
+  } else {
+    r.a = *reinterpret_cast<const uint4*>(g);
+    if (two) r.b = *reinterpret_cast<const uint4*>(g + 16);
+  }
+}
 
 // Position of a thread's row in the swizzled 8-bit tile buffers: constant for the thread's lifetime.  A panel is
 // 128 rows of 2^pw_shift bytes; the 16-byte chunk index of a row is XORed with address bits 7.. (the swizzle the
@@ -486,22 +500,25 @@ __device__ __forceinline__ void epi_row_setup(const UmmaParams& p, EpiTile& t) {
   t.swz = ((t.row_base >> 7) & (uint32_t)p.pmask) << 4;
 }
 
-// One 16-column chunk of one accumulator row.  kOut: Q8_U8, Q8_S8, Q8_S32 or Q8_F32.  kRes: kResNone, kResTma
-// (a residual from the tile buffer if p.res_mode says so, else none: decided at run time), kResGlobal (fp32 outputs) or
-// kResRows (8-bit rows that TMA cannot address: as kResTma, but the warps fill and empty the buffer themselves).  Fewer
+// One 16-column chunk of one accumulator row.  kOut: Q8_U8, Q8_S8, Q8_S32 or Q8_F32.  kRes: kResNone, kResVec
+// (a residual in `rv` if p.res_mode says so, else none: decided at run time), kResGlobal (fp32 outputs) or
+// kResRows (8-bit rows that 16-byte accesses cannot address: the warps move them through the tile buffer).  Fewer
 // distinct kernels matter more than one uniform branch per chunk: a launch of another kernel function than
 // the one before it starts with cold instruction caches, which costs a layer of a network 2 to 6 us, so the
-// layers with and without a residual sum share their kernels.  (One straight-line arm per case, chosen per
-// chunk or per row, made the register allocator spill.)
+// layers with and without a residual sum share their kernels.  (One straight-line copy of the rows' code per case runs 30 %
+// fewer instructions, but 3 % of ResNet-50 slower: 700 -> 730 us, 56x56 bottleneck 30.8 -> 33.9 us.)
 //   v = float(acc + bias) * s;  v += float(res) * s_res;  v = max(v, 0);  y = clamp(Round(v))
 // Each step is one IEEE fp32 operation (the library is built without FMA contraction).
 // kUniform: one multiplier for all channels (scale_count 1, `us`), else one per channel from shared memory.  A broadcast
 // load of four words takes the shared-memory port four passes like any other 512-byte load, and the loads of bias and
 // multiplier are what the epilogue waits for most.
+// Returns the sixteen bytes of an 8-bit output; wider outputs are stored here.
 template <int kOut, int kRes, bool kUniform>
-__device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTile& t, int ch, const int (&raw)[16], const float us) {
+__device__ __forceinline__ uint4 epilogue_chunk(const UmmaParams& p, const EpiTile& t, int ch, const int (&raw)[16], const float us,
+                                                const uint4 rv) {
   const int c16 = ch * 16;
   const int nb = t.n0 + c16;
+  uint4 o = make_uint4(0u, 0u, 0u, 0u);
   int acc[16];
   {
     const int4* bp = reinterpret_cast<const int4*>(t.s_bias + nb);
@@ -525,13 +542,7 @@ __device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTil
           if (j < valid) yp[j] = acc[j];
       }
     }
-    return;
-  }
-  // position of this thread's 16 bytes inside the swizzled 8-bit tile buffer
-  uint32_t off = 0;
-  if (kOut == Q8_U8 || kOut == Q8_S8 || (kRes == kResTma && p.res_mode == kResTma)) {
-    const int pn = c16 >> p.pw_shift;
-    off = t.row_base + (((uint32_t)(c16 & ((1 << p.pw_shift) - 1))) ^ t.swz) + (uint32_t)pn * ((uint32_t)kBM << p.pw_shift);
+    return o;
   }
   unsigned long long v2[8];  // v[2i], v[2i + 1]
   float v[16];
@@ -546,20 +557,9 @@ __device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTil
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) unpack_f2(v2[j], v[2 * j], v[2 * j + 1]);
-  unsigned int rw[4] = {0u, 0u, 0u, 0u};
-  if (kRes == kResRows ? p.res_mode != kResNone : (kRes == kResTma && (kOut == Q8_U8 || kOut == Q8_S8))) {
-    // the tile buffer always exists for 8-bit outputs: its bytes are read ahead of the (uniform) branch on
-    // whether they are a residual, so that the load is in flight with those of bias and scale
-    const uint4 rv = *reinterpret_cast<const uint4*>(t.buf + off);
-    rw[0] = rv.x; rw[1] = rv.y; rw[2] = rv.z; rw[3] = rv.w;
-  }
-  if (kRes == kResGlobal || ((kRes == kResTma || kRes == kResRows) && p.res_mode != kResNone)) {
-    if (kRes == kResTma || kRes == kResRows) {
-      if (kOut != Q8_U8 && kOut != Q8_S8) {
-        const uint4 rv = *reinterpret_cast<const uint4*>(t.buf + off);
-        rw[0] = rv.x; rw[1] = rv.y; rw[2] = rv.z; rw[3] = rv.w;
-      }
-    } else if (t.row_ok && nb < p.K) {
+  if (kRes == kResGlobal || ((kRes == kResVec || kRes == kResRows) && p.res_mode != kResNone)) {
+    unsigned int rw[4] = {rv.x, rv.y, rv.z, rv.w};
+    if (kRes == kResGlobal && t.row_ok && nb < p.K) {
       const int valid = min(16, p.K - nb);
       const unsigned char* rp = p.res + (size_t)t.m * p.K + nb;
 #pragma unroll
@@ -601,7 +601,7 @@ __device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTil
           if (j < valid) yp[j] = v[j];
       }
     }
-    return;
+    return o;
   }
   // 8-bit output: the saturating pack clamps to [0,255] (which also is the ReLU) or [-128,127]
   if (kOut == Q8_S8 && p.relu) {
@@ -611,58 +611,77 @@ __device__ __forceinline__ void epilogue_chunk(const UmmaParams& p, const EpiTil
   int z[16];
 #pragma unroll
   for (int j = 0; j < 16; ++j) z[j] = __float2int_rn(v[j]);
-  uint4 o;
   o.x = pack4_sat<kOut == Q8_S8>(z[0], z[1], z[2], z[3]);
   o.y = pack4_sat<kOut == Q8_S8>(z[4], z[5], z[6], z[7]);
   o.z = pack4_sat<kOut == Q8_S8>(z[8], z[9], z[10], z[11]);
   o.w = pack4_sat<kOut == Q8_S8>(z[12], z[13], z[14], z[15]);
-  if (t.smem_ok) *reinterpret_cast<uint4*>(t.buf + off) = o;
+  return o;
 }
 
-// All chunks of one accumulator row, TMEM loads one chunk ahead of the arithmetic.  The accumulator
-// is released (acc_empty) as soon as its last chunk is in registers.
-template <int kOut, int kRes, bool kPair, bool kUniform>
+// Byte offset of a 16-byte chunk of this thread's row inside a swizzled 8-bit tile in shared memory.
+__device__ __forceinline__ uint32_t tile_offset(const UmmaParams& p, const EpiTile& t, int ch) {
+  const int c16 = ch * 16;
+  return t.row_base + (((uint32_t)(c16 & ((1 << p.pw_shift) - 1))) ^ t.swz) + (uint32_t)(c16 >> p.pw_shift) * ((uint32_t)kBM << p.pw_shift);
+}
+
+// All chunks of one accumulator row, TMEM loads one chunk ahead of the arithmetic, residual bytes one pair of chunks ahead
+// (`r` holds the first pair on entry).  The accumulator is released (acc_empty) as soon as its last chunk is in registers.
+// 8-bit results go straight to global memory, 32 bytes a lane, or with kTile into the shared-memory tile t.buf.
+template <int kOut, int kRes, bool kPair, bool kUniform, bool kTile>
 __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile& t, uint32_t taddr, uint32_t acc_empty_bar,
-                                             int lane, const int ch0, const int nchunk) {
+                                             int lane, const int ch0, const int nchunk, ResPair r) {
   // chunks ch0 .. nchunk-1 of 16 columns each
+  constexpr bool k8 = kOut == Q8_U8 || kOut == Q8_S8;
   int ra[16], rb[16];
   // passed through a warp-wide reduction, which tells the compiler that the value is the same in all lanes (1x1 64->256
   // at 56x56, batch 64: 18.6 us with the loads, 18.2 us without the reduction, 17.2 us with it; 3x3 + 1x1 pair 32.0 /
   // 30.9 / 30.3 us)
   const float us = kUniform ? __uint_as_float(__reduce_or_sync(0xffffffffu, __float_as_uint(t.scale))) : 0.0f;
-  if (ch0 >= nchunk) {  // no columns for this warp in this tile: it still hands the accumulator back
+  auto release = [&] {  // every accumulator value of this warp is in registers: hand the TMEM buffer back
     tcgen05_fence_before();
     __syncwarp();
     if (lane == 0) { if constexpr (kPair) mbar_arrive_cluster(acc_empty_bar); else mbar_arrive(acc_empty_bar); }
+  };
+  if (ch0 >= nchunk) {  // no columns for this warp in this tile: it still hands the accumulator back
+    release();
     return;
   }
+  auto given = [&](int ch, const uint4& v) {  // residual bytes of a row moved through the tile buffer
+    if (kRes == kResRows && p.res_mode != kResNone) return *reinterpret_cast<const uint4*>(t.buf + tile_offset(p, t, ch));
+    return v;
+  };
   tmem_ld_16(taddr + ch0 * 16, ra);
 #pragma unroll 1
   for (int ch = ch0; ch < nchunk; ch += 2) {
     tmem_ld_wait(ra);
-    const bool more1 = ch + 1 < nchunk;
+    const bool more1 = ch + 1 < nchunk, more2 = ch + 2 < nchunk;
     if (more1) tmem_ld_16(taddr + (ch + 1) * 16, rb);
-    else {
-      // every accumulator value of this warp is in registers: hand the TMEM buffer back
-      tcgen05_fence_before();
-      __syncwarp();
-      if (lane == 0) { if constexpr (kPair) mbar_arrive_cluster(acc_empty_bar); else mbar_arrive(acc_empty_bar); }
-    }
-    epilogue_chunk<kOut, kRes, kUniform>(p, t, ch, ra, us);
+    else release();
+    ResPair next;
+    if (kRes == kResVec && p.res_mode != kResNone && more2) load_residual(p, t, ch + 2, nchunk, next);
+    const uint4 o0 = epilogue_chunk<kOut, kRes, kUniform>(p, t, ch, ra, us, given(ch, r.a));
+    if (kTile && t.smem_ok) *reinterpret_cast<uint4*>(t.buf + tile_offset(p, t, ch)) = o0;
+    uint4 o1 = make_uint4(0u, 0u, 0u, 0u);
     if (more1) {
       tmem_ld_wait(rb);
-      const bool more2 = ch + 2 < nchunk;
       if (more2) tmem_ld_16(taddr + (ch + 2) * 16, ra);
-      else {
-        tcgen05_fence_before();
-        __syncwarp();
-        if (lane == 0) { if constexpr (kPair) mbar_arrive_cluster(acc_empty_bar); else mbar_arrive(acc_empty_bar); }
-      }
-      epilogue_chunk<kOut, kRes, kUniform>(p, t, ch + 1, rb, us);
+      else release();
+      o1 = epilogue_chunk<kOut, kRes, kUniform>(p, t, ch + 1, rb, us, given(ch + 1, r.b));
+      if (kTile && t.smem_ok) *reinterpret_cast<uint4*>(t.buf + tile_offset(p, t, ch + 1)) = o1;
     }
+    if (k8 && !kTile && t.row_ok) {
+      const int nb = t.n0 + ch * 16;
+      unsigned char* g = t.yrow + ch * 16;
+      if (t.wide && more1 && nb + 16 < p.K) {
+        store_32(g, o0, o1);
+      } else {
+        if (nb < p.K) *reinterpret_cast<uint4*>(g) = o0;
+        if (more1 && nb + 16 < p.K) *reinterpret_cast<uint4*>(g + 16) = o1;
+      }
+    }
+    if (kRes == kResVec) r = next;
   }
 }
-
 // 8-bit tensors whose rows TMA cannot address (channel counts, pitches, offsets or pointers off the 16-byte grid): a warp
 // moves the rows of its 32 accumulator rows between global memory and the group's tile buffer itself.  Neighbouring lanes
 // take neighbouring words of a row, `lpr` lanes a row (a power of two that covers it, so that narrow rows share a pass);
@@ -691,7 +710,7 @@ __device__ __forceinline__ uint32_t row_buf_offset(const UmmaParams& p, int srow
 __device__ __forceinline__ void rows_in(const UmmaParams& p, const EpiTile& t, const RowMove& mv, int lane) {
   constexpr int U = 4;
   const int lpr = 1 << mv.lpr_shift, sub = lane & (lpr - 1), per_pass = 32 >> mv.lpr_shift;
-  const unsigned char* mine = p.res + t.m * p.K + t.n0 + mv.c0;
+  const unsigned char* mine = p.res + (long long)t.m * p.K + t.n0 + mv.c0;
 #pragma unroll 1
   for (int r0 = 0; r0 < 32; r0 += U * per_pass) {
     uintptr_t at[U];
@@ -726,7 +745,7 @@ __device__ __forceinline__ void rows_in(const UmmaParams& p, const EpiTile& t, c
 // them by the lane whose row it is (partial words in the loop over rows doubled its length).  All lanes call it.
 __device__ __forceinline__ void rows_out(const UmmaParams& p, const EpiTile& t, const RowMove& mv, int lane) {
   const int lpr = 1 << mv.lpr_shift, sub = lane & (lpr - 1);
-  unsigned char* mine = static_cast<unsigned char*>(p.y) + t.m * p.ldc + p.c_off + t.n0 + mv.c0;
+  unsigned char* mine = static_cast<unsigned char*>(p.y) + (long long)t.m * p.ldc + p.c_off + t.n0 + mv.c0;
   for (int r0 = 0; r0 < 32; r0 += 32 >> mv.lpr_shift) {
     const int r = r0 + (lane >> mv.lpr_shift);
     unsigned char* g = reinterpret_cast<unsigned char*>(__shfl_sync(0xffffffffu, (unsigned long long)mine, r));
@@ -950,7 +969,7 @@ int pick_bk(int C) {
 
 // Tile width: the multiple of 16 (power-of-two panels keep the 8-bit tile layout simple) that pads
 // Cout least; short reductions are bandwidth bound and take narrower tiles, which leaves room for
-// four TMEM accumulators and more tile buffers.
+// four TMEM accumulators.
 int pick_bn(int K, int kgemm) {
   const int cap = kgemm <= 640 ? 128 : 256;
   const double k_steps = (kgemm + 31) / 32, k_iters = (kgemm + 127) / 128;
@@ -995,7 +1014,7 @@ FastDiv make_fastdiv(int d) {
 //   Q8_PDL 0/1 dependent launch, Q8_HALO 0/1 halo tiles, Q8_BN tile width (multiple of 16), Q8_LANES 2/3 MMA warps,
 //   Q8_SPLIT 0/1 column-split epilogue (only where the plan allows it), Q8_G 2/4 epilogue groups, Q8_BRES 0 weights
 //   not resident, Q8_CTA2 0 no CTA pairs, Q8_CTA2MIN pair-mode threshold, Q8_BT taps per weight-ring
-//   stage, Q8_KB channel blocks per A stage, Q8_NBUF tile buffers per group, Q8_BSTAGES / Q8_STAGES ring depths (at
+//   stage, Q8_KB channel blocks per A stage, Q8_BSTAGES / Q8_STAGES ring depths (at
 //   most what fits), Q8_GRID number of CTAs (at most the default).
 int tune_env(const char* name, int dflt, int lo, int hi) {
 #ifdef Q8_TUNE_KNOBS
