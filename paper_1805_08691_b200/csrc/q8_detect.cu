@@ -6,7 +6,7 @@
 // in a fixed order (the library is built without contraction; fused steps are written as fused):
 //   * L2 normalisation across channels on 8-bit codes (one warp per pixel, integer sum of squares by dp4a);
 //   * Q_8(max(a + b, 0), q): the FP32 sum, ReLU and re-quantization of two dequantized convolution outputs;
-//   * detection output: box decoding and softmax (one thread per box), per (image, class) candidate selection by a
+//   * detection output: box decoding and softmax (exponentials only for boxes that can hold a candidate), per (image, class) candidate selection by a
 //     bitonic sort in shared memory and greedy suppression over a bit matrix of overlaps, per-image selection of
 //     the best detections.
 #include <atomic>
@@ -182,7 +182,7 @@ __device__ __forceinline__ float exp_fixed_neg(float x) {
 }
 
 constexpr int kMaxSources = 8;
-constexpr int kRegClasses = 24;   // class counts up to this keep a box's logits in registers
+constexpr int kRegClasses = 24;   // class counts up to this keep a block's logits in shared memory
 struct DetSources {
   const float* loc[kMaxSources];
   const float* conf[kMaxSources];
@@ -192,27 +192,15 @@ struct DetSources {
   int n;
 };
 
-// One thread per (image, prior): decoded corner box and the softmax of its class logits.
+// Decoded corner boxes and class probabilities:
 //   cx = (v0 l0) pw + pcx, cy = (v1 l1) ph + pcy, w = exp(v2 l2) pw, h = exp(v3 l3) ph, corners = centre -+ half
 //   e_c = exp(x_c - max x), p_c = e_c / sum_c e_c (sum in class order)
-// boxes: [N][P] float4.  Only candidates (p_c > conf_thresh, c not the background) leave the kernel: bit p of
-// masks[n][c] says whether box p is one, and only then prob[n][c][p] is written; e_c below 0.99 conf_thresh sum cannot
-// be one (the quotient is off by 2^-24 at most), which saves its division.
-// The logits of a warp's 32 boxes travel through shared memory: a thread per box would touch 21 lines with every load
-// (20.9 us at batch 32, 8732 boxes, 21 classes, against 28 MB of input).
-constexpr int kDecThreads = 256;
+// boxes: [N][P] float4.  Only candidates (p_c > conf_thresh, c not the background) leave the kernels: bit p of
+// masks[n][c] says whether box p is one, and only then prob[n][c][p] is written, and boxes[n][p] for boxes that may hold one.
+// e_c below 0.99 conf_thresh sum cannot be one (the quotient is off by 2^-24 at most), which saves its division.
 
-__global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __grid_constant__ DetSources src, const float4* __restrict__ priors,
-                                                                     float v0, float v1, float v2, float v3, int P, int classes,
-                                                                     int background, float conf_thresh, float4* __restrict__ boxes,
-                                                                     float* __restrict__ prob, unsigned int* __restrict__ masks) {
-  __shared__ float stage[kDecThreads / 32][32 * kRegClasses];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int n = blockIdx.y, lane = threadIdx.x & 31, PW = (P + 31) >> 5;
-  const int p = blockIdx.x * kDecThreads + (int)threadIdx.x;
-  if ((p & ~31) >= P) return;  // whole warps
-  const bool live = p < P;
-  const int q = live ? p : P - 1;
+// Prior q of image n: its regression and class values.
+__device__ __forceinline__ void det_source(const DetSources& src, int n, int q, int classes, const float** l, const float** x) {
   int s = 0;
 #pragma unroll
   for (int j = 1; j < kMaxSources; ++j)
@@ -220,91 +208,167 @@ __global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __gri
   const int local = q - src.first[s];
   const int cell = local / src.boxes[s], b = local - cell * src.boxes[s];
   const size_t pix = (size_t)n * src.cells[s] + cell;
-  const float* l = src.loc[s] + pix * src.loc_stride[s] + b * 4;
-  const float* x = src.conf[s] + pix * src.conf_stride[s] + (size_t)b * classes;
-  const bool in_regs = classes <= kRegClasses;
-  if (in_regs) {
-    float* st = stage[threadIdx.x >> 5];
-    const float* x0 = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), 0));
-    if (__all_sync(0xffffffffu, x == x0 + lane * classes)) {  // the warp's boxes lie one after the other
-      float t[kRegClasses];
-#pragma unroll
-      for (int c = 0; c < kRegClasses; ++c)
-        if (c < classes) t[c] = __ldg(x0 + c * 32 + lane);
-#pragma unroll
-      for (int c = 0; c < kRegClasses; ++c)
-        if (c < classes) st[c * 32 + lane] = t[c];
-    } else {
-    const unsigned int inv = 65536u / (unsigned)classes + 1u;  // k / classes for k < 32 * 24
-    for (int c0 = 0; c0 < classes; c0 += 8) {  // eight loads in flight
-      float t[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = (c0 + u) * 32 + lane, box = min((int)(((unsigned)k * inv) >> 16), 31);
-        const float* xb = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), box));
-        if (c0 + u < classes) t[u] = __ldg(xb + (k - box * classes));
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (c0 + u < classes) st[(c0 + u) * 32 + lane] = t[u];
-    }
-    }
-  }
-  const float4 pr = __ldg(priors + q);
+  *l = src.loc[s] + pix * src.loc_stride[s] + b * 4;
+  *x = src.conf[s] + pix * src.conf_stride[s] + (size_t)b * classes;
+}
+
+__device__ __forceinline__ float4 det_box(const float* l, const float4 pr, float v0, float v1, float v2, float v3) {
   const float cx = __fadd_rn(__fmul_rn(__fmul_rn(v0, l[0]), pr.z), pr.x);
   const float cy = __fadd_rn(__fmul_rn(__fmul_rn(v1, l[1]), pr.w), pr.y);
   const float w = __fmul_rn(exp_fixed(__fmul_rn(v2, l[2])), pr.z);
   const float h = __fmul_rn(exp_fixed(__fmul_rn(v3, l[3])), pr.w);
   const float hw = __fmul_rn(w, 0.5f), hh = __fmul_rn(h, 0.5f);
-  if (live) boxes[(size_t)n * P + p] = make_float4(__fsub_rn(cx, hw), __fsub_rn(cy, hh), __fadd_rn(cx, hw), __fadd_rn(cy, hh));
+  return make_float4(__fsub_rn(cx, hw), __fsub_rn(cy, hh), __fadd_rn(cx, hw), __fadd_rn(cy, hh));
+}
+
+constexpr int kDecThreads = 256;
+
+// Up to kRegClasses classes.  A block takes 256 boxes of an image, whose logits travel through shared memory (a thread per
+// box would touch 21 lines with every load).  Most boxes of a detector are background and need no exponential: the largest
+// term of the sum is exp(0) = 1, so p_c <= e_c, and a box whose foreground logits all lie `cutoff` = ln(conf_thresh), less a
+// margin for the recipe's roundings, or more below its largest has no candidate.  What is left (one box in six at a
+// threshold of 0.01) is listed, and the block's threads share its (box, class) pairs.  Comparisons are written so that a NaN
+// lists its box.  One box per thread with all of its exponentials was bound by issue (1291 warp instructions per 32 boxes,
+// 790 with a list but loads through registers, five blocks per SM): detection output of 32 images, 8732 boxes, 21 classes,
+// replayed from a graph 45.8 -> 39.8 -> 36.7 us with eight resident blocks.
+__global__ void __launch_bounds__(kDecThreads, 8) decode_listed_kernel(const __grid_constant__ DetSources src, const float4* __restrict__ priors,
+                                                                       float v0, float v1, float v2, float v3, int P, int classes,
+                                                                       int background, float conf_thresh, float cutoff, float4* __restrict__ boxes,
+                                                                       float* __restrict__ prob, unsigned int* __restrict__ masks) {
+  __shared__ __align__(16) float stage[kDecThreads * kRegClasses];
+  __shared__ float top[kDecThreads], total[kDecThreads];
+  __shared__ unsigned int bits[kRegClasses][kDecThreads / 32];
+  __shared__ unsigned short list[kDecThreads];
+  __shared__ int listed;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int n = blockIdx.y, lane = threadIdx.x & 31, PW = (P + 31) >> 5, tid = (int)threadIdx.x;
+  const int p0 = blockIdx.x * kDecThreads, p = p0 + tid;
+  const bool live = p < P;
+  const float *l, *x;
+  det_source(src, n, live ? p : P - 1, classes, &l, &x);
+  if (tid == 0) listed = 0;
+  if (tid < kRegClasses * (kDecThreads / 32)) bits[tid / (kDecThreads / 32)][tid % (kDecThreads / 32)] = 0u;
+  if ((p & ~31) < P) {  // whole warps
+    float* st = stage + (tid & ~31) * classes;
+    const float* x0 = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), 0));
+    if (__all_sync(0xffffffffu, x == x0 + lane * classes)) {  // the warp's boxes lie one after the other
+      // (asynchronous copies hold no registers: all blocks of 32 images of 8732 boxes are resident at once)
+      if ((reinterpret_cast<unsigned long long>(x0) & 15u) == 0) {
+        for (int c = lane; c < classes * 8; c += 32)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned int)__cvta_generic_to_shared(st + 4 * c)), "l"(x0 + 4 * c) : "memory");
+      } else {
+        for (int c = lane; c < classes * 32; c += 32)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned int)__cvta_generic_to_shared(st + c)), "l"(x0 + c) : "memory");
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+    } else {
+      const unsigned int inv = 65536u / (unsigned)classes + 1u;  // k / classes for k < 32 * 24
+      for (int c0 = 0; c0 < classes; c0 += 8) {  // eight loads in flight
+        float t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = (c0 + u) * 32 + lane, box = min((int)(((unsigned)k * inv) >> 16), 31);
+          const float* xb = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), box));
+          if (c0 + u < classes) t[u] = __ldg(xb + (k - box * classes));
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c0 + u < classes) st[(c0 + u) * 32 + lane] = t[u];
+      }
+    }
+  }
+  __syncthreads();
+  if (live) {
+    // the largest foreground logit against the largest of all, which is that or the background's
+    const float* xs = stage + tid * classes;
+    float f = -INFINITY;
+    const int bg = background < 0 ? classes : background;
+#pragma unroll 4
+    for (int c = 0; c < bg; ++c) f = fmaxf(f, xs[c]);
+#pragma unroll 4
+    for (int c = bg + 1; c < classes; ++c) f = fmaxf(f, xs[c]);
+    const float m = bg < classes ? fmaxf(f, xs[bg]) : f;
+    if (!(__fsub_rn(f, m) < cutoff)) list[atomicAdd(&listed, 1)] = (unsigned short)tid;
+  }
+  __syncthreads();
+  const int count = listed, items = count * classes;
+  if (tid < count) {  // the largest logit as the sum's terms see it (a NaN in front stays)
+    const int b = list[tid];
+    const float* xs = stage + b * classes;
+    float m = xs[0];
+#pragma unroll 4
+    for (int c = 1; c < classes; ++c) m = xs[c] > m ? xs[c] : m;
+    top[b] = m;
+  }
+  if (kDecThreads - 1 - tid < count) {  // its box, by other warps where the list is short
+    const int q = p0 + list[kDecThreads - 1 - tid];
+    det_source(src, n, q, classes, &l, &x);
+    boxes[(size_t)n * P + q] = det_box(l, __ldg(priors + q), v0, v1, v2, v3);
+  }
+  __syncthreads();
+  const unsigned int inv = (1u << 20) / (unsigned)classes + 1u;  // i / classes for i < 256 classes, classes <= 24
+  for (int i = tid; i < items; i += kDecThreads) {
+    const int k = (int)(((unsigned)i * inv) >> 20), c = i - k * classes, b = list[k];
+    float* xs = stage + b * classes + c;
+    *xs = exp_fixed_neg(__fsub_rn(*xs, top[b]));
+  }
+  __syncthreads();
+  if (tid < count) {
+    const int b = list[tid];
+    const float* e = stage + b * classes;
+    float sum = 0.0f;
+#pragma unroll 4
+    for (int c = 0; c < classes; ++c) sum = __fadd_rn(sum, e[c]);
+    total[b] = sum;
+  }
+  __syncthreads();
+  for (int i = tid; i < items; i += kDecThreads) {
+    const int k = (int)(((unsigned)i * inv) >> 20), c = i - k * classes, b = list[k];
+    const float e = stage[b * classes + c], sum = total[b];
+    if (c == background || e < 0.99f * conf_thresh * sum) continue;
+    const float v = __fdiv_rn(e, sum);
+    if (!(v > conf_thresh)) continue;
+    prob[((size_t)n * classes + c) * P + p0 + b] = v;
+    atomicOr(&bits[c][b >> 5], 1u << (b & 31));
+  }
+  __syncthreads();
+  if (tid < classes * (kDecThreads / 32)) {
+    const int c = tid / (kDecThreads / 32), w = tid % (kDecThreads / 32), at = (p0 >> 5) + w;
+    if (at < PW) masks[((size_t)n * classes + c) * PW + at] = bits[c][w];
+  }
+}
+
+// Any number of classes: one thread per box, its exponentials formed twice.
+__global__ void __launch_bounds__(kDecThreads) decode_softmax_kernel(const __grid_constant__ DetSources src, const float4* __restrict__ priors,
+                                                                     float v0, float v1, float v2, float v3, int P, int classes,
+                                                                     int background, float conf_thresh, float4* __restrict__ boxes,
+                                                                     float* __restrict__ prob, unsigned int* __restrict__ masks) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int n = blockIdx.y, lane = threadIdx.x & 31, PW = (P + 31) >> 5;
+  const int p = blockIdx.x * kDecThreads + (int)threadIdx.x;
+  if ((p & ~31) >= P) return;  // whole warps
+  const bool live = p < P;
+  const int q = live ? p : P - 1;
+  const float *l, *x;
+  det_source(src, n, q, classes, &l, &x);
+  if (live) boxes[(size_t)n * P + p] = det_box(l, __ldg(priors + q), v0, v1, v2, v3);
   float* pr_out = prob + (size_t)n * classes * P + p;
   unsigned int* mk = masks + (size_t)n * classes * PW + (p >> 5);
-  // the candidate bits of class c
-  auto emit = [&](int c, float e, float sum, float floor_e) -> unsigned int {
+  float m = x[0];
+  for (int c = 1; c < classes; ++c) m = x[c] > m ? x[c] : m;
+  float sum = 0.0f;
+  for (int c = 0; c < classes; ++c) sum = __fadd_rn(sum, exp_fixed_neg(__fsub_rn(x[c], m)));
+  const float floor_e = 0.99f * conf_thresh * sum;
+  for (int c = 0; c < classes; ++c) {
+    const float e = exp_fixed_neg(__fsub_rn(x[c], m));
     bool cand = live && !(e < floor_e) && c != background;
-    if (!__any_sync(0xffffffffu, cand)) return 0u;
     if (cand) {
       const float v = __fdiv_rn(e, sum);
       cand = v > conf_thresh;
       if (cand) pr_out[(size_t)c * P] = v;
     }
-    return __ballot_sync(0xffffffffu, cand);
-  };
-  if (in_regs) {
-    __syncwarp();
-    const float* xs = stage[threadIdx.x >> 5] + lane * classes;
-    float e[kRegClasses];
-#pragma unroll
-    for (int c = 0; c < kRegClasses; ++c) e[c] = c < classes ? xs[c] : -FLT_MAX;
-    float m = e[0];
-#pragma unroll
-    for (int c = 1; c < kRegClasses; ++c) m = (c < classes && e[c] > m) ? e[c] : m;
-    float sum = 0.0f;
-#pragma unroll
-    for (int c = 0; c < kRegClasses; ++c)
-      if (c < classes) {
-        e[c] = exp_fixed_neg(__fsub_rn(e[c], m));
-        sum = __fadd_rn(sum, e[c]);
-      }
-    const float floor_e = 0.99f * conf_thresh * sum;
-    unsigned int word = 0;  // lane c keeps the bits of class c
-#pragma unroll
-    for (int c = 0; c < kRegClasses; ++c)
-      if (c < classes) {
-        const unsigned int bits = emit(c, e[c], sum, floor_e);
-        if (lane == c) word = bits;
-      }
-    if (lane < classes) mk[(size_t)lane * PW] = word;
-  } else {
-    float m = x[0];
-    for (int c = 1; c < classes; ++c) m = x[c] > m ? x[c] : m;
-    float sum = 0.0f;
-    for (int c = 0; c < classes; ++c) sum = __fadd_rn(sum, exp_fixed_neg(__fsub_rn(x[c], m)));
-    const float floor_e = 0.99f * conf_thresh * sum;
-    for (int c = 0; c < classes; ++c) {
-      const unsigned int bits = emit(c, exp_fixed_neg(__fsub_rn(x[c], m)), sum, floor_e);
-      if (lane == 0) mk[(size_t)c * PW] = bits;
-    }
+    const unsigned int word = __ballot_sync(0xffffffffu, cand);
+    if (lane == 0) mk[(size_t)c * PW] = word;
   }
 }
 
@@ -818,10 +882,18 @@ int q8_detection_output(int n_sources, const float* const* loc, const int* loc_s
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(ws + L.keys);
   unsigned int* masks = reinterpret_cast<unsigned int*>(ws + L.masks);
   int* kcount = reinterpret_cast<int*>(ws + L.counts);
-  decode_softmax_kernel<<<dim3((unsigned)((P + kDecThreads - 1) / kDecThreads), (unsigned)N), kDecThreads, 0, s>>>(
-      src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2], variances[3], (int)P, classes, background,
-      conf_thresh, boxes, prob, masks);
-  int rc2 = check_launch("decode_softmax_kernel");
+  const dim3 dec_grid((unsigned)((P + kDecThreads - 1) / kDecThreads), (unsigned)N);
+  if (classes <= kRegClasses) {
+    // (where the recipe clamps its argument every class may pass)
+    const double ln = std::log((double)conf_thresh) - 1e-4;
+    const float cutoff = ln > -86.5 ? (float)(ln - 1e-5) : -INFINITY;
+    decode_listed_kernel<<<dec_grid, kDecThreads, 0, s>>>(src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2],
+                                                          variances[3], (int)P, classes, background, conf_thresh, cutoff, boxes, prob, masks);
+  } else {
+    decode_softmax_kernel<<<dec_grid, kDecThreads, 0, s>>>(src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2],
+                                                           variances[3], (int)P, classes, background, conf_thresh, boxes, prob, masks);
+  }
+  int rc2 = check_launch("decode kernel");
   if (rc2 != Q8_OK) return rc2;
   const int fg = classes - (background >= 0 ? 1 : 0);
   const int dev = current_device();

@@ -172,3 +172,26 @@ def test_detection_output_selection_limits(q8, shape):
     conf[:, ::7] = conf[:, :1]                                         # equal probabilities
     _compare(q8, loc, conf, priors, [P], [1], background=background, conf_thresh=conf_thresh, nms_thresh=nms_thresh,
              nms_top_k=top, keep_top_k=keep)
+
+
+@pytest.mark.parametrize("thresh", [0.0, 1e-40, 1e-38, 1e-30, 0.01, 0.9])
+@pytest.mark.parametrize("background", [0, 2, -1])
+def test_detection_output_at_the_listing_limit(q8, thresh, background):
+    """Boxes whose best class lies around ln(threshold) below the largest logit, in steps down to single roundings, far below
+    it, and with infinite and undefined logits: whether a box can hold a candidate is decided before any exponential."""
+    g = np.random.default_rng(3)
+    P, classes = 1000, 5
+    centre, size = g.uniform(0.1, 0.9, (P, 2)), g.uniform(0.02, 0.1, (P, 2))
+    priors = np.concatenate([centre, size], 1).astype(np.float32)
+    conf = np.full((2, P, classes), -200.0, np.float32)
+    ln = np.log(max(thresh, 1e-45))
+    top = g.uniform(-3, 3, (2, P)).astype(np.float32)
+    conf[..., max(background, 0)] = top
+    delta = g.choice([0.0, 1e-6, 1e-5, 1e-4, 1e-3, 0.1, 1.0, 20.0], (2, P)) * g.choice([-1, 1], (2, P))
+    conf[..., 3] = np.minimum(top + ln + delta, top + 0.5)
+    conf[:, ::50, 1] = np.inf
+    conf[:, 1::50, 4] = -np.inf
+    conf[:, 2::50, 0] = np.nan
+    conf[:, 3::50, 4] = np.nan
+    conf[:, 4::50] = -np.inf
+    _compare(q8, np.zeros((2, P, 4), np.float32), conf, priors, [P], [1], background=background, conf_thresh=thresh)
