@@ -1,10 +1,12 @@
-"""ctypes binding of libq8.so: argument marshalling only.
+"""Binding of libq8.so: argument marshalling only, by ctypes, and for the calls that a program makes per layer or per batch by
+a native module (csrc/q8_python.cpp).
 
 Every function has the name and meaning of the C entry point declared in include/q8.h; tensors
 are torch CUDA tensors used purely as device memory, and work is enqueued on torch's current
 stream.  There is no CPU path: importing this module without the compiled library raises.
 """
 import ctypes as C
+import importlib.util
 import os
 import shutil
 
@@ -19,6 +21,7 @@ Q8_OK = 0
 STATUS_NAMES = {0: "Q8_OK", 1: "Q8_ERR_INVALID_ARG", 2: "Q8_ERR_UNSUPPORTED", 3: "Q8_ERR_ALIGNMENT",
                 4: "Q8_ERR_WORKSPACE", 5: "Q8_ERR_CUDA", 6: "Q8_ERR_TIMEOUT", 7: "Q8_ERR_NONFINITE"}
 TORCH_DTYPES = {Q8_U8: torch.uint8, Q8_S8: torch.int8, Q8_S32: torch.int32, Q8_F32: torch.float32}
+_INT_TYPES = {torch.uint8: Q8_U8, torch.int8: Q8_S8, torch.int32: Q8_S32}
 EXPORTS = ["q8_version", "q8_last_error", "q8_read_status", "q8_calibrate_maxabs", "q8_factor", "q8_requant_scale",
            "q8_bias_factor", "q8_quantize", "q8_quantize_pad_channels", "q8_dequantize", "q8_fold_bn",
            "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d_query_plan", "q8_conv2d", "q8_static_workspace_bytes",
@@ -48,8 +51,8 @@ def _load():
     path = _build.LIB
     if shutil.which("nvcc") is not None:
         path = _build.build()
-    if not os.path.exists(path):
-        raise ImportError(f"{path} is missing and nvcc is not available to build it; "
+    if not (os.path.exists(path) and os.path.exists(_build.NATIVE)):
+        raise ImportError(f"{path} or {_build.NATIVE} is missing and nvcc is not available to build it; "
                           "run `python -m paper_1805_08691_b200.build` on a machine with CUDA 12.9")
     return C.CDLL(path)
 
@@ -99,6 +102,19 @@ lib.q8_record_free.argtypes = [_vp]
 for _n in EXPORTS[2:]:
     getattr(lib, _n).restype = C.c_int
 lib.q8_static_workspace_bytes.restype = C.c_size_t
+
+
+def _load_native():
+    spec = importlib.util.spec_from_file_location("_q8native", _build.NATIVE)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    module.bind(*(C.cast(f, C.c_void_p).value for f in (lib.q8_conv2d, lib.q8_conv2d_then_1x1, lib.q8_calibrate_maxabs, lib.q8_quantize,
+                                                        lib.q8_dequantize, lib.q8_detection_output_workspace_bytes, lib.q8_detection_output)))
+    return module
+
+
+_native = _load_native()
+_native_conv2d, _native_then_1x1 = _native.conv2d, _native.then_1x1
 
 
 def _check(rc):
@@ -161,7 +177,9 @@ def q8_record_free(graph):
 
 def q8_calibrate_maxabs(x, running_max):
     assert x.dtype == torch.float32 and running_max.dtype == torch.float32 and running_max.numel() == 1
-    _check(lib.q8_calibrate_maxabs(_dev(x, "x"), x.numel(), _dev(running_max, "running_max"), _stream()))
+    rc = _native.maxabs(x, running_max)
+    if rc:
+        _check(rc)
 
 
 def q8_factor(maxabs, p):
@@ -187,7 +205,9 @@ def q8_quantize(x, q, out_type, out=None):
     if out is None:
         out = torch.empty(x.shape, dtype=TORCH_DTYPES[out_type], device=x.device)
     assert out.dtype == TORCH_DTYPES[out_type] and out.numel() == x.numel()
-    _check(lib.q8_quantize(_dev(x, "x"), x.numel(), q, out_type, _dev(out, "out"), _stream()))
+    rc = _native.quantize(x, q, out_type, out)
+    if rc:
+        _check(rc)
     return out
 
 
@@ -212,10 +232,12 @@ def q8_quantize_pad_image(x, W_pad, C_pad, q, out_type, out=None):
 
 
 def q8_dequantize(z, q, out=None):
-    in_type = {torch.uint8: Q8_U8, torch.int8: Q8_S8, torch.int32: Q8_S32}[z.dtype]
+    in_type = _INT_TYPES[z.dtype]
     if out is None:
         out = torch.empty(z.shape, dtype=torch.float32, device=z.device)
-    _check(lib.q8_dequantize(_dev(z, "z"), in_type, z.numel(), q, _dev(out, "out"), _stream()))
+    rc = _native.dequantize(z, in_type, q, out)
+    if rc:
+        _check(rc)
     return out
 
 
@@ -263,10 +285,9 @@ def q8_conv2d(d, x, w, bias, scale, residual=None, residual_scale=0.0, y=None, w
     if y is None:
         P, Q = conv_out_shape(d)
         y = torch.empty((d.N, P, Q, d.y_ldc or d.K), dtype=TORCH_DTYPES[d.y_type], device=x.device)
-    ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    _check(lib.q8_conv2d(C.byref(d), _dev(x, "x"), _dev(w, "w"), _dev(bias, "bias"), _dev(scale, "scale"),
-                         _dev(residual, "residual"), residual_scale, _dev(y, "y"), _dev(workspace, "workspace"),
-                         ws_bytes, _stream()))
+    rc = _native_conv2d(d, x, w, bias, scale, residual, residual_scale, y, workspace)
+    if rc:
+        _check(rc)
     return y
 
 
@@ -281,9 +302,9 @@ def q8_conv2d_then_1x1(d1, d2, x, w1, bias1, scale1, w2, bias2, scale2, residual
     if y is None:
         P, Q = conv_out_shape(d2)
         y = torch.empty((d2.N, P, Q, d2.y_ldc or d2.K), dtype=TORCH_DTYPES[d2.y_type], device=x.device)
-    _check(lib.q8_conv2d_then_1x1(C.byref(d1), C.byref(d2), _dev(x, "x"), _dev(w1, "w1"), _dev(bias1, "bias1"),
-                                  _dev(scale1, "scale1"), _dev(w2, "w2"), _dev(bias2, "bias2"), _dev(scale2, "scale2"),
-                                  _dev(residual, "residual"), residual_scale, _dev(y, "y"), _stream()))
+    rc = _native_then_1x1(d1, d2, x, w1, bias1, scale1, w2, bias2, scale2, residual, residual_scale, y)
+    if rc:
+        _check(rc)
     return y
 
 
@@ -400,50 +421,26 @@ def q8_detection_output_workspace_bytes(N, P, classes, background, nms_top_k, ke
     return n.value
 
 
-def _cell_view(t, what):
-    """(pointer, cell stride in floats, cells per image) of a CUDA fp32 tensor [N, cells..., values] whose cells lie a
-    fixed stride apart (a contiguous tensor, or a slice of the last dimension of one)."""
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.float32 and t.dim() >= 2 and t.stride(-1) == 1):
-        raise TypeError(f"{what}: expected a CUDA fp32 tensor with unit stride in its last dimension")
-    if t.dim() == 2:
-        return t.data_ptr(), int(t.stride(0)), 1
-    stride = int(t.stride(-2))
-    for i in range(t.dim() - 2):
-        if t.shape[i] > 1 and t.stride(i) != t.stride(i + 1) * t.shape[i + 1]:
-            raise TypeError(f"{what}: cells are not a fixed stride apart")
-    cells = 1
-    for v in t.shape[1:-1]:
-        cells *= int(v)
-    return t.data_ptr(), stride, cells
-
-
 def q8_detection_output(sources, priors, variances, classes, background=0, conf_thresh=0.01, nms_thresh=0.45,
                         nms_top_k=400, keep_top_k=200, workspace=None, out=None, counts=None):
     """sources: list of (loc, conf, boxes_per_cell) with loc [N, cells..., boxes * 4] and conf [N, cells...,
     boxes * classes] CUDA fp32 tensors, contiguous or slices of the last dimension of a wider tensor (a merged
     head).  priors: CUDA fp32 [P, 4].  Returns (rows [N, keep_top_k, 6], counts [N])."""
-    N = int(sources[0][0].shape[0])
-    n = len(sources)
-    locp, confp = (C.c_void_p * n)(), (C.c_void_p * n)()
-    lstr, cstr, cells, boxes = (C.c_int * n)(), (C.c_int * n)(), (C.c_int * n)(), (C.c_int * n)()
-    P = 0
-    for i, (loc, conf, b) in enumerate(sources):
-        locp[i], lstr[i], cells[i] = _cell_view(loc, "loc")
-        confp[i], cstr[i], ccells = _cell_view(conf, "conf")
-        if ccells != cells[i] or int(conf.shape[0]) != N or int(loc.shape[0]) != N:
-            raise ValueError("loc and conf of a source must cover the same cells of the same images")
-        boxes[i] = int(b)
-        P += cells[i] * int(b)
-    dev = sources[0][0].device
-    nbytes = q8_detection_output_workspace_bytes(N, P, classes, background, nms_top_k, keep_top_k)
+    first = sources[0][0]
     if workspace is None:
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        P = 0
+        for loc, _, b in sources:
+            cells = 1
+            for v in loc.shape[1:-1]:
+                cells *= int(v)
+            P += cells * int(b)
+        nbytes = q8_detection_output_workspace_bytes(int(first.shape[0]), P, classes, background, nms_top_k, keep_top_k)
+        workspace = torch.empty(nbytes, dtype=torch.uint8, device=first.device)
     if out is None:
-        out = torch.empty((N, keep_top_k, 6), dtype=torch.float32, device=dev)
+        out = torch.empty((int(first.shape[0]), max(keep_top_k, 0), 6), dtype=torch.float32, device=first.device)
     if counts is None:
-        counts = torch.empty(N, dtype=torch.int32, device=dev)
-    var = (C.c_float * 4)(*[float(v) for v in variances])
-    _check(lib.q8_detection_output(n, locp, lstr, confp, cstr, cells, boxes, _dev(priors, "priors"), var, N, classes, background,
-                                   conf_thresh, nms_thresh, nms_top_k, keep_top_k, _dev(workspace, "workspace"), workspace.numel(),
-                                   _dev(out, "out"), _dev(counts, "counts"), _stream()))
+        counts = torch.empty(int(first.shape[0]), dtype=torch.int32, device=first.device)
+    rc = _native.detect(sources, priors, variances, classes, background, conf_thresh, nms_thresh, nms_top_k, keep_top_k, workspace, out, counts)
+    if rc:
+        _check(rc)
     return out, counts

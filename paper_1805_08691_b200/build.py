@@ -1,21 +1,34 @@
-"""Compile libq8.so (CUDA kernels + C ABI) for sm_100a with nvcc, in-tree."""
+"""Compile libq8.so (CUDA kernels + C ABI) for sm_100a with nvcc, and the module that marshals torch tensors into its most
+frequent calls (_q8native.so), both in-tree."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libq8.so")
+NATIVE = os.path.join(HERE, "_q8native.so")
 SOURCES = ["q8_api.cu", "q8_elementwise.cu", "q8_conv_direct.cu", "q8_conv_splitk.cu", "q8_conv_static.cu", "q8_conv_umma.cu", "q8_conv_fused.cu", "q8_conv_gather.cu", "q8_mma_rate.cu", "q8_selftest.cu", "q8_detect.cu", "q8_record.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-fmad=false",
          "-Xcompiler", "-fPIC,-ffp-contract=off,-fno-fast-math", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 
 
+def _native_command():
+    import torch  # only its headers and libraries: the module is linked against the torch that will load it
+    t = os.path.dirname(torch.__file__)
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *(f"-I{d}" for d in (os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(t, "include"),
+                                 os.path.join(t, "include", "torch", "csrc", "api", "include"), "/usr/local/cuda/include")),
+            os.path.join(CSRC, "q8_python.cpp"), "-o", NATIVE, "-L" + os.path.join(t, "lib"),
+            "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(NATIVE)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "q8.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -33,6 +46,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
+    procs.append(("q8_python.cpp", subprocess.Popen(_native_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, pr in procs:
         out, _ = pr.communicate()
@@ -40,7 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(out)
         failed |= pr.returncode != 0
     if failed:
-        raise RuntimeError("nvcc failed")
+        raise RuntimeError("the compiler failed")
     subprocess.run(["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB, *objs], check=True)
     return LIB
 

@@ -178,3 +178,21 @@ def test_recording_requests_are_checked_on_the_host():
     assert q8.lib.q8_record_replay(None, None) == 1
     assert q8.lib.q8_record_end(1, (C.c_void_p * 1)(), None) == 1
     q8.q8_record_free(None)
+
+
+def test_marshalled_calls_refuse_what_they_cannot_pass():
+    """Host tensors, views and objects that are no tensors are refused with the argument's name, before any call."""
+    import torch
+    d = q8.make_conv_desc(1, 4, 4, 16, 16, 1, 1)
+    x = torch.zeros((1, 4, 4, 16), dtype=torch.uint8)
+    w, y = torch.zeros((16, 1, 1, 16), dtype=torch.int8), torch.zeros((1, 4, 4, 16), dtype=torch.uint8)
+    for bad in (x, x.permute(0, 2, 1, 3), 3, [1]):
+        with pytest.raises(TypeError, match="^x: expected a contiguous CUDA tensor"):
+            q8.q8_conv2d(d, bad, w, None, None, y=y)
+    with pytest.raises(TypeError, match="q8_conv_desc"):
+        q8.q8_conv2d(q8.q8_conv_plan(), x, w, None, None, y=y)
+    with pytest.raises(TypeError, match="^out: expected|^x: expected"):
+        q8.q8_quantize(torch.zeros(4), 1.0, q8.Q8_U8)
+    with pytest.raises(TypeError, match="^loc: expected a CUDA fp32 tensor"):
+        q8.q8_detection_output([(torch.zeros(1, 4, 4), torch.zeros(1, 4, 3), 1)], torch.zeros(4, 4), (0.1,) * 4, 3,
+                               workspace=torch.zeros(1, dtype=torch.uint8), out=torch.zeros(1), counts=torch.zeros(1))
