@@ -118,11 +118,13 @@ bool short_rows(const ConvArgs& a) {
 // The kernel a call takes, from its descriptor and the alignment of its pointers; `why` is set where the TMA-fed one is
 // not taken.  That kernel may still find no tile that fits (umma_fits, or kPlanNoFit from its launch); route_off_tma then
 // says what takes its place.
-enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRouteTma };
+enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRoutePacked, kRouteTma };
 
 Route route_off_tma(const ConvArgs& a) {
   if (a.d.algo == Q8_ALGO_UMMA) return kRouteRefused;
-  return gather_addressable(a.d) && gather_us(a) < direct_us(a) ? kRouteGather : kRouteDirect;
+  const double direct = direct_us(a), gather = gather_addressable(a.d) ? gather_us(a) : direct;
+  if (packed_eligible(a.d, a.P, a.Q) && packed_us(a) < (gather < direct ? gather : direct)) return kRoutePacked;
+  return gather < direct ? kRouteGather : kRouteDirect;
 }
 
 Route conv_route(const ConvArgs& a, const char** why) {
@@ -218,7 +220,7 @@ int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan
   Route route = conv_route(a, &why);
   if (route == kRouteTma && !umma_describe(a, plan)) { route = route_off_tma(a); why = "no tile shape of this layer fits in shared memory"; }
   if (route == kRouteRefused) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
-  plan->kernel = route == kRouteTma ? Q8_KERNEL_TMA : (route == kRouteGather ? Q8_KERNEL_GATHER : Q8_KERNEL_DIRECT);
+  plan->kernel = route == kRouteTma ? Q8_KERNEL_TMA : (route == kRouteDirect ? Q8_KERNEL_DIRECT : Q8_KERNEL_GATHER);
   return Q8_OK;
 }
 
@@ -251,6 +253,11 @@ int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32
     why = "no tile shape of this layer fits in shared memory";
   }
   if (route == kRouteRefused) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
+  if (route == kRoutePacked) {
+    rc = launch_conv_packed(a);
+    if (rc != kPlanNoFit) return rc;
+    route = gather_addressable(a.d) && gather_us(a) < direct_us(a) ? kRouteGather : kRouteDirect;
+  }
   return route == kRouteGather ? launch_conv_gather(a) : launch_conv_direct(a);
 }
 

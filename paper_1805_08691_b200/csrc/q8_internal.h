@@ -77,6 +77,10 @@ int launch_conv_direct(const ConvArgs& a);
 bool gather_addressable(const q8_conv_desc& d);
 double gather_us(const ConvArgs& a);  // its estimated time
 int launch_conv_gather(const ConvArgs& a);
+// Tensor-core kernel that packs rows of few input channels from contiguous spans of the input (q8_conv_packed.cu).
+bool packed_eligible(const q8_conv_desc& d, int P, int Q);
+double packed_us(const ConvArgs& a);  // its estimated time
+int launch_conv_packed(const ConvArgs& a);
 // A stride-1 convolution followed by a 1x1 convolution over its output, in one launch (q8_conv_fused.cu).
 // Descriptors validated by the caller; `why` names the first reason a pair cannot run fused.
 bool fused_pair_eligible(const q8_conv_desc& d1, const q8_conv_desc& d2, const char** why);
