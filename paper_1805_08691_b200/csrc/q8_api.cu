@@ -123,7 +123,7 @@ enum Route { kRouteRefused, kRouteDirect, kRouteGather, kRoutePacked, kRouteTma 
 Route route_off_tma(const ConvArgs& a) {
   if (a.d.algo == Q8_ALGO_UMMA) return kRouteRefused;
   const double direct = direct_us(a), gather = gather_addressable(a.d) ? gather_us(a) : direct;
-  if (packed_eligible(a.d, a.P, a.Q) && packed_us(a) < (gather < direct ? gather : direct)) return kRoutePacked;
+  if (packed_better(a)) return kRoutePacked;
   return gather < direct ? kRouteGather : kRouteDirect;
 }
 

@@ -13,7 +13,8 @@
 // other tensor-core kernels.
 //
 // The gathering kernel, which took these layers before, fetches every 16-byte chunk of a run from global memory with five
-// predicated loads and masks: 5560 warp instructions per tile of 3x3/2 on three channels, 64 bytes of reduction for 27.
+// predicated loads and masks: 5560 warp instructions per tile of 3x3/2 on three channels, 64 bytes of reduction for 27
+// (3 -> 32 channels on 8 x 299x299 12.3 us, here 7.8 us, of which about 3 are the chain of a launch).
 #include <type_traits>
 
 #include "q8_umma_common.cuh"
@@ -40,10 +41,10 @@ struct PackedParams {
   int row_bytes;             // W * C
   int bkb, lg_cpb, nblk;     // bytes per K block (32, 64 or 128), log2 of its 16-byte chunks, number of blocks
   int ksteps, last_ksteps;   // K steps of a block, of the last one
-  int m_tiles, n_tiles;
+  int m_tiles;
   unsigned int span_cap, margin, off_a, a_bytes, off_span, off_chan, b_block_bytes, swz_mask;
   int acc_stride, tmem_cols, res_vec, store_vec;
-  FastDiv fd_q, fd_pq;
+  FastDiv fd_q, fd_pq, fd_words;
 };
 
 // First input row (of all images' rows, one after the other) and one past the last that the pixels m0 .. m1 read.
@@ -105,7 +106,7 @@ __device__ __forceinline__ void pack_row(const PackedParams& p, const unsigned c
 template <int kL, bool kMasked>
 __device__ __forceinline__ void pack_rows(const PackedParams& p, const unsigned char* span, unsigned char* dst, int row, int at0, int vl, int vh,
                                           int h0) {
-  if (p.R == 1) pack_row<kL, 1, kMasked>(p, span, dst, row, at0, vl, vh, h0);
+  if (kL == 3 && p.R == 1) pack_row<kL, kL == 3 ? 1 : 3, kMasked>(p, span, dst, row, at0, vl, vh, h0);
   else if (p.R == 3) pack_row<kL, 3, kMasked>(p, span, dst, row, at0, vl, vh, h0);
   else if (p.R == 5) pack_row<kL, 5, kMasked>(p, span, dst, row, at0, vl, vh, h0);
   else pack_row<kL, 7, kMasked>(p, span, dst, row, at0, vl, vh, h0);
@@ -158,14 +159,16 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
       s_bias[i] = (p.u.bias && i < p.u.K) ? p.u.bias[i] : 0;
       s_scale[i] = p.u.scale ? (p.u.scale_count == 1 ? p.u.scale[0] : (i < p.u.K ? p.u.scale[i] : 0.f)) : 0.f;
     }
-  } else if (warp >= kPkFirstPack) {
-    // weights: row n of a tile holds the `reduction` bytes of filter n and zeros, word by word
-    const int t = (int)threadIdx.x - kPkFirstPack * 32, words = p.nblk * p.bkb / 4, total = p.u.k_pad * words;
+  }
+  if (warp < kPkMmaWarp || warp >= kPkFirstPack) {
+    // weights: row n of the tile holds the `reduction` bytes of filter n and zeros; a word per thread and turn, four in flight
+    constexpr int kStagers = (kPkMmaWarp + 4 * kPkGroups) * 32;
+    const int t = warp < kPkMmaWarp ? (int)threadIdx.x : (int)threadIdx.x - 64, words = p.nblk << (p.lg_cpb + 2), items = p.u.k_pad * words;
     const uintptr_t end = reinterpret_cast<uintptr_t>(p.w) + (size_t)p.u.K * p.reduction;
-    for (int i = t; i < total; i += kPkGroups * kGroupThreads) {
-      const int n = i / words, kw = i - n * words;
+#pragma unroll 4
+    for (int i = t; i < items; i += kStagers) {
+      const int n = p.fd_words.div(i), kw = i - n * words, bytes = min(p.reduction - 4 * kw, 4);
       unsigned int v = 0;
-      const int bytes = min(p.reduction - 4 * kw, 4);
       if (n < p.u.K && bytes > 0) {
         const uintptr_t at = reinterpret_cast<uintptr_t>(p.w) + (size_t)n * p.reduction + 4 * kw;
         const unsigned int* g = reinterpret_cast<const unsigned int*>(at & ~(uintptr_t)3);
@@ -173,11 +176,9 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
         v = __funnelshift_r(g[0], hi, 8u * (unsigned)(at & 3));
         if (bytes < 4) v &= (1u << (8 * bytes)) - 1u;
       }
-      const int blk = kw * 4 / p.bkb, col = kw * 4 - blk * p.bkb;
-      const int nt = n / p.u.bn, row = n - nt * p.u.bn;
-      const uint32_t off = (uint32_t)(row * p.bkb + (col & ~15));
-      *reinterpret_cast<unsigned int*>(base_ptr + (size_t)(nt * p.nblk + blk) * p.b_block_bytes + (off ^ (((off >> 7) & p.swz_mask) << 4)) +
-                                       (col & 15)) = v;
+      const int blk = kw >> (p.lg_cpb + 2), col = 4 * kw - (blk << (p.lg_cpb + 4));
+      const uint32_t off = (uint32_t)(n * p.bkb + (col & ~15));
+      *reinterpret_cast<unsigned int*>(base_ptr + (size_t)blk * p.b_block_bytes + (off ^ (((off >> 7) & p.swz_mask) << 4)) + (col & 15)) = v;
     }
     fence_proxy_async_smem();
   }
@@ -246,20 +247,18 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
     bool ok = true;
     for (int tile = first_tile; tile < p.m_tiles && ok; tile += step) {
       if (!mbar_wait(smem_u32(&a_full[g]), par, abortp)) { ok = false; break; }
-      for (int nt = 0; nt < p.n_tiles; ++nt) {
-        if (!mbar_wait(smem_u32(&acc_empty[ab]), apar, abortp)) { ok = false; break; }
-        tcgen05_fence_after();
-        if (elect_one()) {
-          uint32_t ad = a_d0 + g * a16, bd = b_d0 + (uint32_t)(nt * p.nblk) * bblk16;
-          for (int blk = 0; blk < p.nblk; ++blk, ad += ablk16, bd += bblk16) {
-            const int ks = blk == p.nblk - 1 ? p.last_ksteps : p.ksteps;
-            for (int k = 0; k < ks; ++k)
-              umma_i8(tmem_base + ab * (uint32_t)p.acc_stride, ad + 2 * k, bd + 2 * k, p.u.desc_hi, p.u.idesc, blk | k ? 1u : 0u);
-          }
-          umma_commit(smem_u32(&acc_full[ab]));
+      if (!mbar_wait(smem_u32(&acc_empty[ab]), apar, abortp)) { ok = false; break; }
+      tcgen05_fence_after();
+      if (elect_one()) {
+        uint32_t ad = a_d0 + g * a16, bd = b_d0;
+        for (int blk = 0; blk < p.nblk; ++blk, ad += ablk16, bd += bblk16) {
+          const int ks = blk == p.nblk - 1 ? p.last_ksteps : p.ksteps;
+          for (int k = 0; k < ks; ++k)
+            umma_i8(tmem_base + ab * (uint32_t)p.acc_stride, ad + 2 * k, bd + 2 * k, p.u.desc_hi, p.u.idesc, blk | k ? 1u : 0u);
         }
-        if (++ab == kPkEpiGroups) { ab = 0; apar ^= 1u; }
+        umma_commit(smem_u32(&acc_full[ab]));
       }
+      if (++ab == kPkEpiGroups) { ab = 0; apar ^= 1u; }
       if (elect_one()) umma_commit(smem_u32(&a_empty[g]));
       if (++g == kPkStages) { g = 0; par ^= 1u; }
     }
@@ -282,18 +281,14 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
     t.smem_ok = true;
     t.row_base = t.swz = 0;
     uint32_t apar = 0;
-    int seq = 0;  // (tile, columns) pairs of this CTA so far
-    for (int tile = first_tile; tile < p.m_tiles; tile += step)
-      for (int nt = 0; nt < p.n_tiles; ++nt, ++seq) {
-        if ((seq & (kPkEpiGroups - 1)) != g) continue;
+    for (int tile = first_tile + g * step; tile < p.m_tiles; tile += kPkEpiGroups * step) {
         if (!mbar_wait(smem_u32(&acc_full[g]), apar, abortp)) {
           if (lane == 0) { abort_flag = 1; atomicOr(p.u.status, kTimeoutEpilogue); }
-          tile = p.m_tiles;
           break;
         }
         apar ^= 1u;
         tcgen05_fence_after();
-        t.n0 = nt * p.u.bn;
+        t.n0 = 0;
         t.m = tile * kBM + row;
         t.row_ok = t.m < p.u.M;
         const int chunks = p.u.bn >> 4;
@@ -402,17 +397,26 @@ long long span_rows(const q8_conv_desc& d, int Q) {
   const long long out_rows = (kBM - 2 + Q) / Q + 1;
   return (out_rows + 2) * d.stride_h + 2ll * (d.R - 1) * d.dil_h + d.pad_h + 2;
 }
-}  // namespace
-
 bool packed_eligible(const q8_conv_desc& d, int P, int Q) {
   const long long red = (long long)d.R * d.S * d.C, row = (long long)d.W * d.C, pads = ((long long)d.pad_w + (long long)d.S) * d.C;
   auto compiled = [](int v) { return v == 1 || v == 3 || v == 5 || v == 7; };
-  return d.C == 3 && compiled(d.R) && compiled(d.S) && (d.dil_w == 1 || d.S == 1) && red <= kPkMaxReduction && (long long)P * Q >= kBM && d.K <= 512 && pads <= 1024 &&
+  return d.C == 3 && compiled(d.R) && compiled(d.S) && (d.R > 1 || d.S == 1) && (d.dil_w == 1 || d.S == 1) && red <= kPkMaxReduction &&
+         (long long)P * Q >= kBM && d.K <= 128 && pads <= 1024 &&
          d.pad_h < (1 << 20) && (long long)d.R * d.dil_h < (1 << 20) && span_rows(d, Q) * row + 32 <= (long long)kPkMaxSpan &&
          (long long)d.N * d.H < (1ll << 31) && (d.H - 1ll + d.pad_h) * row < (1ll << 30);
 }
+}  // namespace
 
-double packed_us(const ConvArgs& a) { return 0.0; }
+// Where it is faster than the kernels that took such layers: one tile of columns (weights are staged word by word, and what is
+// gathered again for every further tile is little), rows stored in 16-byte pieces, half of the SMs at work, and not a single
+// run of 15 or 21 bytes (1xS), which the gathering kernel fetches densely as well (1x7 of 3 -> 112 on 7 x 58x60: 5.4 there, 6.2
+// us here).  Over 160 random layers of these forms, replayed from a graph, 1.31 times faster in the mean, from 2.7 times
+// (5x5 of 3 -> 16 on 30 x 197x199 89 -> 33 us) to as fast (5x5 of 3 -> 80 on 108x108 6.1 us both).
+bool packed_better(const ConvArgs& a) {
+  const int grid = a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8 ? 16 : 4;
+  return packed_eligible(a.d, a.P, a.Q) && a.M > (long long)kBM * sm_count() / 2 && a.d.K % grid == 0 && aligned16(a.y) && a.ldc % grid == 0 &&
+         a.c_off % grid == 0;
+}
 
 int launch_conv_packed(const ConvArgs& a) {
   const q8_conv_desc& d = a.d;
@@ -431,7 +435,6 @@ int launch_conv_packed(const ConvArgs& a) {
   const int grid16 = out8 ? 16 : 4;
   u.y_vec = aligned16(a.y) && a.ldc % grid16 == 0 && a.c_off % grid16 == 0;
   p.store_vec = u.y_vec;
-  // (a tile's first channel is a multiple of 16: pairs of chunks start on 32-byte lines where tiles are of 32)
   u.y_wide = out8 && (reinterpret_cast<uintptr_t>(a.y) & 31u) == 0 && a.ldc % 32 == 0 && a.c_off % 32 == 0;
   p.res_vec = d.K % 16 == 0 && aligned16(a.residual);
   p.x = static_cast<const unsigned char*>(a.x);
@@ -447,22 +450,19 @@ int launch_conv_packed(const ConvArgs& a) {
   p.ksteps = p.bkb / 32;
   p.last_ksteps = (p.reduction - (p.nblk - 1) * p.bkb + 31) / 32;
   p.swz_mask = p.bkb == 128 ? 7u : (p.bkb == 64 ? 3u : 1u);
-  p.n_tiles = (d.K + 127) / 128;
-  u.bn = ((d.K + p.n_tiles - 1) / p.n_tiles + 15) / 16 * 16;
-  p.n_tiles = (d.K + u.bn - 1) / u.bn;
-  u.k_pad = p.n_tiles * u.bn;
-  if (p.n_tiles > 1 && u.bn % 32) u.y_wide = 0;
+  u.bn = (d.K + 15) / 16 * 16;
+  u.k_pad = u.bn;
   p.m_tiles = (int)((a.M + kBM - 1) / kBM);
   p.acc_stride = 32;
   while (p.acc_stride < u.bn) p.acc_stride *= 2;
   p.tmem_cols = kPkEpiGroups * p.acc_stride;
-  p.fd_q = make_fastdiv(a.Q); p.fd_pq = make_fastdiv(u.PQ);
+  p.fd_q = make_fastdiv(a.Q); p.fd_pq = make_fastdiv(u.PQ); p.fd_words = make_fastdiv(p.nblk << (p.lg_cpb + 2));
   p.b_block_bytes = round_up((unsigned)(u.bn * p.bkb), 1024u);
   p.a_bytes = (unsigned)(p.nblk * kBM * p.bkb);
   // runs that start left of the image or end right of it are read (and masked) up to this far outside the span
   p.margin = round_up((unsigned)((d.pad_w + d.S) * d.C) + 16u, 128u);
   p.span_cap = round_up((unsigned)(span_rows(d, a.Q) * p.row_bytes + 32), 128u);
-  p.off_a = (unsigned)(p.n_tiles * p.nblk) * p.b_block_bytes;
+  p.off_a = (unsigned)p.nblk * p.b_block_bytes;
   p.off_span = p.off_a + (unsigned)kPkStages * p.a_bytes;
   p.off_chan = round_up(p.off_span + (unsigned)kPkStages * (p.span_cap + 2u * p.margin), 1024u);
   const size_t dyn = 1024u + p.off_chan + round_up((unsigned)u.k_pad * 8u, 1024u);

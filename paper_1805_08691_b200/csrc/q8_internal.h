@@ -77,9 +77,9 @@ int launch_conv_direct(const ConvArgs& a);
 bool gather_addressable(const q8_conv_desc& d);
 double gather_us(const ConvArgs& a);  // its estimated time
 int launch_conv_gather(const ConvArgs& a);
-// Tensor-core kernel that packs rows of few input channels from contiguous spans of the input (q8_conv_packed.cu).
-bool packed_eligible(const q8_conv_desc& d, int P, int Q);
-double packed_us(const ConvArgs& a);  // its estimated time
+// Tensor-core kernel for three-channel images that packs its operand rows from contiguous spans of the input
+// (q8_conv_packed.cu); whether a layer takes it.
+bool packed_better(const ConvArgs& a);
 int launch_conv_packed(const ConvArgs& a);
 // A stride-1 convolution followed by a 1x1 convolution over its output, in one launch (q8_conv_fused.cu).
 // Descriptors validated by the caller; `why` names the first reason a pair cannot run fused.

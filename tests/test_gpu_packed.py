@@ -13,20 +13,20 @@ OT = {U8: o.U8, S8: o.S8, S32: o.S32, F32: o.F32}
 
 CASES = [
     # name, N,H,W,C,K,R,S,strides,pads,dil_h, x signed, y type, residual, per channel, extra channels per pixel, input shift
-    ("c3_3x3s2", 3, 99, 97, 3, 32, 3, 3, (2, 2), (0, 0), 1, True, U8, False, False, 0, 0),
-    ("c3_3x3_pad", 2, 40, 37, 3, 64, 3, 3, (1, 1), (1, 1), 1, True, U8, True, False, 0, 1),
-    ("c3_7x7s2_pad3", 2, 64, 62, 3, 64, 7, 7, (2, 2), (3, 3), 1, True, S8, False, True, 0, 2),
-    ("c3_5x5_k500", 1, 30, 31, 3, 500, 5, 5, (1, 1), (2, 2), 1, False, U8, True, False, 0, 0),
-    ("c3_1x7_f32", 2, 33, 40, 3, 24, 1, 7, (1, 1), (0, 3), 1, False, F32, True, True, 0, 3),
-    ("c3_7x1_runs_of_three", 2, 33, 40, 3, 20, 7, 1, (1, 1), (3, 0), 1, False, U8, False, False, 5, 0),
-    ("c3_1x1", 4, 30, 30, 3, 8, 1, 1, (1, 1), (0, 0), 1, False, S32, False, False, 0, 1),
-    ("c3_3x5_strides_3_1", 7, 26, 24, 3, 33, 3, 5, (3, 1), (2, 0), 1, False, U8, False, False, 0, 0),
-    ("c3_5x3_dil_h2", 2, 30, 29, 3, 40, 5, 3, (1, 2), (2, 1), 2, False, U8, False, False, 0, 0),
-    ("c3_7x3_s8_residual", 2, 17, 18, 3, 48, 7, 3, (1, 1), (3, 1), 1, True, S8, True, False, 0, 0),
-    ("c3_1x5", 1, 16, 40, 3, 130, 1, 5, (1, 1), (0, 2), 1, False, U8, False, False, 0, 1),
-    ("c3_5x7", 3, 21, 22, 3, 96, 5, 7, (1, 1), (0, 3), 1, True, U8, False, True, 32, 2),
+    ("c3_3x3s2", 5, 99, 97, 3, 32, 3, 3, (2, 2), (0, 0), 1, True, U8, False, False, 0, 0),
+    ("c3_3x3_pad", 8, 40, 37, 3, 64, 3, 3, (1, 1), (1, 1), 1, True, U8, True, False, 0, 1),
+    ("c3_7x7s2_pad3", 11, 64, 62, 3, 64, 7, 7, (2, 2), (3, 3), 1, True, S8, False, True, 0, 2),
+    ("c3_5x5_k128", 11, 30, 31, 3, 128, 5, 5, (1, 1), (2, 2), 1, False, U8, True, False, 0, 0),
+    ("c3_1x7_f32", 8, 33, 40, 3, 24, 1, 7, (1, 1), (0, 3), 1, False, F32, True, True, 0, 3),
+    ("c3_7x1_runs_of_three", 8, 33, 40, 3, 80, 7, 1, (1, 1), (3, 0), 1, False, U8, False, False, 32, 0),
+    ("c3_1x1", 12, 30, 30, 3, 8, 1, 1, (1, 1), (0, 0), 1, False, S32, False, False, 0, 1),
+    ("c3_3x5_strides_3_1", 50, 26, 24, 3, 32, 3, 5, (3, 1), (2, 0), 1, False, U8, False, False, 0, 0),
+    ("c3_5x3_dil_h2", 26, 30, 29, 3, 48, 5, 3, (1, 2), (2, 1), 2, False, U8, False, False, 0, 0),
+    ("c3_7x3_s8_residual", 32, 17, 18, 3, 48, 7, 3, (1, 1), (3, 1), 1, True, S8, True, False, 0, 0),
+    ("c3_1x5", 16, 16, 40, 3, 112, 1, 5, (1, 1), (0, 2), 1, False, U8, False, False, 0, 1),
+    ("c3_5x7", 30, 21, 22, 3, 96, 5, 7, (1, 1), (0, 3), 1, True, U8, False, True, 32, 2),
     ("many_tiles_c3", 8, 150, 150, 3, 32, 3, 3, (1, 1), (1, 1), 1, True, U8, False, False, 0, 0),
-    ("wide_padding", 2, 14, 14, 3, 16, 3, 3, (1, 1), (7, 9), 1, True, U8, False, False, 0, 0),
+    ("wide_padding", 13, 14, 14, 3, 16, 3, 3, (1, 1), (7, 9), 1, True, U8, False, False, 0, 0),
 ]
 
 
