@@ -203,7 +203,9 @@ int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo);
  * device the plan is that of a B200).  Errors: Q8_ERR_INVALID_ARG; Q8_ERR_UNSUPPORTED where the call is refused. */
 typedef enum q8_conv_kernel { Q8_KERNEL_DIRECT = 0, Q8_KERNEL_GATHER = 1, Q8_KERNEL_TMA = 2 } q8_conv_kernel;
 typedef struct q8_conv_plan {
-  int32_t kernel;           /* q8_conv_kernel; the fields below are zero unless it is Q8_KERNEL_TMA */
+  int32_t kernel;           /* q8_conv_kernel (Q8_KERNEL_GATHER: tensor cores on operands that no TMA load brings, gathered by
+                             * chunks or, for three-channel images, packed from whole rows); the fields below are zero unless
+                             * it is Q8_KERNEL_TMA */
   int32_t tile_n;           /* output channels of a tile */
   int32_t operand;          /* activations as 0: a matrix, 1: im2col loads, 2: halo patches */
   int32_t splits;           /* parts of the reduction, 1: not split */
