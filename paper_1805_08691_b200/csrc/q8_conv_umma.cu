@@ -162,10 +162,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   if constexpr (kCta2) cta_rank = __shfl_sync(0xffffffffu, (int)cluster_ctarank(), 0);
   const int vblock = kCta2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int vgrid = kCta2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  // work items of this CTA: first_item, first_item + item_step, ... below total_tiles (the two of a twin CTA lie side by side)
-  const bool twin = !kCta2 && p.twin != 0;
-  const int first_item = twin ? 2 * vblock : vblock, item_step = twin ? 1 : vgrid;
-  const int total_tiles = twin ? min(p.m_tiles, first_item + 2) : p.m_tiles * p.n_tiles * p.splits;
+  const int total_tiles = p.m_tiles * p.n_tiles * p.splits;  // work items
 
   // Programmatic dependent launch: the next kernel of the stream may be scheduled onto SMs as they fall idle
   // (it waits below, like this one, before it touches global memory), and this kernel's own set-up (barriers,
@@ -250,7 +247,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   if (warp == 0) {
     // ------------------------------------------------------------------ A / B producer (whole warp; an elected lane issues)
     TileIterT<kCta2> ti;
-    ti.init(p, first_item, item_step, cta_rank);
+    ti.init(p, vblock, vgrid, cta_rank);
     const uint32_t nstages = (uint32_t)p.stages, nbst = (uint32_t)p.b_stages;
     const uint32_t afull0 = smem_u32(&a_full[0]), aempty0 = smem_u32(&a_empty[0]);
     const uint32_t bfull0 = smem_u32(&b_full[0]), bempty0 = smem_u32(&b_empty[0]);
@@ -282,12 +279,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
           for (int c = 0; c < p.C_pad; c += p.bk, dst += (uint32_t)p.taps * p.b_tile_bytes) tma_load_3d(dst, &tmB, bar, c, nt * p.bn, 0);
       }
     }
-    if (twin) {
-      TwinLoads tl;
-      tl.base = base; tl.a_full = afull0; tl.a_empty = aempty0; tl.b_full = bfull0; tl.b_empty = bempty0;
-      tl.first_tile = first_item; tl.total_tiles = total_tiles; tl.abortp = abortp;
-      ok = producer_role_twin(p, &tmA, &tmB, tl);
-    } else if (p.a_mode == kAHalo) {
+    if (p.a_mode == kAHalo) {
       const uint32_t b_tx = (uint32_t)p.b_T * p.b_tile_bytes;
       for (; ti.tile < total_tiles && ok; ti.next(p)) {
         const int n0 = ti.nt * p.bn + (kCta2 ? cta_rank * (p.bn >> 1) : 0);
@@ -382,7 +374,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     const int who = warp - 1;
     MmaRoleArgs ra;
     ra.base = base; ra.tmem_base = tmem_base; ra.total_tiles = total_tiles; ra.abortp = abortp;
-    ra.first_tile = first_item; ra.tile_step = item_step;
+    ra.first_tile = (int)blockIdx.x; ra.tile_step = (int)gridDim.x;
     ra.a_full = smem_u32(&a_full[0]); ra.a_empty = smem_u32(&a_empty[0]);
     ra.b_full = smem_u32(&b_full[0]); ra.b_empty = smem_u32(&b_empty[0]);
     ra.acc_full = smem_u32(&acc_full[0]); ra.acc_empty = smem_u32(&acc_empty[0]);
@@ -392,8 +384,6 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       // two issuing warps
     } else if constexpr (kCta2) {
       if (cta_rank == 0) ok = mma_role_pair(p, ra, who, vblock, vgrid);
-    } else if (twin) {
-      if (who == 0) ok = mma_role_twin(p, ra);
     } else {
       ok = mma_role(p, ra, who);
     }
@@ -444,7 +434,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     }
     uint32_t ab = (uint32_t)team % nacc, acc_par = ((uint32_t)team / nacc) & 1u;
     TileIterT<kCta2> ti;
-    ti.init(p, first_item + team * item_step, tile_step * item_step, cta_rank);
+    ti.init(p, vblock + team * vgrid, tile_step * vgrid, cta_rank);
     for (; ti.tile < total_tiles; ti.next(p)) {
       auto place = [&] {  // the tile's pixel and columns of this thread
         t.n0 = ti.nt * p.bn;
@@ -872,15 +862,6 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
     }
   }
-  // Two m tiles of a CTA at once where every CTA has at most two: one pass of the weights serves both, and zero K steps of
-  // the last channel block are left out, which gains nothing while the loads of the weights bound a tile.  Tiles of 144 to 192
-  // columns: 1x7 160->160 at 17x17, batch 64 12.3 -> 11.4 us, 3x3 14.6 -> 12.6 us.  Narrower ones load several taps per operation
-  // and overlap two tiles' epilogues (128 columns 6.5 -> 7.5 us as twins), with 256 the tensor pipe bounds (13.7 -> 14.7 us).
-  // The roles of twin CTAs are functions of their own, not inlined: inlined they cost every other layer of the kernel 3 to 6 %.
-  p.twin = p.a_mode == kAHalo && !paired && p.b_mode == kBRing && !p.cta2 && splits == 1 && p.n_tiles == 1 && BN > 128 && BN <= 192 &&
-           p.m_tiles > sm_count() && p.m_tiles <= 2 * sm_count();
-  p.twin = tune_env("Q8_TWIN", p.twin, 0, p.twin);
-  p.last_ksteps = (c_eff - (p.c_blocks - 1) * BK + 31) / 32;
   const unsigned row_bytes = rows ? (unsigned)(p.epi_split ? 1 : G) * p.tile8_bytes : 0u;
   p.b_T = 1;
   p.b_chunks = p.taps;
@@ -923,9 +904,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   unsigned rest = budget - bres_bytes - row_bytes;
   p.b_stages = 0;
   if (p.b_mode == kBRing) {
-    // twin tiles: two channel blocks' patches in flight where that leaves the ring its minimum
-    if (p.twin && rest < 4u * p.a_stage_bytes + 3u * p.b_sub_bytes) p.twin = 0;
-    int bst = (int)((rest - (p.twin ? 4u : 2u) * p.a_stage_bytes) / p.b_sub_bytes);
+    int bst = (int)((rest - 2u * p.a_stage_bytes) / p.b_sub_bytes);
     if (bst > kMaxBStages) bst = kMaxBStages;
     p.b_stages = tune_env("Q8_BSTAGES", bst, 2, bst > 2 ? bst : 2);
     rest -= (unsigned)p.b_stages * p.b_sub_bytes;
@@ -1047,8 +1026,7 @@ int launch_planned(const ConvArgs& a, int splits) {
 
   const long long tiles = (long long)p.m_tiles * p.n_tiles * splits;  // work items
   int grid = (int)(tiles < sm_count() ? tiles : sm_count());
-  if (p.twin) grid = (p.m_tiles + 1) / 2;
-  grid = tune_env("Q8_GRID", grid, p.twin ? grid : 1, grid);
+  grid = tune_env("Q8_GRID", grid, 1, grid);
   if (p.cta2) {  // one cluster of two CTAs per work item in flight
     const long long pairs = sm_count() / 2;
     grid = 2 * (int)(tiles < pairs ? tiles : pairs);

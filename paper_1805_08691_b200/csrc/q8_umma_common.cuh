@@ -79,8 +79,6 @@ struct UmmaParams {
   // patch descriptor moves by in16 (16-byte units) from one tap to the next and by out16 from one group to the next
   unsigned int in16, out16;
   int tap_inner;
-  int twin;                  // halo, weight ring: a CTA runs two m tiles at once on one pass of the weights (see plan_tiles)
-  int last_ksteps;           // ... K steps of the last channel block that hold a channel
   int mma_lanes;             // MMA-issuing warps: 3 with four accumulators, else 2 (see plan_tiles)
   int pair_shift;            // cta2: log2 of the epilogue groups that share the columns of a tile
   int epi_split;             // 1: every epilogue group takes a share of the columns of every tile (short launches)
@@ -925,101 +923,6 @@ __device__ __forceinline__ bool mma_role(const UmmaParams& p, const MmaRoleArgs&
       bs += skip_b;
       while (bs >= nbst) { bs -= nbst; bphase ^= 1u; }
       bring_d = bring_d0 + bs * bsub16;
-    }
-  }
-  return true;
-}
-
-// ksteps instructions, any number up to 4.
-__device__ __forceinline__ void umma_i8_steps(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                              uint32_t accumulate_first, int ksteps) {
-  umma_i8(d_tmem, a_lo, b_lo, hi, idesc, accumulate_first);
-  if (ksteps > 1) umma_i8_acc(d_tmem, a_lo + 2, b_lo + 2, hi, idesc);
-  if (ksteps > 2) umma_i8_acc(d_tmem, a_lo + 4, b_lo + 4, hi, idesc);
-  if (ksteps > 3) umma_i8_acc(d_tmem, a_lo + 6, b_lo + 6, hi, idesc);
-}
-
-// Two m tiles of one CTA at once: every weight tile of the ring is multiplied with the patches of both.  Their patches lie in
-// consecutive stages, their accumulators are 0 and 1.  One issuing warp, one pass, so no barrier is used twice here but those
-// of the stages.
-__device__ __noinline__ bool mma_role_twin(const UmmaParams& p, const MmaRoleArgs& r) {
-  const bool two = r.first_tile + 1 < r.total_tiles;
-  const uint32_t nstages = (uint32_t)p.stages, nbst = (uint32_t)p.b_stages, hi = p.desc_hi, idesc = p.idesc;
-  const uint32_t a_d0 = kDescLbo | (((r.base + p.off_a) >> 4) & 0x3fffu), bring_d0 = kDescLbo | (((r.base + p.off_bring) >> 4) & 0x3fffu);
-  const uint32_t stage16 = p.a_stage_bytes >> 4, bsub16 = p.b_sub_bytes >> 4, btile16 = p.b_tile_bytes >> 4;
-  const uint32_t acc0 = r.tmem_base, acc1 = r.tmem_base + (uint32_t)p.acc_stride;
-  const int taps = p.taps, inner = p.tap_inner, bT = p.b_T, c_blocks = p.c_blocks, all_ksteps = p.ksteps, last_ksteps = p.last_ksteps;
-  const uint32_t in16 = p.in16, out16 = p.out16;
-  uint32_t stage = 0, phase = 0, bs = 0, bphase = 0, accum = 0;
-  for (int cb = 0; cb < c_blocks; ++cb) {
-    const int ksteps = cb == c_blocks - 1 ? last_ksteps : all_ksteps;
-    const uint32_t s0 = stage, d0 = a_d0 + stage * stage16;
-    if (!mbar_wait(r.a_full + stage * 8u, phase, r.abortp)) return false;
-    if (++stage == nstages) { stage = 0; phase ^= 1u; }
-    const uint32_t s1 = stage, d1 = a_d0 + stage * stage16;
-    if (two) {
-      if (!mbar_wait(r.a_full + stage * 8u, phase, r.abortp)) return false;
-      if (++stage == nstages) { stage = 0; phase ^= 1u; }
-    }
-    uint32_t row = 0, at = 0;  // offset of the filter row's first tap, of this tap, in both patches
-    int left = inner;
-    for (int tap0 = 0; tap0 < taps; tap0 += bT) {
-      if (!mbar_wait(r.b_full + bs * 8u, bphase, r.abortp)) return false;
-      tcgen05_fence_after();
-      const int nt = min(bT, taps - tap0);
-      uint32_t bd = bring_d0 + bs * bsub16;
-      for (int t = 0; t < nt; ++t, bd += btile16) {
-        if (elect_one()) {
-          umma_i8_steps(acc0, d0 + at, bd, hi, idesc, accum, ksteps);
-          if (two) umma_i8_steps(acc1, d1 + at, bd, hi, idesc, accum, ksteps);
-        }
-        accum = 1;
-        at += in16;
-        if (--left == 0) { left = inner; row += out16; at = row; }
-      }
-      if (elect_one()) umma_commit(r.b_empty + bs * 8u);
-      if (++bs == nbst) { bs = 0; bphase ^= 1u; }
-    }
-    if (elect_one()) {
-      umma_commit(r.a_empty + s0 * 8u);
-      if (two) umma_commit(r.a_empty + s1 * 8u);
-    }
-  }
-  if (elect_one()) {
-    umma_commit(r.acc_full);
-    if (two) umma_commit(r.acc_full + 8u);
-  }
-  return true;
-}
-
-// ... and their loads: per channel block the patches of both tiles, then the weights once.
-struct TwinLoads { uint32_t base, a_full, a_empty, b_full, b_empty; int first_tile, total_tiles; volatile int* abortp; };
-__device__ __noinline__ bool producer_role_twin(const UmmaParams& p, const CUtensorMap* tmA, const CUtensorMap* tmB, const TwinLoads& r) {
-  TileIterT<false> t0, t1;
-  t0.init(p, r.first_tile, 1);
-  t1 = t0;
-  t1.next(p);
-  const int both = t1.tile < r.total_tiles ? 2 : 1;
-  uint32_t stage = 0, phase = 1, bs = 0, bphase = 1;
-  for (int c = 0; c < p.C_pad; c += p.bk) {
-    for (int i = 0; i < both; ++i) {
-      if (!mbar_wait(r.a_empty + stage * 8u, phase, r.abortp)) return false;
-      if (elect_one()) {
-        const uint32_t bar = r.a_full + stage * 8u;
-        mbar_arrive_expect_tx(bar, p.a_sub_bytes);
-        tma_load_4d(r.base + p.off_a + stage * p.a_stage_bytes, tmA, bar, c, (i ? t1.qt : t0.qt) * p.tw - p.pad_w,
-                    (i ? t1.pt : t0.pt) * p.th * p.stride_h - p.pad_h, i ? t1.img : t0.img);
-      }
-      if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
-    }
-    for (int tap = 0; tap < p.taps; tap += p.b_T) {
-      if (!mbar_wait(r.b_empty + bs * 8u, bphase, r.abortp)) return false;
-      if (elect_one()) {
-        const uint32_t bar = r.b_full + bs * 8u;
-        mbar_arrive_expect_tx(bar, (uint32_t)p.b_T * p.b_tile_bytes);
-        tma_load_3d(r.base + p.off_bring + bs * p.b_sub_bytes, tmB, bar, c, 0, tap);
-      }
-      if (++bs == (uint32_t)p.b_stages) { bs = 0; bphase ^= 1u; }
     }
   }
   return true;
