@@ -8,18 +8,25 @@
 //   layer 1:  D1[128 rows of one halo tile, Cout1]   = patch (TMA, shifted descriptors per tap) x W1^T
 //             E1: + bias1, * scale1, ReLU, round, clamp -> T[slot] (u8/s8, [128][Cout1], swizzled)
 //   layer 2:  D2[128, 128-column chunk j of Cout2]   = T[slot] x W2[chunk j]^T          for every chunk j
-//             E2: + bias2, * scale2, + residual * s_res, ReLU, round, clamp -> global memory
+//             E2: + bias2, * scale2, + residual * s_res, ReLU, round, clamp -> global memory, by TMA or by the epilogue
 //
 // Warps (whole warps walk the schedules, an elected lane issues):
 //   0      TMA producer of layer 1 (input patches, weight ring), and of all resident weights before the kernel
 //          orders itself behind its predecessor in the stream;
 //   1      MMA issue of layer 1 (owns the TMEM allocation);
 //   2      MMA issue of layer 2;
-//   3      no role after the prologue (the epilogue groups start at a multiple of four warps);
+//   3      tile buffers of layer 2, where used: residual tiles in (TMA), finished output tiles out (TMA store);
 //   4-7    E1, one group of four warps;
 //   8-19   E2, three groups of four warps; group g owns accumulator g of layer 2 and every third chunk.
 // TMEM (512 columns): three layer-2 accumulators of 128 columns, the rest holds one to two layer-1 accumulators.
 // Every hand-off is an mbarrier with a bounded wait (status word + drain on expiry), as in q8_conv_umma.cu.
+//
+// Layer 2's bytes, two ways.  With tile buffers, warp 3 brings residual rows in and sends output rows out by TMA as whole lines;
+// without, the epilogue loads and stores its rows itself, which saves the hand-offs.  Buffers pay where a CTA has many items and
+// there is room for two per E2 group, so that the copies run behind the arithmetic; with one per group they never won.
+// Measured with a residual, per launch, inputs not in L2, buffers against none:
+//   56x56 64->64->256   batch 4: 8.1 / 7.8 us, 8 (3 items per CTA): 9.7 / 9.8, 16 (6): 13.0 / 15.0, 32: 19.4 / 23.7, 64: 31.0 / 41.2;
+//   28x28 128->128->512 (room for one per group)  batch 1: 8.5 / 8.3, 8: 10.8 / 9.9, 16: 15.4 / 14.0, 32: 20.5 / 19.2, 64: 28.3 / 28.4.
 #include "q8_umma_common.cuh"
 
 namespace q8 {
@@ -30,34 +37,56 @@ constexpr int kFE2Groups = 3;
 constexpr int kFThreads = (kFCtrlWarps + 4 + 4 * kFE2Groups) * 32;  // 640
 constexpr int kFAcc2Cols = 128;                                      // columns of one layer-2 accumulator
 constexpr int kFMaxTb = 4;                                           // slots of the intermediate tile ring
+constexpr int kFSlots = 6;                                           // layer-2 tile buffers, two per E2 group
+constexpr int kFBufMinItems = 4;                                     // items per CTA above which buffers are used
 
 struct FusedParams {
   UmmaParams l1;  // layer 1: halo tiles, one tile of columns (bn = Cout1), one MMA warp; its 8-bit tile fields
                   // (pw_shift, pmask) describe the intermediate tile T
-  UmmaParams l2;  // layer 2: bn = chunk width, n_tiles = chunks, bk = ksteps * 32 = Cout1; y / ldc / c_off / residual
-                  // as in the single-layer kernel
+  UmmaParams l2;  // layer 2: bn = chunk width, n_tiles = chunks, bk = ksteps * 32 = Cout1; 8-bit tile fields
+                  // describe the output tile buffers; y / ldc / c_off / residual as in the single-layer kernel
   int ntb;                       // slots of the T ring
   unsigned int off_w2, off_tb;   // resident W2 tiles, T ring (from the 1 KiB aligned base)
   unsigned int tb_bytes;         // 128 * Cout1
   unsigned int off_chan2;        // bias2 / scale2 staging
+  int nslots;                    // layer-2 tile buffers (6; 0: the epilogue moves the rows itself)
+  unsigned int res_tx_bytes;     // bytes one residual tile load delivers
   int acc1_col;                  // first TMEM column of the layer-1 accumulators
 };
 
-template <int kOut1, int kOut2, bool kUniform>
+// One (m tile, chunk) item of layer 2 in this CTA's sequence, with the tile's image coordinates.
+struct ItemIter {
+  TileIterT<false> ti;
+  int j, left;
+  __device__ __forceinline__ void init(const UmmaParams& l1, int t0, int j0, int count) {
+    ti.init(l1, t0, 1);
+    j = j0;
+    left = count;
+  }
+  __device__ __forceinline__ bool done() const { return left <= 0; }
+  __device__ __forceinline__ void next(const UmmaParams& l1, int chunks) {
+    --left;
+    if (++j == chunks) { j = 0; ti.next(l1); }
+  }
+};
+
+template <int kOut1, int kOut2, bool kUniform, bool kBufs>
 __global__ void __launch_bounds__(kFThreads, 1)
     conv_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
-                      const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ FusedParams p) {
+                      const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmRes,
+                      const __grid_constant__ CUtensorMap tmY, const __grid_constant__ FusedParams p) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long a_full[kMaxStages], a_empty[kMaxStages];
   __shared__ __align__(8) unsigned long long b_full[kMaxBStages], b_empty[kMaxBStages];
   __shared__ __align__(8) unsigned long long acc1_full[2], acc1_empty[2];
   __shared__ __align__(8) unsigned long long acc2_full[kFE2Groups], acc2_empty[kFE2Groups];
   __shared__ __align__(8) unsigned long long tb_full[kFMaxTb], tb_empty[kFMaxTb];
+  __shared__ __align__(8) unsigned long long buf_full[kFSlots], store_ready[kFSlots];
   __shared__ __align__(8) unsigned long long w1_full, w2_full, mma_turn;
   __shared__ uint32_t tmem_holder;
   __shared__ int abort_flag;
 
-  // dynamic smem: [W1 resident] [W2 resident] [A stages] [W1 ring] [T ring] [bias1, scale1] [bias2, scale2]
+  // dynamic smem: [W1 resident] [W2 resident] [A stages] [W1 ring] [T ring] [layer-2 tile buffers] [bias1, scale1] [bias2, scale2]
   const uint32_t raw_base = smem_u32(smem_raw);
   const uint32_t base = (raw_base + 1023u) & ~1023u;
   unsigned char* const base_ptr = smem_raw + (base - raw_base);
@@ -148,6 +177,11 @@ __global__ void __launch_bounds__(kFThreads, 1)
     } else if (warp == 2) {
       if (lane < kFE2Groups) { mbar_init(smem_u32(&acc2_full[lane]), 1); mbar_init(smem_u32(&acc2_empty[lane]), 4); }
       else if (lane >= 8 && lane - 8 < p.ntb) { mbar_init(smem_u32(&tb_full[lane - 8]), kGroupThreads); mbar_init(smem_u32(&tb_empty[lane - 8]), 1); }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    } else if (kBufs && warp == 3) {
+      if (lane < p.nslots) { mbar_init(smem_u32(&buf_full[lane]), 1); mbar_init(smem_u32(&store_ready[lane]), kGroupThreads); }
+      else if (lane == 16 && p.l2.res_mode == kResVec) prefetch_tensormap(&tmRes);
+      else if (lane == 17) prefetch_tensormap(&tmY);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tcgen05_fence_before();
@@ -240,6 +274,57 @@ __global__ void __launch_bounds__(kFThreads, 1)
       if (++slot == ntb) { slot = 0; tpar ^= 1u; }
     }
     if (!ok && lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutMma); }
+  } else if (kBufs && warp == 3) {
+    // ------------------------------------------------------------------ layer-2 tile buffers: residual in, output out
+    // Item i of the CTA's sequence uses buffer i % nslots.  A buffer goes: residual tile arrives (buf_full) -> an E2
+    // group turns it into the output tile (store_ready) -> TMA store -> once the store has read it, the residual
+    // of item i + nslots is loaded into it.
+    const UmmaParams& q = p.l2;
+    const uint32_t bfull0 = smem_u32(&buf_full[0]), ready0 = smem_u32(&store_ready[0]);
+    const uint32_t nslots = (uint32_t)p.nslots;
+    const int pw = 1 << q.pw_shift;
+    const uint32_t panel_bytes = (uint32_t)kBM << q.pw_shift;
+    const UmmaParams& h = p.l1;  // tile geometry
+    auto fill_buffer = [&](const ItemIter& it, uint32_t s) {
+      const uint32_t bar = bfull0 + s * 8u;
+      if (q.res_mode == kResVec) {
+        uint32_t dst = base + q.off_bufs + s * q.tile8_bytes;
+        mbar_arrive_expect_tx(bar, p.res_tx_bytes);
+        for (int pn = 0, c = it.j * q.bn; pn < q.panels; ++pn, c += pw, dst += panel_bytes)
+          tma_load_4d(dst, &tmRes, bar, c, it.ti.qt * h.tw, it.ti.pt * h.th, it.ti.img);
+      } else {
+        mbar_arrive(bar);
+      }
+    };
+    ItemIter ld, st;
+    ld.init(h, t0, j0, my_items);
+    st.init(h, t0, j0, my_items);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (elect_one())
+      for (uint32_t s = 0; s < nslots && !ld.done(); ++s, ld.next(h, chunks)) fill_buffer(ld, s);
+    else
+      for (uint32_t s = 0; s < nslots && !ld.done(); ++s) ld.next(h, chunks);
+    uint32_t slot = 0, spar = 0;
+    int prev_slot = -1;
+    bool ok = true;
+    for (; !st.done(); st.next(h, chunks)) {
+      if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
+      if (elect_one()) {
+        uint32_t src = base + q.off_bufs + slot * q.tile8_bytes;
+        for (int pn = 0, c = q.c_off + st.j * q.bn; pn < q.panels; ++pn, c += pw, src += panel_bytes)
+          tma_store_4d(&tmY, src, c, st.ti.qt * h.tw, st.ti.pt * h.th, st.ti.img);
+        bulk_commit();
+        // A buffer takes its next residual once its store has read it; the load is left until the next store, which
+        // keeps this warp free.
+        bulk_wait_read<1>();
+        if (prev_slot >= 0 && !ld.done()) fill_buffer(ld, (uint32_t)prev_slot);
+      }
+      if (prev_slot >= 0 && !ld.done()) ld.next(h, chunks);
+      prev_slot = (int)slot;
+      if (++slot == nslots) { slot = 0; spar ^= 1u; }
+    }
+    if (elect_one()) bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
+    if (!ok && lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutStore); }
   } else if (warp >= kFCtrlWarps && warp < kFCtrlWarps + 4) {
     // ------------------------------------------------------------------ E1: layer-1 accumulator -> T[slot]
     const UmmaParams& q = p.l1;
@@ -252,9 +337,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     t.smem_ok = pp < q.th && qq < q.tw;
     t.srow = t.smem_ok ? pp * q.tw + qq : 0;
     epi_row_setup(q, t);
-    t.n0 = 0; t.y_off = 0; t.m = 0; t.row_ok = false;
-    t.yrow = nullptr; t.rrow = nullptr; t.wide = t.res_wide = false;
-    const ResPair none = {};
+    t.n0 = 0; t.y_off = 0; t.m = 0; t.row_ok = false; t.yrow = nullptr; t.rrow = nullptr; t.wide = t.res_wide = false;
     const uint32_t accf0 = smem_u32(&acc1_full[0]), acce0 = smem_u32(&acc1_empty[0]);
     const uint32_t tbf0 = smem_u32(&tb_full[0]), tbe0 = smem_u32(&tb_empty[0]);
     const uint32_t nacc = (uint32_t)q.nacc, ntb = (uint32_t)p.ntb;
@@ -270,13 +353,13 @@ __global__ void __launch_bounds__(kFThreads, 1)
       tcgen05_fence_after();
       t.buf = base_ptr + p.off_tb + (size_t)slot * p.tb_bytes;
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)p.acc1_col + ab * (uint32_t)q.acc_stride;
-      epilogue_row<kOut1, kResNone, false, kUniform, true>(q, t, taddr, acce0 + ab * 8u, lane, 0, nchunk, none);
+      epilogue_row<kOut1, kResNone, false, kUniform, true>(q, t, taddr, acce0 + ab * 8u, lane, 0, nchunk, ResPair{});
       fence_proxy_async_smem();  // the tile is read by the tensor core (async proxy)
       mbar_arrive(tbf0 + slot * 8u);
       if (++ab == nacc) { ab = 0; apar ^= 1u; }
       if (++slot == ntb) { slot = 0; tpar ^= 1u; }
     }
-  } else if (warp >= kFCtrlWarps) {
+  } else if (!kBufs && warp >= kFCtrlWarps) {
     // ------------------------------------------------------------------ E2 groups: layer-2 accumulator g -> global memory
     const UmmaParams& q = p.l2;
     const UmmaParams& h = p.l1;  // tile geometry
@@ -318,6 +401,46 @@ __global__ void __launch_bounds__(kFThreads, 1)
       epilogue_row<kOut2, kResVec, false, kUniform, false>(q, t, taddr, acce, lane, 0, nchunk, rp);
       apar ^= 1u;
     }
+  } else if (kBufs && warp >= kFCtrlWarps) {
+    // ------------------------------------------------------------------ E2 groups: layer-2 accumulator g -> tile buffer
+    const UmmaParams& q = p.l2;
+    const int g = (warp - kFCtrlWarps - 4) >> 2;
+    const int quad = warp & 3, row = quad * 32 + lane;
+    EpiTile t;
+    t.s_bias = s_bias2;
+    t.s_scale = s_scale2;
+    t.scale = s_scale2[0];
+    t.srow = row;                               // T rows are the tile's pixels in dense order
+    t.smem_ok = row < p.l1.th * p.l1.tw;
+    epi_row_setup(q, t);
+    t.y_off = 0; t.m = 0; t.row_ok = false; t.yrow = nullptr; t.rrow = nullptr; t.wide = t.res_wide = false;
+    const uint32_t accf = smem_u32(&acc2_full[g]), acce = smem_u32(&acc2_empty[g]);
+    const uint32_t bfull0 = smem_u32(&buf_full[0]), ready0 = smem_u32(&store_ready[0]);
+    const uint32_t nslots = (uint32_t)p.nslots;
+    const int items = my_items;
+    uint32_t apar = 0, slot = (uint32_t)g % nslots, spar = ((uint32_t)g / nslots) & 1u;
+    int j = (j0 + g) % chunks;
+    const int nchunk = q.bn >> 4;
+    const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)g * (uint32_t)kFAcc2Cols;
+    for (int i = g; i < items; i += kFE2Groups) {
+      bool ok = mbar_wait(accf, apar, abortp);
+      if (ok) ok = mbar_wait(bfull0 + slot * 8u, spar, abortp);
+      if (!ok) {
+        if (lane0) { abort_flag = 1; atomicOr(p.l1.status, kTimeoutEpilogue); }
+        break;
+      }
+      tcgen05_fence_after();
+      t.n0 = j * q.bn;
+      t.buf = base_ptr + q.off_bufs + (size_t)slot * q.tile8_bytes;
+      epilogue_row<kOut2, kResRows, false, kUniform, true>(q, t, taddr, acce, lane, 0, nchunk, ResPair{});
+      fence_proxy_async_smem();
+      mbar_arrive(ready0 + slot * 8u);
+      apar ^= 1u;
+      slot += (uint32_t)kFE2Groups;
+      while (slot >= nslots) { slot -= nslots; spar ^= 1u; }
+      j += kFE2Groups;
+      while (j >= chunks) j -= chunks;
+    }
   }
 
   tcgen05_fence_before();
@@ -329,10 +452,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
   }
 }
 
-template <int kOut1, int kOut2, bool kUniform>
-int launch_fused_variant(const CUtensorMap& tmA, const CUtensorMap& tmB1, const CUtensorMap& tmB2,
-                         const FusedParams& p, size_t dyn, int grid, cudaStream_t stream) {
-  auto kernel = conv_fused_kernel<kOut1, kOut2, kUniform>;
+template <int kOut1, int kOut2, bool kUniform, bool kBufs>
+int launch_fused_variant(const CUtensorMap& tmA, const CUtensorMap& tmB1, const CUtensorMap& tmB2, const CUtensorMap& tmRes,
+                         const CUtensorMap& tmY, const FusedParams& p, size_t dyn, int grid, cudaStream_t stream) {
+  auto kernel = conv_fused_kernel<kOut1, kOut2, kUniform, kBufs>;
   static std::atomic<bool> configured[kMaxDevices];
   const int dev = current_device();
   if (dev < 0 || !configured[dev].load(std::memory_order_acquire)) {
@@ -355,7 +478,7 @@ int launch_fused_variant(const CUtensorMap& tmA, const CUtensorMap& tmB1, const 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB1, tmB2, p);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB1, tmB2, tmRes, tmY, p);
   if (le != cudaSuccess) {
     cudaGetLastError();
     return fail(Q8_ERR_CUDA, "conv_fused: launch failed (%s; grid %d, shared memory %zu)", cudaGetErrorString(le), grid, dyn);
@@ -434,9 +557,16 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   b.bn = BN2; b.bk = d1.K; b.ksteps = d1.K / 32;
   b.K = d2.K; b.M = a.M; b.P = P; b.Q = Q; b.PQ = P * Q;
   b.n_tiles = (d2.K + BN2 - 1) / BN2;
-  b.k_pad = b.n_tiles * BN2;
   b.fd_ntiles = make_fastdiv(b.n_tiles);
+  b.k_pad = b.n_tiles * BN2;
+  int pw = BN2 & -BN2;
+  if (pw > 128) pw = 128;
+  while ((1 << b.pw_shift) < pw) ++b.pw_shift;
+  b.pmask = pw == 128 ? 7 : (pw == 64 ? 3 : (pw == 32 ? 1 : 0));
+  b.panels = BN2 / pw;
+  b.tile8_bytes = (unsigned)(kBM * BN2);
   b.b_tile_bytes = (unsigned)(BN2 * d1.K);
+  pl.p.res_tx_bytes = (unsigned)BN2 * (unsigned)(ht.tw * ht.th);
   b.relu = d2.relu; b.y_type = d2.y_type; b.y_vec = 1;
   b.scale_count = d2.scale_count;
   b.ldc = ldc; b.c_off = d2.y_c_offset;
@@ -452,9 +582,10 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   a.a_stage_bytes = round_up(reach > a.a_sub_bytes ? reach : a.a_sub_bytes, 1024u);
   pl.p.tb_bytes = (unsigned)(kBM * BN1);
   const unsigned w2_bytes = round_up(w2_all, 1024u);
-  // weights of layer 1 resident when that leaves room for two patch stages and two T slots
+  // weights of layer 1 resident when that leaves room for two patch stages, two T slots and three tile buffers (what
+  // a pair must leave free to be accepted, whichever way its bytes go)
   const bool resident = w1_all <= 80u * 1024u && a.b_tile_bytes % (8u * BK1) == 0 &&
-                        budget >= round_up(w1_all, 1024u) + w2_bytes + 2u * a.a_stage_bytes + 2u * pl.p.tb_bytes;
+                        budget >= round_up(w1_all, 1024u) + w2_bytes + 2u * a.a_stage_bytes + 2u * pl.p.tb_bytes + 3u * b.tile8_bytes;
   a.b_mode = resident ? kBResident : kBRing;
   const unsigned w1_bytes = resident ? round_up(w1_all, 1024u) : 0u;
   a.b_T = 1; a.b_chunks = a.taps;
@@ -462,7 +593,7 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   if (!resident) {
     if (a.b_tile_bytes % (8u * BK1)) { *why = "weight tiles of the first layer do not keep the swizzle alignment"; return false; }
     // ring stages of several taps (one TMA operation each), two of them
-    const unsigned fixed = w2_bytes + 2u * a.a_stage_bytes + 1u * pl.p.tb_bytes;
+    const unsigned fixed = w2_bytes + 2u * a.a_stage_bytes + 1u * pl.p.tb_bytes + 3u * b.tile8_bytes;
     const unsigned avail = budget > fixed ? budget - fixed : 0u;
     int T = (int)(48u * 1024u / a.b_tile_bytes);
     if (T > (int)(avail / (2u * a.b_tile_bytes))) T = (int)(avail / (2u * a.b_tile_bytes));
@@ -474,11 +605,18 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
     a.b_sub_bytes = round_up((unsigned)a.b_T * a.b_tile_bytes, 1024u);
     ring_min = 2u * a.b_sub_bytes;
   }
-  const unsigned need_min = w1_bytes + w2_bytes + 2u * a.a_stage_bytes + ring_min + 1u * pl.p.tb_bytes;
+  const unsigned need_min = w1_bytes + w2_bytes + 2u * a.a_stage_bytes + ring_min + 1u * pl.p.tb_bytes + 3u * b.tile8_bytes;
   if (budget < need_min) { *why = "the layer pair does not fit in shared memory"; return false; }
   unsigned rest = budget - need_min;
   pl.p.ntb = 1;
+  pl.p.nslots = 0;
+  rest += 3u * b.tile8_bytes;
   if (rest >= pl.p.tb_bytes) { pl.p.ntb = 2; rest -= pl.p.tb_bytes; }
+  if ((long long)a.m_tiles * b.n_tiles > (long long)kFBufMinItems * sm_count() &&
+      rest >= (unsigned)kFSlots * b.tile8_bytes + a.a_stage_bytes) {  // where this line lies: see the head of the file
+    pl.p.nslots = kFSlots;
+    rest -= (unsigned)kFSlots * b.tile8_bytes;
+  }
   a.b_stages = 0;
   if (!resident) {
     a.b_stages = 2;
@@ -490,7 +628,8 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   a.off_a = w1_bytes + w2_bytes;
   a.off_bring = a.off_a + (unsigned)a.stages * a.a_stage_bytes;
   pl.p.off_tb = a.off_bring + (unsigned)a.b_stages * a.b_sub_bytes;
-  a.off_chan = pl.p.off_tb + (unsigned)pl.p.ntb * pl.p.tb_bytes;
+  b.off_bufs = pl.p.off_tb + (unsigned)pl.p.ntb * pl.p.tb_bytes;
+  a.off_chan = b.off_bufs + (unsigned)pl.p.nslots * b.tile8_bytes;
   pl.p.off_chan2 = a.off_chan + chan1;
   pl.dyn = 1024u + pl.p.off_chan2 + chan2;
   if (pl.dyn > (size_t)(kSmemLimit - kStaticSmemReserve)) { *why = "the layer pair does not fit in shared memory"; return false; }
@@ -528,7 +667,7 @@ int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void
   if (residual && !aligned16(residual)) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d_then_1x1: residual not 16-byte aligned");
   FusedParams& p = pl.p;
   const HaloTile& ht = pl.ht;
-  const int BK1 = pl.BK1;
+  const int BK1 = pl.BK1, P = pl.P, Q = pl.Q;
   p.l1.bias = bias1; p.l1.scale = scale1; p.l1.status = status;
   p.l2.bias = bias2; p.l2.scale = scale2; p.l2.status = status;
   p.l2.res = static_cast<const unsigned char*>(residual);
@@ -538,7 +677,8 @@ int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void
   p.l2.res_scale = residual_scale;
   p.l2.y = y;
 
-  CUtensorMap tmA, tmB1, tmB2;
+  CUtensorMap tmA, tmB1, tmB2, tmRes, tmY;
+  memset(&tmRes, 0, sizeof(tmRes));
   const cuuint32_t ones[4] = {1, 1, 1, 1};
   CUresult cr;
   {
@@ -567,14 +707,33 @@ int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void
                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for_bytes(d1.K), CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_fused: second weight tensor map rejected (CUresult %d)", (int)cr);
   }
+  const int pw = 1 << p.l2.pw_shift;
+  auto encode_rows = [&](CUtensorMap* tm, void* ptr, int channels, int ld, CUtensorMapL2promotion promo) -> CUresult {
+    cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)Q, (cuuint64_t)P, (cuuint64_t)d1.N};
+    cuuint64_t strides[3] = {(cuuint64_t)ld, (cuuint64_t)Q * ld, (cuuint64_t)P * Q * ld};
+    cuuint32_t box[4] = {(cuuint32_t)pw, (cuuint32_t)ht.tw, (cuuint32_t)ht.th, 1};
+    return fn.tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, ptr, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    swizzle_for_bytes(pw), promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  if (residual) {
+    cr = encode_rows(&tmRes, const_cast<void*>(residual), d2.K, d2.K, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+    if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_fused: residual tensor map rejected (CUresult %d)", (int)cr);
+  }
+  cr = encode_rows(&tmY, y, p.l2.c_off + d2.K, p.l2.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
+  if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_fused: output tensor map rejected (CUresult %d)", (int)cr);
+
   const long long items = (long long)p.l1.m_tiles * p.l2.n_tiles;
   const int grid = (int)(items < sm_count() ? items : sm_count());
   // one multiplier per tensor in both layers, or per-channel arrays (a lone one is staged once per channel)
   const bool uniform = d1.scale_count == 1 && d2.scale_count == 1;
 #define Q8_FUSED(OUT1, OUT2)                                                                                           \
   do {                                                                                                                 \
-    if (uniform) return launch_fused_variant<OUT1, OUT2, true>(tmA, tmB1, tmB2, p, pl.dyn, grid, stream);  \
-    return launch_fused_variant<OUT1, OUT2, false>(tmA, tmB1, tmB2, p, pl.dyn, grid, stream);              \
+    if (p.nslots) {                                                                                                    \
+      if (uniform) return launch_fused_variant<OUT1, OUT2, true, true>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream); \
+      return launch_fused_variant<OUT1, OUT2, false, true>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);      \
+    }                                                                                                                  \
+    if (uniform) return launch_fused_variant<OUT1, OUT2, true, false>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream); \
+    return launch_fused_variant<OUT1, OUT2, false, false>(tmA, tmB1, tmB2, tmRes, tmY, p, pl.dyn, grid, stream);       \
   } while (0)
   if (d1.y_type == Q8_U8) {
     if (d2.y_type == Q8_U8) Q8_FUSED(Q8_U8, Q8_U8);

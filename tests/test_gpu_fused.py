@@ -118,3 +118,19 @@ def test_ineligible_pairs_are_refused_with_a_reason(q8):
     with pytest.raises(q8.Q8Error) as e:
         q8.q8_conv2d_then_1x1(d1, d2, x, w1, None, s, w2, None, s)
     assert e.value.code == 2 and "32, 64 or 128" in str(e.value)
+
+
+# 56x56 64->64->256 has 56 items of layer 2 per image: both sides of four items per block, where tile buffers take over
+@pytest.mark.parametrize("N", [10, 11, 12])
+def test_fused_pair_on_both_sides_of_the_buffer_rule(q8, N):
+    g = np.random.default_rng(N)
+    x, r = (torch.from_numpy(g.integers(0, 256, (N, 56, 56, c), dtype=np.uint8)).cuda() for c in (64, 256))
+    w1, w2 = (torch.from_numpy(g.integers(-128, 128, s).astype(np.int8)).cuda() for s in ((64, 3, 3, 64), (256, 1, 1, 64)))
+    s1, s2 = torch.tensor([3e-4], device="cuda"), torch.tensor([2e-4], device="cuda")
+    d1 = q8.make_conv_desc(N, 56, 56, 64, 64, 3, 3, (1, 1), (1, 1), (1, 1), U8, U8, U8, True)
+    d2 = q8.make_conv_desc(N, 56, 56, 64, 256, 1, 1, (1, 1), (0, 0), (1, 1), U8, U8, U8, True, 1)
+    y = q8.q8_conv2d_then_1x1(d1, d2, x, w1, None, s1, w2, None, s2, r, 0.37)
+    mid = o.conv2d(x.cpu().numpy(), w1.cpu().numpy(), None, np.float32(3e-4), pad=(1, 1), relu=True, threads=8)
+    acc = o.conv_acc(mid, w2.cpu().numpy(), None, (1, 1), (0, 0), (1, 1), threads=8)
+    q8.q8_read_status()
+    assert np.array_equal(y.cpu().numpy(), o.epilogue(acc, np.float32(2e-4), r.cpu().numpy(), 0.37, True, o.U8))
