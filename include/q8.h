@@ -216,6 +216,12 @@ typedef struct q8_conv_plan {
 } q8_conv_plan;
 int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan);
 
+/* How many tile buffers in shared memory a block of the TMA-fed kernel, or with `then_1x1` a block of
+ * q8_conv2d_then_1x1(d, then_1x1), moves its 8-bit rows through: 0 where the epilogue accesses global memory itself.
+ * Given and answered as q8_conv2d_query_plan; `residual` is that of the call (of the 1x1 layer in a pair).
+ * Errors: Q8_ERR_INVALID_ARG.  Host only. */
+int q8_conv2d_query_row_buffers(const q8_conv_desc* d, const q8_conv_desc* then_1x1, int residual, int* buffers);
+
 /* x: device NHWC (x_type).  w: device KRSC s8.  bias: device s32[K] or NULL.
  * scale: device fp32[scale_count].  residual: device [N,P,Q,K] dense (res_type)
  * or NULL.  y: device, see above.  workspace: device, 16-byte aligned, workspace_bytes long, or NULL.

@@ -24,7 +24,7 @@ TORCH_DTYPES = {Q8_U8: torch.uint8, Q8_S8: torch.int8, Q8_S32: torch.int32, Q8_F
 _INT_TYPES = {torch.uint8: Q8_U8, torch.int8: Q8_S8, torch.int32: Q8_S32}
 EXPORTS = ["q8_version", "q8_last_error", "q8_read_status", "q8_calibrate_maxabs", "q8_factor", "q8_requant_scale",
            "q8_bias_factor", "q8_quantize", "q8_quantize_pad_channels", "q8_dequantize", "q8_fold_bn",
-           "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d_query_plan", "q8_conv2d", "q8_static_workspace_bytes",
+           "q8_conv2d_workspace_bytes", "q8_conv2d_query_algo", "q8_conv2d_query_plan", "q8_conv2d_query_row_buffers", "q8_conv2d", "q8_static_workspace_bytes",
            "q8_conv2d_static_workspace", "q8_conv2d_then_1x1_supported", "q8_conv2d_then_1x1", "q8_int8_mma_rate", "q8_selftest_bounded_wait", "q8_concat", "q8_concat_branch", "q8_calibrate_maxabs_rows", "q8_quantize_rows", "q8_quantize_pad_image", "q8_pool_out_extent",
            "q8_maxpool2d", "q8_avgpool2d", "q8_l2norm", "q8_add_relu_quantize", "q8_detection_output_workspace_bytes",
            "q8_detection_output", "q8_record_begin", "q8_record_end", "q8_record_replay", "q8_record_free"]
@@ -75,6 +75,7 @@ lib.q8_fold_bn.argtypes = [_vp] * 6 + [C.c_double, _i, _sz, _vp, _vp, _vp]
 lib.q8_conv2d_workspace_bytes.argtypes = [C.POINTER(q8_conv_desc), C.POINTER(_sz)]
 lib.q8_conv2d_query_algo.argtypes = [C.POINTER(q8_conv_desc), _ip]
 lib.q8_conv2d_query_plan.argtypes = [C.POINTER(q8_conv_desc), _i, C.POINTER(q8_conv_plan)]
+lib.q8_conv2d_query_row_buffers.argtypes = [C.POINTER(q8_conv_desc), C.POINTER(q8_conv_desc), _i, C.POINTER(_i)]
 lib.q8_conv2d.argtypes = [C.POINTER(q8_conv_desc), _vp, _vp, _vp, _vp, _vp, _f, _vp, _vp, _sz, _vp]
 lib.q8_static_workspace_bytes.argtypes = []
 lib.q8_selftest_bounded_wait.argtypes = [C.c_uint, _vp]
@@ -279,6 +280,12 @@ def q8_conv2d_query_plan(d, residual=False):
     p = q8_conv_plan()
     _check(lib.q8_conv2d_query_plan(C.byref(d), int(residual), C.byref(p)))
     return p
+
+
+def q8_conv2d_query_row_buffers(d, then_1x1=None, residual=False):
+    n = C.c_int()
+    _check(lib.q8_conv2d_query_row_buffers(C.byref(d), None if then_1x1 is None else C.byref(then_1x1), int(residual), C.byref(n)))
+    return n.value
 
 
 def q8_conv2d(d, x, w, bias, scale, residual=None, residual_scale=0.0, y=None, workspace=None):

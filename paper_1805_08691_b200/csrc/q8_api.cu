@@ -224,6 +224,24 @@ int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan
   return Q8_OK;
 }
 
+int q8_conv2d_query_row_buffers(const q8_conv_desc* d, const q8_conv_desc* then_1x1, int residual, int* buffers) {
+  clear_error();
+  ConvArgs a;
+  int rc = described_call(d, residual != 0, &a);
+  if (rc != Q8_OK) return rc;
+  if (!buffers) return fail(Q8_ERR_INVALID_ARG, "q8_conv2d_query_row_buffers: null pointer");
+  if (then_1x1) {
+    int P, Q;
+    rc = validate_desc(then_1x1, &P, &Q);
+    if (rc != Q8_OK) return rc;
+    *buffers = fused_row_buffers(*d, *then_1x1, residual != 0);
+    return Q8_OK;
+  }
+  const char* why = nullptr;
+  *buffers = conv_route(a, &why) == kRouteTma ? umma_row_buffers(a) : 0;
+  return Q8_OK;
+}
+
 int q8_conv2d(const q8_conv_desc* d, const void* x, const int8_t* w, const int32_t* bias, const float* scale,
               const void* residual, float residual_scale, void* y, void* workspace, size_t workspace_bytes,
               void* stream) {

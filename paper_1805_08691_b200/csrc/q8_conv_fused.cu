@@ -654,6 +654,11 @@ bool fused_pair_eligible(const q8_conv_desc& d1, const q8_conv_desc& d2, const c
   return plan_fused(d1, d2, nullptr, why);
 }
 
+int fused_row_buffers(const q8_conv_desc& d1, const q8_conv_desc& d2, bool) {
+  FusedPlan pl;
+  return plan_fused(d1, d2, &pl, nullptr) ? pl.p.nslots : 0;
+}
+
 int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void* x, const int8_t* w1, const int32_t* bias1,
                       const float* scale1, const int8_t* w2, const int32_t* bias2, const float* scale2, const void* residual,
                       float residual_scale, void* y, cudaStream_t stream) {

@@ -35,14 +35,14 @@
 //                owns one accumulator row: tcgen05.ld, + bias, requantise, + residual, ReLU, round,
 //                clamp, straight to global memory; residual bytes come from there the same way, a pair of
 //                16-column chunks ahead.
-// The epilogue moved its bytes by TMA before (residual tiles into shared-memory buffers, finished tiles out of them): a
-// copy of a 128-row box occupies the copy engine for some 400 cycles, beside those of the operands, and the store of the
-// last tile, through two barriers and another warp, ended 0.8 us after its arithmetic.  Now that is 0.2 us (14x14 256->256
-// 3x3, batch 64: from the last accumulator to the end of the CTA 2.0 -> 1.8 us in all, since 32 rows a pitch apart keep the
-// load/store unit for 47 cycles an instruction; tiles of 16 columns on one image 0.9 -> 0.6 us), and the shared memory of the buffers holds operands: ResNet-50 batch 1 285 -> 252 us, batch
-// 64 722 -> 702 us, Inception-v3 batch 64 1226 -> 1164 us, 14x14 bottleneck batch 64 33.1 -> 30.6 us.  Measured and not kept:
-// rows exchanged through shared memory so that two lanes share one (64 contiguous bytes an access): 14x14 bottleneck 33.3 us,
-// 56x56 41 us; four lanes a row by tcgen05.ld.16x128b and weight rows in permuted order: 32.3 and 44 us.
+// Where the rows are most of a launch (see buffered()), another instantiation moves them by TMA: warp 4 hands tile buffers in
+// shared memory to the epilogue groups, filled with the residual tile when there is one, the groups turn them into output
+// tiles in place, warp 5 stores those and recycles the buffers; the groups are warps 6 and up.
+// Without buffers there are two hand-offs less behind the last tile, whose store ended 0.8 us after its arithmetic with them and
+// ends 0.2 us after it now (14x14 256->256 3x3, batch 64), and their shared memory holds operands: ResNet-50 batch 1 285 -> 252
+// us, batch 64 722 -> 702 us, Inception-v3 batch 64 1226 -> 1164 us, 14x14 bottleneck batch 64 33.1 -> 30.6 us.  Measured and not
+// kept: rows exchanged through shared memory so that two lanes share one (64 contiguous bytes an access): 14x14 bottleneck 33.3
+// us, 56x56 41 us; four lanes a row by tcgen05.ld.16x128b and weight rows in permuted order: 32.3 and 44 us.
 // The kernel is launched with programmatic stream serialization: its set-up overlaps the tail of the kernel
 // before it, and every global access comes after griddepcontrol.wait.
 // All hand-offs are mbarriers, there is no block-wide barrier after the prologue.  Every wait is
@@ -135,20 +135,40 @@ __device__ __forceinline__ bool mma_role_pair(const UmmaParams& p, const MmaRole
 // G epilogue groups; one instantiation per output type and residual source keeps a single epilogue
 // body in each kernel (several of them in one kernel made the register allocator spill).
 // kCta2: the CTA-pair variant (its cta_group::2 instructions make the kernel launchable as clusters of two only).
+// kRes = kResTma: 8-bit rows, a residual's in and the output's out, move by TMA through tile buffers in shared memory.
+template <int kRes>
+constexpr int kCtrlOf = kRes == kResTma ? kCtrlWarps + 2 : kCtrlWarps;  // control warps
+template <bool kBufs>
+struct RowMaps {};           // tensor maps of the residual's and the output's tiles
+template <>
+struct RowMaps<true> { CUtensorMap res, y; };
+constexpr int kFillWarp = kCtrlWarps, kStoreWarp = kCtrlWarps + 1;
+template <bool kBufs>
+__device__ __forceinline__ void prefetch_maps(const RowMaps<kBufs>& maps, bool residual) {
+  if constexpr (kBufs) {
+    if (residual) prefetch_tensormap(&maps.res);
+    prefetch_tensormap(&maps.y);
+  }
+}
+
 template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
-__global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
+__global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
     conv_umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                     const __grid_constant__ UmmaParams p) {
+                     const __grid_constant__ UmmaParams p, const __grid_constant__ RowMaps<kRes == kResTma> maps) {
+  constexpr bool kBufs = kRes == kResTma;
+  constexpr int kCtrl = kCtrlOf<kRes>, kCtrlT = kCtrl * 32;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long a_full[kMaxStages], a_empty[kMaxStages];
   __shared__ __align__(8) unsigned long long b_full[kMaxBStages], b_empty[kMaxBStages];
   __shared__ __align__(8) unsigned long long acc_full[kMaxAcc], acc_empty[kMaxAcc];
+  // per buffer: residual arrived (or none to come), output tile read by its store, output tile written
+  __shared__ __align__(8) unsigned long long buf_full[kBufs ? kMaxSlots : 1], buf_empty[kBufs ? kMaxSlots : 1], store_ready[kBufs ? kMaxSlots : 1];
   __shared__ __align__(8) unsigned long long bres_full;
   __shared__ __align__(8) unsigned long long mma_turn[kMmaWarps];
   __shared__ uint32_t tmem_holder;
   __shared__ int abort_flag;
 
-  // dynamic smem: [resident weights] [A stages] [weight ring] [tile buffers of moved rows] [bias, scale]
+  // dynamic smem: [resident weights] [A stages] [weight ring] [8-bit tile buffers] [bias, scale]
   const uint32_t raw_base = smem_u32(smem_raw);
   const uint32_t base = (raw_base + 1023u) & ~1023u;
   unsigned char* const base_ptr = smem_raw + (base - raw_base);
@@ -163,6 +183,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   const int vblock = kCta2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int vgrid = kCta2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const int total_tiles = p.m_tiles * p.n_tiles * p.splits;  // work items
+  const int slots = (kCta2 ? G >> p.pair_shift : G) * p.nbuf;  // tile buffers of the CTA, used round robin
 
   // Programmatic dependent launch: the next kernel of the stream may be scheduled onto SMs as they fall idle
   // (it waits below, like this one, before it touches global memory), and this kernel's own set-up (barriers,
@@ -176,14 +197,14 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
   // control warps meet on barrier 1 among themselves and start; the epilogue warps first touch every line of the
   // kernel parameters (the control warps' first reads of them would otherwise miss the constant cache one after
   // the other), fetch bias and scale, and join on barrier 3, which the control warps only signal.
-  const int nthreads = kCtrlThreads + G * kGroupThreads;
-  if (!kCta2 && warp >= kCtrlWarps) {
+  const int nthreads = kCtrlT + G * kGroupThreads;
+  if (!kCta2 && warp >= kCtrl) {
     const unsigned int* words = reinterpret_cast<const unsigned int*>(&p);
     unsigned int touched = 0;
-    for (int i = ((int)threadIdx.x - kCtrlThreads) * 16; i < (int)(sizeof(UmmaParams) / 4); i += G * kGroupThreads * 16) touched ^= words[i];
+    for (int i = ((int)threadIdx.x - kCtrlT) * 16; i < (int)(sizeof(UmmaParams) / 4); i += G * kGroupThreads * 16) touched ^= words[i];
     asm volatile("" ::"r"(touched));
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = (int)threadIdx.x - kCtrlThreads; i < p.k_pad; i += G * kGroupThreads) {
+    for (int i = (int)threadIdx.x - kCtrlT; i < p.k_pad; i += G * kGroupThreads) {
       s_bias[i] = (p.bias && i < p.K) ? p.bias[i] : 0;
       s_scale[i] = p.scale ? (p.scale_count == 1 ? p.scale[0] : (i < p.K ? p.scale[i] : 0.f)) : 0.f;
     }
@@ -203,7 +224,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       cluster_sync_all();  // the peer's barriers exist before anything signals them
       asm volatile("bar.arrive 1, %0;" ::"r"(nthreads) : "memory");
     } else {
-      asm volatile("bar.arrive 1, %0;" ::"r"(kCtrlThreads) : "memory");
+      asm volatile("bar.arrive 1, %0;" ::"r"(kCtrlT) : "memory");
       asm volatile("bar.arrive 3, %0;" ::"r"(nthreads) : "memory");
     }
   } else {
@@ -211,6 +232,13 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       // one arrival per epilogue warp that reads the accumulator: a group's four, or all of them in split mode
       if (lane < p.nacc) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), kCta2 ? 8 << p.pair_shift : (p.epi_split ? 4 * G : 4)); }
       else if (lane >= 8 && lane - 8 < kMmaWarps) mbar_init(smem_u32(&mma_turn[lane - 8]), 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    } else if (kBufs && warp == kFillWarp) {
+      if (lane < slots) { mbar_init(smem_u32(&buf_full[lane]), 1); mbar_init(smem_u32(&buf_empty[lane]), 1); }
+      else if (lane == 16) prefetch_maps(maps, p.res_mode != kResNone);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    } else if (kBufs && warp == kStoreWarp) {
+      if (lane < slots) mbar_init(smem_u32(&store_ready[lane]), kCta2 ? kGroupThreads << p.pair_shift : kGroupThreads);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -237,7 +265,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     } else {
       tcgen05_fence_before();
       asm volatile("bar.arrive 3, %0;" ::"r"(nthreads) : "memory");      // the epilogue warps wait for this set-up
-      asm volatile("bar.sync 1, %0;" ::"r"(kCtrlThreads) : "memory");    // the control warps only for each other
+      asm volatile("bar.sync 1, %0;" ::"r"(kCtrlT) : "memory");    // the control warps only for each other
     }
     tcgen05_fence_after();
   }
@@ -256,7 +284,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     uint32_t bs = 0, bphase = 0, b_dst = bring0;
     bool ok = true;
     // Everything the previous kernel wrote is visible from here.  The roles wait for it themselves, as late as they
-    // touch global memory, so that their set-up runs while that kernel drains; the MMA warps and the store warp only
+    // touch global memory, so that their set-up runs while that kernel drains; the MMA warps (and the store warp) only
     // ever follow loads of this warp and need no wait of their own.
     if constexpr (!kCta2) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.b_mode == kBResident) {
@@ -391,9 +419,92 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       abort_flag = 1;
       atomicOr(p.status, kTimeoutMma);
     }
+  } else if (kBufs && warp == kFillWarp) {
+    // ------------------------------------------------------------------ tile buffers to the epilogue, with their residual tile
+    if constexpr (kBufs) {
+      TileIterT<kCta2> ti;
+      ti.init(p, vblock, vgrid, cta_rank);
+      const uint32_t bfull0 = smem_u32(&buf_full[0]), bempty0 = smem_u32(&buf_empty[0]);
+      const uint32_t nslots = (uint32_t)slots;
+      uint32_t slot = 0, par = 1;  // tile lt of the CTA's sequence uses buffer lt % slots
+      bool ok = true;
+      const int pw = 1 << p.pw_shift;
+      const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
+      if constexpr (!kCta2) asm volatile("griddepcontrol.wait;" ::: "memory");
+      for (; ti.tile < total_tiles; ti.next(p)) {
+        if (!mbar_wait(bempty0 + slot * 8u, par, abortp)) { ok = false; break; }
+        const uint32_t bar = bfull0 + slot * 8u;
+        if (!elect_one()) {
+        } else if (p.res_mode != kResNone && ti.valid) {
+          uint32_t dst = base + p.off_bufs + slot * p.tile8_bytes;
+          mbar_arrive_expect_tx(bar, p.res_tx_bytes);
+          if (p.a_mode == kAHalo) {
+            for (int pn = 0, c = ti.nt * p.bn; pn < p.panels; ++pn, c += pw, dst += panel_bytes) tma_load_4d(dst, &maps.res, bar, c, ti.qt * p.tw, ti.pt * p.th, ti.img);
+          } else {
+            for (int pn = 0, c = ti.nt * p.bn; pn < p.panels; ++pn, c += pw, dst += panel_bytes) tma_load_2d(dst, &maps.res, bar, c, ti.mt * kBM);
+          }
+        } else {
+          mbar_arrive(bar);
+        }
+        if (++slot == nslots) { slot = 0; par ^= 1u; }
+      }
+      if (!ok && lane0) {
+        abort_flag = 1;
+        atomicOr(p.status, kTimeoutResidual);
+      }
+    }
+  } else if (kBufs && warp == kStoreWarp) {
+    // ------------------------------------------------------------------ finished tiles to global memory, buffers back
+    if constexpr (kBufs) {
+      TileIterT<kCta2> ti;
+      ti.init(p, vblock, vgrid, cta_rank);
+      const uint32_t bempty0 = smem_u32(&buf_empty[0]), ready0 = smem_u32(&store_ready[0]);
+      const uint32_t nslots = (uint32_t)slots;
+      uint32_t slot = 0, spar = 0;
+      int prev_slot = -1;
+      const bool one_each = p.nbuf == 1;
+      bool ok = true;
+      const int pw = 1 << p.pw_shift;
+      const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
+      for (; ti.tile < total_tiles; ti.next(p)) {
+        if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
+        if (elect_one()) {
+          uint32_t src = base + p.off_bufs + slot * p.tile8_bytes;
+          if (!ti.valid) {
+            // second tile of the last pair of an odd count: nothing to store
+          } else if (p.a_mode == kAHalo) {
+            for (int pn = 0, c = p.c_off + ti.nt * p.bn; pn < p.panels; ++pn, c += pw, src += panel_bytes) tma_store_4d(&maps.y, src, c, ti.qt * p.tw, ti.pt * p.th, ti.img);
+          } else {
+            for (int pn = 0, c = p.c_off + ti.nt * p.bn; pn < p.panels; ++pn, c += pw, src += panel_bytes) tma_store_2d(&maps.y, src, c, ti.mt * kBM);
+          }
+          bulk_commit();
+          if (one_each) {
+            // one buffer per group: its group waits for it, so it is handed back as soon as it has been read (3x3
+            // 128->192 at 73x73, batch 64, two groups: 66.0 -> 62.3 us; with more buffers the wait would only hold up
+            // this warp)
+            bulk_wait_read<0>();
+            mbar_arrive(bempty0 + slot * 8u);
+          } else {
+            // the store before this one has read its buffer: hand that buffer back
+            bulk_wait_read<1>();
+            if (prev_slot >= 0) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
+          }
+          prev_slot = (int)slot;
+        }
+        if (++slot == nslots) { slot = 0; spar ^= 1u; }
+      }
+      if (elect_one()) {
+        bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
+        if (prev_slot >= 0 && !one_each) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
+      }
+      if (!ok && lane0) {
+        abort_flag = 1;
+        atomicOr(p.status, kTimeoutStore);
+      }
+    }
   } else {
     // ------------------------------------------------------------------ epilogue groups
-    const int g = (warp - kCtrlWarps) >> 2;
+    const int g = (warp - kCtrl) >> 2;
     const int quad = warp & 3;  // TMEM lane quadrant this warp may read
     const int row = quad * 32 + lane;  // accumulator row of this thread
     EpiTile t;
@@ -422,7 +533,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
     const uint32_t nacc = (uint32_t)p.nacc;
     // split mode: every group works on every tile and takes the chunks [ch0, ch1) of its columns, so that a
     // launch with one or two tiles per CTA does not leave three of four groups idle
-    const bool split = p.epi_split != 0;
+    const bool split = !kBufs && p.epi_split != 0;
     const int team = kCta2 ? g >> p.pair_shift : (split ? 0 : g);
     const int tile_step = kCta2 ? G >> p.pair_shift : (split ? 1 : G);
     const int nchunk_all = p.bn >> 4;
@@ -433,6 +544,7 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       ch1 = ((member + 1) * nchunk_all) >> p.pair_shift;
     }
     uint32_t ab = (uint32_t)team % nacc, acc_par = ((uint32_t)team / nacc) & 1u;
+    uint32_t slot = (uint32_t)team, slot_par = 0;
     TileIterT<kCta2> ti;
     ti.init(p, vblock + team * vgrid, tile_step * vgrid, cta_rank);
     for (; ti.tile < total_tiles; ti.next(p)) {
@@ -451,7 +563,9 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       place();
       ResPair rp = {};
       RowMove mv;
-      if constexpr (kRes == kResRows) {  // one buffer per group, shared where groups share tiles: their columns are disjoint
+      if constexpr (kBufs) {
+        t.buf = base_ptr + p.off_bufs + (size_t)slot * p.tile8_bytes;
+      } else if constexpr (kRes == kResRows) {  // one buffer per group, shared where groups share tiles: their columns are disjoint
         t.buf = base_ptr + p.off_bufs + (split ? (size_t)0 : (size_t)g * p.tile8_bytes);
         mv.init(p, t.n0, ch0, ch1);
         if (p.res_mode != kResNone) rows_in(p, t, mv, lane);  // while the accumulator is being formed
@@ -463,7 +577,9 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
         t.rrow = p.res + (long long)t.m * p.K + t.n0;
         if (kRes == kResVec && p.res_mode != kResNone) load_residual(p, t, ch0, ch1, rp);  // the first bytes, likewise
       }
-      if (!mbar_wait(accf0 + ab * 8u, acc_par, abortp)) {
+      bool ok = mbar_wait(accf0 + ab * 8u, acc_par, abortp);
+      if (kBufs && ok) ok = mbar_wait(smem_u32(&buf_full[0]) + slot * 8u, slot_par, abortp);
+      if (!ok) {
         if (lane == 0) {
           abort_flag = 1;
           atomicOr(p.status, kTimeoutEpilogue);
@@ -472,7 +588,13 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
       }
       tcgen05_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * (uint32_t)p.acc_stride;
-      epilogue_row<kOut, kRes, kCta2, kUniform, kRes == kResRows>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1, rp);
+      epilogue_row<kOut, kRes, kCta2, kUniform, kBufs || kRes == kResRows>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1, rp);
+      if constexpr (kBufs) {
+        fence_proxy_async_smem();  // this thread's reads and writes of the buffer are done; the store reads it
+        mbar_arrive(smem_u32(&store_ready[0]) + slot * 8u);
+        slot += (uint32_t)tile_step;
+        if (slot >= (uint32_t)slots) { slot -= (uint32_t)slots; slot_par ^= 1u; }
+      }
       if constexpr (kRes == kResRows) {
         __syncwarp();
         rows_out(p, t, mv, lane);
@@ -496,7 +618,11 @@ __global__ void __launch_bounds__(kCtrlThreads + G * kGroupThreads, 1)
 
 // ------------------------------------------------------------------------------------------ host
 template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
-int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaParams& p, size_t dyn, int grid, cudaStream_t stream) {
+int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const RowMaps<true>& row_maps, const UmmaParams& p, size_t dyn, int grid,
+                   cudaStream_t stream) {
+  constexpr int kThreads = kCtrlOf<kRes> * 32 + G * kGroupThreads;
+  RowMaps<kRes == kResTma> maps;
+  if constexpr (kRes == kResTma) maps = row_maps;
   auto kernel = conv_umma_kernel<G, kOut, kRes, kCta2, kUniform>;
   static std::atomic<bool> configured[kMaxDevices];  // per instantiation and device (the attribute is per device)
   const int dev = current_device();
@@ -514,7 +640,7 @@ int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaPar
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)(kCtrlThreads + G * kGroupThreads));
+  cfg.blockDim = dim3((unsigned)kThreads);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = stream;
   // let this kernel's set-up overlap the tail of the kernel before it in the stream
@@ -531,37 +657,40 @@ int launch_variant(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaPar
     attr[pdl].val.clusterDim.z = 1;
     cfg.numAttrs = pdl + 1;
   }
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB, p);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tmA, tmB, p, maps);
   if (le != cudaSuccess) {
     cudaGetLastError();
     return fail(Q8_ERR_CUDA, "conv_umma: launch failed (%s; grid %d, block %d, shared memory %zu, cluster %d)", cudaGetErrorString(le),
-                grid, kCtrlThreads + G * kGroupThreads, dyn, p.cta2 ? 2 : 1);
+                grid, kThreads, dyn, p.cta2 ? 2 : 1);
   }
   return check_launch("conv_umma_kernel");
 }
 
 template <int G>
-int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const UmmaParams& p, bool rows, size_t dyn, int grid, cudaStream_t stream) {
-#define Q8_LAUNCH(OUT, RES)                                                                                       \
-  do {                                                                                                            \
-    if (p.scale_count == 1) return launch_variant<G, OUT, RES, false, true>(tmA, tmB, p, dyn, grid, stream); \
-    return launch_variant<G, OUT, RES, false, false>(tmA, tmB, p, dyn, grid, stream);                 \
+int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const RowMaps<true>& maps, const UmmaParams& p, bool rows, size_t dyn, int grid,
+                  cudaStream_t stream) {
+#define Q8_LAUNCH(OUT, RES)                                                                                          \
+  do {                                                                                                               \
+    if (p.scale_count == 1) return launch_variant<G, OUT, RES, false, true>(tmA, tmB, maps, p, dyn, grid, stream);   \
+    return launch_variant<G, OUT, RES, false, false>(tmA, tmB, maps, p, dyn, grid, stream);                          \
   } while (0)
-  // kResVec stands for "a residual through the tile buffers, or none"
+  // kResTma and kResVec stand for "a residual, or none"
   const bool global_res = p.res_mode == kResGlobal;
   if (p.y_type == Q8_U8) {
     if (rows) Q8_LAUNCH(Q8_U8, kResRows);
+    if (p.nbuf) Q8_LAUNCH(Q8_U8, kResTma);
     Q8_LAUNCH(Q8_U8, kResVec);
   }
   if (p.y_type == Q8_S8) {
     if (rows) Q8_LAUNCH(Q8_S8, kResRows);
+    if (p.nbuf) Q8_LAUNCH(Q8_S8, kResTma);
     Q8_LAUNCH(Q8_S8, kResVec);
   }
   if (p.y_type == Q8_F32) {
     if (global_res) Q8_LAUNCH(Q8_F32, kResGlobal);
     Q8_LAUNCH(Q8_F32, kResVec);
   }
-  return launch_variant<G, Q8_S32, kResVec, false, false>(tmA, tmB, p, dyn, grid, stream);
+  return launch_variant<G, Q8_S32, kResVec, false, false>(tmA, tmB, maps, p, dyn, grid, stream);
 #undef Q8_LAUNCH
 }
 
@@ -627,7 +756,7 @@ struct UmmaPlan {
   size_t dyn;
 };
 
-bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, UmmaPlan* plan);
+bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, bool allow_bufs, UmmaPlan* plan);
 
 // Tries tile shapes from the preferred one down: halo patches of dilated filters on wide channel blocks can
 // exceed shared memory, narrower channel blocks shrink them; im2col loads need the least, where they are open.
@@ -635,7 +764,7 @@ bool plan_conv(const ConvArgs& a, int splits, UmmaPlan* plan) {
   static const struct { int bk_cap; bool halo; } kTries[] = {{128, true}, {64, true}, {32, true}, {128, false}, {64, false}};
   const char* why;
   for (const auto& t : kTries)
-    if ((t.halo || is_plain(a.d) || im2col_open(a.d, &why)) && plan_tiles(a, splits, t.bk_cap, t.halo, plan)) return true;
+    if ((t.halo || is_plain(a.d) || im2col_open(a.d, &why)) && plan_tiles(a, splits, t.bk_cap, t.halo, true, plan)) return true;
   return false;
 }
 
@@ -708,6 +837,13 @@ bool umma_describe(const ConvArgs& a, q8_conv_plan* out) {
   return true;
 }
 
+int umma_row_buffers(const ConvArgs& a) {
+  UmmaPlan plan;
+  if (umma_splits(a) > 1 || !plan_conv(a, 1, &plan)) return 0;
+  const UmmaParams& p = plan.p;
+  return (p.cta2 ? plan.G >> p.pair_shift : plan.G) * p.nbuf;
+}
+
 int launch_conv_umma(const ConvArgs& a) {
   const int splits = a.workspace && aligned16(a.workspace) ? split_parts(a) : 1;
   if (splits > 1 && a.workspace_bytes >= (size_t)splits * (size_t)a.M * a.d.K * sizeof(int)) {
@@ -719,12 +855,44 @@ int launch_conv_umma(const ConvArgs& a) {
 }
 
 namespace {
-bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, UmmaPlan* plan) {
+// Whether the 8-bit rows of a layer go through tile buffers, `two` of which fit per epilogue group or else one.
+//
+// Without them a warp's access touches 32 rows a pitch apart, which keeps the load/store unit busy in proportion to the bytes
+// of the rows; with them the copy engine moves whole lines, at the price of two more hand-offs at the end of a CTA and of
+// shared memory.  So buffers are for CTAs with many tiles, wide ones and short reductions, where rows and not operands are
+// the launch, more so with a residual, whose bytes count again.  Inputs not in L2, buffers against none (us):
+//   1x1 64->256 at 56x56 with a residual: batch 8 (2.6 tiles a CTA) 8.1 / 7.9, 16 (5.3) 10.9 / 12.9, 32 16.0 / 21.3, 64 25.9 / 39.4;
+//     without one: batch 16 8.4 / 8.4, 32 11.5 / 12.0, 64 18.1 / 20.3; 32 columns never gain (32->32 at 112x112, batch 64 24.7 /
+//     22.6; 256->32 at 56x56 with a residual 14.2 / 13.5);
+//   room for one buffer per group only: 1x1 256->256 at 56x56, batch 64 27.4 / 23.0 (too few operand stages are left), with a
+//     residual 31.7 / 43.4; 128->512 at 28x28 with one 19.2 / 21.4, without 12.6 / 12.6;
+//   halo tiles: 3x3 64->64 at 56x56, batch 64 12.3 / 13.3, batch 32 9.1 / 8.7; 32->96 at 112x112 with a residual, batch 8 (6 tiles a
+//     CTA) 12.3 / 11.1, 64 46.3 / 55.7; pairs at 75x75, batch 32 128->192 32.2 / 34.5, 128->256 40.1 / 38.9;
+//   tiles shared by all groups: 1x1 128->512 at 28x28, batch 8 with a residual 6.3 / 7.1, without 5.5 / 5.6.  They take none all
+//     the same: a launch of another kernel function than the one before it starts slower, and in ResNet-50 at batch 16 that
+//     costs more than it gives (402 -> 410 us; batch 32 501 -> 508).  The other lines lie where the networks gain or stay: SSD-300
+//     at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64.
+// Over 2131 layers the rule is on average 3.0 % below no buffers at all (34 % at best).
+bool buffered(const ConvArgs& a, const UmmaParams& p, bool two) {
+  const bool residual = a.residual != nullptr, plain = p.a_mode == kAPlain, wide = a.ldc % 32 == 0 && a.c_off % 32 == 0;
+  const int reduction = a.d.R * a.d.S * a.d.C, ctas = p.cta2 ? sm_count() / 2 : sm_count();
+  const long long items = (long long)p.m_tiles * p.n_tiles;
+  auto more_than = [&](int per_cta) { return items > (long long)per_cta * ctas; };
+  if (p.splits > 1 || p.epi_split) return false;
+  const bool broad = p.bn > 128 && p.bn < 256;
+  if (p.bn < 64 || reduction > (residual || broad ? 1152 : 864)) return false;
+  if (residual) return more_than(plain || p.n_tiles > 1 || p.bn > 128 ? 4 : 8);
+  if (p.bn < 96) return !plain && two && more_than(12);
+  if (!plain) return more_than(two || (broad && p.cta2) ? 8 : 12);
+  return ((two || reduction <= 128) && more_than(12)) || (!wide && reduction <= 288 && more_than(8));  // (!wide: twice the accesses)
+}
+
+bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, bool allow_bufs, UmmaPlan* plan) {
   const q8_conv_desc& d = a.d;
   const bool out8 = d.y_type == Q8_U8 || d.y_type == Q8_S8;
   int res_mode = kResNone;
   if (a.residual) res_mode = (d.K % 16 == 0 && aligned16(a.residual)) ? kResVec : (out8 ? kResRows : kResGlobal);
-  // 8-bit rows that TMA cannot address are moved by the epilogue warps, in both directions if in one
+  // 8-bit rows that 16-byte accesses cannot address are moved by the epilogue warps in words, in both directions if in one
   const bool rows = out8 && (rows_off_tma(a) || res_mode == kResRows);
   if (rows && a.residual) res_mode = kResRows;
   UmmaParams& p = plan->p;
@@ -810,7 +978,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   p.b_tile_bytes = (unsigned)(BN * BK);
   p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
 
-  // ---- shared memory plan: [resident weights] [A stages] [weight ring] [tile buffers of moved rows] [bias, scale]
+  // ---- shared memory plan: [resident weights] [A stages] [weight ring] [8-bit tile buffers] [bias, scale]
   // Launches with at most two work items per CTA cannot keep several groups busy on different tiles: there all
   // four groups share every tile, each taking a quarter of its columns (any tile width, both accumulators).
   {
@@ -862,6 +1030,8 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
     }
   }
+  const bool use_bufs = allow_bufs && out8 && !rows && tune_env("Q8_BUFS", buffered(a, p, true) || buffered(a, p, false), 0, 1);
+  const unsigned teams = (unsigned)(p.cta2 ? G >> p.pair_shift : G);
   const unsigned row_bytes = rows ? (unsigned)(p.epi_split ? 1 : G) * p.tile8_bytes : 0u;
   p.b_T = 1;
   p.b_chunks = p.taps;
@@ -876,8 +1046,8 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
     if (p.b_mode == kBRing && p.b_tile_bytes % (8u * BK) == 0 && (p.nacc >= 4 || p.cta2)) {
       // Weight ring stages of several filter taps, one TMA operation each (the copy engine spends ~600 cycles
       // per operation whatever its size): as many taps as fit in about 48 KiB while two such stages fit beside
-      // two activation stages and one tile buffer per epilogue group, spread evenly over a channel block.
-      const unsigned fixed = bres_bytes + row_bytes + 2u * p.a_stage_bytes;
+      // two activation stages and the tile buffers, spread evenly over a channel block.
+      const unsigned fixed = bres_bytes + row_bytes + (use_bufs ? teams * p.tile8_bytes : 0u) + 2u * p.a_stage_bytes;
       const unsigned avail = budget > fixed ? budget - fixed : 0u;
       int T = (int)(48u * 1024u / p.b_tile_bytes);
       if (T > (int)(avail / (2u * p.b_tile_bytes))) T = (int)(avail / (2u * p.b_tile_bytes));
@@ -900,8 +1070,17 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
     p.a_stage_bytes = (unsigned)p.kb * unit;
     min_pipe = 2u * p.a_stage_bytes;
   }
-  if (budget < bres_bytes + row_bytes + min_pipe) return false;
-  unsigned rest = budget - bres_bytes - row_bytes;
+  p.nbuf = 0;
+  if (use_bufs) {
+    // two buffers per group (team) when that still leaves a comfortable pipeline
+    const bool fit = budget >= bres_bytes + teams * p.tile8_bytes + min_pipe;
+    const bool two = budget >= bres_bytes + 2u * teams * p.tile8_bytes + 2u * min_pipe && 2 * teams <= (unsigned)kMaxSlots;
+    if (!fit || !tune_env("Q8_BUFS", buffered(a, p, two), 0, 1)) return plan_tiles(a, splits, bk_cap, allow_halo, false, plan);
+    p.nbuf = two ? 2 : 1;
+  }
+  const unsigned buf_bytes = row_bytes + teams * (unsigned)p.nbuf * p.tile8_bytes;
+  if (budget < bres_bytes + buf_bytes + min_pipe) return false;
+  unsigned rest = budget - bres_bytes - buf_bytes;
   p.b_stages = 0;
   if (p.b_mode == kBRing) {
     int bst = (int)((rest - 2u * p.a_stage_bytes) / p.b_sub_bytes);
@@ -915,7 +1094,7 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, Umma
   p.off_a = bres_bytes;
   p.off_bring = p.off_a + (unsigned)p.stages * p.a_stage_bytes;
   p.off_bufs = p.off_bring + (unsigned)p.b_stages * p.b_sub_bytes;
-  p.off_chan = p.off_bufs + row_bytes;
+  p.off_chan = p.off_bufs + buf_bytes;
   size_t dyn = 1024u + p.off_chan + chan_bytes;
   if (dyn > (size_t)(kSmemLimit - kStaticSmemReserve)) return false;
   // at least 120 KiB so that one CTA owns an SM and with it the whole TMEM
@@ -999,6 +1178,37 @@ int launch_planned(const ConvArgs& a, int splits) {
   }
   if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: weight tensor map rejected (CUresult %d)", (int)cr);
 
+  // 8-bit tiles through buffers: [M][channels] matrices, or for halo tiles (channels, Q, P, N) tensors whose TH x TW box
+  // lands as TH*TW dense rows.  The output map ends at the last channel this layer owns, a multiple of 16 (stores are
+  // clipped in units of 16 bytes), so the store clips ragged Cout tiles and never touches a neighbouring slice of a
+  // concatenated tensor.
+  RowMaps<true> maps;
+  memset(&maps, 0, sizeof(maps));
+  if (p.nbuf) {
+    const int pw = 1 << p.pw_shift;
+    auto encode_rows = [&](CUtensorMap* tm, void* ptr, int channels, int ld, CUtensorMapL2promotion promo) -> CUresult {
+      if (p.a_mode == kAHalo) {
+        cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)a.Q, (cuuint64_t)a.P, (cuuint64_t)d.N};
+        cuuint64_t strides[3] = {(cuuint64_t)ld, (cuuint64_t)a.Q * ld, (cuuint64_t)a.P * a.Q * ld};
+        cuuint32_t box[4] = {(cuuint32_t)pw, (cuuint32_t)ht.tw, (cuuint32_t)ht.th, 1};
+        return fn.tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, ptr, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        swizzle_for_bytes(pw), promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      }
+      cuuint64_t dims[2] = {(cuuint64_t)channels, (cuuint64_t)a.M};
+      cuuint64_t strides[1] = {(cuuint64_t)ld};
+      cuuint32_t box[2] = {(cuuint32_t)pw, (cuuint32_t)kBM};
+      return fn.tiled(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, ptr, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      swizzle_for_bytes(pw), promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    if (a.residual) {
+      cr = encode_rows(&maps.res, const_cast<void*>(a.residual), d.K, d.K, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+      if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: residual tensor map rejected (CUresult %d)", (int)cr);
+    }
+    cr = encode_rows(&maps.y, a.y, a.c_off + d.K, a.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
+    if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: output tensor map rejected (CUresult %d)", (int)cr);
+    p.res_tx_bytes = (unsigned)BN * (p.a_mode == kAHalo ? (unsigned)(ht.tw * ht.th) : (unsigned)kBM);
+  }
+
   // instruction descriptor: D = s32 (2 << 4); A format at bit 7 (0 = u8, 1 = s8); B = s8 at bit 10;
   // both operands K-major; N/8 at bit 17; M/16 at bit 24.
   p.idesc = (2u << 4) | ((d.x_type == Q8_S8 ? 1u : 0u) << 7) | (1u << 10) | ((unsigned)(BN >> 3) << 17) |
@@ -1032,15 +1242,17 @@ int launch_planned(const ConvArgs& a, int splits) {
     grid = 2 * (int)(tiles < pairs ? tiles : pairs);
   }
   if (p.cta2) {
-    // planned only for 8-bit outputs, residual by TMA or none.  These are the large 3x3 layers, which seldom
-    // take a residual: their kernels keep that choice at compile time.
+    // planned only for 8-bit outputs on the 16-byte grid.  These are the large 3x3 layers, which seldom take a
+    // residual: without tile buffers their kernels keep that choice at compile time.
 #define Q8_PAIR_LAUNCH(GG, OUT, RES)                                                                                      \
   do {                                                                                                                   \
-    if (p.scale_count == 1) return launch_variant<GG, OUT, RES, true, true>(tmA, tmB, p, dyn, grid, a.stream); \
-    return launch_variant<GG, OUT, RES, true, false>(tmA, tmB, p, dyn, grid, a.stream);                      \
+    if (p.scale_count == 1) return launch_variant<GG, OUT, RES, true, true>(tmA, tmB, maps, p, dyn, grid, a.stream); \
+    return launch_variant<GG, OUT, RES, true, false>(tmA, tmB, maps, p, dyn, grid, a.stream);                      \
   } while (0)
 #define Q8_PAIR(GG)                                                                                                      \
   do {                                                                                                                   \
+    if (p.nbuf && d.y_type == Q8_U8) Q8_PAIR_LAUNCH(GG, Q8_U8, kResTma);                                                 \
+    if (p.nbuf) Q8_PAIR_LAUNCH(GG, Q8_S8, kResTma);                                                                      \
     if (d.y_type == Q8_U8 && res_mode == kResVec) Q8_PAIR_LAUNCH(GG, Q8_U8, kResVec);                                    \
     if (d.y_type == Q8_U8) Q8_PAIR_LAUNCH(GG, Q8_U8, kResNone);                                                          \
     if (res_mode == kResVec) Q8_PAIR_LAUNCH(GG, Q8_S8, kResVec);                                                         \
@@ -1050,8 +1262,8 @@ int launch_planned(const ConvArgs& a, int splits) {
 #undef Q8_PAIR
 #undef Q8_PAIR_LAUNCH
   }
-  if (G == 2) return launch_groups<2>(tmA, tmB, p, rows, dyn, grid, a.stream);
-  return launch_groups<4>(tmA, tmB, p, rows, dyn, grid, a.stream);
+  if (G == 2) return launch_groups<2>(tmA, tmB, maps, p, rows, dyn, grid, a.stream);
+  return launch_groups<4>(tmA, tmB, maps, p, rows, dyn, grid, a.stream);
 }
 }  // namespace
 

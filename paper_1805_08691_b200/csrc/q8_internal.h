@@ -63,6 +63,7 @@ bool rows_off_tma(const ConvArgs& a);
 // Whether one of its tile shapes fits the layer, and which (decided without a device).
 bool umma_fits(const ConvArgs& a);
 bool umma_describe(const ConvArgs& a, q8_conv_plan* out);
+int umma_row_buffers(const ConvArgs& a);  // tile buffers of a CTA that TMA fills and empties; 0: the epilogue moves its rows itself
 // kPlanNoFit (nothing recorded as an error) where none does, else a q8_status.
 constexpr int kPlanNoFit = -1000;
 int launch_conv_umma(const ConvArgs& a);
@@ -84,6 +85,7 @@ int launch_conv_packed(const ConvArgs& a);
 // A stride-1 convolution followed by a 1x1 convolution over its output, in one launch (q8_conv_fused.cu).
 // Descriptors validated by the caller; `why` names the first reason a pair cannot run fused.
 bool fused_pair_eligible(const q8_conv_desc& d1, const q8_conv_desc& d2, const char** why);
+int fused_row_buffers(const q8_conv_desc& d1, const q8_conv_desc& d2, bool residual);  // of a block; 0: rows by the epilogue
 int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void* x, const int8_t* w1, const int32_t* bias1,
                       const float* scale1, const int8_t* w2, const int32_t* bias2, const float* scale2, const void* residual,
                       float residual_scale, void* y, cudaStream_t stream);

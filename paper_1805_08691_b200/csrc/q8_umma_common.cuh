@@ -23,6 +23,7 @@ constexpr int kGroupThreads = 128;      // one epilogue group
 constexpr int kMaxStages = 8;           // A stages
 constexpr int kMaxBStages = 8;          // weight ring
 constexpr int kMaxAcc = 4;
+constexpr int kMaxSlots = 8;            // 8-bit tile buffers over all groups
 constexpr int kMaxTaps = 64;            // halo mode: filter taps (one TMA box holds all taps of resident weights)
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 constexpr int kSmemLimit = 232448;                           // 227 KiB opt-in maximum per CTA
@@ -32,10 +33,11 @@ enum StatusBits : unsigned int {
   kTimeoutProducer = 1u,
   kTimeoutMma = 2u,
   kTimeoutEpilogue = 4u,
+  kTimeoutResidual = 8u,
   kTimeoutStore = 16u,
 };
 
-enum ResMode : int { kResNone = 0, kResVec = 1, kResGlobal = 2, kResRows = 3 };
+enum ResMode : int { kResNone = 0, kResVec = 1, kResGlobal = 2, kResRows = 3, kResTma = 4 };
 enum AMode : int { kAPlain = 0, kAIm2col = 1, kAHalo = 2 };
 enum BMode : int { kBStage = 0, kBResident = 1, kBRing = 2 };
 
@@ -86,6 +88,8 @@ struct UmmaParams {
   int b_T, b_chunks;         // weight ring: filter taps per ring stage (one TMA operation), stages per channel block
   unsigned int a_stage_bytes;
   unsigned int tile8_bytes;
+  int nbuf;                  // 8-bit tile buffers per epilogue group or team that TMA fills and empties (0: none)
+  unsigned int res_tx_bytes; // bytes one residual tile load delivers
   unsigned int off_a, off_bring, off_bufs, off_chan;  // from the 1 KiB aligned base; resident weights at 0
   int pw_shift, pmask, panels;  // 8-bit tiles live in smem as panels of 2^pw_shift bytes per row
   int k_pad;                 // n_tiles * bn channels of bias/scale staged in smem
@@ -281,6 +285,11 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t sr
                ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
                : "memory");
 }
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(map), "r"(src), "r"(c0), "r"(c1)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
@@ -459,7 +468,7 @@ struct EpiTile {
   const int* s_bias;       // smem, k_pad entries
   const float* s_scale;    // smem, k_pad entries
   float scale;             // the first of them: the multiplier of every channel when there is one per tensor
-  unsigned char* buf;      // 8-bit tile in shared memory (kTile, kResRows)
+  unsigned char* buf;      // 8-bit tile in shared memory (kTile)
   unsigned char* yrow;     // this thread's row of the 8-bit output, at the tile's first channel
   const unsigned char* rrow;  // ... of the residual
   bool wide, res_wide;     // pairs of chunks of those rows start on 32-byte lines
@@ -510,8 +519,9 @@ __device__ __forceinline__ void epi_row_setup(const UmmaParams& p, EpiTile& t) {
 }
 
 // One 16-column chunk of one accumulator row.  kOut: Q8_U8, Q8_S8, Q8_S32 or Q8_F32.  kRes: kResNone, kResVec
-// (a residual in `rv` if p.res_mode says so, else none: decided at run time), kResGlobal (fp32 outputs) or
-// kResRows (8-bit rows that 16-byte accesses cannot address: the warps move them through the tile buffer).  Fewer
+// (a residual in `rv` if p.res_mode says so, else none: decided at run time), kResGlobal (fp32 outputs), kResRows
+// (8-bit rows that 16-byte accesses cannot address: the warps move them through a tile buffer) or kResTma (TMA moves them
+// through one).  Fewer
 // distinct kernels matter more than one uniform branch per chunk: a launch of another kernel function than
 // the one before it starts with cold instruction caches, which costs a layer of a network 2 to 6 us, so the
 // layers with and without a residual sum share their kernels.  (One straight-line copy of the rows' code per case runs 30 %
@@ -566,7 +576,7 @@ __device__ __forceinline__ uint4 epilogue_chunk(const UmmaParams& p, const EpiTi
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) unpack_f2(v2[j], v[2 * j], v[2 * j + 1]);
-  if (kRes == kResGlobal || ((kRes == kResVec || kRes == kResRows) && p.res_mode != kResNone)) {
+  if (kRes == kResGlobal || ((kRes == kResVec || kRes == kResRows || kRes == kResTma) && p.res_mode != kResNone)) {
     unsigned int rw[4] = {rv.x, rv.y, rv.z, rv.w};
     if (kRes == kResGlobal && t.row_ok && nb < p.K) {
       const int valid = min(16, p.K - nb);
@@ -656,7 +666,8 @@ __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile&
     return;
   }
   auto given = [&](int ch, const uint4& v) {  // residual bytes of a row moved through the tile buffer
-    if (kRes == kResRows && p.res_mode != kResNone) return *reinterpret_cast<const uint4*>(t.buf + tile_offset(p, t, ch));
+    // (a buffer that TMA fills holds the residual or nothing: its bytes are read ahead of the uniform branch on which)
+    if (kRes == kResTma || (kRes == kResRows && p.res_mode != kResNone)) return *reinterpret_cast<const uint4*>(t.buf + tile_offset(p, t, ch));
     return v;
   };
   tmem_ld_16(taddr + ch0 * 16, ra);
@@ -691,7 +702,7 @@ __device__ __forceinline__ void epilogue_row(const UmmaParams& p, const EpiTile&
     if (kRes == kResVec) r = next;
   }
 }
-// 8-bit tensors whose rows TMA cannot address (channel counts, pitches, offsets or pointers off the 16-byte grid): a warp
+// 8-bit tensors whose rows 16-byte accesses cannot address (channel counts, pitches, offsets or pointers off that grid): a warp
 // moves the rows of its 32 accumulator rows between global memory and the group's tile buffer itself.  Neighbouring lanes
 // take neighbouring words of a row, `lpr` lanes a row (a power of two that covers it, so that narrow rows share a pass);
 // the global words are aligned ones, the buffer's follow from two of them by a funnel shift.  Only words that hold a byte

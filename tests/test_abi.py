@@ -196,3 +196,19 @@ def test_marshalled_calls_refuse_what_they_cannot_pass():
     with pytest.raises(TypeError, match="^loc: expected a CUDA fp32 tensor"):
         q8.q8_detection_output([(torch.zeros(1, 4, 4), torch.zeros(1, 4, 3), 1)], torch.zeros(4, 4), (0.1,) * 4, 3,
                                workspace=torch.zeros(1, dtype=torch.uint8), out=torch.zeros(1), counts=torch.zeros(1))
+
+
+@pytest.mark.parametrize("N,HW,C,K,R,residual,buffers", [
+    (64, 56, 64, 256, 1, True, 8), (64, 56, 64, 256, 1, False, 8),     # the expanding layers of early residual blocks
+    (64, 28, 128, 512, 1, True, 4), (64, 14, 256, 1024, 1, True, 4),   # weights resident: room for one a group
+    (32, 150, 64, 128, 3, False, 4), (64, 56, 64, 64, 3, False, 8),
+    (8, 28, 128, 512, 1, True, 0), (8, 56, 64, 256, 1, True, 0),       # few tiles a block
+    (16, 56, 64, 256, 1, False, 0), (64, 56, 256, 256, 1, False, 0),   # no residual: the same, or operands need the memory
+    (32, 75, 256, 256, 3, False, 0), (64, 56, 256, 32, 1, True, 0),    # long reductions, narrow tiles
+], ids=str)
+def test_layers_bound_by_their_rows_take_tile_buffers(N, HW, C, K, R, residual, buffers):
+    d = q8.make_conv_desc(N, HW, HW, C, K, R, R, (1, 1), (R // 2, R // 2), relu=True)
+    assert q8.q8_conv2d_query_row_buffers(d, None, residual) == buffers
+    for y_type in (2, 3):   # 32-bit outputs are stored by the epilogue
+        d.y_type = y_type
+        assert q8.q8_conv2d_query_row_buffers(d, None, residual and y_type == 3) == 0
