@@ -22,11 +22,19 @@
 // Every hand-off is an mbarrier with a bounded wait (status word + drain on expiry), as in q8_conv_umma.cu.
 //
 // Layer 2's bytes, two ways.  With tile buffers, warp 3 brings residual rows in and sends output rows out by TMA as whole lines;
-// without, the epilogue loads and stores its rows itself, which saves the hand-offs.  Buffers pay where a CTA has many items and
-// there is room for two per E2 group, so that the copies run behind the arithmetic; with one per group they never won.
-// Measured with a residual, per launch, inputs not in L2, buffers against none:
-//   56x56 64->64->256   batch 4: 8.1 / 7.8 us, 8 (3 items per CTA): 9.7 / 9.8, 16 (6): 13.0 / 15.0, 32: 19.4 / 23.7, 64: 31.0 / 41.2;
-//   28x28 128->128->512 (room for one per group)  batch 1: 8.5 / 8.3, 8: 10.8 / 9.9, 16: 15.4 / 14.0, 32: 20.5 / 19.2, 64: 28.3 / 28.4.
+// without, the epilogue loads and stores its rows itself, which saves the hand-offs.  Buffers pay where a block has many items
+// (tiles of 128 columns of layer 2) and its rows, not layer 1, are the work; row_buffers() draws the line.  Per launch, inputs
+// not in L2, buffers against none (us):
+//   two buffers per E2 group, 56x56 64->64->256: batch 4 8.1 / 7.9, 8 (3 items a block) 9.9 / 10.3, 16 (6) 13.1 / 15.1, 32 19.5 /
+//     24.1, 64 31.1 / 41.8; without a residual 7.3 / 6.9, 8.8 / 8.6, 10.9 / 11.0, 15.4 / 16.2, 24.6 / 26.9; 64->64->128 (one item of
+//     layer 2 per tile of layer 1) with one, batch 16 10.8 / 10.8, 32 16.0 / 15.5, 64 24.9 / 24.7;
+//   one per group, layer 1's weights resident, 56x56 with a residual: 128->64->256 batch 16 14.5 / 16.2, 64 37.7 / 44.4, 64->128->512
+//     batch 8 (6) 15.4 / 16.3, 64 66.2 / 79.2; without one 128->64->256 batch 64 29.5 / 29.1, 64->128->256 35.8 / 38.3;
+//   one per group, weights streamed, with a residual: 256->64->256 at 56x56, batch 64 54.0 / 53.8, 256->64->512 71.0 / 84.0;
+//     128->128->512 at 28x28, batch 64 (12 items) within 1 %, but in ResNet-50, its inputs in L2, 679 us without and 685 with them.
+// Over 1532 pairs the rule is on average 0.4 % off the better form.
+#include <climits>
+
 #include "q8_umma_common.cuh"
 
 namespace q8 {
@@ -37,8 +45,7 @@ constexpr int kFE2Groups = 3;
 constexpr int kFThreads = (kFCtrlWarps + 4 + 4 * kFE2Groups) * 32;  // 640
 constexpr int kFAcc2Cols = 128;                                      // columns of one layer-2 accumulator
 constexpr int kFMaxTb = 4;                                           // slots of the intermediate tile ring
-constexpr int kFSlots = 6;                                           // layer-2 tile buffers, two per E2 group
-constexpr int kFBufMinItems = 4;                                     // items per CTA above which buffers are used
+constexpr int kFSlots = 6;                                           // layer-2 tile buffers at most, two per E2 group
 
 struct FusedParams {
   UmmaParams l1;  // layer 1: halo tiles, one tile of columns (bn = Cout1), one MMA warp; its 8-bit tile fields
@@ -49,7 +56,7 @@ struct FusedParams {
   unsigned int off_w2, off_tb;   // resident W2 tiles, T ring (from the 1 KiB aligned base)
   unsigned int tb_bytes;         // 128 * Cout1
   unsigned int off_chan2;        // bias2 / scale2 staging
-  int nslots;                    // layer-2 tile buffers (6; 0: the epilogue moves the rows itself)
+  int nslots;                    // layer-2 tile buffers (3 or 6; 0: the epilogue moves the rows itself)
   unsigned int res_tx_bytes;     // bytes one residual tile load delivers
   int acc1_col;                  // first TMEM column of the layer-1 accumulators
 };
@@ -306,6 +313,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       for (uint32_t s = 0; s < nslots && !ld.done(); ++s) ld.next(h, chunks);
     uint32_t slot = 0, spar = 0;
     int prev_slot = -1;
+    const bool one_each = p.nslots == kFE2Groups;
     bool ok = true;
     for (; !st.done(); st.next(h, chunks)) {
       if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
@@ -314,12 +322,18 @@ __global__ void __launch_bounds__(kFThreads, 1)
         for (int pn = 0, c = q.c_off + st.j * q.bn; pn < q.panels; ++pn, c += pw, src += panel_bytes)
           tma_store_4d(&tmY, src, c, st.ti.qt * h.tw, st.ti.pt * h.th, st.ti.img);
         bulk_commit();
-        // A buffer takes its next residual once its store has read it; the load is left until the next store, which
-        // keeps this warp free.
-        bulk_wait_read<1>();
-        if (prev_slot >= 0 && !ld.done()) fill_buffer(ld, (uint32_t)prev_slot);
+        // A buffer takes its next residual once its store has read it.  With one buffer per group the group waits for
+        // that residual, so the load goes out at once (28x28 pair, batch 64: 26.4 -> 25.7 us); with two it is left until
+        // the next store, which keeps this warp free (56x56 pair: 31.0 against 32.5 us).
+        if (one_each) {
+          bulk_wait_read<0>();
+          if (!ld.done()) fill_buffer(ld, slot);
+        } else {
+          bulk_wait_read<1>();
+          if (prev_slot >= 0 && !ld.done()) fill_buffer(ld, (uint32_t)prev_slot);
+        }
       }
-      if (prev_slot >= 0 && !ld.done()) ld.next(h, chunks);
+      if ((one_each || prev_slot >= 0) && !ld.done()) ld.next(h, chunks);
       prev_slot = (int)slot;
       if (++slot == nslots) { slot = 0; spar ^= 1u; }
     }
@@ -432,7 +446,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       tcgen05_fence_after();
       t.n0 = j * q.bn;
       t.buf = base_ptr + q.off_bufs + (size_t)slot * q.tile8_bytes;
-      epilogue_row<kOut2, kResRows, false, kUniform, true>(q, t, taddr, acce, lane, 0, nchunk, ResPair{});
+      epilogue_row<kOut2, kResTma, false, kUniform, true>(q, t, taddr, acce, lane, 0, nchunk, ResPair{});
       fence_proxy_async_smem();
       mbar_arrive(ready0 + slot * 8u);
       apar ^= 1u;
@@ -494,7 +508,20 @@ struct FusedPlan {
   size_t dyn;
 };
 
-bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, const char** why) {
+// Layer-2 tile buffers of a block: kFSlots where `two` fit per E2 group, else one each, or none (see the head of the file).
+int row_buffers(const UmmaParams& a, const UmmaParams& b, bool residual, bool two) {
+  const long long items = (long long)a.m_tiles * b.n_tiles;
+  const bool streamed = a.b_mode != kBResident, chunks = b.n_tiles > 1;
+  int above = INT_MAX;  // items per block
+  const int steps = a.k_iters * a.ksteps * a.bn / b.n_tiles;  // layer-1 weights streamed per item, in 32 bytes
+  if (streamed) { if (residual && steps <= 1152) above = steps > 576 && a.bn == 128 ? 16 : 8; }
+  else if (residual) above = chunks || a.bn == 128 ? 4 : 8;
+  else if (two && chunks) above = 4;
+  else if (a.bn == 128) above = 6;
+  return tune_env("Q8_FBUFS", items > (long long)above * sm_count(), 0, 1) ? (two ? kFSlots : kFE2Groups) : 0;
+}
+
+bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, bool residual, FusedPlan* out, const char** why) {
   const char* dummy;
   if (!why) why = &dummy;
   const int P = conv_out_extent(d1.H, d1.pad_h, d1.dil_h, d1.R, d1.stride_h), Q = conv_out_extent(d1.W, d1.pad_w, d1.dil_w, d1.S, d1.stride_w);
@@ -607,16 +634,14 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
   }
   const unsigned need_min = w1_bytes + w2_bytes + 2u * a.a_stage_bytes + ring_min + 1u * pl.p.tb_bytes + 3u * b.tile8_bytes;
   if (budget < need_min) { *why = "the layer pair does not fit in shared memory"; return false; }
-  unsigned rest = budget - need_min;
+  unsigned rest = budget - need_min;  // beside three tile buffers
+  const unsigned after_tb = rest >= pl.p.tb_bytes ? rest - pl.p.tb_bytes : rest;
+  const bool two = after_tb >= (unsigned)(kFSlots - kFE2Groups) * b.tile8_bytes + a.a_stage_bytes;
+  pl.p.nslots = row_buffers(a, b, residual, two);
+  if (!pl.p.nslots) rest += (unsigned)kFE2Groups * b.tile8_bytes;
   pl.p.ntb = 1;
-  pl.p.nslots = 0;
-  rest += 3u * b.tile8_bytes;
   if (rest >= pl.p.tb_bytes) { pl.p.ntb = 2; rest -= pl.p.tb_bytes; }
-  if ((long long)a.m_tiles * b.n_tiles > (long long)kFBufMinItems * sm_count() &&
-      rest >= (unsigned)kFSlots * b.tile8_bytes + a.a_stage_bytes) {  // where this line lies: see the head of the file
-    pl.p.nslots = kFSlots;
-    rest -= (unsigned)kFSlots * b.tile8_bytes;
-  }
+  if (pl.p.nslots == kFSlots) rest -= (unsigned)(kFSlots - kFE2Groups) * b.tile8_bytes;
   a.b_stages = 0;
   if (!resident) {
     a.b_stages = 2;
@@ -651,12 +676,12 @@ bool plan_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, FusedPlan* out, 
 }  // namespace
 
 bool fused_pair_eligible(const q8_conv_desc& d1, const q8_conv_desc& d2, const char** why) {
-  return plan_fused(d1, d2, nullptr, why);
+  return plan_fused(d1, d2, false, nullptr, why);
 }
 
-int fused_row_buffers(const q8_conv_desc& d1, const q8_conv_desc& d2, bool) {
+int fused_row_buffers(const q8_conv_desc& d1, const q8_conv_desc& d2, bool residual) {
   FusedPlan pl;
-  return plan_fused(d1, d2, &pl, nullptr) ? pl.p.nslots : 0;
+  return plan_fused(d1, d2, residual, &pl, nullptr) ? pl.p.nslots : 0;
 }
 
 int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void* x, const int8_t* w1, const int32_t* bias1,
@@ -668,7 +693,7 @@ int launch_conv_fused(const q8_conv_desc& d1, const q8_conv_desc& d2, const void
   if (!status) return fail(Q8_ERR_CUDA, "conv_fused: status word not available");
   FusedPlan pl;
   const char* why = "";
-  if (!plan_fused(d1, d2, &pl, &why)) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d_then_1x1: %s", why);
+  if (!plan_fused(d1, d2, residual != nullptr, &pl, &why)) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d_then_1x1: %s", why);
   if (residual && !aligned16(residual)) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d_then_1x1: residual not 16-byte aligned");
   FusedParams& p = pl.p;
   const HaloTile& ht = pl.ht;

@@ -212,3 +212,15 @@ def test_layers_bound_by_their_rows_take_tile_buffers(N, HW, C, K, R, residual, 
     for y_type in (2, 3):   # 32-bit outputs are stored by the epilogue
         d.y_type = y_type
         assert q8.q8_conv2d_query_row_buffers(d, None, residual and y_type == 3) == 0
+
+
+@pytest.mark.parametrize("N,HW,C1,K1,K2,residual,buffers", [
+    (64, 56, 64, 64, 256, True, 6), (64, 56, 64, 64, 256, False, 6), (4, 56, 64, 64, 256, True, 0),
+    (64, 56, 128, 64, 256, True, 3), (32, 56, 64, 128, 512, True, 3),      # one a group, weights of the first layer resident
+    (64, 56, 128, 128, 512, True, 3), (64, 28, 128, 128, 512, True, 0),    # streamed
+    (64, 56, 128, 64, 256, False, 0), (64, 56, 64, 64, 128, False, 0),     # the first layer is most of the work
+], ids=str)
+def test_pairs_bound_by_their_rows_take_tile_buffers(N, HW, C1, K1, K2, residual, buffers):
+    d1 = q8.make_conv_desc(N, HW, HW, C1, K1, 3, 3, (1, 1), (1, 1), relu=True)
+    d2 = q8.make_conv_desc(N, HW, HW, K1, K2, 1, 1, relu=True)
+    assert q8.q8_conv2d_query_row_buffers(d1, d2, residual) == buffers

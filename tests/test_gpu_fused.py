@@ -134,3 +134,53 @@ def test_fused_pair_on_both_sides_of_the_buffer_rule(q8, N):
     acc = o.conv_acc(mid, w2.cpu().numpy(), None, (1, 1), (0, 0), (1, 1), threads=8)
     q8.q8_read_status()
     assert np.array_equal(y.cpu().numpy(), o.epilogue(acc, np.float32(2e-4), r.cpu().numpy(), 0.37, True, o.U8))
+
+
+BUFFERED = [
+    # name, H,W, C1, K1, dil, K2, x signed, type between, out type, residual, relu2, per channel, pitch - K2, offset, buffers, batches
+    ("two_a_group_ragged_edges", 37, 41, 64, 64, 1, 256, False, U8, U8, None, True, True, 0, 0, 6, 2),
+    ("two_a_group_ragged_chunk", 28, 28, 64, 64, 1, 192, False, U8, U8, "u8", True, False, 0, 0, 6, 2),
+    ("two_a_group_signed", 28, 28, 64, 64, 1, 256, True, S8, S8, "s8", False, True, 0, 0, 6, 2),
+    ("two_a_group_signed_between", 29, 27, 32, 32, 1, 256, True, S8, U8, "u8", True, False, 0, 0, 6, 2),
+    ("two_a_group_slice", 28, 28, 64, 64, 1, 256, False, U8, S8, "u8", False, False, 96, 32, 6, 2),
+    ("two_a_group_dilated", 40, 40, 64, 64, 2, 256, False, U8, U8, "u8", True, True, 16, 16, 6, 2),
+    ("one_a_group_no_residual", 28, 28, 64, 128, 1, 256, False, U8, U8, None, True, False, 0, 0, 3, 1),
+    ("one_a_group_one_chunk", 30, 31, 64, 128, 1, 112, False, U8, S8, "s8", True, True, 16, 0, 3, 1),
+    ("one_a_group_streamed_weights", 28, 28, 128, 128, 1, 512, False, U8, U8, "u8", True, True, 0, 0, 3, 1),
+]
+
+
+@pytest.mark.parametrize("case", BUFFERED, ids=[c[0] for c in BUFFERED])
+def test_fused_pair_through_tile_buffers(q8, case):
+    """The smallest batch whose blocks have enough items for tile buffers, or twice that, so that every buffer is used again."""
+    name, H, W, C1, K1, dil, K2, xs8, t_type, ytype, res, relu2, per_channel, extra, off, buffers, times = case
+    ldc = K2 + extra
+
+    def descs(N):
+        return (q8.make_conv_desc(N, H, W, C1, K1, 3, 3, (1, 1), (dil, dil), (dil, dil), S8 if xs8 else U8, U8, t_type, t_type == U8),
+                q8.make_conv_desc(N, H, W, K1, K2, 1, 1, (1, 1), (0, 0), (1, 1), t_type, S8 if res == "s8" else U8, ytype, relu2,
+                                  K2 if per_channel else 1, ldc, off))
+    N = next(n for n in range(1, 257) if q8.q8_conv2d_query_row_buffers(*descs(n), res is not None))
+    assert q8.q8_conv2d_query_row_buffers(*descs(N - 1 or 1), res is not None) == 0
+    N *= times
+    d1, d2 = descs(N)
+    assert q8.q8_conv2d_query_row_buffers(d1, d2, res is not None) == buffers
+    g = np.random.default_rng(sum(map(ord, name)))
+    x = g.integers(0, 256, (N, H, W, C1), dtype=np.uint8).view(np.int8 if xs8 else np.uint8)
+    w1, w2 = (g.integers(-128, 128, s).astype(np.int8) for s in ((K1, 3, 3, C1), (K2, 1, 1, K1)))
+    b1, b2 = (g.integers(-5000, 5000, k).astype(np.int32) for k in (K1, K2))
+    acc1 = o.conv_acc(x, w1, b1, (1, 1), (dil, dil), (dil, dil), threads=8)
+    s1 = np.float32(200.0 / max(1, np.abs(acc1).max()))
+    acc2 = o.conv_acc(o.epilogue(acc1, s1, None, 0.0, t_type == U8, OT[t_type]), w2, b2, (1, 1), (0, 0), (1, 1), threads=8)
+    s2 = (g.uniform(0.5, 1.5, K2 if per_channel else 1) * 150.0 / max(1, np.abs(acc2).max())).astype(np.float32)
+    resid = None if res is None else g.integers(0, 256, acc2.shape, dtype=np.uint8).view(np.int8 if res == "s8" else np.uint8)
+    rs = 0.37 if res else 0.0
+    want = o.epilogue(acc2, s2 if per_channel else s2[0], resid, rs, relu2, OT[ytype])
+    y = torch.full((N, H, W, ldc), 7, dtype=q8.TORCH_DTYPES[ytype], device="cuda")
+    args = (_cuda(x), _cuda(w1), _cuda(b1), torch.tensor([s1], device="cuda"), _cuda(w2), _cuda(b2), _cuda(s2))
+    for _ in range(2):   # twice: the second launch follows the first in the stream
+        q8.q8_conv2d_then_1x1(d1, d2, *args, None if resid is None else _cuda(resid), rs, y)
+    q8.q8_read_status()
+    got = y.cpu().numpy()
+    assert np.array_equal(got[..., off:off + K2], want)
+    assert (got[..., :off] == 7).all() and (got[..., off + K2:] == 7).all()
