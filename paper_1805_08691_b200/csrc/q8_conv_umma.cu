@@ -871,7 +871,8 @@ namespace {
 //   tiles shared by all groups: 1x1 128->512 at 28x28, batch 8 with a residual 6.3 / 7.1, without 5.5 / 5.6.  They take none all
 //     the same: a launch of another kernel function than the one before it starts slower, and in ResNet-50 at batch 16 that
 //     costs more than it gives (402 -> 410 us; batch 32 501 -> 508).  The other lines lie where the networks gain or stay: SSD-300
-//     at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64.
+//     at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64
+//     (matrices without a residual, taken from 12 tiles a CTA, still cost ResNet-50 at batch 40 551 -> 554 us).
 // Over 2131 layers the rule is on average 3.0 % below no buffers at all (34 % at best).
 bool buffered(const ConvArgs& a, const UmmaParams& p, bool two) {
   const bool residual = a.residual != nullptr, plain = p.a_mode == kAPlain, wide = a.ldc % 32 == 0 && a.c_off % 32 == 0;
@@ -884,7 +885,7 @@ bool buffered(const ConvArgs& a, const UmmaParams& p, bool two) {
   if (residual) return more_than(plain || p.n_tiles > 1 || p.bn > 128 ? 4 : 8);
   if (p.bn < 96) return !plain && two && more_than(12);
   if (!plain) return more_than(two || (broad && p.cta2) ? 8 : 12);
-  return ((two || reduction <= 128) && more_than(12)) || (!wide && reduction <= 288 && more_than(8));  // (!wide: twice the accesses)
+  return ((two || reduction <= 128) && more_than(16)) || (!wide && reduction <= 288 && more_than(8));  // (!wide: twice the accesses)
 }
 
 bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, bool allow_bufs, UmmaPlan* plan) {

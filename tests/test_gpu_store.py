@@ -61,7 +61,7 @@ def test_rows_in_global_memory_match_oracle(q8, case):
 
 BUFFERED = [
     # name, N,H,W,C,K,R,stride,pad, y type, residual, per channel, pitch - K, channel offset, tile width, CTA pair, buffers
-    ("matrix_no_residual", 35, 57, 57, 64, 256, 1, 1, 0, S8, None, False, 0, 0, 128, 0, 8),
+    ("matrix_no_residual", 47, 57, 57, 64, 256, 1, 1, 0, S8, None, False, 0, 0, 128, 0, 8),
     ("matrix_slice_s8_residual", 12, 57, 57, 64, 256, 1, 1, 0, S8, "s8", True, 48, 16, 128, 0, 8),
     ("matrix_one_a_group", 12, 57, 57, 256, 256, 1, 1, 0, U8, "u8", False, 0, 0, 128, 0, 4),
     ("ragged_columns_208", 25, 57, 57, 32, 208, 1, 1, 0, U8, "u8", True, 16, 0, 112, 0, 8),
