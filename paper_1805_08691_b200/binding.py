@@ -433,20 +433,16 @@ def q8_detection_output(sources, priors, variances, classes, background=0, conf_
     """sources: list of (loc, conf, boxes_per_cell) with loc [N, cells..., boxes * 4] and conf [N, cells...,
     boxes * classes] CUDA fp32 tensors, contiguous or slices of the last dimension of a wider tensor (a merged
     head).  priors: CUDA fp32 [P, 4].  Returns (rows [N, keep_top_k, 6], counts [N])."""
-    first = sources[0][0]
-    if workspace is None:
-        P = 0
-        for loc, _, b in sources:
-            cells = 1
-            for v in loc.shape[1:-1]:
-                cells *= int(v)
-            P += cells * int(b)
-        nbytes = q8_detection_output_workspace_bytes(int(first.shape[0]), P, classes, background, nms_top_k, keep_top_k)
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=first.device)
-    if out is None:
-        out = torch.empty((int(first.shape[0]), max(keep_top_k, 0), 6), dtype=torch.float32, device=first.device)
-    if counts is None:
-        counts = torch.empty(int(first.shape[0]), dtype=torch.int32, device=first.device)
+    if workspace is None or out is None or counts is None:
+        N, P = _native.detect_size(sources)
+        nbytes = q8_detection_output_workspace_bytes(N, P, classes, background, nms_top_k, keep_top_k)
+        dev = sources[0][0].device
+        if workspace is None:
+            workspace = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        if out is None:
+            out = torch.empty((N, keep_top_k, 6), dtype=torch.float32, device=dev)
+        if counts is None:
+            counts = torch.empty(N, dtype=torch.int32, device=dev)
     rc = _native.detect(sources, priors, variances, classes, background, conf_thresh, nms_thresh, nms_top_k, keep_top_k, workspace, out, counts)
     if rc:
         _check(rc)

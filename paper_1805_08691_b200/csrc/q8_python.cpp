@@ -9,6 +9,7 @@
 #include <torch/csrc/utils/object_ptr.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "q8.h"
 
@@ -194,44 +195,74 @@ bool cell_view(PyObject* o, const char* what, const float** p, int* stride, int*
   return true;
 }
 
-constexpr Py_ssize_t kMaxSources = 64;  // the library takes fewer and says so
+// The sources of a detection output, a sequence of (loc, conf, boxes per cell); what int() takes counts boxes.
+struct Sources {
+  std::vector<const float*> loc, conf;
+  std::vector<int> ls, cs, cells, boxes;
+  int64_t images = 0;
+  long long P = 0;   // boxes per image
+
+  bool parse(PyObject* sources) {
+    THPObjectPtr seq(PySequence_Fast(sources, "sources: expected a sequence"));
+    if (!seq) return false;
+    const Py_ssize_t k = PySequence_Fast_GET_SIZE(seq.get());
+    loc.resize(k); conf.resize(k);
+    ls.resize(k); cs.resize(k); cells.resize(k); boxes.resize(k);
+    for (Py_ssize_t i = 0; i < k; ++i) {
+      THPObjectPtr item(PySequence_Fast(PySequence_Fast_GET_ITEM(seq.get(), i), "sources: expected (loc, conf, boxes per cell)"));
+      if (!item) return false;
+      if (PySequence_Fast_GET_SIZE(item.get()) != 3) { PyErr_SetString(PyExc_ValueError, "sources: expected (loc, conf, boxes per cell)"); return false; }
+      PyObject** e = PySequence_Fast_ITEMS(item.get());
+      int ccells;
+      int64_t ni, nc;
+      if (!cell_view(e[0], "loc", &loc[i], &ls[i], &cells[i], &ni) || !cell_view(e[1], "conf", &conf[i], &cs[i], &ccells, &nc)) return false;
+      if (i == 0) images = ni;
+      if (ccells != cells[i] || nc != images || ni != images) {
+        PyErr_SetString(PyExc_ValueError, "loc and conf of a source must cover the same cells of the same images");
+        return false;
+      }
+      THPObjectPtr count(PyNumber_Long(e[2]));
+      if (!count || !number(count.get(), &boxes[i])) return false;
+      P += (long long)cells[i] * boxes[i];
+    }
+    return true;
+  }
+  int boxes_per_image() const { return (int)(P > 0x7fffffff ? 0x7fffffff : P); }
+};
+
+// (sources) -> (images, boxes per image)
+PyObject* py_detect_size(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (!count(n, 1)) return nullptr;
+  HANDLE_TH_ERRORS
+  Sources src;
+  if (!src.parse(a[0])) return nullptr;
+  return Py_BuildValue("Li", (long long)src.images, src.boxes_per_image());
+  END_HANDLE_TH_ERRORS
+}
+
+// Up to four numbers, what float() takes; those not given are zero.
+bool variances(PyObject* o, float (&var)[4]) {
+  THPObjectPtr vars(PySequence_Fast(o, "variances: expected a sequence"));
+  if (!vars) return false;
+  const Py_ssize_t k = PySequence_Fast_GET_SIZE(vars.get());
+  if (k > 4) { PyErr_SetString(PyExc_IndexError, "variances: more than four values"); return false; }
+  for (Py_ssize_t i = 0; i < 4; ++i) {
+    var[i] = 0.0f;
+    if (i >= k) continue;
+    THPObjectPtr v(PyNumber_Float(PySequence_Fast_GET_ITEM(vars.get(), i)));
+    if (!v || !number(v.get(), &var[i])) return false;
+  }
+  return true;
+}
 
 // (sources, priors, variances, classes, background, conf_thresh, nms_thresh, nms_top_k, keep_top_k, workspace, out, counts)
-// -> status.  out and counts are given; sources is a sequence of (loc, conf, boxes per cell).
+// -> status.  workspace, out and counts are given.
 PyObject* py_detect(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!count(n, 12)) return nullptr;
   HANDLE_TH_ERRORS
-  PyObject* seq = PySequence_Fast(a[0], "sources: expected a sequence");
-  if (!seq) return nullptr;
-  THPObjectPtr hold(seq);
-  const Py_ssize_t k = PySequence_Fast_GET_SIZE(seq);
-  if (k > kMaxSources) { PyErr_SetString(PyExc_ValueError, "sources: too many"); return nullptr; }
-  const float *loc[kMaxSources], *conf[kMaxSources];
-  int ls[kMaxSources], cs[kMaxSources], cells[kMaxSources], boxes[kMaxSources];
-  int64_t images = 0;
-  long long P = 0;
-  for (Py_ssize_t i = 0; i < k; ++i) {
-    THPObjectPtr item(PySequence_Fast(PySequence_Fast_GET_ITEM(seq, i), "sources: expected (loc, conf, boxes per cell)"));
-    if (!item) return nullptr;
-    if (PySequence_Fast_GET_SIZE(item.get()) != 3) { PyErr_SetString(PyExc_ValueError, "sources: expected (loc, conf, boxes per cell)"); return nullptr; }
-    PyObject** e = PySequence_Fast_ITEMS(item.get());
-    int ccells;
-    int64_t ni, nc;
-    if (!cell_view(e[0], "loc", &loc[i], &ls[i], &cells[i], &ni) || !cell_view(e[1], "conf", &conf[i], &cs[i], &ccells, &nc)) return nullptr;
-    if (i == 0) images = ni;
-    if (ccells != cells[i] || nc != images || ni != images) {
-      PyErr_SetString(PyExc_ValueError, "loc and conf of a source must cover the same cells of the same images");
-      return nullptr;
-    }
-    if (!number(e[2], &boxes[i])) return nullptr;
-    P += (long long)cells[i] * boxes[i];
-  }
-  THPObjectPtr vars(PySequence_Fast(a[2], "variances: expected a sequence"));
-  if (!vars) return nullptr;
+  Sources src;
   float var[4];
-  if (PySequence_Fast_GET_SIZE(vars.get()) != 4) { PyErr_SetString(PyExc_ValueError, "variances: expected four values"); return nullptr; }
-  for (int i = 0; i < 4; ++i)
-    if (!number(PySequence_Fast_GET_ITEM(vars.get(), i), &var[i])) return nullptr;
+  if (!src.parse(a[0]) || !variances(a[2], var)) return nullptr;
   void *priors, *ws, *out, *counts;
   int classes, background, top, keep;
   float ct, nt;
@@ -242,10 +273,11 @@ PyObject* py_detect(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void* s = current_stream();
   return call([&] {
     size_t need;
-    const int rc = g_q8.det_bytes((int)images, (int)(P > 0x7fffffff ? 0x7fffffff : P), classes, background, top, keep, &need);
+    const int rc = g_q8.det_bytes((int)src.images, src.boxes_per_image(), classes, background, top, keep, &need);
     if (rc != Q8_OK) return rc;
-    return g_q8.detect((int)k, loc, ls, conf, cs, cells, boxes, static_cast<const float*>(priors), var, (int)images, classes, background, ct, nt,
-                       top, keep, ws, ws_bytes, static_cast<float*>(out), static_cast<int32_t*>(counts), s);
+    return g_q8.detect((int)src.loc.size(), src.loc.data(), src.ls.data(), src.conf.data(), src.cs.data(), src.cells.data(), src.boxes.data(),
+                       static_cast<const float*>(priors), var, (int)src.images, classes, background, ct, nt, top, keep, ws, ws_bytes,
+                       static_cast<float*>(out), static_cast<int32_t*>(counts), s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -271,7 +303,8 @@ PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
 #define Q8_METHOD(name, f) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(f)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {Q8_METHOD("bind", py_bind),         Q8_METHOD("conv2d", py_conv2d),     Q8_METHOD("then_1x1", py_then_1x1),
                          Q8_METHOD("maxabs", py_maxabs),     Q8_METHOD("quantize", py_quantize), Q8_METHOD("dequantize", py_dequantize),
-                         Q8_METHOD("detect", py_detect),     {nullptr, nullptr, 0, nullptr}};
+                         Q8_METHOD("detect", py_detect),     Q8_METHOD("detect_size", py_detect_size),
+                         {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_q8native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

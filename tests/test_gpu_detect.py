@@ -195,3 +195,30 @@ def test_detection_output_at_the_listing_limit(q8, thresh, background):
     conf[:, 3::50, 4] = np.nan
     conf[:, 4::50] = -np.inf
     _compare(q8, np.zeros((2, P, 4), np.float32), conf, priors, [P], [1], background=background, conf_thresh=thresh)
+
+
+def test_detection_output_takes_what_converts(q8):
+    """Box counts that int() takes, variances that float() takes, fewer than four of them (the others are zero); too many
+    sources, and more boxes than fit, are the library's errors; with scratch and outputs given or not."""
+    g = np.random.default_rng(9)
+    loc, conf = _cuda(g.normal(0, 1, (2, 60, 8)).astype(np.float32)), _cuda(g.normal(0, 2, (2, 60, 8)).astype(np.float32))
+    priors = _cuda(g.uniform(0.2, 0.8, (120, 4)).astype(np.float32))
+    kw = dict(background=0, nms_top_k=50, keep_top_k=20)
+    want = q8.q8_detection_output([(loc, conf, 2)], priors, (0.1, 0.1, 0.2, 0.0), 4, **kw)
+    ws = torch.empty(q8.q8_detection_output_workspace_bytes(2, 120, 4, 0, 50, 20), dtype=torch.uint8, device="cuda")
+    given = dict(workspace=ws, out=torch.empty_like(want[0]), counts=torch.empty_like(want[1]))
+    for b, v in ((2.0, (0.1, 0.1, 0.2)), (np.float32(2.9), [np.float64(0.1), 0.1, "0.2"]), (torch.tensor(2), torch.tensor([0.1, 0.1, 0.2, 0.0]))):
+        for extra in ({}, given):
+            got = q8.q8_detection_output([[loc, conf, b]], priors, v, 4, **kw, **extra)
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    with pytest.raises(IndexError):
+        q8.q8_detection_output([(loc, conf, 2)], priors, (0.1,) * 5, 4, **kw)
+    for extra in ({}, given):
+        for sources, code in (([(loc, conf, 2)] * 70, 1), ([(loc, conf, 400)], 2)):
+            with pytest.raises(q8.Q8Error) as e:
+                q8.q8_detection_output(sources, priors, (0.1,) * 4, 4, **kw, **extra)
+            assert e.value.code == code
+        with pytest.raises(ValueError, match="same cells"):
+            q8.q8_detection_output([(loc, conf[:, :9].contiguous(), 2)], priors, (0.1,) * 4, 4, **kw, **extra)
+        with pytest.raises(TypeError, match="^conf: expected"):
+            q8.q8_detection_output([(loc, conf.double(), 2)], priors, (0.1,) * 4, 4, **kw, **extra)
