@@ -125,15 +125,24 @@ PyObject* py_then_1x1(PyObject*, PyObject* const* a, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-size_t numel(PyObject* o) { return (size_t)THPVariable_Unpack(o).numel(); }
+// The elements of a tensor; anything else has the error of its attribute (dev() has let nothing but None through).
+bool numel(PyObject* o, size_t* n) {
+  if (THPVariable_Check(o)) {
+    *n = (size_t)THPVariable_Unpack(o).numel();
+    return true;
+  }
+  THPObjectPtr attr(PyObject_GetAttrString(o, "numel"));
+  if (attr) PyErr_SetString(PyExc_TypeError, "expected a tensor");
+  return false;
+}
 
 // (x, running_max) -> status
 PyObject* py_maxabs(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!count(n, 2)) return nullptr;
   HANDLE_TH_ERRORS
   void *x, *m;
-  if (!dev(a[0], "x", &x) || !dev(a[1], "running_max", &m)) return nullptr;
-  const size_t k = numel(a[0]);
+  size_t k;
+  if (!dev(a[0], "x", &x) || !dev(a[1], "running_max", &m) || !numel(a[0], &k)) return nullptr;
   void* s = current_stream();
   return call([&] { return g_q8.maxabs(static_cast<const float*>(x), k, static_cast<float*>(m), s); });
   END_HANDLE_TH_ERRORS
@@ -146,8 +155,8 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void *x, *out;
   float q;
   int type;
-  if (!dev(a[0], "x", &x) || !number(a[1], &q) || !number(a[2], &type) || !dev(a[3], "out", &out)) return nullptr;
-  const size_t k = numel(a[0]);
+  size_t k;
+  if (!dev(a[0], "x", &x) || !number(a[1], &q) || !number(a[2], &type) || !dev(a[3], "out", &out) || !numel(a[0], &k)) return nullptr;
   void* s = current_stream();
   return call([&] { return g_q8.quantize(static_cast<const float*>(x), k, q, type, out, s); });
   END_HANDLE_TH_ERRORS
@@ -160,8 +169,8 @@ PyObject* py_dequantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void *z, *out;
   float q;
   int type;
-  if (!dev(a[0], "z", &z) || !number(a[1], &type) || !number(a[2], &q) || !dev(a[3], "out", &out)) return nullptr;
-  const size_t k = numel(a[0]);
+  size_t k;
+  if (!dev(a[0], "z", &z) || !number(a[1], &type) || !number(a[2], &q) || !dev(a[3], "out", &out) || !numel(a[0], &k)) return nullptr;
   void* s = current_stream();
   return call([&] { return g_q8.dequantize(z, type, k, q, static_cast<float*>(out), s); });
   END_HANDLE_TH_ERRORS
@@ -269,7 +278,8 @@ PyObject* py_detect(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!dev(a[1], "priors", &priors) || !number(a[3], &classes) || !number(a[4], &background) || !number(a[5], &ct) || !number(a[6], &nt) ||
       !number(a[7], &top) || !number(a[8], &keep) || !dev(a[9], "workspace", &ws) || !dev(a[10], "out", &out) || !dev(a[11], "counts", &counts))
     return nullptr;
-  const size_t ws_bytes = a[9] == Py_None ? 0 : numel(a[9]);
+  size_t ws_bytes;
+  if (!numel(a[9], &ws_bytes)) return nullptr;
   void* s = current_stream();
   return call([&] {
     size_t need;

@@ -224,3 +224,21 @@ def test_pairs_bound_by_their_rows_take_tile_buffers(N, HW, C1, K1, K2, residual
     d1 = q8.make_conv_desc(N, HW, HW, C1, K1, 3, 3, (1, 1), (1, 1), relu=True)
     d2 = q8.make_conv_desc(N, HW, HW, K1, K2, 1, 1, relu=True)
     assert q8.q8_conv2d_query_row_buffers(d1, d2, residual) == buffers
+
+
+def test_marshalled_calls_refuse_none_without_assertions():
+    """In an interpreter that runs no assertions: an error of the argument, not an access to what it is not."""
+    code = """if True:
+        import torch, paper_1805_08691_b200 as q8
+        from paper_1805_08691_b200 import binding
+        for call in (lambda: binding._native.maxabs(None, None), lambda: binding._native.quantize(None, 1.0, q8.Q8_U8, None),
+                     lambda: binding._native.dequantize(None, q8.Q8_U8, 1.0, None), lambda: q8.q8_calibrate_maxabs(None, None)):
+            try:
+                call()
+            except AttributeError as e:
+                if "numel" not in str(e):
+                    raise
+            else:
+                raise SystemExit("no error")
+        """
+    assert subprocess.run([sys.executable, "-O", "-c", code], cwd=ROOT).returncode == 0
