@@ -110,7 +110,7 @@ def _load_native():
     module = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(module)
     module.bind(*(C.cast(f, C.c_void_p).value for f in (lib.q8_conv2d, lib.q8_conv2d_then_1x1, lib.q8_calibrate_maxabs, lib.q8_quantize,
-                                                        lib.q8_dequantize, lib.q8_detection_output_workspace_bytes, lib.q8_detection_output)))
+                                                        lib.q8_dequantize, lib.q8_detection_output_workspace_bytes, lib.q8_detection_output)), q8_conv_desc)
     return module
 
 

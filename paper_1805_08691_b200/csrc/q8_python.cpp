@@ -43,14 +43,16 @@ bool dev(PyObject* o, const char* what, void** p) {
   return false;
 }
 
-// A ctypes structure's bytes.
+PyObject* g_desc_type = nullptr;  // the binding's ctypes structure
+
+// The bytes of a descriptor, an instance of that structure or of a class derived from it.
 struct Bytes {
   Py_buffer b{};
   bool ok = false;
-  explicit Bytes(PyObject* o) { ok = PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) == 0; }
+  explicit Bytes(PyObject* o) { ok = PyObject_IsInstance(o, g_desc_type) == 1 && PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) == 0; }
   ~Bytes() { if (ok) PyBuffer_Release(&b); }
   const q8_conv_desc* desc() const {
-    if (ok && (size_t)b.len == sizeof(q8_conv_desc)) return static_cast<const q8_conv_desc*>(b.buf);
+    if (ok && (size_t)b.len >= sizeof(q8_conv_desc)) return static_cast<const q8_conv_desc*>(b.buf);
     if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "expected a q8_conv_desc");
     return nullptr;
   }
@@ -292,14 +294,18 @@ PyObject* py_detect(PyObject*, PyObject* const* a, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-// (addresses of the entry points, in the order of Entry)
+// (addresses of the entry points, in the order of Entry, the descriptors' class)
 PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  if (!count(n, 7)) return nullptr;
+  if (!count(n, 8)) return nullptr;
   void* p[7];
   for (int i = 0; i < 7; ++i) {
     p[i] = PyLong_AsVoidPtr(a[i]);
     if (!p[i]) return nullptr;
   }
+  PyObject* old = g_desc_type;
+  Py_INCREF(a[7]);
+  g_desc_type = a[7];
+  Py_XDECREF(old);
   g_q8.conv2d = reinterpret_cast<decltype(g_q8.conv2d)>(p[0]);
   g_q8.then_1x1 = reinterpret_cast<decltype(g_q8.then_1x1)>(p[1]);
   g_q8.maxabs = reinterpret_cast<decltype(g_q8.maxabs)>(p[2]);

@@ -189,8 +189,14 @@ def test_marshalled_calls_refuse_what_they_cannot_pass():
     for bad in (x, x.permute(0, 2, 1, 3), 3, [1]):
         with pytest.raises(TypeError, match="^x: expected a contiguous CUDA tensor"):
             q8.q8_conv2d(d, bad, w, None, None, y=y)
-    with pytest.raises(TypeError, match="q8_conv_desc"):
-        q8.q8_conv2d(q8.q8_conv_plan(), x, w, None, None, y=y)
+    for no_desc in (q8.q8_conv_plan(), bytes(d), bytearray(d), C.byref(d)):
+        with pytest.raises(TypeError, match="q8_conv_desc"):
+            q8.q8_conv2d(no_desc, x, w, None, None, y=y)
+
+    class wider(q8.q8_conv_desc):
+        _fields_ = [("note", C.c_int32)]
+    with pytest.raises(TypeError, match="^x: expected"):   # a derived structure is one
+        q8.q8_conv2d(wider(*bytes(21)), x, w, None, None, y=y)
     with pytest.raises(TypeError, match="^out: expected|^x: expected"):
         q8.q8_quantize(torch.zeros(4), 1.0, q8.Q8_U8)
     with pytest.raises(TypeError, match="^loc: expected a CUDA fp32 tensor"):
