@@ -51,8 +51,8 @@ def _load():
     path = _build.LIB
     if shutil.which("nvcc") is not None:
         path = _build.build()
-    if not (os.path.exists(path) and os.path.exists(_build.NATIVE)):
-        raise ImportError(f"{path} or {_build.NATIVE} is missing and nvcc is not available to build it; "
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing and nvcc is not available to build it; "
                           "run `python -m paper_1805_08691_b200.build` on a machine with CUDA 12.9")
     return C.CDLL(path)
 
@@ -106,7 +106,13 @@ lib.q8_static_workspace_bytes.restype = C.c_size_t
 
 
 def _load_native():
-    spec = importlib.util.spec_from_file_location("_q8native", _build.NATIVE)
+    path = _build.native_path()
+    if not os.path.exists(path):   # (libq8.so came without it, or with that of another torch)
+        try:
+            path = _build.build_native()
+        except RuntimeError as e:
+            raise ImportError(f"{path}, the marshalling module for this torch, is missing and cannot be built here: {e}") from None
+    spec = importlib.util.spec_from_file_location("_q8native", path)
     module = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(module)
     module.bind(*(C.cast(f, C.c_void_p).value for f in (lib.q8_conv2d, lib.q8_conv2d_then_1x1, lib.q8_calibrate_maxabs, lib.q8_quantize,

@@ -248,3 +248,27 @@ def test_marshalled_calls_refuse_none_without_assertions():
                 raise SystemExit("no error")
         """
     assert subprocess.run([sys.executable, "-O", "-c", code], cwd=ROOT).returncode == 0
+
+
+def test_marshalling_module_belongs_to_one_torch(monkeypatch):
+    """Another torch asks for another file, which is built by a C++ compiler alone; without one the import says what is missing."""
+    from paper_1805_08691_b200 import build
+    import torch
+    mine = build.native_path()
+    assert os.path.exists(mine) and not build._native_stale()
+    monkeypatch.setattr(torch, "__version__", "0.1+other")
+    assert build.native_path() != mine and build._native_stale()
+    monkeypatch.setattr(build.shutil, "which", lambda name: None)
+    with pytest.raises(RuntimeError, match="compiler"):
+        build.build_native()
+    code = """if True:
+        import torch
+        torch.__version__ = "0.1+other"
+        try:
+            import paper_1805_08691_b200
+        except ImportError as e:
+            raise SystemExit(0 if "for this torch" in str(e) else 2)
+        raise SystemExit("imported a module of another torch")
+        """
+    env = dict(os.environ, PATH="/nonexistent", CXX="/nonexistent")
+    assert subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env).returncode == 0
