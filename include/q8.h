@@ -204,10 +204,10 @@ int q8_conv2d_query_algo(const q8_conv_desc* d, int* algo);
 typedef enum q8_conv_kernel { Q8_KERNEL_DIRECT = 0, Q8_KERNEL_GATHER = 1, Q8_KERNEL_TMA = 2 } q8_conv_kernel;
 typedef struct q8_conv_plan {
   int32_t kernel;           /* q8_conv_kernel (Q8_KERNEL_GATHER: tensor cores on operands that no TMA load brings, gathered by
-                             * chunks or, for three-channel images, packed from whole rows); the fields below are zero unless
-                             * it is Q8_KERNEL_TMA */
+                             * chunks or, for three-channel images, packed from whole rows); but for `operand`, the fields
+                             * below are zero unless it is Q8_KERNEL_TMA */
   int32_t tile_n;           /* output channels of a tile */
-  int32_t operand;          /* activations as 0: a matrix, 1: im2col loads, 2: halo patches */
+  int32_t operand;          /* activations as 0: a matrix, 1: im2col loads, 2: halo patches; Q8_KERNEL_GATHER: 0 by chunks, 3 packed */
   int32_t splits;           /* parts of the reduction, 1: not split */
   int32_t weights;          /* 0: staged with the activations, 1: resident in shared memory, 2: in a ring of their own */
   int32_t cta_pair;         /* 1: CTA pairs share the weights of a tile */

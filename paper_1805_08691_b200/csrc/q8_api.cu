@@ -104,12 +104,12 @@ double direct_us(const ConvArgs& a) {
   return 2.4 + outputs * (9.0 + 0.22 * chain) + chain * (0.033 + 0.019 * apart) + (taps > 1 ? 0.1 * seen : 0.0) + 0.03 * taps;
 }
 
-// 8-bit rows that TMA cannot store, short ones with short reductions: gathering the operands (or the direct kernel) costs
+// 8-bit rows off the 16-byte grid, short ones with short reductions: gathering the operands (or the direct kernel) costs
 // less than the kernel that moves such rows through shared memory, whose start-up is longer.  The gathering kernel's time
 // grows faster, by the bytes that its producers fetch (reduction x pixels) and by every 16 columns that it stores byte by
 // byte, which is what the limits are in (1x1 64 -> 9 at 56x56: batch 4 3.9 against 4.6 us, batch 16 5.0 against 5.5, batch 32
-// 7.2 against 7.1; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).  Over 870 random layers whose rows TMA
-// cannot store, the kernel taken is on average 0.9 % off the fastest of the three.
+// 7.2 against 7.1; 32 -> 31 on one 8x8 image 4.2 against 4.7, 12x12 5.6 against 4.6).  Over 870 random layers with such
+// rows, the kernel taken is on average 0.9 % off the fastest of the three.
 bool short_rows(const ConvArgs& a) {
   const long long products = (long long)a.d.R * a.d.S * a.d.C;
   return products <= 64 && (a.d.K <= 16 ? products * a.M <= 4000000 : a.d.K <= 32 && a.M <= 128);
@@ -221,6 +221,7 @@ int q8_conv2d_query_plan(const q8_conv_desc* d, int residual, q8_conv_plan* plan
   if (route == kRouteTma && !umma_describe(a, plan)) { route = route_off_tma(a); why = "no tile shape of this layer fits in shared memory"; }
   if (route == kRouteRefused) return fail(Q8_ERR_UNSUPPORTED, "q8_conv2d: tensor-core kernel not eligible: %s", why);
   plan->kernel = route == kRouteTma ? Q8_KERNEL_TMA : (route == kRouteDirect ? Q8_KERNEL_DIRECT : Q8_KERNEL_GATHER);
+  if (route == kRoutePacked) plan->operand = 3;
   return Q8_OK;
 }
 

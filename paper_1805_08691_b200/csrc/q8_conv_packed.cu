@@ -6,7 +6,7 @@
 // across the end of an image), which one bulk copy brings into shared memory.  A thread per pixel then packs the pixel's
 // R runs of S C bytes densely, in the order in which the weights of a filter lie in memory, into its row of the K-major
 // swizzled tile that tcgen05.mma reads: unaligned words of the span by funnel shifts, joined by shifts that are compile-time
-// constants (filters of 1, 3, 5 or 7 rows and columns).  Bytes outside the image are masked to zero, the exact code of 0.0.
+// constants (filters of 3, 5 or 7 rows and 1, 3, 5 or 7 columns, and 1x1).  Bytes outside the image are masked to zero, the exact code of 0.0.
 //
 // Roles: warps 0-15 four epilogue groups, each with its accumulator (thread = accumulator row), warp 16 MMA issue and TMEM, warp
 // 17 bulk copies, warps 18-25 two packing groups on alternate tiles.  Weights are resident.  All waits are bounded as in the
@@ -34,16 +34,16 @@ struct PackedParams {
   UmmaParams u;              // what the epilogue reads: M, K, bn, bias, scale, residual, output
   const unsigned char* x;
   const unsigned char* w;
-  int H, W, C, rows;         // rows: N * H
+  int H, W, C;
   int stride_h, stride_w, pad_h, pad_w, dil_h;
-  int R, run_len, words;     // runs (filter rows), bytes of a run, 32-bit words of a packed row that hold a byte
+  int R, run_len;            // runs (filter rows), bytes of a run
   int reduction;             // R * run_len
   int row_bytes;             // W * C
   int bkb, lg_cpb, nblk;     // bytes per K block (32, 64 or 128), log2 of its 16-byte chunks, number of blocks
   int ksteps, last_ksteps;   // K steps of a block, of the last one
   int m_tiles;
   unsigned int span_cap, margin, off_a, a_bytes, off_span, off_chan, b_block_bytes, swz_mask;
-  int acc_stride, tmem_cols, res_vec, store_vec;
+  int acc_stride, tmem_cols, res_vec;
   FastDiv fd_q, fd_pq, fd_words;
 };
 
@@ -309,17 +309,6 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
           }
           return rv;
         };
-        auto store = [&](int nb, int valid, const uint4& o) {
-          unsigned char* yp = static_cast<unsigned char*>(p.u.y) + (size_t)t.m * p.u.ldc + p.u.c_off + nb;
-          if (p.store_vec && valid == 16) {
-            *reinterpret_cast<uint4*>(yp) = o;
-          } else {
-            const unsigned int q[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (j < valid) yp[j] = (unsigned char)(q[j >> 2] >> (8 * (j & 3)));
-          }
-        };
         for (int ch = 0; ch < chunks; ch += 2) {
           const bool two = ch + 1 < chunks;
           tmem_ld_16(taddr + ch * 16, ra);
@@ -337,11 +326,13 @@ __global__ void __launch_bounds__(kPkThreads, 1) conv_packed_kernel(const __grid
           uint4 o1 = make_uint4(0u, 0u, 0u, 0u);
           if (two) o1 = epilogue_chunk<kOut, kRes, kUniform>(p.u, t, ch + 1, rb, us, r1);
           if (kOut == Q8_U8 || kOut == Q8_S8) {
+            // (rows are stored in 16-byte pieces, see packed_better: a chunk of a row is all there or not)
+            unsigned char* yp = static_cast<unsigned char*>(p.u.y) + (size_t)t.m * p.u.ldc + p.u.c_off + nb;
             if (p.u.y_wide && v1 == 16) {
-              store_32(static_cast<unsigned char*>(p.u.y) + (size_t)t.m * p.u.ldc + p.u.c_off + nb, o0, o1);
+              store_32(yp, o0, o1);
             } else {
-              if (v0 > 0) store(nb, v0, o0);
-              if (v1 > 0) store(nb + 16, v1, o1);
+              if (v0 > 0) *reinterpret_cast<uint4*>(yp) = o0;
+              if (v1 > 0) *reinterpret_cast<uint4*>(yp + 16) = o1;
             }
           }
           __syncwarp();
@@ -408,10 +399,10 @@ bool packed_eligible(const q8_conv_desc& d, int P, int Q) {
 }  // namespace
 
 // Where it is faster than the kernels that took such layers: one tile of columns (weights are staged word by word, and what is
-// gathered again for every further tile is little), rows stored in 16-byte pieces, half of the SMs at work, and not a single
-// run of 15 or 21 bytes (1xS), which the gathering kernel fetches densely as well (1x7 of 3 -> 112 on 7 x 58x60: 5.4 there, 6.2
-// us here).  Over 160 random layers of these forms, replayed from a graph, 1.31 times faster in the mean, from 2.7 times
-// (5x5 of 3 -> 16 on 30 x 197x199 89 -> 33 us) to as fast (5x5 of 3 -> 80 on 108x108 6.1 us both).
+// gathered again for every further tile is little), rows stored in 16-byte pieces (the kernel relies on it), half of the SMs at
+// work, and not a single run of several columns (1xS), which the gathering kernel fetches densely as well (1x7 of 3 -> 112 on
+// 7 x 58x60: 5.4 there, 6.2 us here).  Over 160 random layers of these forms, replayed from a graph, 1.31 times faster in the
+// mean, from 2.7 times (5x5 of 3 -> 16 on 30 x 197x199 89 -> 33 us) to as fast (5x5 of 3 -> 80 on 108x108 6.1 us both).
 bool packed_better(const ConvArgs& a) {
   const int grid = a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8 ? 16 : 4;
   return packed_eligible(a.d, a.P, a.Q) && a.M > (long long)kBM * sm_count() / 2 && a.d.K % grid == 0 && aligned16(a.y) && a.ldc % grid == 0 &&
@@ -432,16 +423,14 @@ int launch_conv_packed(const ConvArgs& a) {
   u.res_mode = a.residual ? kResVec : kResNone;
   u.res_signed = d.res_type == Q8_S8; u.res_scale = a.residual_scale;
   u.y = a.y; u.y_type = d.y_type; u.ldc = a.ldc; u.c_off = a.c_off; u.relu = d.relu;
-  const int grid16 = out8 ? 16 : 4;
-  u.y_vec = aligned16(a.y) && a.ldc % grid16 == 0 && a.c_off % grid16 == 0;
-  p.store_vec = u.y_vec;
+  u.y_vec = 1;
   u.y_wide = out8 && (reinterpret_cast<uintptr_t>(a.y) & 31u) == 0 && a.ldc % 32 == 0 && a.c_off % 32 == 0;
   p.res_vec = d.K % 16 == 0 && aligned16(a.residual);
   p.x = static_cast<const unsigned char*>(a.x);
   p.w = reinterpret_cast<const unsigned char*>(a.w);
-  p.H = d.H; p.W = d.W; p.C = d.C; p.rows = d.N * d.H;
+  p.H = d.H; p.W = d.W; p.C = d.C;
   p.stride_h = d.stride_h; p.stride_w = d.stride_w; p.pad_h = d.pad_h; p.pad_w = d.pad_w; p.dil_h = d.dil_h;
-  p.R = d.R; p.run_len = d.S * d.C; p.reduction = d.R * p.run_len; p.words = (p.reduction + 3) / 4;
+  p.R = d.R; p.run_len = d.S * d.C; p.reduction = d.R * p.run_len;
   p.row_bytes = d.W * d.C;
   const int chunks = (p.reduction + 15) / 16;
   p.lg_cpb = chunks <= 2 ? 1 : (chunks <= 4 ? 2 : 3);

@@ -272,3 +272,11 @@ def test_marshalling_module_belongs_to_one_torch(monkeypatch):
         """
     env = dict(os.environ, PATH="/nonexistent", CXX="/nonexistent")
     assert subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env).returncode == 0
+
+
+@pytest.mark.parametrize("shape,operand", [((8, 99, 99, 3, 32, 3, 3), 3), ((8, 99, 99, 3, 64, 7, 1), 3), ((8, 99, 99, 3, 32, 1, 1), 3),
+                                           ((8, 99, 99, 3, 32, 1, 7), 0), ((8, 99, 99, 4, 32, 3, 3), 0), ((8, 99, 99, 3, 24, 3, 3), 0),
+                                           ((8, 99, 99, 3, 144, 3, 3), 0), ((1, 60, 60, 3, 32, 3, 3), 0)], ids=str)
+def test_plan_tells_packed_operands_from_gathered_ones(shape, operand):
+    plan = q8.q8_conv2d_query_plan(q8.make_conv_desc(*shape, x_type=q8.Q8_S8))
+    assert plan.kernel == q8.Q8_KERNEL_GATHER and plan.operand == operand

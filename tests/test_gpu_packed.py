@@ -1,6 +1,7 @@
 """GPU parity of the tensor-core convolution that packs rows of three-channel images, against the CPU oracle, bit-exact: every
-run length and number of runs, one and several K blocks, tiles across image ends, padding on
-all sides, dilation along H, unaligned inputs and outputs, several tiles of columns, every output type."""
+run length and number of runs, one and several K blocks, tiles across image ends, padding on all sides, dilation along H,
+inputs and residuals off the 16-byte grid, slices of wider outputs, channel counts off the 16-column chunks, every output type
+with and without a residual, one multiplier and one per channel.  Filters of one row and several columns are gathered."""
 import numpy as np
 import pytest
 import torch
@@ -27,7 +28,15 @@ CASES = [
     ("c3_5x7", 30, 21, 22, 3, 96, 5, 7, (1, 1), (0, 3), 1, True, U8, False, True, 32, 2),
     ("many_tiles_c3", 8, 150, 150, 3, 32, 3, 3, (1, 1), (1, 1), 1, True, U8, False, False, 0, 0),
     ("wide_padding", 13, 14, 14, 3, 16, 3, 3, (1, 1), (7, 9), 1, True, U8, False, False, 0, 0),
+    ("c3_3x3_f32", 6, 45, 47, 3, 36, 3, 3, (1, 1), (1, 1), 1, True, F32, False, False, 8, 2),
+    ("c3_7x7s2_f32_residual", 11, 64, 62, 3, 64, 7, 7, (2, 2), (3, 3), 1, False, F32, True, False, 0, 0),
+    ("c3_5x5_f32_per_channel", 11, 31, 30, 3, 112, 5, 5, (1, 1), (2, 2), 1, True, F32, False, True, 0, 1),
+    ("c3_3x1_f32_residual_off_per_channel", 12, 33, 40, 3, 44, 3, 1, (1, 1), (1, 0), 1, True, F32, True, True, 8, 0),
+    ("c3_3x3_s32", 6, 45, 47, 3, 20, 3, 3, (1, 1), (1, 1), 1, True, S32, False, False, 8, 0),
+    ("c3_3x3_residual_off", 8, 40, 37, 3, 48, 3, 3, (1, 1), (1, 1), 1, True, U8, True, False, 32, 0),
+    ("c3_7x7s2_s8_residual_off", 9, 64, 66, 3, 32, 7, 7, (2, 2), (3, 3), 1, False, S8, True, True, 0, 3),
 ]
+GATHERED = ("c3_1x7_f32", "c3_1x5")
 
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
@@ -44,12 +53,18 @@ def test_packed_matches_oracle(q8, case):
     want = o.epilogue(acc, scale if per_channel else scale[0], resid, 0.37 if res else 0.0, True, OT[ytype])
     d = q8.make_conv_desc(N, H, W, C, K, R, S, st, pad, (dil_h, 1), S8 if xs8 else U8, U8, ytype, True,
                           K if per_channel else 1, K + extra, extra // 2)
-    assert q8.q8_conv2d_query_plan(d, res).kernel == q8.Q8_KERNEL_GATHER
+    plan = q8.q8_conv2d_query_plan(d, res)
+    assert plan.kernel == q8.Q8_KERNEL_GATHER and plan.operand == (0 if name in GATHERED else 3)
     xb = torch.zeros(x.size + 3, dtype=torch.uint8, device="cuda")
     xb[shift:shift + x.size] = torch.from_numpy(x.view(np.uint8).ravel()).cuda()
+    rd, off = None, 1 if "residual_off" in name else 0
+    if res:
+        rb = torch.zeros(resid.size + 1, dtype=torch.uint8, device="cuda")
+        rd = rb[off:off + resid.size].view(N, P, Q, K)
+        rd.copy_(torch.from_numpy(resid).cuda())
     y = torch.full((N, P, Q, K + extra), 7, dtype=q8.TORCH_DTYPES[ytype], device="cuda")
     q8.q8_conv2d(d, xb[shift:shift + x.size].view(N, H, W, C), torch.from_numpy(w).cuda(), torch.from_numpy(bias).cuda(),
-                 torch.from_numpy(scale).cuda(), torch.from_numpy(resid).cuda() if res else None, 0.37 if res else 0.0, y)
+                 torch.from_numpy(scale).cuda(), rd, 0.37 if res else 0.0, y)
     q8.q8_read_status()
     got = y.cpu().numpy()
     lo, hi = extra // 2, extra // 2 + K
