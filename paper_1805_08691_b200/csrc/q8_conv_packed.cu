@@ -403,8 +403,12 @@ bool packed_eligible(const q8_conv_desc& d, int P, int Q) {
 // work, and not a single run of several columns (1xS), which the gathering kernel fetches densely as well (1x7 of 3 -> 112 on
 // 7 x 58x60: 5.4 there, 6.2 us here).  Over 160 random layers of these forms, replayed from a graph, 1.31 times faster in the
 // mean, from 2.7 times (5x5 of 3 -> 16 on 30 x 197x199 89 -> 33 us) to as fast (5x5 of 3 -> 80 on 108x108 6.1 us both).
+// 32-bit outputs of more than 48 channels that end inside a 16-column chunk store that chunk word by word: up to three tiles
+// per CTA still faster (85 random layers: 1.1 times), slower beyond (3x3 of 3 -> 104 on 10 x 258x258 172 against 118 us gathered;
+// 3x7 of 3 -> 60 on 25 x 172x174 149 against 108), while whole chunks and narrower outputs gain at any size (1.2 and 1.4 times).
 bool packed_better(const ConvArgs& a) {
   const int grid = a.d.y_type == Q8_U8 || a.d.y_type == Q8_S8 ? 16 : 4;
+  if (grid == 4 && a.d.K % 16 && a.d.K > 48 && a.M > 3ll * kBM * sm_count()) return false;
   return packed_eligible(a.d, a.P, a.Q) && a.M > (long long)kBM * sm_count() / 2 && a.d.K % grid == 0 && aligned16(a.y) && a.ldc % grid == 0 &&
          a.c_off % grid == 0;
 }

@@ -280,3 +280,12 @@ def test_marshalling_module_belongs_to_one_torch(monkeypatch):
 def test_plan_tells_packed_operands_from_gathered_ones(shape, operand):
     plan = q8.q8_conv2d_query_plan(q8.make_conv_desc(*shape, x_type=q8.Q8_S8))
     assert plan.kernel == q8.Q8_KERNEL_GATHER and plan.operand == operand
+
+
+@pytest.mark.parametrize("N,K,operand", [(10, 104, 0), (10, 52, 0), (1, 104, 0), (10, 48, 3), (10, 112, 3), (10, 44, 3)], ids=str)
+@pytest.mark.parametrize("y_type", [2, 3])
+def test_long_layers_with_ragged_32_bit_rows_are_gathered(y_type, N, K, operand):
+    d = q8.make_conv_desc(N, 258, 258, 3, K, 3, 3, pad=(1, 1), y_type=y_type)
+    assert q8.q8_conv2d_query_plan(d).operand == operand
+    d.N, d.H = 1, 200   # 3.0 tiles a block
+    assert q8.q8_conv2d_query_plan(d).operand == 3

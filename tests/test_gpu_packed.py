@@ -33,6 +33,7 @@ CASES = [
     ("c3_5x5_f32_per_channel", 11, 31, 30, 3, 112, 5, 5, (1, 1), (2, 2), 1, True, F32, False, True, 0, 1),
     ("c3_3x1_f32_residual_off_per_channel", 12, 33, 40, 3, 44, 3, 1, (1, 1), (1, 0), 1, True, F32, True, True, 8, 0),
     ("c3_3x3_s32", 6, 45, 47, 3, 20, 3, 3, (1, 1), (1, 1), 1, True, S32, False, False, 8, 0),
+    ("c3_3x3_s32_k52", 6, 45, 47, 3, 52, 3, 3, (1, 1), (1, 1), 1, False, S32, False, False, 0, 1),
     ("c3_3x3_residual_off", 8, 40, 37, 3, 48, 3, 3, (1, 1), (1, 1), 1, True, U8, True, False, 32, 0),
     ("c3_7x7s2_s8_residual_off", 9, 64, 66, 3, 32, 7, 7, (2, 2), (3, 3), 1, False, S8, True, True, 0, 3),
 ]
