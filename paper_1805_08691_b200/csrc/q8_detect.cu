@@ -222,33 +222,37 @@ __device__ __forceinline__ float4 det_box(const float* l, const float4 pr, float
 }
 
 constexpr int kDecThreads = 256;
+constexpr int kDecFew = 64;  // boxes of a block where there are few
 
-// Up to kRegClasses classes.  A block takes 256 boxes of an image, whose logits travel through shared memory (a thread per
+// Up to kRegClasses classes.  A block takes kBoxes boxes of an image (256, or 64 where there are few), whose logits travel through shared memory (a thread per
 // box would touch 21 lines with every load).  Most boxes of a detector are background and need no exponential: the largest
 // term of the sum is exp(0) = 1, so p_c <= e_c, and a box whose foreground logits all lie `cutoff` = ln(conf_thresh), less a
 // margin for the recipe's roundings, or more below its largest has no candidate.  What is left (one box in six at a
-// threshold of 0.01) is listed, and the block's threads share its (box, class) pairs.  Comparisons are written so that a NaN
-// lists its box.  One box per thread with all of its exponentials was bound by issue (1291 warp instructions per 32 boxes,
+// threshold of 0.01) is listed, and the block's threads share its (box, class) pairs.  A NaN among a
+// box's logits makes its sum a NaN, so no class of it passes, whether the maxima (which skip a NaN) list it or not; infinities of
+// one sign compare by a NaN difference, which lists.  One box per thread with all of its exponentials was bound by issue (1291 warp instructions per 32 boxes,
 // 790 with a list but loads through registers, five blocks per SM): detection output of 32 images, 8732 boxes, 21 classes,
 // replayed from a graph 45.8 -> 39.8 -> 36.7 us with eight resident blocks.
+template <int kBoxes>
 __global__ void __launch_bounds__(kDecThreads, 8) decode_listed_kernel(const __grid_constant__ DetSources src, const float4* __restrict__ priors,
                                                                        float v0, float v1, float v2, float v3, int P, int classes,
                                                                        int background, float conf_thresh, float cutoff, float4* __restrict__ boxes,
                                                                        float* __restrict__ prob, unsigned int* __restrict__ masks) {
-  __shared__ __align__(16) float stage[kDecThreads * kRegClasses];
-  __shared__ float top[kDecThreads], total[kDecThreads];
-  __shared__ unsigned int bits[kRegClasses][kDecThreads / 32];
-  __shared__ unsigned short list[kDecThreads];
+  constexpr int kWords = kBoxes / 32;
+  __shared__ __align__(16) float stage[kBoxes * kRegClasses];
+  __shared__ float top[kBoxes], total[kBoxes];
+  __shared__ unsigned int bits[kRegClasses][kWords];
+  __shared__ unsigned short list[kBoxes];
   __shared__ int listed;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int n = blockIdx.y, lane = threadIdx.x & 31, PW = (P + 31) >> 5, tid = (int)threadIdx.x;
-  const int p0 = blockIdx.x * kDecThreads, p = p0 + tid;
-  const bool live = p < P;
+  const int p0 = blockIdx.x * kBoxes, p = p0 + tid;
+  const bool mine = tid < kBoxes, live = mine && p < P;
   const float *l, *x;
   det_source(src, n, live ? p : P - 1, classes, &l, &x);
   if (tid == 0) listed = 0;
-  if (tid < kRegClasses * (kDecThreads / 32)) bits[tid / (kDecThreads / 32)][tid % (kDecThreads / 32)] = 0u;
-  if ((p & ~31) < P) {  // whole warps
+  if (tid < kRegClasses * kWords) bits[tid / kWords][tid % kWords] = 0u;
+  if (mine && (p & ~31) < P) {  // whole warps
     float* st = stage + (tid & ~31) * classes;
     const float* x0 = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), 0));
     if (__all_sync(0xffffffffu, x == x0 + lane * classes)) {  // the warp's boxes lie one after the other
@@ -332,8 +336,8 @@ __global__ void __launch_bounds__(kDecThreads, 8) decode_listed_kernel(const __g
     atomicOr(&bits[c][b >> 5], 1u << (b & 31));
   }
   __syncthreads();
-  if (tid < classes * (kDecThreads / 32)) {
-    const int c = tid / (kDecThreads / 32), w = tid % (kDecThreads / 32), at = (p0 >> 5) + w;
+  if (tid < classes * kWords) {
+    const int c = tid / kWords, w = tid % kWords, at = (p0 >> 5) + w;
     if (at < PW) masks[((size_t)n * classes + c) * PW + at] = bits[c][w];
   }
 }
@@ -902,8 +906,14 @@ int q8_detection_output(int n_sources, const float* const* loc, const int* loc_s
     // (where the recipe clamps its argument every class may pass)
     const double ln = std::log((double)conf_thresh) - 1e-4;
     const float cutoff = ln > -86.5 ? (float)(ln - 1e-5) : -INFINITY;
-    decode_listed_kernel<<<dec_grid, kDecThreads, 0, s>>>(src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2],
-                                                          variances[3], (int)P, classes, background, conf_thresh, cutoff, boxes, prob, masks);
+    // Where a quarter of the SMs can take 64 boxes each they do: a thread's share of the (box, class) pairs is a fourth (963
+    // boxes with flat logits at a threshold of 0.3: 15.9 -> 13.1 us).  No further: the blocks of the next launch find room as
+    // these leave it, and beside more of them they pile up on the SMs that are free (2 images of 8732 boxes 111 -> 223 us).
+    const dim3 few_grid((unsigned)((P + kDecFew - 1) / kDecFew), (unsigned)N);
+    const bool few = (long long)few_grid.x * N * 4 <= sm_count();
+    (few ? decode_listed_kernel<kDecFew> : decode_listed_kernel<kDecThreads>)<<<few ? few_grid : dec_grid, kDecThreads, 0, s>>>(
+        src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2], variances[3], (int)P, classes, background,
+        conf_thresh, cutoff, boxes, prob, masks);
   } else {
     decode_softmax_kernel<<<dec_grid, kDecThreads, 0, s>>>(src, reinterpret_cast<const float4*>(d_priors), variances[0], variances[1], variances[2],
                                                            variances[3], (int)P, classes, background, conf_thresh, boxes, prob, masks);

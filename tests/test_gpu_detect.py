@@ -197,6 +197,22 @@ def test_detection_output_at_the_listing_limit(q8, thresh, background):
     _compare(q8, np.zeros((2, P, 4), np.float32), conf, priors, [P], [1], background=background, conf_thresh=thresh)
 
 
+@pytest.mark.parametrize("N,P,classes", [(1, 1, 2), (1, 63, 24), (1, 65, 21), (37, 64, 5), (38, 64, 5), (1, 2368, 21), (1, 2369, 21), (13, 190, 7)])
+@pytest.mark.parametrize("spread,thresh", [(0.3, 0.3), (3.0, 0.01)])
+def test_detection_output_on_both_sides_of_few_boxes(q8, N, P, classes, spread, thresh):
+    """64 boxes a block up to a quarter of the SMs, 256 beyond; all boxes listed, or some; infinite and undefined logits."""
+    g = np.random.default_rng(N * P + classes)
+    centre, size = g.uniform(0.1, 0.9, (P, 2)), g.uniform(0.02, 0.2, (P, 2))
+    priors = np.concatenate([centre, size], 1).astype(np.float32)
+    conf = g.normal(0, spread, (N, P, classes)).astype(np.float32)
+    conf[:, 5::41, 1] = np.inf
+    conf[:, 6::41, 0] = np.nan
+    conf[:, 7::41, classes - 1] = np.nan
+    conf[:, 8::41] = -np.inf
+    _compare(q8, g.normal(0, 0.3, (N, P, 4)).astype(np.float32), conf, priors, [P], [1], background=g.integers(-1, classes - 1).item(),
+             conf_thresh=thresh, nms_thresh=0.45, nms_top_k=60, keep_top_k=50)
+
+
 def test_detection_output_takes_what_converts(q8):
     """Box counts that int() takes, variances that float() takes, fewer than four of them (the others are zero); too many
     sources, and more boxes than fit, are the library's errors; with scratch and outputs given or not."""
