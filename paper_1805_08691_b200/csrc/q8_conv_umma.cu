@@ -144,10 +144,10 @@ template <>
 struct RowMaps<true> { CUtensorMap res, y; };
 constexpr int kFillWarp = kCtrlWarps, kStoreWarp = kCtrlWarps + 1;
 template <bool kBufs>
-__device__ __forceinline__ void prefetch_maps(const RowMaps<kBufs>& maps, bool residual) {
+__device__ __forceinline__ void prefetch_maps(const RowMaps<kBufs>& maps, bool residual, bool out8) {
   if constexpr (kBufs) {
     if (residual) prefetch_tensormap(&maps.res);
-    prefetch_tensormap(&maps.y);
+    if (out8) prefetch_tensormap(&maps.y);
   }
 }
 
@@ -155,7 +155,7 @@ template <int G, int kOut, int kRes, bool kCta2, bool kUniform>
 __global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
     conv_umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ UmmaParams p, const __grid_constant__ RowMaps<kRes == kResTma> maps) {
-  constexpr bool kBufs = kRes == kResTma;
+  constexpr bool kBufs = kRes == kResTma, k8 = kOut == Q8_U8 || kOut == Q8_S8;
   constexpr int kCtrl = kCtrlOf<kRes>, kCtrlT = kCtrl * 32;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long a_full[kMaxStages], a_empty[kMaxStages];
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (kBufs && warp == kFillWarp) {
       if (lane < slots) { mbar_init(smem_u32(&buf_full[lane]), 1); mbar_init(smem_u32(&buf_empty[lane]), 1); }
-      else if (lane == 16) prefetch_maps(maps, p.res_mode != kResNone);
+      else if (lane == 16) prefetch_maps(maps, p.res_mode != kResNone, k8);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (kBufs && warp == kStoreWarp) {
       if (lane < slots) mbar_init(smem_u32(&store_ready[lane]), kCta2 ? kGroupThreads << p.pair_shift : kGroupThreads);
@@ -468,7 +468,9 @@ __global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
       const uint32_t panel_bytes = (uint32_t)kBM << p.pw_shift;
       for (; ti.tile < total_tiles; ti.next(p)) {
         if (!mbar_wait(ready0 + slot * 8u, spar, abortp)) { ok = false; break; }
-        if (elect_one()) {
+        if (!k8) {
+          if (elect_one()) mbar_arrive(bempty0 + slot * 8u);  // (32-bit rows are stored by the epilogue: the residual has been read)
+        } else if (elect_one()) {
           uint32_t src = base + p.off_bufs + slot * p.tile8_bytes;
           if (!ti.valid) {
             // second tile of the last pair of an odd count: nothing to store
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
         }
         if (++slot == nslots) { slot = 0; spar ^= 1u; }
       }
-      if (elect_one()) {
+      if (k8 && elect_one()) {
         bulk_wait_read<0>();  // the CTA's shared memory must outlive the reads of its last stores
         if (prev_slot >= 0 && !one_each) mbar_arrive(bempty0 + (uint32_t)prev_slot * 8u);
       }
@@ -588,9 +590,9 @@ __global__ void __launch_bounds__(kCtrlOf<kRes> * 32 + G * kGroupThreads, 1)
       }
       tcgen05_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * (uint32_t)p.acc_stride;
-      epilogue_row<kOut, kRes, kCta2, kUniform, kBufs || kRes == kResRows>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1, rp);
+      epilogue_row<kOut, kRes, kCta2, kUniform, (kBufs && k8) || kRes == kResRows>(p, t, taddr, acce0 + ab * 8u, lane, ch0, ch1, rp);
       if constexpr (kBufs) {
-        fence_proxy_async_smem();  // this thread's reads and writes of the buffer are done; the store reads it
+        if (k8) fence_proxy_async_smem();  // this thread's reads and writes of the buffer are done; the store reads it
         mbar_arrive(smem_u32(&store_ready[0]) + slot * 8u);
         slot += (uint32_t)tile_step;
         if (slot >= (uint32_t)slots) { slot -= (uint32_t)slots; slot_par ^= 1u; }
@@ -688,6 +690,7 @@ int launch_groups(const CUtensorMap& tmA, const CUtensorMap& tmB, const RowMaps<
   }
   if (p.y_type == Q8_F32) {
     if (global_res) Q8_LAUNCH(Q8_F32, kResGlobal);
+    if (p.nbuf) Q8_LAUNCH(Q8_F32, kResTma);
     Q8_LAUNCH(Q8_F32, kResVec);
   }
   return launch_variant<G, Q8_S32, kResVec, false, false>(tmA, tmB, maps, p, dyn, grid, stream);
@@ -873,13 +876,18 @@ namespace {
 //     costs more than it gives (402 -> 410 us; batch 32 501 -> 508).  The other lines lie where the networks gain or stay: SSD-300
 //     at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64
 //     (matrices without a residual, taken from 12 tiles a CTA, still cost ResNet-50 at batch 40 551 -> 554 us).
+// 32-bit outputs are stored by the epilogue; a residual of theirs (8-bit) comes through buffers already from one tile a CTA, in
+// groups of their own: 408 layers 3.6 % faster in the mean, 1x1 256->512 at 112x112, batch 4 51.8 -> 46.5 us, 3x3 256->512 at 56x56,
+// batch 16 73.7 -> 64.4.
 // Over 2131 layers the rule is on average 3.0 % below no buffers at all (34 % at best).
 bool buffered(const ConvArgs& a, const UmmaParams& p, bool two) {
   const bool residual = a.residual != nullptr, plain = p.a_mode == kAPlain, wide = a.ldc % 32 == 0 && a.c_off % 32 == 0;
   const int reduction = a.d.R * a.d.S * a.d.C, ctas = p.cta2 ? sm_count() / 2 : sm_count();
   const long long items = (long long)p.m_tiles * p.n_tiles;
   auto more_than = [&](int per_cta) { return items > (long long)per_cta * ctas; };
-  if (p.splits > 1 || p.epi_split) return false;
+  if (p.splits > 1) return false;
+  if (a.d.y_type == Q8_F32) return p.bn > 64 ? more_than(1) : (p.bn == 64 && more_than(8));
+  if (p.epi_split) return false;
   const bool broad = p.bn > 128 && p.bn < 256;
   if (p.bn < 64 || reduction > (residual || broad ? 1152 : 864)) return false;
   if (residual) return more_than(plain || p.n_tiles > 1 || p.bn > 128 ? 4 : 8);
@@ -1031,7 +1039,11 @@ bool plan_tiles(const ConvArgs& a, int splits, int bk_cap, bool allow_halo, bool
       p.b_sub_bytes = round_up(p.b_tile_bytes, 1024u);
     }
   }
-  const bool use_bufs = allow_bufs && out8 && !rows && tune_env("Q8_BUFS", buffered(a, p, true) || buffered(a, p, false), 0, 1);
+  const bool use_bufs = allow_bufs && (out8 ? !rows : d.y_type == Q8_F32 && res_mode == kResVec) && tune_env("Q8_BUFS", buffered(a, p, true) || buffered(a, p, false), 0, 1);
+  if (use_bufs && p.epi_split) {
+    p.epi_split = 0;
+    if (BN > 128 || G > p.nacc) G = 2;
+  }
   const unsigned teams = (unsigned)(p.cta2 ? G >> p.pair_shift : G);
   const unsigned row_bytes = rows ? (unsigned)(p.epi_split ? 1 : G) * p.tile8_bytes : 0u;
   p.b_T = 1;
@@ -1205,8 +1217,10 @@ int launch_planned(const ConvArgs& a, int splits) {
       cr = encode_rows(&maps.res, const_cast<void*>(a.residual), d.K, d.K, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
       if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: residual tensor map rejected (CUresult %d)", (int)cr);
     }
-    cr = encode_rows(&maps.y, a.y, a.c_off + d.K, a.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
-    if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: output tensor map rejected (CUresult %d)", (int)cr);
+    if (out8) {
+      cr = encode_rows(&maps.y, a.y, a.c_off + d.K, a.ldc, CU_TENSOR_MAP_L2_PROMOTION_NONE);
+      if (cr != CUDA_SUCCESS) return fail(Q8_ERR_CUDA, "conv_umma: output tensor map rejected (CUresult %d)", (int)cr);
+    }
     p.res_tx_bytes = (unsigned)BN * (p.a_mode == kAHalo ? (unsigned)(ht.tw * ht.th) : (unsigned)kBM);
   }
 

@@ -217,7 +217,14 @@ def test_layers_bound_by_their_rows_take_tile_buffers(N, HW, C, K, R, residual, 
     assert q8.q8_conv2d_query_row_buffers(d, None, residual) == buffers
     for y_type in (2, 3):   # 32-bit outputs are stored by the epilogue
         d.y_type = y_type
-        assert q8.q8_conv2d_query_row_buffers(d, None, residual and y_type == 3) == 0
+        assert q8.q8_conv2d_query_row_buffers(d, None, False) == 0
+
+
+@pytest.mark.parametrize("N,HW,C,K,R,buffers", [(1, 112, 64, 256, 1, 8), (1, 56, 64, 128, 1, 0), (16, 56, 256, 512, 3, 2), (16, 56, 64, 64, 1, 0),
+                                                (64, 56, 64, 64, 1, 8), (64, 56, 64, 32, 1, 0)], ids=str)
+def test_residuals_of_fp32_outputs_come_through_tile_buffers(N, HW, C, K, R, buffers):
+    d = q8.make_conv_desc(N, HW, HW, C, K, R, R, (1, 1), (R // 2, R // 2), y_type=q8.Q8_F32)
+    assert q8.q8_conv2d_query_row_buffers(d, None, True) == buffers
 
 
 @pytest.mark.parametrize("N,HW,C1,K1,K2,residual,buffers", [

@@ -2,7 +2,7 @@
 offsets and pointers on the 16-byte grid but off the 32-byte one, odd numbers of 16-column chunks, residual rows of another
 alignment than the output's, one tile and several per CTA, CTA pairs.  Through tile buffers (long launches with wide tiles and
 short reductions): every operand path, one and two buffers a group, ragged tiles of rows and of columns, channel
-slices, with and without a residual.  Bytes beside the rows stay as they are."""
+slices, with and without a residual; residuals of fp32 outputs.  Bytes beside the rows stay as they are."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +10,7 @@ import torch
 import oracle as o
 
 pytestmark = pytest.mark.gpu
-U8, S8 = 0, 1
+U8, S8, F32 = 0, 1, 3
 
 CASES = [
     # name, N,H,W,C,K,R,pad, y type, residual, pitch - K, channel offset, output shift, residual shift (bytes)
@@ -73,6 +73,11 @@ BUFFERED = [
     ("im2col", 30, 75, 75, 32, 256, 3, 2, 0, U8, "s8", False, 0, 0, 128, 0, 4),
     ("pairs_odd_tiles", 23, 37, 41, 64, 256, 3, 1, 1, U8, "u8", True, 16, 16, 128, 1, 4),
     ("pairs_no_residual", 70, 37, 41, 64, 256, 3, 1, 1, S8, None, False, 0, 0, 128, 1, 4),
+    ("matrix_f32", 12, 57, 57, 64, 256, 1, 1, 0, F32, "u8", False, 8, 4, 128, 0, 8),
+    ("matrix_f32_two_tiles", 4, 57, 57, 64, 256, 1, 1, 0, F32, "s8", True, 0, 0, 128, 0, 8),
+    ("matrix_f32_64_columns", 60, 57, 57, 32, 64, 1, 1, 0, F32, "u8", True, 0, 0, 64, 0, 8),
+    ("halo_f32_ragged_edges", 22, 37, 41, 32, 192, 3, 1, 1, F32, "s8", True, 4, 0, 96, 0, 8),
+    ("halo_f32_256_columns", 25, 28, 28, 128, 256, 3, 1, 1, F32, "u8", False, 0, 0, 256, 0, 2),
     ("pairs_shared_groups", 47, 37, 41, 128, 160, 3, 1, 1, S8, "s8", False, 0, 0, 160, 1, 2),
 ]
 
@@ -93,7 +98,7 @@ def test_rows_through_tile_buffers_match_oracle(q8, case):
     acc = o.conv_acc(x, w, bias, (st, st), (pad, pad), (1, 1), threads=8)
     resid = None if res is None else g.integers(0, 256, acc.shape, dtype=np.uint8).view(np.int8 if res == "s8" else np.uint8)
     scale = (g.uniform(0.5, 1.5, K if per_channel else 1) * 100.0 / max(1, np.abs(acc).max())).astype(np.float32)
-    want = o.epilogue(acc, scale if per_channel else scale[0], resid, 0.37, ytype == U8, o.U8 if ytype == U8 else o.S8)
+    want = o.epilogue(acc, scale if per_channel else scale[0], resid, 0.37, ytype == U8, {U8: o.U8, S8: o.S8, F32: o.F32}[ytype])
     args = [torch.from_numpy(a).cuda() for a in (x, w, bias, scale)]
     rd = None if resid is None else torch.from_numpy(resid).cuda()
     y = torch.full((*acc.shape[:3], ldc), 7, dtype=q8.TORCH_DTYPES[ytype], device="cuda")
@@ -101,5 +106,5 @@ def test_rows_through_tile_buffers_match_oracle(q8, case):
         q8.q8_conv2d(d, *args, rd, 0.37 if res else 0.0, y)
     q8.q8_read_status()
     got = y.cpu().numpy()
-    assert np.array_equal(got[..., c_off:c_off + K], want)
+    assert np.ascontiguousarray(got[..., c_off:c_off + K]).tobytes() == want.tobytes()
     assert (got[..., :c_off] == 7).all() and (got[..., c_off + K:] == 7).all()
