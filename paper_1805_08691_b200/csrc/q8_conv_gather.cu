@@ -17,10 +17,10 @@
 // activations.  All waits are bounded as in the other tensor-core kernels.
 //
 // Bound by the instructions of its warps (3x3/2 of 3 -> 32 channels: 5560 per tile of 128 pixels over all roles, issue slots
-// 58 % busy, tensor pipe 1 %, nothing else near a limit; profiles/conv_gather_first_layer.md), hence no division
-// per chunk, rows per thread fixed at compile time and branch-free loads.  Measured against the CUDA-core kernel:
-// 3x3/2 of 3 -> 32 channels on 8 x 299x299 157.7 -> 12.2 us, 7x7/2 of 3 -> 64 on 224x224 134 -> 7.7 us,
-// 3x3 of 100 -> 120 on 8 x 28x28 963 -> 26 us, 1x1 of 200 -> 500 at 14x14 32.8 -> 10.2 us.
+// 58 % busy, tensor pipe 1 %, nothing else near a limit), hence no division per chunk, rows per thread fixed at compile time
+// and branch-free loads.  Measured against the CUDA-core kernel: 3x3/2 of 3 -> 32 channels on 8 x 299x299 157.7 ->
+// 12.2 us, 7x7/2 of 3 -> 64 on 224x224 134 -> 7.7 us, 3x3 of 100 -> 120 on 8 x 28x28 963 -> 26 us, 1x1 of 200 -> 500 at 14x14
+// 32.8 -> 10.2 us.
 #include "q8_umma_common.cuh"
 
 namespace q8 {

@@ -864,22 +864,22 @@ namespace {
 // of the rows; with them the copy engine moves whole lines, at the price of two more hand-offs at the end of a CTA and of
 // shared memory.  So buffers are for CTAs with many tiles, wide ones and short reductions, where rows and not operands are
 // the launch, more so with a residual, whose bytes count again.  Inputs not in L2, buffers against none (us):
-//   1x1 64->256 at 56x56 with a residual: batch 8 (2.6 tiles a CTA) 8.1 / 7.9, 16 (5.3) 10.9 / 12.9, 32 16.0 / 21.3, 64 25.9 / 39.4;
-//     without one: batch 16 8.4 / 8.4, 32 11.5 / 12.0, 64 18.1 / 20.3; 32 columns never gain (32->32 at 112x112, batch 64 24.7 /
-//     22.6; 256->32 at 56x56 with a residual 14.2 / 13.5);
+//   1x1 64->256 at 56x56 with a residual: batch 8 (2.6 tiles a CTA) 8.1 / 7.9, 16 (5.3) 10.9 / 12.9, 32 16.0 / 21.3, 64 25.9 /
+//     39.4; without one: batch 16 8.4 / 8.4, 32 11.5 / 12.0, 64 18.1 / 20.3; 32 columns never gain (32->32 at 112x112, batch 64
+//     24.7 / 22.6; 256->32 at 56x56 with a residual 14.2 / 13.5);
 //   room for one buffer per group only: 1x1 256->256 at 56x56, batch 64 27.4 / 23.0 (too few operand stages are left), with a
 //     residual 31.7 / 43.4; 128->512 at 28x28 with one 19.2 / 21.4, without 12.6 / 12.6;
-//   halo tiles: 3x3 64->64 at 56x56, batch 64 12.3 / 13.3, batch 32 9.1 / 8.7; 32->96 at 112x112 with a residual, batch 8 (6 tiles a
-//     CTA) 12.3 / 11.1, 64 46.3 / 55.7; pairs at 75x75, batch 32 128->192 32.2 / 34.5, 128->256 40.1 / 38.9;
-//   tiles shared by all groups: 1x1 128->512 at 28x28, batch 8 with a residual 6.3 / 7.1, without 5.5 / 5.6.  They take none all
-//     the same: a launch of another kernel function than the one before it starts slower, and in ResNet-50 at batch 16 that
-//     costs more than it gives (402 -> 410 us; batch 32 501 -> 508).  The other lines lie where the networks gain or stay: SSD-300
-//     at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64
-//     (matrices without a residual, taken from 12 tiles a CTA, still cost ResNet-50 at batch 40 551 -> 554 us).
+//   halo tiles: 3x3 64->64 at 56x56, batch 64 12.3 / 13.3, batch 32 9.1 / 8.7; 32->96 at 112x112 with a residual, batch 8 (6
+//     tiles a CTA) 12.3 / 11.1, 64 46.3 / 55.7; pairs at 75x75, batch 32 128->192 32.2 / 34.5, 128->256 40.1 / 38.9;
+//   tiles shared by all groups: 1x1 128->512 at 28x28, batch 8 with a residual 6.3 / 7.1, without 5.5 / 5.6.
+// Shared tiles take none all the same: a launch of another kernel function than the one before it starts slower, and in
+// ResNet-50 at batch 16 that costs more than it gives (402 -> 410 us; batch 32 501 -> 508).  The other lines lie where the
+// networks gain or stay: SSD-300 at batch 32 1095 -> 1076 us, ResNet-50 and Inception-v3 within 0.3 % from batch 8 to 64
+// (matrices without a residual, taken from 12 tiles a CTA, still cost ResNet-50 at batch 40 551 -> 554 us).
 // 32-bit outputs are stored by the epilogue; a residual of theirs (8-bit) comes through buffers already from one tile a CTA, in
-// groups of their own: 408 layers 3.6 % faster in the mean, 1x1 256->512 at 112x112, batch 4 51.8 -> 46.5 us, 3x3 256->512 at 56x56,
-// batch 16 73.7 -> 64.4.
-// Over 2131 layers the rule is on average 3.0 % below no buffers at all (34 % at best).
+// groups of their own: 408 layers 3.6 % faster in the mean, 1x1 256->512 at 112x112, batch 4 51.8 -> 46.5 us, 3x3 256->512 at
+// 56x56, batch 16 73.7 -> 64.4.
+// Over 2131 layers with 8-bit outputs the rule is on average 3.0 % below no buffers at all (34 % at best).
 bool buffered(const ConvArgs& a, const UmmaParams& p, bool two) {
   const bool residual = a.residual != nullptr, plain = p.a_mode == kAPlain, wide = a.ldc % 32 == 0 && a.c_off % 32 == 0;
   const int reduction = a.d.R * a.d.S * a.d.C, ctas = p.cta2 ? sm_count() / 2 : sm_count();

@@ -224,15 +224,15 @@ __device__ __forceinline__ float4 det_box(const float* l, const float4 pr, float
 constexpr int kDecThreads = 256;
 constexpr int kDecFew = 64;  // boxes of a block where there are few
 
-// Up to kRegClasses classes.  A block takes kBoxes boxes of an image (256, or 64 where there are few), whose logits travel through shared memory (a thread per
-// box would touch 21 lines with every load).  Most boxes of a detector are background and need no exponential: the largest
-// term of the sum is exp(0) = 1, so p_c <= e_c, and a box whose foreground logits all lie `cutoff` = ln(conf_thresh), less a
-// margin for the recipe's roundings, or more below its largest has no candidate.  What is left (one box in six at a
-// threshold of 0.01) is listed, and the block's threads share its (box, class) pairs.  A NaN among a
-// box's logits makes its sum a NaN, so no class of it passes, whether the maxima (which skip a NaN) list it or not; infinities of
-// one sign compare by a NaN difference, which lists.  One box per thread with all of its exponentials was bound by issue (1291 warp instructions per 32 boxes,
-// 790 with a list but loads through registers, five blocks per SM): detection output of 32 images, 8732 boxes, 21 classes,
-// replayed from a graph 45.8 -> 39.8 -> 36.7 us with eight resident blocks.
+// Up to kRegClasses classes.  A block takes kBoxes boxes of an image (256, or 64 where there are few), whose logits travel
+// through shared memory (a thread per box would touch 21 lines with every load).  Most boxes of a detector are background and
+// need no exponential: the largest term of the sum is exp(0) = 1, so p_c <= e_c, and a box whose foreground logits all lie
+// `cutoff` = ln(conf_thresh), less a margin for the recipe's roundings, or more below its largest has no candidate.  What is
+// left (one box in six at a threshold of 0.01) is listed, and the block's threads share its (box, class) pairs.  A NaN among a
+// box's logits makes its sum a NaN, so no class of it passes, whether the maxima (which skip a NaN) list it or not; infinities
+// of one sign compare by a NaN difference, which lists.  One box per thread with all of its exponentials was bound by issue
+// (1291 warp instructions per 32 boxes, 790 with a list but loads through registers, five blocks per SM): detection output of
+// 32 images, 8732 boxes, 21 classes, replayed from a graph 45.8 -> 39.8 -> 36.7 us with eight resident blocks.
 template <int kBoxes>
 __global__ void __launch_bounds__(kDecThreads, 8) decode_listed_kernel(const __grid_constant__ DetSources src, const float4* __restrict__ priors,
                                                                        float v0, float v1, float v2, float v3, int P, int classes,

@@ -595,8 +595,8 @@ __device__ __forceinline__ uint4 epilogue_chunk(const UmmaParams& p, const EpiTi
       const unsigned int w = rw[j >> 1] ^ sign_mask;
       const float r0 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u | (unsigned)((2 * j) & 3)));
       const float r1 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u | (unsigned)((2 * j + 1) & 3)));
-      // the sum stays scalar: the assembler contracts a packed multiply followed by a packed add into one
-      // fused operation (one rounding instead of two), which would break the two-rounding definition
+      // the sum stays scalar: with a packed multiply followed by a packed add a bit-exact test saw one rounding instead of
+      // two, as of a fused operation, which would break the two-rounding definition
       float t0, t1;
       unpack_f2(fmul2(fsub2(pack_f2(r0, r1), magic2), rs2), t0, t1);
       v[2 * j] = __fadd_rn(v[2 * j], t0);
