@@ -296,3 +296,17 @@ def test_long_layers_with_ragged_32_bit_rows_are_gathered(y_type, N, K, operand)
     assert q8.q8_conv2d_query_plan(d).operand == operand
     d.N, d.H = 1, 200   # 3.0 tiles a block
     assert q8.q8_conv2d_query_plan(d).operand == 3
+
+
+def test_row_buffer_query_checks_what_it_is_given():
+    d1 = q8.make_conv_desc(64, 56, 56, 64, 64, 3, 3, pad=(1, 1), relu=True)
+    d2 = q8.make_conv_desc(64, 56, 56, 64, 256, 1, 1, relu=True)
+    n = C.c_int(-1)
+    assert q8.lib.q8_conv2d_query_row_buffers(C.byref(d1), None, 0, None) == 1
+    assert q8.lib.q8_conv2d_query_row_buffers(None, None, 0, C.byref(n)) == 1 and n.value == -1
+    bad = q8.make_conv_desc(64, 56, 56, 64, 0, 1, 1)
+    assert _code(q8.q8_conv2d_query_row_buffers, bad) == 1 and _code(q8.q8_conv2d_query_row_buffers, d1, bad) == 1
+    d1.K = d2.C = 256   # a pair that does not run as one launch
+    assert q8.q8_conv2d_query_row_buffers(d1, d2, True) == 0
+    d2.algo = q8.Q8_ALGO_DIRECT
+    assert q8.q8_conv2d_query_row_buffers(d2, None, True) == 0
